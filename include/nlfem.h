@@ -120,7 +120,9 @@ typedef struct {
     int32_t *col_idx;               /* [nnz] */
     double *val;                    /* [nnz] */
     int64_t n_pairs;                /* element pairs (T_a, T_b) with a non-empty region for some outer point */
-    int64_t n_qp_pairs;             /* (outer point, inner point) evaluations performed */
+    int64_t n_qp_pairs;             /* (outer point, inner point) pairs of the quadrature sums (the constant kernel
+                                       takes a region's inner sum from its moments, which the inner rules integrate
+                                       exactly, not point by point) */
     int64_t n_inter;                /* (T_a, q, T_b) triples with a non-empty region */
     void *priv;                     /* library state (pattern, candidate lists); do not touch */
 } nl_csr;

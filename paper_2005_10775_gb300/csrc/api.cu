@@ -186,13 +186,12 @@ nl_status nl_validate(nl_ctx *ctx, const nl_mesh *m, const nl_config *c)
 // Bound on the sum over all T_b of s0(x, T_b) = int_{region(x) cap T_b} gamma(x, y) dy at any
 // outer point x: every region of x lies in B(x, delta + h_max) (the shifted, barycenter and
 // overlap balls included), so the sum is at most kc pi (delta + h_max)^2 for a constant kernel
-// and c 2 pi (delta + h_max) for c / |x - y| (the integral of 1/r over the disc); here with a
+// (returned without kc: the constant kernel's sums are areas) and c 2 pi (delta + h_max) for c / |x - y| (the integral of 1/r over the disc); here with a
 // margin of 1.25 (twice that for the singular kernel's quadrature).
 static double s0_sum_bound(const nl_config &c, double hmax)
 {
     const double r = c.delta + hmax, pi = 3.14159265358979323846;
-    return c.kernel == NL_KERNEL_INV_DIST ? 2.5 * fabs(c.kernel_c) * 2.0 * pi * r
-                                          : 1.25 * fabs(c.kernel_c) * pi * r * r;
+    return c.kernel == NL_KERNEL_INV_DIST ? 2.5 * fabs(c.kernel_c) * 2.0 * pi * r : 1.25 * pi * r * r;
 }
 
 static double abs_weight_sum(int rule)
@@ -211,6 +210,25 @@ float nl_outer_abs_weight(const nl_plan *P)
     if (P->cfg.outer == NL_RULE_SWITCH47)
         return (float)fmax(abs_weight_sum(NL_RULE_GAUSS4), abs_weight_sum(NL_RULE_PAPER7));
     return (float)abs_weight_sum(P->cfg.outer);
+}
+
+// are the polygon's vertices R (cos 2 pi k / N, sin 2 pi k / N)?
+static bool ngon_regular(const nl_plan *P)
+{
+    const int N = P->cfg.ngon_n;
+    const double *o = P->ngon_host.data();
+    const double R = sqrt(o[0] * o[0] + o[1] * o[1]);
+    bool reg = R > 0.0;
+    for (int k = 0; k < N && reg; k++) {
+        const double th = 2.0 * M_PI * k / N;
+        reg = fabs(o[2 * k] - R * cos(th)) <= 1e-12 * R && fabs(o[2 * k + 1] - R * sin(th)) <= 1e-12 * R;
+    }
+    return reg;
+}
+
+int nl_const_ball(const nl_plan *P)
+{
+    return P->cfg.ball == NL_BALL_NGON && !ngon_regular(P) ? nlq::kBallNgonAny : P->cfg.ball;
 }
 
 nl_status nl_fill_args(nl_ctx *ctx, const nl_plan *P, nlq::NumArgs &A, bool stats)
@@ -266,12 +284,16 @@ nl_status nl_fill_args(nl_ctx *ctx, const nl_plan *P, nlq::NumArgs &A, bool stat
     A.kc = c.kernel_c;
     A.kcf = (float)c.kernel_c;
     {
-        // grid of the boundary kernel's fixed-point sums of s0 per outer point: the bound,
-        // rounded up to a power of two 2^e, maps to 2^30
+        // grid of the fixed-point sums of s0 per outer point (constant kernel: of the regions' areas):
+        // the bound, rounded up to a power of two 2^e, maps to 2^30
         const double bound = s0_sum_bound(c, P->hmax);
         int e = 0;
         frexp(bound > 1e-30 ? bound : 1e-30, &e);   // bound < 2^e
         A.s0q_grid = (float)ldexp(1.0, 30 - e);
+        // FP64 sums of areas: 2^50 on a power of two above the largest area a triangle of
+        // barycentre radius r_max can have (27/8 of the equilateral one's r^2 is above 3 sqrt(3)/4)
+        frexp(4.0 * P->rmax * P->rmax, &e);
+        A.area_grid = ldexp(1.0, 50 - e);
     }
     A.geo.delta = c.delta;
     A.geo.deltaf = (float)c.delta;
@@ -308,16 +330,14 @@ nl_status nl_fill_args(nl_ctx *ctx, const nl_plan *P, nlq::NumArgs &A, bool stat
     A.geo.tau = (float)tau;
     A.geo.inv_tau = (float)(1.0 / tau);
     if (c.ball == NL_BALL_NGON) {
-        // regular polygon R (cos 2 pi k / N, sin 2 pi k / N)?  (enables the angular pass window)
         const int N = c.ngon_n;
         const double *o = P->ngon_host.data();
+        A.geo.regular = ngon_regular(P) ? 1 : 0;   // enables the angular pass window and k_const's walk
         const double R = sqrt(o[0] * o[0] + o[1] * o[1]);
-        bool reg = R > 0.0;
-        for (int k = 0; k < N && reg; k++) {
-            const double th = 2.0 * M_PI * k / N;
-            reg = fabs(o[2 * k] - R * cos(th)) <= 1e-12 * R && fabs(o[2 * k + 1] - R * sin(th)) <= 1e-12 * R;
-        }
-        A.geo.regular = reg ? 1 : 0;
+        A.geo.poly_r2 = (float)(R * R);
+        A.geo.poly_side = (float)(2.0 * R * sin(M_PI / N));
+        A.geo.poly_m = (float)(2.0 * R * sin(M_PI / N) * tau);
+        A.geo.inv_sector = (float)(N / (2.0 * M_PI));
         double m1 = 0.0;
         for (int k = 0; k < N; k++) m1 = fmax(m1, fabs(o[2 * k]) + fabs(o[2 * k + 1]));
         A.geo.r2 = (float)(2.0 * m1);
@@ -382,7 +402,8 @@ nl_status run_numeric(nl_ctx *ctx, nl_plan *P, bool stats, bool one_stream = fal
     nlq::NumArgs A;
     nl_status s = nl_fill_args(ctx, P, A, stats);
     if (s != NL_OK) return s;
-    if (P->cfg.prec == NL_PREC_FP64) return nl_launch_numeric_f64(ctx, A, P->cfg.ball, one_stream);
+    const int ball = P->cfg.kernel == NL_KERNEL_CONST ? nl_const_ball(P) : P->cfg.ball;
+    if (P->cfg.prec == NL_PREC_FP64) return nl_launch_numeric_f64(ctx, A, ball, one_stream);
     if (!P->defer) {
         const int cap = nl_defer_cap(P->E) > P->defer_min ? nl_defer_cap(P->E) : P->defer_min;
         nlq::DeferItem *q = nullptr;
@@ -414,7 +435,7 @@ nl_status run_numeric(nl_ctx *ctx, nl_plan *P, bool stats, bool one_stream = fal
             A.otab = (nlq::OuterPt *)P->otab;
         }
     }
-    return nl_launch_numeric_f32(ctx, A, P->cfg.ball, one_stream);
+    return nl_launch_numeric_f32(ctx, A, ball, one_stream);
 }
 
 }  // namespace

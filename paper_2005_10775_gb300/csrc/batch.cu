@@ -308,7 +308,7 @@ nl_status launch_numeric(nl_ctx *ctx, nl_batch *b, bool set_attr)
                       : nl_launch_boundary_batch_f32(ctx, l.ball, l.inv, g.dA, l.items, l.n_items, c, l.blocks,
                                                      set_attr);
         if (s == NL_OK && l.defer)
-            s = nl_launch_deferred_batch_f32(ctx, l.ball, g.dA, l.defer, b->counters + nl + k, l.defer_cap);
+            s = nl_launch_deferred_batch_f32(ctx, l.ball, l.inv, g.dA, l.defer, b->counters + nl + k, l.defer_cap);
         if (s != NL_OK) return s;
     }
     return NL_OK;
@@ -709,11 +709,13 @@ nl_status nl_batch_create(nl_ctx *ctx, int32_t n, const nl_mesh *meshes, const n
         const int pg = (int)b->pgroups.size() - 1;
         Launch li;
         li.prec = pg;
-        li.probs = g.probs;
+        // the constant kernel's launches do their interior candidates too
+        for (int i : g.probs)
+            if (b->P[i]->cfg.kernel == NL_KERNEL_INV_DIST) li.probs.push_back(i);
         b->launches.push_back(li);
         for (int i : g.probs) {
-            const int ball = b->P[i]->cfg.ball;
             const bool inv = b->P[i]->cfg.kernel == NL_KERNEL_INV_DIST;
+            const int ball = inv ? b->P[i]->cfg.ball : nl_const_ball(b->P[i]);
             Launch *l = nullptr;
             for (Launch &x : b->launches)
                 if (x.prec == pg && x.ball == ball && x.inv == inv) l = &x;
@@ -826,6 +828,8 @@ nl_status nl_batch_create(nl_ctx *ctx, int32_t n, const nl_mesh *meshes, const n
             a.tslot = P->tslot;
             a.val = outs[i].val;
             a.err = P->err;
+            a.split = P->cfg.kernel == NL_KERNEL_CONST ? P->nbr_split : nullptr;
+            a.kc = P->cfg.kernel_c;
             a.area = P->area;
             a.fxe = P->fxe;
             a.ws = nl_outer_abs_weight(P);

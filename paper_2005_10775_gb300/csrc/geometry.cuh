@@ -68,6 +68,8 @@ struct GeoParams {
     float r2;             // 2 max_k |o_k|_1
     float o1max;          // max_k |o_k|_1
     float sector, rin_tau; // 2 pi / N; inradius - tau
+    float inv_sector;      // N / 2 pi
+    float poly_r2, poly_side, poly_m;   // regular polygon: circumradius^2, edge length, its orientation margin
     float deltaf;          // delta in FP32
 };
 
@@ -464,34 +466,19 @@ __device__ __forceinline__ float dist2_origin_triangle(const F2 d[3])
 
 // rin: radius of the disc that lies inside the kept region for sure (delta, or the
 // polygon's inradius); rout: radius of a disc containing it (delta)
-// The triangle with vertices d (relative to the origin, every vertex farther than sqrt(r2))
-// lies farther than sqrt(r2) from the origin: the origin is outside it and no edge comes closer.
-// An edge p -> q whose closest point is interior (0 < n = -p.e < e.e) is at squared distance
-// |p|^2 - n^2 / e.e; the test multiplies through by e.e (no division).
-__device__ __forceinline__ bool triangle_beyond(const F2 d[3], float r2)
-{
-    const float o0 = d[0].x * d[1].y - d[0].y * d[1].x;
-    const float o1 = d[1].x * d[2].y - d[1].y * d[2].x;
-    const float o2 = d[2].x * d[0].y - d[2].y * d[0].x;
-    if (o0 >= 0.f && o1 >= 0.f && o2 >= 0.f) return false;
-#pragma unroll
-    for (int i = 0; i < 3; i++) {
-        const F2 p = d[i], q = d[(i + 1) % 3];
-        const float ex = q.x - p.x, ey = q.y - p.y;
-        const float n = -(p.x * ex + p.y * ey), ee = ex * ex + ey * ey;
-        if (n > 0.f && n < ee && (p.x * p.x + p.y * p.y) * ee - n * n <= r2 * ee) return false;
-    }
-    return true;
-}
-
+// The empty test asks whether the triangle lies beyond the tangent at the disc's point in the
+// direction of the triangle's barycentre (m_i = d_i . c, c the sum of the vertices: every m_i >
+// sqrt(rout_p2) |c|).  It misses 1 % of the triangles that lie outside the disc (they come out as
+// regions without a crossing), takes no branch and half the instructions of the edges' distances.
 __device__ __forceinline__ int classify_vertices(const F2 d[3], float rin_m2, float rout_p2)
 {
-    float r0 = d[0].x * d[0].x + d[0].y * d[0].y;
-    float r1 = d[1].x * d[1].x + d[1].y * d[1].y;
-    float r2 = d[2].x * d[2].x + d[2].y * d[2].y;
-    if (fmaxf(r0, fmaxf(r1, r2)) <= rin_m2) return CLS_WHOLE;
-    if (fminf(r0, fminf(r1, r2)) > rout_p2 && triangle_beyond(d, rout_p2)) return CLS_EMPTY;
-    return CLS_EXACT;
+    const float r0 = d[0].x * d[0].x + d[0].y * d[0].y;
+    const float r1 = d[1].x * d[1].x + d[1].y * d[1].y;
+    const float r2 = d[2].x * d[2].x + d[2].y * d[2].y;
+    const float cx = d[0].x + d[1].x + d[2].x, cy = d[0].y + d[1].y + d[2].y;
+    const float m = fminf(d[0].x * cx + d[0].y * cy, fminf(d[1].x * cx + d[1].y * cy, d[2].x * cx + d[2].y * cy));
+    const bool out = m > 0.f && m * m > rout_p2 * (cx * cx + cy * cy);
+    return fmaxf(r0, fmaxf(r1, r2)) <= rin_m2 ? CLS_WHOLE : out ? CLS_EMPTY : CLS_EXACT;
 }
 
 // ---------------------------------------------------------------------------
@@ -763,6 +750,36 @@ __device__ __forceinline__ int ball_region_f32(const F2 d[3], const GeoParams &g
     return m;
 }
 
+// cap_rule in FP32: centroid (cx, cy) and area of the cap over the chord e f, relative to x
+__device__ __forceinline__ void cap_rule_f32(const F2 &e, const F2 &f, const GeoParams &g, float *cx, float *cy,
+                                             float *area)
+{
+    const float delta = g.deltaf;
+    const float ux = f.x - e.x, uy = f.y - e.y;
+    const float chord = sqrtf(ux * ux + uy * uy);
+    const float th = asinf(fminf(chord / (2.f * delta), 1.f));
+    const float u = 2.f * th;
+    float tms;   // 2 th - sin 2 th
+    if (u < 0.5f) {
+        const float u2 = u * u;
+        float term = u * u2 / 6.f, sum = 0.f;
+        for (int k = 1; k <= 6; k++) {
+            sum += term;
+            term *= -u2 / ((2.f * k + 2.f) * (2.f * k + 3.f));
+        }
+        tms = sum;
+    } else {
+        tms = u - sinf(u);
+    }
+    const float st = sinf(th);
+    const float dc = tms > 0.f ? 4.f * delta * st * st * st / (3.f * tms) : delta;
+    const float mx = 0.5f * (e.x + f.x), my = 0.5f * (e.y + f.y);
+    const float im = rsqrtf(mx * mx + my * my);
+    *cx = dc * mx * im;
+    *cy = dc * my * im;
+    *area = delta * delta * tms / (g.cap_printed ? 4.f : 2.f);
+}
+
 // FP32 region of exactcaps (Sec. 5.2, Eq. (areacap)): the certified FP32 walk as for nocaps (a
 // polygon when it has three points or more) and one cap for every exit followed by an entry,
 // each integrated by one point at its centroid with weight its area, as the FP64 cap rule (the
@@ -781,35 +798,11 @@ __device__ __forceinline__ int exactcaps_region_f32(const F2 d[3], const GeoPara
     *ncap = 0;
     if (n < 0) return -1;
     if (n < 2) return 0;
-    const float delta = g.deltaf;
     int nc = 0;
     for (int i = 0; i < n; i++) {
         const int j = i + 1 < n ? i + 1 : 0;
         if (!(walk_tag(tags, i) == 2 && walk_tag(tags, j) == 1) || nc >= 3) continue;
-        const F2 e = {px[i], py[i]}, f = {px[j], py[j]};
-        const float cx = f.x - e.x, cy = f.y - e.y;
-        const float chord = sqrtf(cx * cx + cy * cy);
-        const float th = asinf(fminf(chord / (2.f * delta), 1.f));
-        const float u = 2.f * th;
-        float tms;   // 2 th - sin 2 th
-        if (u < 0.5f) {
-            const float u2 = u * u;
-            float term = u * u2 / 6.f, sum = 0.f;
-            for (int k = 1; k <= 6; k++) {
-                sum += term;
-                term *= -u2 / ((2.f * k + 2.f) * (2.f * k + 3.f));
-            }
-            tms = sum;
-        } else {
-            tms = u - sinf(u);
-        }
-        const float st = sinf(th);
-        const float dc = tms > 0.f ? 4.f * delta * st * st * st / (3.f * tms) : delta;
-        const float mx = 0.5f * (e.x + f.x), my = 0.5f * (e.y + f.y);
-        const float im = rsqrtf(mx * mx + my * my);
-        px[8 + nc] = dc * mx * im;
-        py[8 + nc] = dc * my * im;
-        pe[nc] = delta * delta * tms / (g.cap_printed ? 4.f : 2.f);
+        cap_rule_f32(F2{px[i], py[i]}, F2{px[j], py[j]}, g, &px[8 + nc], &py[8 + nc], &pe[nc]);
         nc++;
     }
     *ncap = nc;

@@ -97,7 +97,7 @@ struct nl_plan {
     int32_t *tri = nullptr;       // [3K]
     double *tx = nullptr, *ty = nullptr;   // [3][K] vertex coordinates per triangle
     double *bx = nullptr, *by = nullptr, *rad = nullptr, *area = nullptr;  // [K]
-    float *akc = nullptr;         // [K] |T| times the kernel constant, rounded to FP32
+    float *akc = nullptr;         // [K] FP32: |T| (constant kernel), |T| times c (singular kernel)
     float *hl = nullptr;          // [16][K] vertex coordinates and barycentre as FP32 hi + lo pairs
     double *ngon = nullptr;       // [2 ngon_n]
     std::vector<double> ngon_host; // host copy of the polygon offsets
@@ -303,7 +303,10 @@ struct ScatterArgs {   // one problem
     const int64_t *tslot;
     double *val;
     int *err;
-    const double *area;   // [K] |T_a| (the FP32 scatter's fixed-point grids)
+    const int64_t *split; // constant kernel: first boundary candidate of each triangle (null: every
+                          // pair's block is in blk)
+    double kc;            // kernel constant
+    const double *area;   // [K] |T| (the interior pairs' blocks, the FP32 scatter's fixed-point grids)
     const int *fxe;       // nl_plan::fxe
     float ws;             // nl_outer_abs_weight
 };

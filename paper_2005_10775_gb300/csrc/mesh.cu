@@ -294,7 +294,7 @@ __global__ void k_candidates(int K, Grid g, float delta, const float4 *__restric
 // interior when every point of T_b lies, with margin, inside the kept region of every outer
 // point of T_a (whole for every q):
 //   mode 0: |bary_a - bary_b| + r_a + r_b <= lim   (lim = r_in - 2 tau: disc or polygon inradius)
-//   mode 1: |bary_a - bary_b| + r_a <= lim         (barycenter ball, lim = delta - 2 tau)
+//   mode 1: |bary_a - bary_b| + max(r_a, r_b) <= lim   (barycenter ball, lim = delta - 2 tau)
 //   mode 2: no interior fast path
 //   mode 3: mode 0 and |bary_a - bary_b| - r_a - 3 r_b > far_margin (singular kernel: no near field)
 // split[a] = index of the first boundary candidate.  Candidate indices of a mesh numbered
@@ -311,7 +311,8 @@ __device__ __forceinline__ bool interior_cand(const float4 &ca, const float4 &cb
     // FP32 with lim already reduced by 1e-5 delta (far above the FP32 rounding): conservative
     const float dx = cb.x - ca.x, dy = cb.y - ca.y;
     const float D = sqrtf(dx * dx + dy * dy);
-    bool in = (mode == 1 ? D + ca.z : D + ca.z + cb.z) <= lim;
+    // the radii enter symmetrically, so (a, b) is interior exactly when (b, a) is (modes 0 and 1)
+    bool in = (mode == 1 ? D + fmaxf(ca.z, cb.z) : D + (ca.z + cb.z)) <= lim;
     // singular kernel: also far from the near field for every outer point
     // (distance >= D - r_a - r_b >= 2 r_b >= diameter of T_b)
     if (mode == 3) in = in && (D - ca.z - 3.0f * cb.z > far_margin);
@@ -542,7 +543,8 @@ nl_status nl_prepare_a(nl_ctx *ctx, const nl_mesh *mesh, const nl_config *cfg, n
     NL_CK(cudaMallocAsync((void **)&T->cf, sizeof(float4) * K, ctx->stream));
     k_prepare<<<(K + 255) / 256, 256, 0, ctx->stream>>>(K, J, (const int32_t *)T->dtri, (const double *)T->dvx,
                                                         (const double *)T->dvy, P->tx, P->ty, P->bx, P->by,
-                                                        P->rad, P->area, T->diam, T->cf, cfg->kernel_c, P->akc,
+                                                        P->rad, P->area, T->diam, T->cf,
+                                                        cfg->kernel == NL_KERNEL_CONST ? 1.0 : cfg->kernel_c, P->akc,
                                                         T->bad); ++ctx->launches;
     k_hilo<<<(K + 255) / 256, 256, 0, ctx->stream>>>(K, P->tx, P->ty, P->bx, P->by, P->hl); ++ctx->launches;
     NL_CK(cudaGetLastError());

@@ -4,9 +4,8 @@
 // weights W_q = w_q |T_a| and barycentric coordinates phi_a(x_q) in shared memory;
 // each lane then takes candidate neighbours T_b in turn and, for every x_q, builds
 // R(x_q, T_b) (geometry.cuh) and its inner sums
-//     s0 = sum w psi,  s1 = sum w psi phi_b,  S2 = sum w psi phi_b phi_b^T
-// over the fan subtriangles (inner rule) and caps (one centroid point), which
-// gives the expansion of (phi_j(x)-phi_j(y))(phi_j'(x)-phi_j'(y)) psi of
+//     s0 = sum w psi,  s1 = sum w psi phi_b,  S2 = sum w psi phi_b phi_b^T,
+// which gives the expansion of (phi_j(x)-phi_j(y))(phi_j'(x)-phi_j'(y)) psi of
 // Eq. (bformhj) over the six local nodes (Sec. 7.2):
 //     M_aa += W s0 phi_a phi_a^T,   M_bb += W S2,   M_ab += W phi_a s1^T
 // (D receives +M_aa, +M_bb, -M_ab and -M_ab^T).  Per candidate pair the lane writes
@@ -14,9 +13,14 @@
 // symmetric) onto T_b's per-triangle sums (FP64 atomics); M_aa is summed over all
 // candidates in FP64 and reduced across the warp.
 //
+// The constant kernel takes its sums from the regions' moments (numeric_const.cuh: k_const does
+// the interior and the boundary candidates).  The singular kernel psi = c / |x - y| takes them
+// from the inner rule on the fan subtriangles (and one centroid point per cap), in k_interior,
+// k_boundary and, in the near field, k_near.
+//
 // T = double: FP64 quadrature.  T = float: the inner sums run in FP32, the boundary
-// kernel's per-pair sums in 32-bit fixed point (exact, order-free integer adds of values
-// rounded to a per-pair grid), and the long sums (M_aa over all neighbours, M_bb over all
+// kernels' per-pair sums in 32-bit fixed point (exact, order-free integer adds of values
+// rounded to a grid), and the long sums (M_aa over all neighbours, M_bb over all
 // pairs of T_b, and D over all pairs in the scatter) in FP64, which compensates the FP32
 // rounding of the short sums.
 #pragma once
@@ -61,7 +65,7 @@ struct NumArgs {
     int64_t E;
     const double *tx, *ty;            // [3][K]
     const double *bx, *by, *area;     // [K]
-    const float *akc;                 // [K] |T| kc in FP32
+    const float *akc;                 // [K] in FP32: |T| (constant kernel), |T| kc (singular kernel)
     const float *hl;                  // [16][K] coordinates as FP32 hi + lo pairs (k_hilo)
     const int64_t *nbr_ptr, *nbr_split;
     const int32_t *nbr_idx;
@@ -104,6 +108,7 @@ struct NumArgs {
     OuterPt *otab;                    // [K][outer.n] outer points as the boundary kernel staged them (read by
                                       // k_near; with the near-field queue only)
     int prob;                         // index of this problem in a batched launch's argument array
+    double area_grid;                 // constant kernel, FP64: scale of the fixed-point sums of areas
     float s0q_grid;                   // FP32 boundary kernel: scale of the fixed-point sums of s0 per
                                       // outer point (a power of two; the bound on a sum maps below 2^30)
 };
@@ -255,23 +260,15 @@ __device__ __forceinline__ void rule_pt(const NumArgs &A, int r, T &p0, T &p1, T
 }
 
 // inner sums over the whole triangle T_b: phi_b at the rule points are the rule's barycentrics.
-// KIN: the kernel type when the caller knows it at compile time (0 constant, 1 c/|x - y|), else
-// -1 (read from A.kernel)
-template <typename T, int KIN = -1>
+// INV: the kernel is c / |x - y| (vertices relative to x: dl if given, else from V), else constant
+template <typename T, bool INV>
 __device__ __forceinline__ void whole_sums(const NumArgs &A, const D2 V[3], T area_kc, D2 x, Sums<T> &S,
                                            int64_t &nqp, const nlg::F2 *dl = nullptr)
 {
     sums_zero(S);
-    const bool inv = KIN < 0 ? (A.kernel == NL_KERNEL_INV_DIST) : (KIN == 1);
     const int n = A.inner.n;
-    T ar = area_kc;
-    // Every (x_q, T_b) evaluates its inner points: for a constant kernel on a whole T_b
-    // they do not depend on x, and the opaque barrier keeps the compiler from hoisting
-    // them out of the outer-point loop (that hoist would skip counted work).
-    if (sizeof(T) == sizeof(float)) asm volatile("" : "+f"(*(float *)&ar));
-    else asm volatile("" : "+d"(*(double *)&ar));
     T lx[3], ly[3];
-    if (inv) {
+    if (INV) {
         if (sizeof(T) == sizeof(float) && dl)   // FP32 coordinates relative to x (no FP64 work)
             for (int i = 0; i < 3; i++) { lx[i] = (T)dl[i].x; ly[i] = (T)dl[i].y; }
         else
@@ -280,8 +277,8 @@ __device__ __forceinline__ void whole_sums(const NumArgs &A, const D2 V[3], T ar
     for (int r = 0; r < n; r++) {
         T p0, p1, p2, w;
         rule_pt<T>(A, r, p0, p1, p2, w);
-        w *= ar;
-        if (inv) {
+        w *= area_kc;
+        if (INV) {
             T dx = p0 * lx[0] + p1 * lx[1] + p2 * lx[2];
             T dy = p0 * ly[0] + p1 * ly[1] + p2 * ly[2];
             w = w / sqrt(dx * dx + dy * dy);
@@ -291,14 +288,14 @@ __device__ __forceinline__ void whole_sums(const NumArgs &A, const D2 V[3], T ar
     nqp += n;
 }
 
+// inner sums over the region R of the singular kernel c / |x - y|
 template <typename T>
 __device__ __forceinline__ void inner_sums(const NumArgs &A, const nlg::Region &R, const D2 V[3], double area_b,
                                            D2 x, Sums<T> &S, int64_t &nqp)
 {
     sums_zero(S);
-    const bool inv = (A.kernel == NL_KERNEL_INV_DIST);
     const RuleTab &ri = A.inner;
-    if (inv && R.nv >= 3 && nlg::is_near(R, V, x)) {
+    if (R.nv >= 3 && nlg::is_near(R, V, x)) {
         BaryMap bm = bary_map(V);
         Sums<double> Sd;
         sums_zero(Sd);
@@ -310,18 +307,13 @@ __device__ __forceinline__ void inner_sums(const NumArgs &A, const nlg::Region &
         // the region is T_b itself: phi_b at the rule points are the rule's barycentrics
         const T ar = (T)area_b;
         T lx[3], ly[3];
-        if (inv)
-            for (int i = 0; i < 3; i++) { lx[i] = (T)(V[i].x - x.x); ly[i] = (T)(V[i].y - x.y); }
+        for (int i = 0; i < 3; i++) { lx[i] = (T)(V[i].x - x.x); ly[i] = (T)(V[i].y - x.y); }
         for (int r = 0; r < ri.n; r++) {
             T p0 = (T)ri.l[r][0], p1 = (T)ri.l[r][1], p2 = (T)ri.l[r][2];
             T w = (T)ri.w[r] * ar;
-            if (inv) {
-                T dx = p0 * lx[0] + p1 * lx[1] + p2 * lx[2];
-                T dy = p0 * ly[0] + p1 * ly[1] + p2 * ly[2];
-                w = w * (T)A.kc / sqrt(dx * dx + dy * dy);
-            } else {
-                w = w * (T)A.kc;
-            }
+            T dx = p0 * lx[0] + p1 * lx[1] + p2 * lx[2];
+            T dy = p0 * ly[0] + p1 * ly[1] + p2 * ly[2];
+            w = w * (T)A.kc / sqrt(dx * dx + dy * dy);
             sums_add<T>(S, w, p0, p1, p2);
         }
         nqp += ri.n;
@@ -351,13 +343,9 @@ __device__ __forceinline__ void inner_sums(const NumArgs &A, const nlg::Region &
                     T p1 = m0 * f0[1] + m1 * fk[1] + m2 * fn[1];
                     T p2 = m0 * f0[2] + m1 * fk[2] + m2 * fn[2];
                     w *= art;
-                    if (inv) {
-                        T dx = m0 * l0x + m1 * lkx + m2 * lnx;
-                        T dy = m0 * l0y + m1 * lky + m2 * lny;
-                        w = w * (T)A.kc / sqrt(dx * dx + dy * dy);
-                    } else {
-                        w = w * (T)A.kc;
-                    }
+                    T dx = m0 * l0x + m1 * lkx + m2 * lnx;
+                    T dy = m0 * l0y + m1 * lky + m2 * lny;
+                    w = w * (T)A.kc / sqrt(dx * dx + dy * dy);
                     sums_add<T>(S, w, p0, p1, p2);
                 }
                 nqp += ri.n;
@@ -369,12 +357,8 @@ __device__ __forceinline__ void inner_sums(const NumArgs &A, const nlg::Region &
             double ph[3];
             bary_of(bm, R.cc[c].x, R.cc[c].y, ph);
             T w = (T)R.cw[c];
-            if (inv) {
-                double dx = R.cc[c].x - x.x, dy = R.cc[c].y - x.y;
-                w = w * (T)(A.kc / sqrt(dx * dx + dy * dy));
-            } else {
-                w = w * (T)A.kc;
-            }
+            double dx = R.cc[c].x - x.x, dy = R.cc[c].y - x.y;
+            w = w * (T)(A.kc / sqrt(dx * dx + dy * dy));
             sums_add<T>(S, w, (T)ph[0], (T)ph[1], (T)ph[2]);
             nqp++;
         }
@@ -382,8 +366,7 @@ __device__ __forceinline__ void inner_sums(const NumArgs &A, const nlg::Region &
 }
 
 // inner sums over a fanned polygon in FP32 coordinates relative to x, held in the lane's columns
-// px / py of a shared buffer (FP32 path; KIN as for whole_sums)
-template <int KIN = -1>
+// px / py of a shared buffer (FP32 path, singular kernel)
 __device__ __forceinline__ void poly_sums_col(const NumArgs &A, nlg::Col px, nlg::Col py, int n, const nlg::F2 &d0,
                                               const nlg::F2 &e1, const nlg::F2 &e2, float inv_det,
                                               Sums<float> &S, int64_t &nqp)
@@ -416,10 +399,8 @@ __device__ __forceinline__ void poly_sums_col(const NumArgs &A, nlg::Col px, nlg
             const float p1 = m0 * f0[1] + m1 * fk[1] + m2 * fn[1];
             const float p2 = m0 * f0[2] + m1 * fk[2] + m2 * fn[2];
             float w = f.w * ar;
-            if (KIN < 0 ? A.kernel == NL_KERNEL_INV_DIST : KIN == 1) {   // psi = c / |y - x|, relative to x
-                const float yx = m0 * x0 + m1 * xk + m2 * xn, yy = m0 * y0 + m1 * yk + m2 * yn;
-                w *= rsqrtf(yx * yx + yy * yy);
-            }
+            const float yx = m0 * x0 + m1 * xk + m2 * xn, yy = m0 * y0 + m1 * yk + m2 * yn;
+            w *= rsqrtf(yx * yx + yy * yy);   // psi = c / |y - x|, relative to x
             sums_add<float>(S, w, p0, p1, p2);
         }
         nqp += nr;
@@ -429,13 +410,12 @@ __device__ __forceinline__ void poly_sums_col(const NumArgs &A, nlg::Col px, nlg
 }
 
 // the same over buffer `which` of a clip buffer (the N-gon clip's output)
-template <int KIN = -1>
 __device__ __forceinline__ void poly_sums_sh(const NumArgs &A, const nlg::ClipBuf &cb, int which, int lane, int n,
                                              const nlg::F2 &d0, const nlg::F2 &e1, const nlg::F2 &e2, float inv_det,
                                              Sums<float> &S, int64_t &nqp)
 {
     nlg::ClipBuf &c = const_cast<nlg::ClipBuf &>(cb);
-    poly_sums_col<KIN>(A, nlg::Col{&c.x[which][0][lane]}, nlg::Col{&c.y[which][0][lane]}, n, d0, e1, e2, inv_det, S,
+    poly_sums_col(A, nlg::Col{&c.x[which][0][lane]}, nlg::Col{&c.y[which][0][lane]}, n, d0, e1, e2, inv_det, S,
                        nqp);
 }
 
@@ -680,13 +660,13 @@ __device__ __forceinline__ bool want_stats(const NumArgs &A)
 }
 
 // ---------------------------------------------------------------------------
-// Interior pairs: T_b is whole for every outer point of T_a (certified when the
+// Interior pairs (singular kernel): T_b is whole for every outer point of T_a (certified when the
 // candidate lists are built), so there is no per-point classification.  k_interior runs
 // concurrently with k_boundary (it fills the boundary kernel's last wave): both add the
 // per-triangle M_aa and statistics atomically onto zeroed outputs; the batched kernels run
 // one after the other and store, then add.
 // ---------------------------------------------------------------------------
-template <typename T, int STS = -1, int KIN = -1>
+template <typename T, int STS = -1>
 __device__ __forceinline__ void interior_outer(const NumArgs &A, int a, const OuterPt *sq, int lane, LaneAcc &acc)
 {
     const int K = A.K;
@@ -700,17 +680,13 @@ __device__ __forceinline__ void interior_outer(const NumArgs &A, int a, const Ou
             continue;
         }
 #endif
-        const bool inv = KIN < 0 ? A.kernel == NL_KERNEL_INV_DIST : KIN == 1;
-        // the FP64 vertices only where the quadrature uses them (singular kernel)
-        D2 Vb[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
-        if (inv)
-            for (int i = 0; i < 3; i++) { Vb[i].x = A.tx[i * K + b]; Vb[i].y = A.ty[i * K + b]; }
+        D2 Vb[3];
+        for (int i = 0; i < 3; i++) { Vb[i].x = A.tx[i * K + b]; Vb[i].y = A.ty[i * K + b]; }
         const T akc = sizeof(T) == sizeof(float) ? (T)A.akc[b] : (T)(A.area[b] * A.kc);
         int q0 = 0, q1 = A.outer.n;
         if (A.switch47) rule_range(A, ba, D2{A.bx[b], A.by[b]}, q0, q1);
         nlg::F2 vl[3];
-        if (inv)
-            for (int i = 0; i < 3; i++) { vl[i].x = (float)(Vb[i].x - ba.x); vl[i].y = (float)(Vb[i].y - ba.y); }
+        for (int i = 0; i < 3; i++) { vl[i].x = (float)(Vb[i].x - ba.x); vl[i].y = (float)(Vb[i].y - ba.y); }
         T v[21];
         for (int i = 0; i < 21; i++) v[i] = 0;
         for (int q = q0; q < q1; q++) {
@@ -718,19 +694,12 @@ __device__ __forceinline__ void interior_outer(const NumArgs &A, int a, const Ou
             Sums<T> S;
             int64_t nq = 0;
             nlg::F2 dl[3];
-            if (inv)
-                for (int i = 0; i < 3; i++) { dl[i].x = vl[i].x - o.lx; dl[i].y = vl[i].y - o.ly; }
-            whole_sums<T, KIN>(A, Vb, akc, D2{o.x, o.y}, S, nq, inv ? dl : nullptr);
+            for (int i = 0; i < 3; i++) { dl[i].x = vl[i].x - o.lx; dl[i].y = vl[i].y - o.ly; }
+            whole_sums<T, true>(A, Vb, akc, D2{o.x, o.y}, S, nq, dl);
             combine<T>(o, S, v);
             acc.qp += nq;
-            if (!A.outer_support) {
-                acc.cnt++;
-                if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, b, q - q0, nlg::KIND_WHOLE, 3, 0);
-            }
-        }
-        if (A.outer_support && q1 > q0) {   // one record per pair: the support is all of T_a
             acc.cnt++;
-            if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, b, 0, nlg::KIND_WHOLE, 3, 0);
+            if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, b, q - q0, nlg::KIND_WHOLE, 3, 0);
         }
         write_pair<T>(A, e, b, q1 > q0, v, acc);
     }
@@ -768,7 +737,7 @@ __device__ __forceinline__ void finish_outer(const NumArgs &A, int a, LaneAcc &a
 }
 
 // five resident 4-warp blocks per SM with float sums (96 registers); double sums unconstrained
-template <typename T, int STS = -1, int KIN = -1>
+template <typename T, int STS = -1>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, sizeof(T) == sizeof(float) ? 5 : 1) k_interior(const NumArgs A)
 {
     __shared__ OuterPt sq_all[kWarpsPerBlock][NL_MAXQ + 8];
@@ -780,7 +749,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, sizeof(T) == sizeof(float
     __syncwarp();
     LaneAcc acc;
     acc_zero(acc);
-    interior_outer<T, STS, KIN>(A, a, sq, lane, acc);
+    interior_outer<T, STS>(A, a, sq, lane, acc);
     finish_outer<STS>(A, a, acc, lane, kAtomicAdd);
 }
 
@@ -797,7 +766,7 @@ struct CandData {
     float vlx[3], vly[3];      // T_b relative to bary_a
     float blx, bly;            // bary_b relative to bary_a
     float e1x, e1y, e2x, e2y, binv;
-    float akcf;                // |T_b| times the kernel constant
+    float akcf;                // |T_b| (constant kernel), |T_b| times c (singular kernel)
     int b, q0;
 };
 
@@ -925,8 +894,7 @@ __device__ __noinline__ bool exact_item_fp64(const NumArgs &A, const CandData &c
                                              int lane);
 
 // inner sums over fan triangle k (vertices 0, k, k + 1) of a polygon held in columns px / py, in
-// FP32 coordinates relative to x (FP32 path; KIN as for whole_sums)
-template <int KIN = -1>
+// FP32 coordinates relative to x (FP32 path, singular kernel)
 __device__ __forceinline__ void fan_tri_sums(const NumArgs &A, nlg::Col px, nlg::Col py, int k, const nlg::F2 &d0,
                                              const nlg::F2 &e1, const nlg::F2 &e2, float inv_det, Sums<float> &S)
 {
@@ -954,10 +922,8 @@ __device__ __forceinline__ void fan_tri_sums(const NumArgs &A, nlg::Col px, nlg:
         const float p1 = m0 * f0[1] + m1 * fk[1] + m2 * fn[1];
         const float p2 = m0 * f0[2] + m1 * fk[2] + m2 * fn[2];
         float w = f.w * ar;
-        if (KIN < 0 ? A.kernel == NL_KERNEL_INV_DIST : KIN == 1) {   // psi = c / |y - x|, relative to x
-            const float yx = m0 * x0 + m1 * xk + m2 * xn, yy = m0 * y0 + m1 * yk + m2 * yn;
-            w *= rsqrtf(yx * yx + yy * yy);
-        }
+        const float yx = m0 * x0 + m1 * xk + m2 * xn, yy = m0 * y0 + m1 * yk + m2 * yn;
+        w *= rsqrtf(yx * yx + yy * yy);   // psi = c / |y - x|, relative to x
         sums_add<float>(S, w, p0, p1, p2);
     }
 }
@@ -965,17 +931,17 @@ __device__ __forceinline__ void fan_tri_sums(const NumArgs &A, nlg::Col px, nlg:
 // FP32 region of one undecided (q, b) of the balls whose region is a polygon (N-gon, nocaps,
 // approxcaps), left in the lane's clip-buffer column (buffer *which): 1 with its vertex count n
 // and kind, 0 empty, -1 the FP64 geometry decides (as exact_item_f32)
-template <int BALL, bool INV>
+template <int BALL>
 __device__ __forceinline__ int exact_region_f32(const NumArgs &A, const CandData &c, const OuterPt &o,
                                                 nlg::ClipBuf &cb, int lane, int &n, int &kind, int &which)
 {
     nlg::F2 dl[3];
     for (int i = 0; i < 3; i++) { dl[i].x = c.vlx[i] - o.lx; dl[i].y = c.vly[i] - o.ly; }
-    if (INV && nlg::near_f32(dl, cand_diam(c), A.geo.tau) != 0) return -1;
+    if (nlg::near_f32(dl, cand_diam(c), A.geo.tau) != 0) return -1;
     which = 0;
     if (BALL == NL_BALL_NGON) {
         bool cut = false;
-        n = nlg::clip_ngon_f32_sh<!INV>(dl, A.geo.err0, A.geo, cb, lane, &which, &cut);
+        n = nlg::clip_ngon_f32_sh<false>(dl, A.geo.err0, A.geo, cb, lane, &which, &cut);
         if (n < 0) return -1;
         if (n < 3) return 0;
         kind = cut ? nlg::KIND_PARTIAL : nlg::KIND_WHOLE;
@@ -991,14 +957,14 @@ __device__ __forceinline__ int exact_region_f32(const NumArgs &A, const CandData
 // lane per item (the N-gon's items go through exact_region_f32 and the spread fans): 1 done (S
 // holds its sums), 0 empty region, -1 the FP64 geometry decides (the singular kernel's near
 // field, an uncertified FP32 choice, FP64 sums or a ball without an FP32 region)
-template <int BALL, typename T, bool INV>
+template <int BALL, typename T>
 __device__ __forceinline__ int exact_item_f32(const NumArgs &A, const CandData &c, const OuterPt &o, Sums<T> &S,
                                               int64_t &nq, int &kind, int &nv, int &ncap, nlg::ClipBuf &cb, int lane)
 {
     if (sizeof(T) == sizeof(float) && (BALL == NL_BALL_NOCAPS || BALL == NL_BALL_APPROXCAPS)) {
         nlg::F2 dl[3];
         for (int i = 0; i < 3; i++) { dl[i].x = c.vlx[i] - o.lx; dl[i].y = c.vly[i] - o.ly; }
-        if (INV && nlg::near_f32(dl, cand_diam(c), A.geo.tau) != 0)
+        if (nlg::near_f32(dl, cand_diam(c), A.geo.tau) != 0)
             return -1;
         int k = nlg::KIND_PARTIAL;
         const int n = nlg::ball_region_f32<BALL>(dl, A.geo, cb, lane, &k);
@@ -1010,10 +976,10 @@ __device__ __forceinline__ int exact_item_f32(const NumArgs &A, const CandData &
             ncap = 0;
             if (k == nlg::KIND_WHOLE) {
                 const D2 Vb[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};   // unused: FP32 coordinates dl
-                whole_sums<T, INV>(A, Vb, cand_akc<T>(A, c), D2{o.x, o.y}, S, nq, dl);
+                whole_sums<T, true>(A, Vb, cand_akc<T>(A, c), D2{o.x, o.y}, S, nq, dl);
             } else {
                 const nlg::F2 e1 = {c.e1x, c.e1y}, e2 = {c.e2x, c.e2y};
-                poly_sums_col<INV>(A, nlg::col(cb.x, lane), nlg::col(cb.y, lane), n, dl[0], e1, e2, c.binv,
+                poly_sums_col(A, nlg::col(cb.x, lane), nlg::col(cb.y, lane), n, dl[0], e1, e2, c.binv,
                                    *(Sums<float> *)&S, nq);
             }
             return 1;
@@ -1022,7 +988,7 @@ __device__ __forceinline__ int exact_item_f32(const NumArgs &A, const CandData &
     if (sizeof(T) == sizeof(float) && BALL == NL_BALL_EXACTCAPS) {
         nlg::F2 dl[3];
         for (int i = 0; i < 3; i++) { dl[i].x = c.vlx[i] - o.lx; dl[i].y = c.vly[i] - o.ly; }
-        if (INV && nlg::near_f32(dl, cand_diam(c), A.geo.tau) != 0)
+        if (nlg::near_f32(dl, cand_diam(c), A.geo.tau) != 0)
             return -1;
         int nc = 0, k = nlg::KIND_PARTIAL;
         const int n = nlg::exactcaps_region_f32(dl, A.geo, cb, lane, &nc, &k);
@@ -1035,18 +1001,18 @@ __device__ __forceinline__ int exact_item_f32(const NumArgs &A, const CandData &
             ncap = nc;
             if (k == nlg::KIND_WHOLE) {
                 const D2 Vb[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};   // unused: FP32 coordinates dl
-                whole_sums<T, INV>(A, Vb, cand_akc<T>(A, c), D2{o.x, o.y}, S, nq, dl);
+                whole_sums<T, true>(A, Vb, cand_akc<T>(A, c), D2{o.x, o.y}, S, nq, dl);
             } else {
                 Sums<float> &Sf = *(Sums<float> *)&S;
                 const nlg::F2 e1 = {c.e1x, c.e1y}, e2 = {c.e2x, c.e2y};
-                if (n >= 3) poly_sums_col<INV>(A, px, py, n, dl[0], e1, e2, c.binv, Sf, nq);
+                if (n >= 3) poly_sums_col(A, px, py, n, dl[0], e1, e2, c.binv, Sf, nq);
                 else sums_zero(Sf);
                 for (int j = 0; j < nc; j++) {   // one point per cap: its centroid, weight its area
                     const float cx = px[8 + j], cy = py[8 + j];
                     const float rx = cx - dl[0].x, ry = cy - dl[0].y;
                     const float l1 = (rx * e2.y - e2.x * ry) * c.binv, l2 = (e1.x * ry - rx * e1.y) * c.binv;
                     float w = pe[j] * A.kcf;
-                    if (INV) w *= rsqrtf(cx * cx + cy * cy);
+                    w *= rsqrtf(cx * cx + cy * cy);
                     sums_add<float>(Sf, w, 1.f - l1 - l2, l1, l2);
                     nq++;
                 }
@@ -1078,10 +1044,7 @@ __device__ __noinline__ bool exact_item_fp64(const NumArgs &A, const CandData &c
     kind = R.kind;
     nv = R.nv;
     ncap = R.ncap;
-    if (R.kind == nlg::KIND_WHOLE && R.ncap == 0 && A.kernel != NL_KERNEL_INV_DIST) {
-        whole_sums<T>(A, Vb, (T)(c64.area * A.kc), x, S, nq);
-    } else if (sizeof(T) == sizeof(float) && R.ncap == 0 && R.nv <= nlg::kClipCap &&
-               (A.kernel == NL_KERNEL_CONST || !nlg::is_near(R, Vb, x))) {
+    if (sizeof(T) == sizeof(float) && R.ncap == 0 && R.nv <= nlg::kClipCap && !nlg::is_near(R, Vb, x)) {
         // FP32 quadrature on the FP64 polygon (coordinates relative to x)
         for (int i = 0; i < R.nv; i++) {
             cb.x[0][i][lane] = (float)(R.P[i].x - x.x);
@@ -1090,8 +1053,7 @@ __device__ __noinline__ bool exact_item_fp64(const NumArgs &A, const CandData &c
         const nlg::F2 d0 = {(float)(Vb[0].x - x.x), (float)(Vb[0].y - x.y)};
         const nlg::F2 e1 = {c.e1x, c.e1y}, e2 = {c.e2x, c.e2y};
         poly_sums_sh(A, cb, 0, lane, R.nv, d0, e1, e2, c.binv, *(Sums<float> *)&S, nq);
-    } else if (sizeof(T) == sizeof(float) && A.kernel == NL_KERNEL_INV_DIST && R.kind == nlg::KIND_WHOLE &&
-               R.ncap == 0) {
+    } else if (sizeof(T) == sizeof(float) && R.kind == nlg::KIND_WHOLE && R.ncap == 0) {
         // a whole T_b in the singular kernel's near field (decided by the FP64 test): the FP32
         // near rule, as k_near integrates the near-field items that FP32 decides
         const nlg::F2 e1 = {c.e1x, c.e1y}, e2 = {c.e2x, c.e2y};
@@ -1111,8 +1073,7 @@ __device__ __noinline__ bool exact_item_fp64(const NumArgs &A, const CandData &c
 // Bound: an item (x_q, T_b) adds W_q la_i s1_j to M_ab and W_q S2_jk to M_bb; with |la_i| <= L_q
 // (the outer point's barycentrics) and 0 <= S2_jk, s1_j <= s0 (inner barycentrics in [0, 1] up to
 // rounding) every sum of the pair is at most B_a s0max, B_a = sum_q |W_q| max(1, L_q).  The region
-// lies in T_b, so s0max = kc |T_b| for a constant kernel; for c / |x - y| the integral over T_b is
-// at most c 2 sqrt(pi |T_b|) (the disc of the same area centred at x), taken twice more for the
+// lies in T_b, and the integral of c / |x - y| over T_b is at most s0max = c 2 sqrt(pi |T_b|) (the disc of the same area centred at x), taken twice more for the
 // quadrature's error.  The bound, rounded up to a power of two 2^e, maps to 2^29: a rounding error
 // of at most 2^-30 of it per item, and sums far from the 2^31 range unless the bound is broken
 // (|sum| >= 2^30 sets error bit 256).
@@ -1127,11 +1088,10 @@ __device__ __forceinline__ float fx_outer_bound(const OuterPt *sq, int n)
     return b * 1.0001f;   // above its own rounding
 }
 
-// grid scale 2^(29 - e) of a pair (outer bound bwa, |T_b| kc = akcf)
-template <bool INV>
+// grid scale 2^(29 - e) of a pair (outer bound bwa, |T_b| c = akcf)
 __device__ __forceinline__ float fx_scale(float bwa, float akcf, float kcf)
 {
-    const float r = INV ? bwa * 4.f * sqrtf(3.14159265f * kcf * akcf) : bwa * akcf;
+    const float r = bwa * 4.f * sqrtf(3.14159265f * kcf * akcf);
     const int e = ((__float_as_int(fmaxf(r, 1e-25f)) >> 23) & 0xff) - 126;   // r < 2^e
     return __int_as_float((127 + 29 - e) << 23);
 }
@@ -1344,9 +1304,8 @@ __device__ __forceinline__ void near_flush(const NumArgs &A, int a, int64_t base
     }
 }
 
-// The boundary candidates of outer triangle a (outer points staged in sh.sq).
-// INV: the kernel is psi = c/|x - y| (near-field split), else the constant kernel.
-template <int BALL, typename T, bool INV, bool NQ = false, int STS = -1>
+// The boundary candidates of outer triangle a (outer points staged in sh.sq), singular kernel.
+template <int BALL, typename T, bool NQ = false, int STS = -1>
 __device__ __forceinline__ void boundary_outer(const NumArgs &A, int a, BoundaryShared<T> &sh, int lane,
                                                LaneAcc &acc)
 {
@@ -1360,7 +1319,6 @@ __device__ __forceinline__ void boundary_outer(const NumArgs &A, int a, Boundary
     const int nq_all = A.outer.n;
     // FP32 sums: the outer bound of the pairs' fixed-point grids
     const float fx_bwa = sizeof(T) == sizeof(float) ? fx_outer_bound(sh.sq, nq_all) : 0.f;
-    const bool inv = INV;
     for (int q = lane; q < NL_MAXQ; q += 32) sh.s0q[q] = 0;
     __syncwarp();
     for (int64_t base = es; base < e1; base += 32) {
@@ -1387,7 +1345,7 @@ __device__ __forceinline__ void boundary_outer(const NumArgs &A, int a, Boundary
         // phase 1: classify every (q, b) in lockstep; queue whole and undecided items.  With a
         // near-field queue (FP32 singular kernel), the near-field whole items of this lane's
         // candidate are only marked (my_near, bit q) and handed to k_near after the round.
-        constexpr bool split_near = INV && NQ && sizeof(T) == sizeof(float);
+        constexpr bool split_near = NQ && sizeof(T) == sizeof(float);
         unsigned my_near = 0;
         int nwhole = 0, nnear = 0;
         for (int q = 0; q < nq_all; q++) {
@@ -1398,7 +1356,7 @@ __device__ __forceinline__ void boundary_outer(const NumArgs &A, int a, Boundary
                 cls = classify_item<BALL, T>(A, c, sh.sq[q], dl);
                 // singular kernel: whole items in the near field take the near rule (certified
                 // in FP32; undecided ones the FP64 path)
-                if (inv && cls == nlg::CLS_WHOLE) {
+                if (cls == nlg::CLS_WHOLE) {
                     const int nr = nlg::near_f32(dl, cand_diam(c), A.geo.tau);
                     cls = nr == 0 ? nlg::CLS_WHOLE : (nr == 1 && sizeof(T) == sizeof(float) ? 3 : nlg::CLS_EXACT);
                     if (cls == 3 && split_near) {
@@ -1428,22 +1386,21 @@ __device__ __forceinline__ void boundary_outer(const NumArgs &A, int a, Boundary
             const OuterPt &o = sh.sq[q];
             // FP64 vertices only where the FP64 quadrature of the singular kernel needs them
             D2 Vb[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
-            if (INV && sizeof(T) == sizeof(double))
+            if (sizeof(T) == sizeof(double))
                 for (int k = 0; k < 3; k++) { Vb[k].x = A.tx[k * K + cd.b]; Vb[k].y = A.ty[k * K + cd.b]; }
             Sums<T> S;
             int64_t nq = 0;
             nlg::F2 dl[3];
-            if (INV)
-                for (int k = 0; k < 3; k++) { dl[k].x = cd.vlx[k] - o.lx; dl[k].y = cd.vly[k] - o.ly; }
-            whole_sums<T, INV>(A, Vb, cand_akc<T>(A, cd), D2{o.x, o.y}, S, nq, INV ? dl : nullptr);
-            block_add<T>(o, S, sh.acc, sh.s0q, own, q, fx_scale<INV>(fx_bwa, cd.akcf, A.kcf), A.s0q_grid);
+            for (int k = 0; k < 3; k++) { dl[k].x = cd.vlx[k] - o.lx; dl[k].y = cd.vly[k] - o.ly; }
+            whole_sums<T, true>(A, Vb, cand_akc<T>(A, cd), D2{o.x, o.y}, S, nq, dl);
+            block_add<T>(o, S, sh.acc, sh.s0q, own, q, fx_scale(fx_bwa, cd.akcf, A.kcf), A.s0q_grid);
             acc.cnt++;
             acc.qp += nq;
             if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, cd.b, q - cd.q0, nlg::KIND_WHOLE, 3, 0);
         }
         __syncwarp();
         // phase 2c: whole items in the singular kernel's near field (FP32 near rule)
-        for (int i = lane; INV && !split_near && i < nnear; i += 32) {
+        for (int i = lane; !split_near && i < nnear; i += 32) {
             const int left = nnear - (i - lane);   // items of this round
             const unsigned rmask = left >= 32 ? 0xffffffffu : ((1u << left) - 1u);
             const unsigned it = sh.wqueue[kQueueCap - 1 - i];
@@ -1462,7 +1419,7 @@ __device__ __forceinline__ void boundary_outer(const NumArgs &A, int a, Boundary
             // an owner lies in the near field of several outer points of one round: the lanes
             // with the same owner sum their blocks by shuffles, one lane per owner adds
             s0q_add<T>(sh.s0q, q, S.s0, A.s0q_grid);
-            warp_owner_add<T>(sh.acc, own, lane, w, fx_scale<INV>(fx_bwa, cd.akcf, A.kcf), rmask);
+            warp_owner_add<T>(sh.acc, own, lane, w, fx_scale(fx_bwa, cd.akcf, A.kcf), rmask);
             acc.cnt++;
             acc.qp += nq;
             if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, cd.b, q - cd.q0, nlg::KIND_WHOLE, 3, 0);
@@ -1471,20 +1428,14 @@ __device__ __forceinline__ void boundary_outer(const NumArgs &A, int a, Boundary
         // items: lanes at different items run the same parts of the clip together.  So the order
         // in which their blocks reach an owner's column depends on the scheduling: FP32 sums are
         // integers there (the same for any order), FP64 blocks may differ in their last bits.
-        // FP32 polygon regions of the N-gon (either kernel) and nocaps: a round of 32 items
-        // builds its regions (a lane per item), then the warp spreads the fan triangles of all 32
-        // polygons over its lanes, each adding its triangle's block onto the owner's column
-        // (integer sums: any order), so the lanes stay busy although the fans have 1 to 4
-        // triangles (nocaps boundary kernel of a K = 23328 problem 3.43 -> 2.20 ms; the N-gon's
-        // numeric phase 5.63 -> 5.51 ms, with the singular kernel 15.9 -> 14.8 ms).  The fan is
-        // the one the lane-per-item drain integrates (from the polygon's first vertex).  The
-        // approxcaps fans (up to 13 triangles with the arc points) keep the lane-per-item drain:
-        // a triangle's lookup and block add then cost about as much as its quadrature (2.68 ->
-        // 3.08 ms spread, 2.95 ms with the owner table; tasks of two to five triangles of one fan
-        // did not pay either).  The owner of each triangle comes from a per-round table
-        // (`ftask`) instead of a binary search over the lanes' first triangles (the N-gon's
-        // numeric phase 5.51 -> 5.38 ms).
-        constexpr bool kSpread = sizeof(T) == sizeof(float) && (BALL == NL_BALL_NGON || (!INV && BALL == NL_BALL_NOCAPS));
+        // FP32 polygon regions of the N-gon: a round of 32 items builds its regions (a lane per
+        // item), then the warp spreads the fan triangles of all 32 polygons over its lanes, each
+        // adding its triangle's block onto the owner's column (integer sums: any order), so the
+        // lanes stay busy although the fans have 1 to 4 triangles (numeric phase at K = 32768,
+        // delta = 0.05: 15.9 -> 14.8 ms).  The fan is the one the lane-per-item drain integrates (from
+        // the polygon's first vertex).  The owner of each triangle comes from a per-round table
+        // (`ftask`).
+        constexpr bool kSpread = sizeof(T) == sizeof(float) && BALL == NL_BALL_NGON;
         if constexpr (kSpread)
         for (int r0 = 0; r0 < nqueue; r0 += 32) {
             const int i = r0 + lane;
@@ -1495,7 +1446,7 @@ __device__ __forceinline__ void boundary_outer(const NumArgs &A, int a, Boundary
                 const CandData &cd = sh.cand[own];
                 const OuterPt &o = sh.sq[q];
                 int n = 0, kind = nlg::KIND_PARTIAL;
-                const int r = exact_region_f32<BALL, INV>(A, cd, o, sh.clip, lane, n, kind, which);
+                const int r = exact_region_f32<BALL>(A, cd, o, sh.clip, lane, n, kind, which);
                 if (r > 0) {
                     m = n - 2;
                     acc.cnt++;
@@ -1506,7 +1457,7 @@ __device__ __forceinline__ void boundary_outer(const NumArgs &A, int a, Boundary
                     int64_t nq = 0;
                     int kd, nv, ncap;
                     if (exact_item_fp64<BALL, T>(A, cd, o, S, nq, kd, nv, ncap, sh.clip, lane)) {
-                        block_add<T>(o, S, sh.acc, sh.s0q, own, q, fx_scale<INV>(fx_bwa, cd.akcf, A.kcf), A.s0q_grid);
+                        block_add<T>(o, S, sh.acc, sh.s0q, own, q, fx_scale(fx_bwa, cd.akcf, A.kcf), A.s0q_grid);
                         acc.cnt++;
                         acc.qp += (uint32_t)nq;
                         if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, cd.b, q - cd.q0, kd, nv, ncap);
@@ -1533,9 +1484,9 @@ __device__ __forceinline__ void boundary_outer(const NumArgs &A, int a, Boundary
                 const int w = sh.fwhich[lo];
                 const nlg::F2 d0 = {cd.vlx[0] - o.lx, cd.vly[0] - o.ly}, e1 = {cd.e1x, cd.e1y}, e2 = {cd.e2x, cd.e2y};
                 Sums<float> S;
-                fan_tri_sums<INV>(A, nlg::Col{&sh.clip.x[w][0][lo]}, nlg::Col{&sh.clip.y[w][0][lo]}, k, d0, e1, e2,
+                fan_tri_sums(A, nlg::Col{&sh.clip.x[w][0][lo]}, nlg::Col{&sh.clip.y[w][0][lo]}, k, d0, e1, e2,
                                   cd.binv, S);
-                block_add<float>(o, S, sh.acc, sh.s0q, own, q, fx_scale<INV>(fx_bwa, cd.akcf, A.kcf), A.s0q_grid);
+                block_add<float>(o, S, sh.acc, sh.s0q, own, q, fx_scale(fx_bwa, cd.akcf, A.kcf), A.s0q_grid);
             }
             __syncwarp();
         }
@@ -1548,24 +1499,24 @@ __device__ __forceinline__ void boundary_outer(const NumArgs &A, int a, Boundary
             Sums<T> S;
             int64_t nq = 0;
             int kind, nv, ncap;
-            int r = exact_item_f32<BALL, T, INV>(A, cd, o, S, nq, kind, nv, ncap, sh.clip, lane);
+            int r = exact_item_f32<BALL, T>(A, cd, o, S, nq, kind, nv, ncap, sh.clip, lane);
             if (r < 0) {
                 if (defer_mark<T>(A, sh, own, q)) continue;
                 r = exact_item_fp64<BALL, T>(A, cd, o, S, nq, kind, nv, ncap, sh.clip, lane) ? 1 : 0;
             }
             if (r == 0) continue;
-            block_add<T>(o, S, sh.acc, sh.s0q, own, q, fx_scale<INV>(fx_bwa, cd.akcf, A.kcf), A.s0q_grid);
+            block_add<T>(o, S, sh.acc, sh.s0q, own, q, fx_scale(fx_bwa, cd.akcf, A.kcf), A.s0q_grid);
             acc.cnt++;
             acc.qp += nq;
             if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, cd.b, q - cd.q0, kind, nv, ncap);
         }
         __syncwarp();
         if (sizeof(T) == sizeof(float) && A.defer) {
-            defer_flush<BALL, T>(A, a, base, sh, lane, fx_scale<INV>(fx_bwa, sh.cand[lane].akcf, A.kcf), acc);
+            defer_flush<BALL, T>(A, a, base, sh, lane, fx_scale(fx_bwa, sh.cand[lane].akcf, A.kcf), acc);
             __syncwarp();
         }
         if constexpr (split_near) {
-            near_flush<T>(A, a, base, my_near, sh, fx_scale<INV>(fx_bwa, sh.cand[lane].akcf, A.kcf), lane, acc);
+            near_flush<T>(A, a, base, my_near, sh, fx_scale(fx_bwa, sh.cand[lane].akcf, A.kcf), lane, acc);
             __syncwarp();
         }
         // phase 3: owners merge the queue's contributions and write their pair
@@ -1573,7 +1524,7 @@ __device__ __forceinline__ void boundary_outer(const NumArgs &A, int a, Boundary
             T v[15];
             if constexpr (sizeof(T) == sizeof(float)) {
                 // back from the pair's grid (an exact power of two)
-                const float inv_s = 1.f / fx_scale<INV>(fx_bwa, sh.cand[lane].akcf, A.kcf);
+                const float inv_s = 1.f / fx_scale(fx_bwa, sh.cand[lane].akcf, A.kcf);
                 bool big = false;
                 for (int k = 0; k < 15; k++) {
                     const int iv = *reinterpret_cast<const int *>(&sh.acc[k][lane]);
@@ -1628,7 +1579,7 @@ __device__ __forceinline__ void support_boundary(const NumArgs &A, int a, int la
         rule_range(A, ba, bb, q0, q1);
         Sums<T> S;
         int64_t nq_in = 0;
-        whole_sums<T>(A, Vb, (T)(A.area[b] * A.kc), bb, S, nq_in);
+        whole_sums<T, false>(A, Vb, (T)(A.area[b] * A.kc), bb, S, nq_in);
         T v[21];
         for (int i = 0; i < 21; i++) v[i] = 0;
         int kind = nlg::KIND_NONE, nv = 0;
@@ -1707,29 +1658,31 @@ __device__ __forceinline__ void support_boundary(const NumArgs &A, int a, int la
     }
 }
 
+}  // namespace nlq
+
+#include "numeric_const.cuh"
+
+namespace nlq {
+
 // boundary candidates of outer triangle a for the ball mode BALL (NQ: the singular kernel's
 // near-field whole items go to the near-field queue)
-template <int BALL, typename T, bool INV, bool NQ = false, int STS = -1>
+template <int BALL, typename T, bool NQ = false, int STS = -1>
 __device__ __forceinline__ void boundary_any(const NumArgs &A, int a, BoundaryShared<T> &sh, int lane, LaneAcc &acc)
 {
-    if constexpr (BALL == NL_BALL_BARY_NOCAPS || BALL == NL_BALL_BARY_APPROXCAPS) {
-        support_boundary<BALL, T>(A, a, lane, sh.clip, acc);
-    } else {
-        stage_outer(A, a, sh.sq, lane);
-        __syncwarp();
-        if (INV && A.otab)   // k_near reads the outer points from here (no FP64 arithmetic per item)
-            for (int q = lane; q < A.outer.n; q += 32) A.otab[(int64_t)a * A.outer.n + q] = sh.sq[q];
-        boundary_outer<BALL, T, INV, NQ, STS>(A, a, sh, lane, acc);
-    }
+    stage_outer(A, a, sh.sq, lane);
+    __syncwarp();
+    if (A.otab)   // k_near reads the outer points from here (no FP64 arithmetic per item)
+        for (int q = lane; q < A.outer.n; q += 32) A.otab[(int64_t)a * A.outer.n + q] = sh.sq[q];
+    boundary_outer<BALL, T, NQ, STS>(A, a, sh, lane, acc);
 }
 
 // resident 4-warp blocks per SM: four with float sums (registers capped at 128, a few hundred
 // bytes of spills), three with double sums
-template <typename T, bool INV>
+template <typename T>
 constexpr int kBoundaryBlocksPerSm = sizeof(T) == sizeof(float) ? 4 : 3;
 
-template <int BALL, typename T, bool INV, bool NQ = false, int STS = -1>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, kBoundaryBlocksPerSm<T, INV>) k_boundary(const NumArgs A)
+template <int BALL, typename T, bool NQ = false, int STS = -1>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, kBoundaryBlocksPerSm<T>) k_boundary(const NumArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BoundaryShared<T> &sh = ((BoundaryShared<T> *)smem_raw)[threadIdx.x >> 5];
@@ -1738,7 +1691,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBoundaryBlocksPerSm<T, I
     if (a >= A.K) return;
     LaneAcc acc;
     acc_zero(acc);
-    boundary_any<BALL, T, INV, NQ, STS>(A, a, sh, lane, acc);
+    boundary_any<BALL, T, NQ, STS>(A, a, sh, lane, acc);
     // k_interior may be running: add atomically onto the zeroed outputs
     finish_outer<STS>(A, a, acc, lane, kAtomicAdd);
 }
@@ -1795,10 +1748,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, sizeof(T) == sizeof(float
     }
 }
 
-// boundary candidates of the problems with ball mode BALL (adds onto k_interior_batch's
-// values, as k_boundary adds onto k_interior's)
-template <int BALL, typename T, bool INV>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, kBoundaryBlocksPerSm<T, INV>)
+// boundary candidates of the singular-kernel problems with ball mode BALL (adds onto
+// k_interior_batch's values, as k_boundary adds onto k_interior's)
+template <int BALL, typename T>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, kBoundaryBlocksPerSm<T>)
     k_boundary_batch(const NumArgs *__restrict__ As, const BatchItem *__restrict__ items, int n_items, int *counter)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1816,8 +1769,32 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBoundaryBlocksPerSm<T, I
         for (int a = w.a0; a < w.a1; a++) {
             LaneAcc acc;
             acc_zero(acc);
-            boundary_any<BALL, T, INV>(A, a, sh, lane, acc);
+            boundary_any<BALL, T>(A, a, sh, lane, acc);
             finish_outer(A, a, acc, lane, kAdd);
+            __syncwarp();
+        }
+    }
+}
+
+// all candidates of the constant-kernel problems with ball mode BALL (as k_const)
+template <int BALL, typename T>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, kConstBlocksPerSm<T>)
+    k_const_batch(const NumArgs *__restrict__ As, const BatchItem *__restrict__ items, int n_items, int *counter)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ConstShared<BALL, T> &sh = ((ConstShared<BALL, T> *)smem_raw)[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    for (int it = next_item(counter, lane); it < n_items; it = next_item(counter, lane)) {
+        const BatchItem w = items[it];
+        const NumArgs &A = As[w.p];
+#ifdef NL_CHECKS
+        if (w.a0 < 0 || w.a1 > A.K || A.nbr_ptr[w.a0] < 0 || A.nbr_ptr[w.a1] > A.E) {
+            atomicOr(A.err, 32);   // debug build: bad work item recorded (bit 32) and skipped
+            continue;
+        }
+#endif
+        for (int a = w.a0; a < w.a1; a++) {
+            const_outer<BALL, T, 0>(A, a, sh, lane);
             __syncwarp();
         }
     }
@@ -1871,26 +1848,31 @@ __device__ __forceinline__ void deferred_item(const NumArgs &A, const DeferItem 
                   (unsigned long long)nlg::record_hash(a, b, q - c.q0, kind, nv, ncap));
 }
 
-template <int BALL>
+template <int BALL, bool INV>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_deferred(const NumArgs A)
 {
-    __shared__ nlg::ClipBuf cb[kWarpsPerBlock];
+    __shared__ nlg::ClipBuf cb[INV ? kWarpsPerBlock : 1];
     const int n = min(*A.defer_n, A.defer_cap);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        deferred_item<BALL>(A, A.defer[i], A.dval, A.defer_cap, i, cb[threadIdx.x >> 5], threadIdx.x & 31);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        if constexpr (INV)
+            deferred_item<BALL>(A, A.defer[i], A.dval, A.defer_cap, i, cb[threadIdx.x >> 5], threadIdx.x & 31);
+        else
+            deferred_const<BALL>(A, A.defer[i], A.dval, A.defer_cap, i);
+    }
 }
 
 // the queue of one batched boundary launch (items of its problems, As indexed by qp >> 8)
-template <int BALL>
+template <int BALL, bool INV>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
     k_deferred_batch(const NumArgs *__restrict__ As, const DeferItem *__restrict__ items, const int *count, int cap)
 {
-    __shared__ nlg::ClipBuf cb[kWarpsPerBlock];
+    __shared__ nlg::ClipBuf cb[INV ? kWarpsPerBlock : 1];
     const int n = min(*count, cap);
     float *dv = defer_values(const_cast<DeferItem *>(items), cap);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const DeferItem d = items[i];
-        deferred_item<BALL>(As[d.qp >> 8], d, dv, cap, i, cb[threadIdx.x >> 5], threadIdx.x & 31);
+        if constexpr (INV) deferred_item<BALL>(As[d.qp >> 8], d, dv, cap, i, cb[threadIdx.x >> 5], threadIdx.x & 31);
+        else deferred_const<BALL>(As[d.qp >> 8], d, dv, cap, i);
     }
 }
 
@@ -2225,6 +2207,8 @@ __global__ void __launch_bounds__(256)
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
+// ball mode of the constant-kernel launches: cfg.ball, or nlq::kBallNgonAny (api.cu)
+int nl_const_ball(const nl_plan *P);
 // kernel arguments of one assembled problem (api.cu)
 nl_status nl_fill_args(nl_ctx *ctx, const nl_plan *P, nlq::NumArgs &A, bool stats);
 
@@ -2247,8 +2231,8 @@ nl_status nl_launch_boundary_batch_f64(nl_ctx *ctx, int ball, bool inv, const nl
                                        const nlq::BatchItem *items, int n_items, int *counter, int blocks,
                                        bool set_attr);
 // the deferred items of one float boundary launch (queue `items`, fill count *count)
-nl_status nl_launch_deferred_batch_f32(nl_ctx *ctx, int ball, const nlq::NumArgs *dA, const nlq::DeferItem *items,
-                                       const int *count, int cap);
+nl_status nl_launch_deferred_batch_f32(nl_ctx *ctx, int ball, bool inv, const nlq::NumArgs *dA,
+                                       const nlq::DeferItem *items, const int *count, int cap);
 // grid of the deferred-item kernels: two blocks per SM (a grid-stride loop covers any count)
 nl_status nl_deferred_blocks(nl_ctx *ctx, int *blocks);
 // resident blocks per SM of the interior launch (ball < 0) or of a boundary launch
@@ -2290,8 +2274,7 @@ template <typename T, int STS = -1>
 nl_status nl_numeric_interior_same(nl_ctx *ctx, const nlq::NumArgs &A, unsigned grid, unsigned threads, nl_status s)
 {
     if (s != NL_OK) return s;
-    if (A.kernel == NL_KERNEL_INV_DIST) nlq::k_interior<T, STS, 1><<<grid, threads, 0, ctx->stream>>>(A);
-    else nlq::k_interior<T, STS, 0><<<grid, threads, 0, ctx->stream>>>(A);
+    nlq::k_interior<T, STS><<<grid, threads, 0, ctx->stream>>>(A);
     ++ctx->launches;
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? NL_OK : nl_cuda_fail(ctx, e, "k_interior launch");
@@ -2303,8 +2286,7 @@ template <typename T, int STS = -1>
 nl_status nl_numeric_interior_join(nl_ctx *ctx, const nlq::NumArgs &A, unsigned grid, unsigned threads, nl_status s)
 {
     if (s == NL_OK) {
-        if (A.kernel == NL_KERNEL_INV_DIST) nlq::k_interior<T, STS, 1><<<grid, threads, 0, ctx->side[0]>>>(A);
-        else nlq::k_interior<T, STS, 0><<<grid, threads, 0, ctx->side[0]>>>(A);
+        nlq::k_interior<T, STS><<<grid, threads, 0, ctx->side[0]>>>(A);
         ++ctx->launches;
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) s = nl_cuda_fail(ctx, e, "k_interior launch");

@@ -5,50 +5,55 @@
 
 namespace {
 
-constexpr size_t kBoundarySmem = sizeof(nlq::BoundaryShared<float>) * nlq::kWarpsPerBlock;
-
-template <int BALL, bool INV>
-nl_status boundary(nl_ctx *ctx, const nlq::NumArgs *dA, const nlq::BatchItem *items, int n_items, int *counter,
-                   int blocks, bool set_attr, int *per_sm)
+// one launch of a persistent kernel; SH: its per-warp shared memory
+template <typename SH, typename K>
+nl_status launch(nl_ctx *ctx, K kernel, const nlq::NumArgs *dA, const nlq::BatchItem *items, int n_items, int *counter,
+                 int blocks, bool set_attr, int *per_sm)
 {
+    const size_t smem = sizeof(SH) * nlq::kWarpsPerBlock;
+    if (per_sm || set_attr)
+        NL_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (per_sm) {
-        NL_CK(cudaFuncSetAttribute(nlq::k_boundary_batch<BALL, float, INV>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBoundarySmem));
-        NL_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, nlq::k_boundary_batch<BALL, float, INV>,
-                                                            nlq::kWarpsPerBlock * 32, kBoundarySmem));
+        NL_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kernel, nlq::kWarpsPerBlock * 32, smem));
         return NL_OK;
     }
-    if (set_attr)
-        NL_CK(cudaFuncSetAttribute(nlq::k_boundary_batch<BALL, float, INV>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBoundarySmem));
-    nlq::k_boundary_batch<BALL, float, INV><<<blocks, nlq::kWarpsPerBlock * 32, kBoundarySmem, ctx->stream>>>(
-        dA, items, n_items, counter);
+    kernel<<<blocks, nlq::kWarpsPerBlock * 32, smem, ctx->stream>>>(dA, items, n_items, counter);
     ++ctx->launches;
     NL_CK(cudaGetLastError());
     return NL_OK;
 }
 
-template <bool INV>
-nl_status boundary_ball(nl_ctx *ctx, int ball, const nlq::NumArgs *dA, const nlq::BatchItem *items, int n_items,
-                        int *counter, int blocks, bool set_attr, int *per_sm)
+template <int BALL>
+nl_status boundary(nl_ctx *ctx, bool inv, const nlq::NumArgs *dA, const nlq::BatchItem *items, int n_items,
+                   int *counter, int blocks, bool set_attr, int *per_sm)
 {
+    if constexpr (BALL != nlq::kBallNgonAny && !nlq::kSupportBall<BALL>)
+        if (inv)
+            return launch<nlq::BoundaryShared<float>>(ctx, nlq::k_boundary_batch<BALL, float>, dA, items, n_items, counter,
+                                                   blocks, set_attr, per_sm);
+    if (inv) return nl_fail(ctx, NL_EINVAL, "unknown ball mode");
+    return launch<nlq::ConstShared<BALL, float>>(ctx, nlq::k_const_batch<BALL, float>, dA, items, n_items, counter, blocks,
+                                              set_attr, per_sm);
+}
+
+nl_status boundary_ball(nl_ctx *ctx, int ball, bool inv, const nlq::NumArgs *dA, const nlq::BatchItem *items,
+                        int n_items, int *counter, int blocks, bool set_attr, int *per_sm)
+{
+#define NL_CASE(B) \
+    case B: return boundary<B>(ctx, inv, dA, items, n_items, counter, blocks, set_attr, per_sm)
     switch (ball) {
-    case NL_BALL_BARYCENTER:
-        return boundary<NL_BALL_BARYCENTER, INV>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_NOCAPS: return boundary<NL_BALL_NOCAPS, INV>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_APPROXCAPS:
-        return boundary<NL_BALL_APPROXCAPS, INV>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_EXACTCAPS:
-        return boundary<NL_BALL_EXACTCAPS, INV>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_NGON: return boundary<NL_BALL_NGON, INV>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_OVERLAP:
-        return boundary<NL_BALL_OVERLAP, INV>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_BARY_NOCAPS:
-        return boundary<NL_BALL_BARY_NOCAPS, false>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_BARY_APPROXCAPS:
-        return boundary<NL_BALL_BARY_APPROXCAPS, false>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
+        NL_CASE(NL_BALL_BARYCENTER);
+        NL_CASE(NL_BALL_NOCAPS);
+        NL_CASE(NL_BALL_APPROXCAPS);
+        NL_CASE(NL_BALL_EXACTCAPS);
+        NL_CASE(NL_BALL_NGON);
+        NL_CASE(nlq::kBallNgonAny);
+        NL_CASE(NL_BALL_OVERLAP);
+        NL_CASE(NL_BALL_BARY_NOCAPS);
+        NL_CASE(NL_BALL_BARY_APPROXCAPS);
     default: return nl_fail(ctx, NL_EINVAL, "unknown ball mode");
     }
+#undef NL_CASE
 }
 
 }  // namespace
@@ -66,32 +71,31 @@ nl_status nl_launch_boundary_batch_f32(nl_ctx *ctx, int ball, bool inv, const nl
                                        const nlq::BatchItem *items, int n_items, int *counter, int blocks,
                                        bool set_attr)
 {
-    return inv ? boundary_ball<true>(ctx, ball, dA, items, n_items, counter, blocks, set_attr, nullptr)
-               : boundary_ball<false>(ctx, ball, dA, items, n_items, counter, blocks, set_attr, nullptr);
+    return boundary_ball(ctx, ball, inv, dA, items, n_items, counter, blocks, set_attr, nullptr);
 }
 
-nl_status nl_launch_deferred_batch_f32(nl_ctx *ctx, int ball, const nlq::NumArgs *dA, const nlq::DeferItem *items,
-                                       const int *count, int cap)
+nl_status nl_launch_deferred_batch_f32(nl_ctx *ctx, int ball, bool inv, const nlq::NumArgs *dA,
+                                       const nlq::DeferItem *items, const int *count, int cap)
 {
     int blocks = 0;
     nl_status s = nl_deferred_blocks(ctx, &blocks);
     if (s != NL_OK) return s;
     const unsigned threads = nlq::kWarpsPerBlock * 32;
-    switch (ball) {
-    case NL_BALL_BARYCENTER:
-        nlq::k_deferred_batch<NL_BALL_BARYCENTER><<<blocks, threads, 0, ctx->stream>>>(dA, items, count, cap); break;
-    case NL_BALL_NOCAPS:
-        nlq::k_deferred_batch<NL_BALL_NOCAPS><<<blocks, threads, 0, ctx->stream>>>(dA, items, count, cap); break;
-    case NL_BALL_APPROXCAPS:
-        nlq::k_deferred_batch<NL_BALL_APPROXCAPS><<<blocks, threads, 0, ctx->stream>>>(dA, items, count, cap); break;
-    case NL_BALL_EXACTCAPS:
-        nlq::k_deferred_batch<NL_BALL_EXACTCAPS><<<blocks, threads, 0, ctx->stream>>>(dA, items, count, cap); break;
-    case NL_BALL_NGON:
-        nlq::k_deferred_batch<NL_BALL_NGON><<<blocks, threads, 0, ctx->stream>>>(dA, items, count, cap); break;
-    case NL_BALL_OVERLAP:
-        nlq::k_deferred_batch<NL_BALL_OVERLAP><<<blocks, threads, 0, ctx->stream>>>(dA, items, count, cap); break;
+#define NL_CASE(B)                                                                                             \
+    case B:                                                                                                    \
+        if (inv) nlq::k_deferred_batch<B, true><<<blocks, threads, 0, ctx->stream>>>(dA, items, count, cap);   \
+        else nlq::k_deferred_batch<B, false><<<blocks, threads, 0, ctx->stream>>>(dA, items, count, cap);      \
+        break
+    switch (ball == nlq::kBallNgonAny ? (int)NL_BALL_NGON : ball) {
+        NL_CASE(NL_BALL_BARYCENTER);
+        NL_CASE(NL_BALL_NOCAPS);
+        NL_CASE(NL_BALL_APPROXCAPS);
+        NL_CASE(NL_BALL_EXACTCAPS);
+        NL_CASE(NL_BALL_NGON);
+        NL_CASE(NL_BALL_OVERLAP);
     default: return nl_fail(ctx, NL_EINVAL, "no deferred items for this ball mode");
     }
+#undef NL_CASE
     ++ctx->launches;
     nlq::k_defer_merge_batch<float><<<blocks, 256, 0, ctx->stream>>>(dA, items, count, cap); ++ctx->launches;
     NL_CK(cudaGetLastError());
@@ -105,6 +109,5 @@ nl_status nl_batch_occupancy_f32(nl_ctx *ctx, int ball, bool inv, int *per_sm)
                                                             nlq::kWarpsPerBlock * 32, 0));
         return NL_OK;
     }
-    return inv ? boundary_ball<true>(ctx, ball, nullptr, nullptr, 0, nullptr, 0, false, per_sm)
-               : boundary_ball<false>(ctx, ball, nullptr, nullptr, 0, nullptr, 0, false, per_sm);
+    return boundary_ball(ctx, ball, inv, nullptr, nullptr, 0, nullptr, 0, false, per_sm);
 }

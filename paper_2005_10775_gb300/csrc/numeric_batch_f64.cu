@@ -5,50 +5,55 @@
 
 namespace {
 
-constexpr size_t kBoundarySmem = sizeof(nlq::BoundaryShared<double>) * nlq::kWarpsPerBlock;
-
-template <int BALL, bool INV>
-nl_status boundary(nl_ctx *ctx, const nlq::NumArgs *dA, const nlq::BatchItem *items, int n_items, int *counter,
-                   int blocks, bool set_attr, int *per_sm)
+// one launch of a persistent kernel; SH: its per-warp shared memory
+template <typename SH, typename K>
+nl_status launch(nl_ctx *ctx, K kernel, const nlq::NumArgs *dA, const nlq::BatchItem *items, int n_items, int *counter,
+                 int blocks, bool set_attr, int *per_sm)
 {
+    const size_t smem = sizeof(SH) * nlq::kWarpsPerBlock;
+    if (per_sm || set_attr)
+        NL_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (per_sm) {
-        NL_CK(cudaFuncSetAttribute(nlq::k_boundary_batch<BALL, double, INV>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBoundarySmem));
-        NL_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, nlq::k_boundary_batch<BALL, double, INV>,
-                                                            nlq::kWarpsPerBlock * 32, kBoundarySmem));
+        NL_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kernel, nlq::kWarpsPerBlock * 32, smem));
         return NL_OK;
     }
-    if (set_attr)
-        NL_CK(cudaFuncSetAttribute(nlq::k_boundary_batch<BALL, double, INV>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBoundarySmem));
-    nlq::k_boundary_batch<BALL, double, INV><<<blocks, nlq::kWarpsPerBlock * 32, kBoundarySmem, ctx->stream>>>(
-        dA, items, n_items, counter);
+    kernel<<<blocks, nlq::kWarpsPerBlock * 32, smem, ctx->stream>>>(dA, items, n_items, counter);
     ++ctx->launches;
     NL_CK(cudaGetLastError());
     return NL_OK;
 }
 
-template <bool INV>
-nl_status boundary_ball(nl_ctx *ctx, int ball, const nlq::NumArgs *dA, const nlq::BatchItem *items, int n_items,
-                        int *counter, int blocks, bool set_attr, int *per_sm)
+template <int BALL>
+nl_status boundary(nl_ctx *ctx, bool inv, const nlq::NumArgs *dA, const nlq::BatchItem *items, int n_items,
+                   int *counter, int blocks, bool set_attr, int *per_sm)
 {
+    if constexpr (BALL != nlq::kBallNgonAny && !nlq::kSupportBall<BALL>)
+        if (inv)
+            return launch<nlq::BoundaryShared<double>>(ctx, nlq::k_boundary_batch<BALL, double>, dA, items, n_items, counter,
+                                                   blocks, set_attr, per_sm);
+    if (inv) return nl_fail(ctx, NL_EINVAL, "unknown ball mode");
+    return launch<nlq::ConstShared<BALL, double>>(ctx, nlq::k_const_batch<BALL, double>, dA, items, n_items, counter, blocks,
+                                              set_attr, per_sm);
+}
+
+nl_status boundary_ball(nl_ctx *ctx, int ball, bool inv, const nlq::NumArgs *dA, const nlq::BatchItem *items,
+                        int n_items, int *counter, int blocks, bool set_attr, int *per_sm)
+{
+#define NL_CASE(B) \
+    case B: return boundary<B>(ctx, inv, dA, items, n_items, counter, blocks, set_attr, per_sm)
     switch (ball) {
-    case NL_BALL_BARYCENTER:
-        return boundary<NL_BALL_BARYCENTER, INV>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_NOCAPS: return boundary<NL_BALL_NOCAPS, INV>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_APPROXCAPS:
-        return boundary<NL_BALL_APPROXCAPS, INV>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_EXACTCAPS:
-        return boundary<NL_BALL_EXACTCAPS, INV>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_NGON: return boundary<NL_BALL_NGON, INV>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_OVERLAP:
-        return boundary<NL_BALL_OVERLAP, INV>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_BARY_NOCAPS:
-        return boundary<NL_BALL_BARY_NOCAPS, false>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
-    case NL_BALL_BARY_APPROXCAPS:
-        return boundary<NL_BALL_BARY_APPROXCAPS, false>(ctx, dA, items, n_items, counter, blocks, set_attr, per_sm);
+        NL_CASE(NL_BALL_BARYCENTER);
+        NL_CASE(NL_BALL_NOCAPS);
+        NL_CASE(NL_BALL_APPROXCAPS);
+        NL_CASE(NL_BALL_EXACTCAPS);
+        NL_CASE(NL_BALL_NGON);
+        NL_CASE(nlq::kBallNgonAny);
+        NL_CASE(NL_BALL_OVERLAP);
+        NL_CASE(NL_BALL_BARY_NOCAPS);
+        NL_CASE(NL_BALL_BARY_APPROXCAPS);
     default: return nl_fail(ctx, NL_EINVAL, "unknown ball mode");
     }
+#undef NL_CASE
 }
 
 }  // namespace
@@ -66,8 +71,7 @@ nl_status nl_launch_boundary_batch_f64(nl_ctx *ctx, int ball, bool inv, const nl
                                        const nlq::BatchItem *items, int n_items, int *counter, int blocks,
                                        bool set_attr)
 {
-    return inv ? boundary_ball<true>(ctx, ball, dA, items, n_items, counter, blocks, set_attr, nullptr)
-               : boundary_ball<false>(ctx, ball, dA, items, n_items, counter, blocks, set_attr, nullptr);
+    return boundary_ball(ctx, ball, inv, dA, items, n_items, counter, blocks, set_attr, nullptr);
 }
 
 nl_status nl_batch_occupancy_f64(nl_ctx *ctx, int ball, bool inv, int *per_sm)
@@ -77,6 +81,5 @@ nl_status nl_batch_occupancy_f64(nl_ctx *ctx, int ball, bool inv, int *per_sm)
                                                             nlq::kWarpsPerBlock * 32, 0));
         return NL_OK;
     }
-    return inv ? boundary_ball<true>(ctx, ball, nullptr, nullptr, 0, nullptr, 0, false, per_sm)
-               : boundary_ball<false>(ctx, ball, nullptr, nullptr, 0, nullptr, 0, false, per_sm);
+    return boundary_ball(ctx, ball, inv, nullptr, nullptr, 0, nullptr, 0, false, per_sm);
 }

@@ -1,0 +1,1057 @@
+// numeric_const.cuh -- numeric phase of the constant kernel psi = c (included by numeric.cuh, whose
+// types it uses).  One kernel, k_const, does a triangle's interior and boundary candidates.
+//
+// With psi = c the inner integrand c (1, phi_b, phi_b phi_b^T) is quadratic on T_b, and every inner
+// rule of the library integrates quadratics exactly, so the rule's sums over a region equal the
+// region's moments.  The moments are taken once per region from its boundary, in T_b's own
+// barycentric coordinates, instead of point by point over a fan: a whole T_b needs no arithmetic
+// beyond its area, and a cut T_b needs the parameters t of its cut edges and one closing chain.
+// n_qp_pairs still counts the rule's points, which the sums stand for.
+//
+// Moments (Mom): with l = (l1, l2) the barycentric coordinates of T_b's vertices 1 and 2, each
+// scaled so that the whole triangle has all six equal to 1:
+//     S0 = int 1 / |T|, S1 = 3 int l1 / |T|, S2 = 3 int l2 / |T|,
+//     S11 = 6 int l1^2 / |T|, S22 = 6 int l2^2 / |T|, S12 = 12 int l1 l2 / |T|.
+// A directed boundary segment p -> q contributes the triangle (0, p, q), 0 = T_b's vertex 0 (Green);
+// pieces of edges 0 and 2 pass through that origin and contribute nothing, and a piece [t0, t1] of
+// edge 1 contributes F(t1) - F(t0) with the polynomials of edge1_add.  T_b's vertices are renumbered
+// per item so that the origin belongs to the region (a vertex inside, or the start of the edge that is
+// cut twice): the contributions are then of the region's own size and nothing cancels, also where the
+// region is a small part of T_b (mom_turn puts the moments back).
+//
+// A pair's block is linear in twelve sums over its outer points (acc rows): P_i,c = sum_q W_q
+// phi_a,i S_c (c = 0, 1, 2) and Q = sum_q W_q (S11, S22, S12); the other entries of M_ab and M_bb
+// follow from phi_0 = 1 - phi_1 - phi_2 and sum_i phi_a,i = 1 (pair_block).
+#pragma once
+
+namespace nlq {
+
+// ball modes of k_const beyond nl_ball: an N-gon whose vertices are not those of a regular polygon
+constexpr int kBallNgonAny = 16;
+
+template <int BALL>
+constexpr int kGeoBall = BALL == kBallNgonAny ? NL_BALL_NGON : BALL;
+
+template <int BALL>
+constexpr bool kSupportBall = BALL == NL_BALL_BARY_NOCAPS || BALL == NL_BALL_BARY_APPROXCAPS;
+
+template <typename T>
+struct Mom {
+    T s0, s1, s2, s11, s22, s12;
+};
+
+template <typename T>
+__device__ __forceinline__ void mom_set(Mom<T> &M, T v)
+{
+    M.s0 = M.s1 = M.s2 = M.s11 = M.s22 = M.s12 = v;
+}
+
+// boundary segment p -> q, (l1, l2) coordinates
+template <typename T>
+__device__ __forceinline__ void seg_add(Mom<T> &M, T p1, T p2, T q1, T q2)
+{
+    const T cr = p1 * q2 - q1 * p2, a1 = p1 + q1, a2 = p2 + q2;
+    M.s0 += cr;
+    M.s1 += cr * a1;
+    M.s2 += cr * a2;
+    M.s11 += cr * (a1 * a1 - p1 * q1);
+    M.s22 += cr * (a2 * a2 - p2 * q2);
+    M.s12 += cr * (a1 * a2 + p1 * p2 + q1 * q2);
+}
+
+// the piece of edge 1 (from (1, 0) to (0, 1)) up to its point (1 - t, t), times sg
+template <typename T>
+__device__ __forceinline__ void edge1_add(Mom<T> &M, T t, T sg)
+{
+    const T st = sg * t, tt = st * t;
+    M.s0 += st;
+    M.s1 += st * ((T)2 - t);
+    M.s2 += tt;
+    M.s11 += st * ((T)3 - t * ((T)3 - t));
+    M.s22 += tt * t;
+    M.s12 += tt * ((T)3 - (T)2 * t);
+}
+
+// a point of weight w (relative to |T|)
+template <typename T>
+__device__ __forceinline__ void point_add(Mom<T> &M, T l1, T l2, T w)
+{
+    M.s0 += w;
+    M.s1 += (T)3 * w * l1;
+    M.s2 += (T)3 * w * l2;
+    M.s11 += (T)6 * w * l1 * l1;
+    M.s22 += (T)6 * w * l2 * l2;
+    M.s12 += (T)12 * w * l1 * l2;
+}
+
+// moments about vertex r's numbering (vertices r, r + 1, r + 2 as 0, 1, 2) to T_b's own
+template <typename T>
+__device__ __forceinline__ void mom_turn(Mom<T> &M, int r)
+{
+    if (r != 0) {
+        const bool one = r == 1;
+        const T s = one ? M.s1 : M.s2, ss = one ? M.s11 : M.s22, s12 = M.s1 + M.s2;
+        const T z = (T)3 * M.s0 - s12, zz = (T)6 * M.s0 - (T)4 * s12 + (M.s11 + M.s22 + M.s12);
+        M.s12 = (T)4 * s - (T)2 * ss - M.s12;
+        M.s1 = one ? z : s;
+        M.s2 = one ? s : z;
+        M.s11 = one ? zz : ss;
+        M.s22 = one ? ss : zz;
+    }
+}
+
+// moments of m about the point p in T_b's own coordinates: those of l + p
+template <typename T>
+__device__ __forceinline__ void mom_shift(Mom<T> &M, T p1, T p2)
+{
+    M.s12 += (T)12 * p1 * p2 * M.s0 + (T)4 * (p1 * M.s2 + p2 * M.s1);
+    M.s11 += p1 * ((T)6 * p1 * M.s0 + (T)4 * M.s1);
+    M.s22 += p2 * ((T)6 * p2 * M.s0 + (T)4 * M.s2);
+    M.s1 += (T)3 * p1 * M.s0;
+    M.s2 += (T)3 * p2 * M.s0;
+}
+
+// M_ab (9) and the upper M_bb (00 11 22 01 02 12) from a pair's sums P, Q and akc = c |T_b|
+template <typename T>
+__device__ __forceinline__ void pair_block(T akc, const T *P, const T *Q, T *mab, T *mbb)
+{
+    const T k3 = akc * (T)(1.0 / 3.0);
+    for (int i = 0; i < 3; i++) {
+        const T m1 = P[3 * i + 1] * k3, m2 = P[3 * i + 2] * k3;
+        mab[3 * i] = akc * P[3 * i] - m1 - m2;
+        mab[3 * i + 1] = m1;
+        mab[3 * i + 2] = m2;
+    }
+    const T k6 = akc * (T)(1.0 / 6.0), k12 = akc * (T)(1.0 / 12.0);
+    const T b11 = k6 * Q[0], b22 = k6 * Q[1], b12 = k12 * Q[2];
+    const T p1 = mab[1] + mab[4] + mab[7], p2 = mab[2] + mab[5] + mab[8];
+    const T p00 = mab[0] + mab[3] + mab[6];   // sum_q W int phi_0
+    const T b01 = p1 - b11 - b12, b02 = p2 - b12 - b22;
+    mbb[0] = p00 - b01 - b02;
+    mbb[1] = b11;
+    mbb[2] = b22;
+    mbb[3] = b01;
+    mbb[4] = b02;
+    mbb[5] = b12;
+}
+
+// FP64 data of a candidate (FP64 path)
+struct Cand64 {
+    double x0, y0, e1x, e1y, e2x, e2y, inv, area;   // vertex 0, edges 0 -> 1 and 0 -> 2, 1 / det, |T|
+};
+struct CandNone {};
+
+template <typename T>
+using CandT = typename std::conditional<sizeof(T) == sizeof(double), Cand64, CandNone>::type;
+
+// Frame of one item: T_b's vertex 0 and edges relative to x, and 1 / det
+template <typename T>
+struct Frame {
+    T rx, ry;   // x - vertex 0
+    T e1x, e1y, e2x, e2y, inv;
+};
+
+template <typename T>
+__device__ __forceinline__ void frame_l(const Frame<T> &f, T px, T py, T &l1, T &l2)   // p relative to x
+{
+    const T cx = px + f.rx, cy = py + f.ry;
+    l1 = (cx * f.e2y - f.e2x * cy) * f.inv;
+    l2 = (f.e1x * cy - cx * f.e1y) * f.inv;
+}
+
+// start p (relative to x) and direction e of edge i
+template <typename T>
+__device__ __forceinline__ void frame_edge(const Frame<T> &f, int i, T &px, T &py, T &ex, T &ey)
+{
+    px = (i == 0 ? (T)0 : i == 1 ? f.e1x : f.e2x) - f.rx;
+    py = (i == 0 ? (T)0 : i == 1 ? f.e1y : f.e2y) - f.ry;
+    ex = i == 0 ? f.e1x : i == 1 ? f.e2x - f.e1x : -f.e2x;
+    ey = i == 0 ? f.e1y : i == 1 ? f.e2y - f.e1y : -f.e2y;
+}
+
+template <typename T>
+__device__ __forceinline__ T quot(T a, T b)
+{
+    if constexpr (sizeof(T) == sizeof(float)) return __fdividef(a, b);
+    else return a / b;
+}
+
+// the barycentric point at parameter t of edge i
+template <typename T>
+__device__ __forceinline__ void edge_l(int i, T t, T &l1, T &l2)
+{
+    const T u = (T)1 - t;
+    l1 = i == 0 ? t : i == 1 ? u : (T)0;
+    l2 = i == 0 ? (T)0 : i == 1 ? t : u;
+}
+
+// ---------------------------------------------------------------------------
+// Which of T_b's vertices lie in the ball (bits of `in`) and which edges with both ends outside
+// cross it twice (bits of `dbl`), in FP32, taken only when FP32 is certain (false: undecided).
+// Every function of the cut items has a single exit: an early return inside a divergent loop
+// moves the point where the warp's lanes meet again to the end of the item (the first version of
+// k_const<N-gon, float> ran 13 of 32 lanes on average for that reason).
+// ---------------------------------------------------------------------------
+// The disc: the predicates and margins of nlg::ball_walk_f32.
+__device__ __forceinline__ bool disc_status(const nlg::F2 d[3], const nlg::GeoParams &g, unsigned &in, unsigned &dbl)
+{
+    in = 0;
+    dbl = 0;
+    bool sure = true;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        const float r = d[i].x * d[i].x + d[i].y * d[i].y;
+        const bool is_in = r <= g.rin_m2;
+        sure = sure && (is_in || r > g.rout_p2);
+        if (is_in) in |= 1u << i;
+    }
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        const int j = (i + 1) % 3;
+        const float ex = d[j].x - d[i].x, ey = d[j].y - d[i].y;
+        const float a = ex * ex + ey * ey, b = d[i].x * ex + d[i].y * ey, cr = d[i].x * ey - d[i].y * ex;
+        // both ends outside and the closest point between them
+        const bool mid = !(((in >> i) | (in >> j)) & 1u) && b < 0.f && -b < a;
+        const bool hits = cr * cr <= g.rin_m2 * a, misses = cr * cr > g.rout_p2 * a;
+        if (mid && hits) dbl |= 1u << i;
+        sure = sure && !(mid && !hits && !misses);
+    }
+    return sure;
+}
+
+// The regular N-gon with corners o_0 .. o_N (o_N = o_0) on the circle of radius^2 g.poly_r2.
+// The line p + t e crosses polygon edge k exactly when it separates corners k and k + 1, that is
+// when its crossing of the circle lies on the arc between them: k comes from the angle of that
+// crossing (arctangent polynomial) and is certain when both corners are farther than tau from
+// the line, on the sides that an exit (entry) needs.  s0, s1: the corners' signed distances to
+// the line times |e|.  Returns k in [0, N); *hit = false when the line misses the circle.
+__device__ __forceinline__ int ngon_edge(const nlg::F2 &p, const nlg::F2 &e, float a, float b, float cr, bool exit_,
+                                         const nlg::GeoParams &g, const float2 *corner, bool *hit, float *s0,
+                                         float *s1)
+{
+    const float disc = a * g.poly_r2 - cr * cr;
+    *hit = disc > 0.f;
+    const float half = sqrtf(fmaxf(disc, 0.f));
+    const float t = __fdividef((exit_ ? half : -half) - b, a);
+    int k = (int)floorf(nlg::atan2_poly(p.y + t * e.y, p.x + t * e.x) * g.inv_sector);
+    if (k < 0) k += g.ngon_n;
+    const float2 o0 = corner[k], o1 = corner[k + 1];
+    *s0 = e.x * (o0.y - p.y) - e.y * (o0.x - p.x);
+    *s1 = e.x * (o1.y - p.y) - e.y * (o1.x - p.x);
+    return k;
+}
+
+// is v inside the N-gon?  v's angle names the polygon edge to test (and the next one, for an angle
+// near a corner): 1 inside, 0 outside, -1 undecided; *w: the direction of an edge v lies beyond
+__device__ __forceinline__ int ngon_holds(const nlg::F2 &v, const nlg::GeoParams &g, const float2 *corner, nlg::F2 *w)
+{
+    const float f = nlg::atan2_poly(v.y, v.x) * g.inv_sector;
+    const float fl = floorf(f);
+    int k = (int)fl, n = f - fl < 0.5f ? k - 1 : k + 1;
+    const int N = g.ngon_n;
+    k += k < 0 ? N : 0;
+    n += n < 0 ? N : 0;
+    n -= n >= N ? N : 0;
+    const float m = g.poly_m;
+    const float2 a0 = corner[k], a1 = corner[k + 1], b0 = corner[n], b1 = corner[n + 1];
+    const float ax = a1.x - a0.x, ay = a1.y - a0.y, bx = b1.x - b0.x, by = b1.y - b0.y;
+    const float oa = ax * (v.y - a0.y) - ay * (v.x - a0.x), ob = bx * (v.y - b0.y) - by * (v.x - b0.x);
+    const bool out_a = oa < -m, out_b = ob < -m;
+    w->x = out_a ? ax : bx;
+    w->y = out_a ? ay : by;
+    return out_a || out_b ? 0 : (oa > m && ob > m ? 1 : -1);
+}
+
+__device__ __forceinline__ bool ngon_status(const nlg::F2 d[3], const nlg::GeoParams &g, const float2 *corner,
+                                            unsigned &in, unsigned &dbl)
+{
+    in = 0;
+    dbl = 0;
+    bool sure = true;
+    unsigned far = 0;
+    nlg::F2 w[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};   // a polygon edge that an outside vertex lies beyond
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        const float r = d[i].x * d[i].x + d[i].y * d[i].y;
+        if (r <= g.rin_m2) in |= 1u << i;
+        else if (r > g.rout_p2) far |= 1u << i;
+    }
+    // vertices between the inscribed and the circumscribed circle: rarely more than one
+    for (unsigned todo = ~(in | far) & 7u; todo; todo &= todo - 1) {
+        const int i = __ffs(todo) - 1;
+        nlg::F2 x;
+        const int h = ngon_holds(i == 0 ? d[0] : i == 1 ? d[1] : d[2], g, corner, &x);
+        sure = sure && h >= 0;
+        if (h > 0) in |= 1u << i;
+        if (i == 0) w[0] = x;
+        if (i == 1) w[1] = x;
+        if (i == 2) w[2] = x;
+    }
+    unsigned pend = 0;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        const int j = (i + 1) % 3;
+        const float ex = d[j].x - d[i].x, ey = d[j].y - d[i].y;
+        const float a = ex * ex + ey * ey, b = d[i].x * ex + d[i].y * ey, cr = d[i].x * ey - d[i].y * ex;
+        const bool both = ((far >> i) & (far >> j) & 1u) != 0;
+        // edges with both ends outside that miss the polygon: the line misses the circle; both ends
+        // beyond the circle and the closest point is one of them; or an end lies beyond a polygon
+        // edge and the edge leads away from it
+        const bool miss = cr * cr > g.rout_p2 * a || (both && !(b < 0.f && -b < a)) ||
+                          (!((far >> i) & 1u) && w[i].x * ey - w[i].y * ex <= 0.f) ||
+                          (!((far >> j) & 1u) && w[j].x * ey - w[j].y * ex >= 0.f);
+        const bool out = !(((in >> i) | (in >> j)) & 1u);
+        const bool hits = both && cr * cr <= g.rin_m2 * a;   // the line meets the inscribed circle
+        if (out && !miss) {
+            if (hits) dbl |= 1u << i;
+            else pend |= 1u << i;
+        }
+    }
+    for (; pend; pend &= pend - 1) {
+        // an outside edge whose line passes between the two circles, or that starts or ends there
+        const int i = __ffs(pend) - 1;
+        const nlg::F2 p = i == 0 ? d[0] : i == 1 ? d[1] : d[2], q = i == 0 ? d[1] : i == 1 ? d[2] : d[0];
+        const nlg::F2 e = {q.x - p.x, q.y - p.y};
+        const float a = e.x * e.x + e.y * e.y, b = p.x * e.x + p.y * e.y, cr = p.x * e.y - p.y * e.x;
+        const float le = sqrtf(a), m = g.tau * le;
+        float n0, n1, x0, x1;
+        bool hit;
+        const int kn = ngon_edge(p, e, a, b, cr, false, g, corner, &hit, &n0, &n1);
+        const int kx = ngon_edge(p, e, a, b, cr, true, g, corner, &hit, &x0, &x1);
+        // every corner on one side of the line: no crossing
+        const bool none = kn == kx && ((n0 > m && n1 > m) || (n0 < -m && n1 < -m));
+        // the line crosses edges kn and kx: between p and q (both outside by tau), or not
+        const float2 on = corner[kn], on1 = corner[kn + 1], ox = corner[kx], ox1 = corner[kx + 1];
+        const float ax = on1.x - on.x, ay = on1.y - on.y, cx = ox1.x - ox.x, cy = ox1.y - ox.y;
+        const float dn = ax * e.y - ay * e.x, dx = cx * e.y - cy * e.x;
+        const float graze = 0.02f * le * g.poly_side;   // below that the crossing's place is too uncertain
+        const float tn = __fdividef(ay * (p.x - on.x) - ax * (p.y - on.y), dn);
+        const float tx = __fdividef(cy * (p.x - ox.x) - cx * (p.y - ox.y), dx);
+        const float mt = __fdividef(g.tau, le);
+        const bool cross = kn != kx && n0 > m && n1 < -m && x0 < -m && x1 > m && fabsf(dn) > graze && fabsf(dx) > graze;
+        const bool inside = cross && tn > mt && tx < 1.f - mt, beyond = cross && (tx < -mt || tn > 1.f + mt);
+        if (hit && inside) dbl |= 1u << i;
+        sure = sure && hit && (none || inside || beyond);
+    }
+    return sure;
+}
+
+// the parameter t of edge (p, e) where it leaves (enters) the disc
+template <typename T>
+__device__ __forceinline__ T disc_cross(T px, T py, T ex, T ey, T r2, bool exit_)
+{
+    const T a = ex * ex + ey * ey, b = px * ex + py * ey, c = px * px + py * py - r2;
+    T ds = b * b - a * c;
+    ds = ds > (T)0 ? ds : (T)0;
+    const T s = sqrt(ds);
+    // roots of a t^2 + 2 b t + c without cancellation: the far one from w, the other from c / w
+    const T w = b > (T)0 ? -(b + s) : s - b;
+    const bool num = exit_ == (b <= (T)0);
+    return quot(num ? w : c, num ? a : w);
+}
+
+// corner k of the polygon in the quadrature's precision
+template <typename T>
+__device__ __forceinline__ void corner_of(const NumArgs &A, const float2 *corner, int k, T &x, T &y)
+{
+    if constexpr (sizeof(T) == sizeof(float)) {
+        const float2 o = corner[k];
+        x = o.x;
+        y = o.y;
+    } else {
+        const int kk = k >= A.geo.ngon_n ? k - A.geo.ngon_n : k;
+        const double2 o = __ldg((const double2 *)A.geo.ngon + kk);
+        x = o.x;
+        y = o.y;
+    }
+}
+
+// Moments of one cut (q, b): the region's structure (vertices in, edges cut, polygon edges met) from
+// certain FP32 predicates, its coordinates in T.  1 done, 0 empty region, -1 the FP64 geometry decides.
+// The vertex count, kind and cap count are those of the FP64 region (the records' content).
+// Every lane of the warp calls it (with data of some item: `live` says whether the lane's counts).
+template <int BALL, typename T>
+__device__ __forceinline__ int cut_item(const NumArgs &A, bool live, const nlg::F2 v[3], const Frame<T> &f0, T inv_area,
+                                        const float2 *corner, Mom<T> &M, int &nv, int &kind, int &ncap)
+{
+    constexpr bool kPoly = BALL == NL_BALL_NGON;
+    const nlg::GeoParams &g = A.geo;
+    unsigned in, dbl;
+    const bool sure = kPoly ? ngon_status(v, g, corner, in, dbl) : disc_status(v, g, in, dbl);
+    // the new vertex 0: the vertex inside, the first of two inside, the start of the edge cut twice
+    const unsigned who = in ? in : dbl;
+    const int rot = (who & 1u) && !(who & 4u && in) ? 0 : who & 4u ? (who & 2u ? 1 : 2) : who & 2u ? 1 : 0;
+    in = ((in >> rot) | (in << (3 - rot))) & 7u;
+    dbl = ((dbl >> rot) | (dbl << (3 - rot))) & 7u;
+    const nlg::F2 d[3] = {rot == 0 ? v[0] : rot == 1 ? v[1] : v[2], rot == 0 ? v[1] : rot == 1 ? v[2] : v[0],
+                          rot == 0 ? v[2] : rot == 1 ? v[0] : v[1]};
+    Frame<T> f = f0;
+    if (rot != 0) {
+        const T ox = rot == 1 ? f0.e1x : f0.e2x, oy = rot == 1 ? f0.e1y : f0.e2y;   // the new vertex 0
+        const T wx = rot == 1 ? f0.e2x : f0.e1x, wy = rot == 1 ? f0.e2y : f0.e1y;   // the other of 1, 2
+        f.rx = f0.rx - ox;
+        f.ry = f0.ry - oy;
+        const T tx = wx - ox, ty = wy - oy;
+        f.e1x = rot == 1 ? tx : -ox;
+        f.e1y = rot == 1 ? ty : -oy;
+        f.e2x = rot == 1 ? -ox : tx;
+        f.e2y = rot == 1 ? -oy : ty;
+    }
+    const unsigned nxt = ((in >> 1) | (in << 2)) & 7u;   // bit i: the end of edge i is inside
+    unsigned X = (in & ~nxt) | dbl;                      // edges that leave the ball
+    const unsigned N = (~in & nxt) | dbl;                // edges that enter it
+    const int narc = __popc(X);
+    int n = __popc(in) + 2 * narc;
+    bool known = sure;
+    if (BALL == NL_BALL_APPROXCAPS) {
+        known = known && g.cap_level <= 2;
+        n += narc * ((1 << g.cap_level) - 1);
+    }
+    bool empty = BALL == NL_BALL_EXACTCAPS ? n < 2 : n < 3;
+    if (kPoly && X == 0u && in != 7u) {
+        // no crossing: empty, unless the polygon lies inside T_b (x inside it)
+        const float o0 = d[0].x * d[1].y - d[0].y * d[1].x, o1 = d[1].x * d[2].y - d[1].y * d[2].x;
+        const float o2 = d[2].x * d[0].y - d[2].y * d[0].x;
+        known = known && !(fminf(o0, fminf(o1, o2)) >= 0.f);
+        empty = true;
+    }
+    // a polygon region with two crossings and no vertex of T_b inside has its corners still to count
+    if (kPoly && X != 0u) empty = false;
+    mom_set(M, in == 7u ? (T)1 : (T)0);
+    ncap = 0;
+    bool go = live && known && !empty;
+    __syncwarp();
+    while (__any_sync(0xffffffffu, go && X != 0u)) {   // one exit and the next entry (rarely more)
+        if (go && X != 0u) {
+            const int i = __ffs(X) - 1;
+            X &= X - 1;
+            // the next edge that enters, along the boundary of T_b
+            const int i1 = i == 2 ? 0 : i + 1, i2 = i1 == 2 ? 0 : i1 + 1;
+            const int j = (N >> i1) & 1u ? i1 : ((N >> i2) & 1u ? i2 : i);
+            T px, py, ex, ey, sx, sy, gx, gy, tx, tn;
+            frame_edge(f, i, px, py, ex, ey);
+            frame_edge(f, j, sx, sy, gx, gy);
+            int kx = 0, kn = 0;
+            if constexpr (kPoly) {
+                float s0, s1, n0, n1;
+                bool hx, hn;
+                const nlg::F2 p = i == 0 ? d[0] : i == 1 ? d[1] : d[2], pe = i == 0 ? d[1] : i == 1 ? d[2] : d[0];
+                const nlg::F2 e = {pe.x - p.x, pe.y - p.y};
+                const float ae = e.x * e.x + e.y * e.y;
+                kx = ngon_edge(p, e, ae, p.x * e.x + p.y * e.y, p.x * e.y - p.y * e.x, true, g, corner, &hx, &s0, &s1);
+                const nlg::F2 q = j == 0 ? d[0] : j == 1 ? d[1] : d[2], qe = j == 0 ? d[1] : j == 1 ? d[2] : d[0];
+                const nlg::F2 h = {qe.x - q.x, qe.y - q.y};
+                const float ah = h.x * h.x + h.y * h.y;
+                kn = ngon_edge(q, h, ah, q.x * h.x + q.y * h.y, q.x * h.y - q.y * h.x, false, g, corner, &hn, &n0, &n1);
+                const float m = g.tau * sqrtf(ae), mh = g.tau * sqrtf(ah);
+                known = hx && hn && s0 < -m && s1 > m && n0 > mh && n1 < -mh;
+                T ox, oy, ux, uy;
+                corner_of<T>(A, corner, kx, ox, oy);
+                corner_of<T>(A, corner, kx + 1, ux, uy);
+                ux -= ox;
+                uy -= oy;
+                tx = quot(uy * (px - ox) - ux * (py - oy), ux * ey - uy * ex);
+                corner_of<T>(A, corner, kn, ox, oy);
+                corner_of<T>(A, corner, kn + 1, ux, uy);
+                ux -= ox;
+                uy -= oy;
+                tn = quot(uy * (sx - ox) - ux * (sy - oy), ux * gy - uy * gx);
+                if (kn == kx) {
+                    // both on one polygon edge: the boundary runs along it from the exit to the entry, or
+                    // (the polygon all but inside T_b) around it
+                    const T run = ((sx + tn * gx) - (px + tx * ex)) * ux + ((sy + tn * gy) - (py + tx * ey)) * uy;
+                    known = known && run > (T)(g.tau * g.poly_side);
+                }
+                go = known;
+            } else {
+                const T r2 = sizeof(T) == sizeof(float) ? (T)(g.deltaf * g.deltaf) : (T)g.d2;
+                tx = disc_cross<T>(px, py, ex, ey, r2, true);
+                tn = disc_cross<T>(sx, sy, gx, gy, r2, false);
+            }
+            if (i == 1) edge1_add(M, tx, (T)1);
+            if (j == 1) edge1_add(M, tn, (T)-1);
+            T l1, l2, q1, q2;
+            edge_l(i, tx, l1, l2);
+            edge_l(j, tn, q1, q2);
+            if constexpr (kPoly) {   // along the polygon's corners
+                int c = kn - kx;
+                c += c < 0 ? g.ngon_n : 0;
+                n += c;
+                for (int k = kx + 1; c > 0; c--, k++) {
+                    if (k >= g.ngon_n) k -= g.ngon_n;
+                    T ox, oy, m1, m2;
+                    corner_of<T>(A, corner, k, ox, oy);
+                    frame_l(f, ox, oy, m1, m2);
+                    seg_add(M, l1, l2, m1, m2);
+                    l1 = m1;
+                    l2 = m2;
+                }
+            }
+            if constexpr (BALL == NL_BALL_APPROXCAPS) {   // along the dyadic arc points
+                if (g.cap_level > 0) {
+                    const T ax = px + tx * ex, ay = py + tx * ey, bx = sx + tn * gx, by = sy + tn * gy;
+                    const T dl = sizeof(T) == sizeof(float) ? (T)g.deltaf : (T)g.delta;
+                    auto mid = [&](T ux, T uy, T &ox, T &oy) {
+                        T s;
+                        if constexpr (sizeof(T) == sizeof(float)) s = dl * rsqrtf(ux * ux + uy * uy);
+                        else s = dl / sqrt(ux * ux + uy * uy);
+                        ox = ux * s;
+                        oy = uy * s;
+                    };
+                    auto to = [&](T x, T y) {
+                        T m1, m2;
+                        frame_l(f, x, y, m1, m2);
+                        seg_add(M, l1, l2, m1, m2);
+                        l1 = m1;
+                        l2 = m2;
+                    };
+                    T mx, my;
+                    mid(ax + bx, ay + by, mx, my);
+                    if (g.cap_level == 2) {
+                        T hx, hy;
+                        mid(ax + mx, ay + my, hx, hy);
+                        to(hx, hy);
+                        to(mx, my);
+                        mid(mx + bx, my + by, hx, hy);
+                        to(hx, hy);
+                    } else {
+                        to(mx, my);
+                    }
+                }
+            }
+            seg_add(M, l1, l2, q1, q2);
+            if constexpr (BALL == NL_BALL_EXACTCAPS) {
+                const T ax = px + tx * ex, ay = py + tx * ey, bx = sx + tn * gx, by = sy + tn * gy;
+                T cx, cy, w;
+                if constexpr (sizeof(T) == sizeof(float)) {
+                    nlg::cap_rule_f32(nlg::F2{ax, ay}, nlg::F2{bx, by}, g, &cx, &cy, &w);
+                } else {
+                    D2 cc;
+                    nlg::cap_rule(D2{ax, ay}, D2{bx, by}, D2{0.0, 0.0}, g.delta, g.cap_printed, &cc, &w);
+                    cx = cc.x;
+                    cy = cc.y;
+                }
+                T c1, c2;
+                frame_l(f, cx, cy, c1, c2);
+                point_add(M, c1, c2, w * inv_area);
+                ncap++;
+            }
+        }
+        __syncwarp();
+    }
+    mom_turn(M, rot);
+    kind = in == 7u ? nlg::KIND_WHOLE : nlg::KIND_PARTIAL;
+    nv = BALL == NL_BALL_EXACTCAPS && n < 3 ? 0 : n;
+    return !known ? -1 : empty ? 0 : 1;
+}
+
+// ---------------------------------------------------------------------------
+// Per-warp shared memory of k_const
+// ---------------------------------------------------------------------------
+struct NoClip {};
+
+template <int BALL, typename T>
+struct ConstShared {
+    static constexpr bool kClip = sizeof(T) == sizeof(float) ? (BALL == kBallNgonAny || kSupportBall<BALL>) : kSupportBall<BALL>;
+    using Fx = typename std::conditional<sizeof(T) == sizeof(float), int, T>::type;   // FP32 sums: fixed point
+    CandT<T> c64[sizeof(T) == sizeof(double) ? 32 : 1];
+    OuterPt sq[NL_MAXQ];
+    CandData cand[32];
+    Fx acc[12][32];            // P (rows 0-8) and Q (9-11) of each lane's pair, value-major
+    Fx s0q[NL_MAXQ];           // per outer point: sum of |T_b| S0 over the cut regions
+    unsigned dmask[32];        // outer points of each lane's candidate whose item the deferred kernel takes
+    float2 corner[65];         // the regular polygon's corners, corner[N] = corner[0]
+    unsigned short queue[32 * NL_MAXQ];   // cut items (owner lane << 8 | q)
+    unsigned char hit[32];     // the lane's pair has a non-empty cut region
+    typename std::conditional<kClip, nlg::ClipBuf, NoClip>::type clip;
+};
+
+// The item's region by the FP64 geometry, its moments in T (from FP64 barycentric coordinates):
+// false for an empty region
+template <int BALL, typename T>
+__device__ __noinline__ bool exact_const_item(const NumArgs &A, int b, const nlg::F2 *dl, double xx, double xy,
+                                              Mom<T> &M, int &nv, int &kind, int &ncap)
+{
+    const CandFp64 c = cand_fp64(A, b);
+    const D2 x = {xx, xy};
+    nlg::Region R;
+    nlg::make_region<kGeoBall<BALL>>(c.V, dl, c.bb, x, A.geo, R);
+    if (R.overflow) atomicOr(A.err, 1);
+    if (R.kind == nlg::KIND_NONE) return false;
+    kind = R.kind;
+    nv = R.nv;
+    ncap = R.ncap;
+    if (kind == nlg::KIND_WHOLE && ncap == 0) {
+        mom_set(M, (T)1);
+        return true;
+    }
+    // in FP64 whatever T (these items are few)
+    const BaryMap bm = bary_map(c.V);
+    Mom<double> S;
+    mom_set(S, 0.0);
+    double phi[3];
+    if (nv >= 3) {
+        const double x0 = R.P[0].x, y0 = R.P[0].y;   // about the polygon's first vertex
+        double p1 = 0.0, p2 = 0.0;
+        for (int i = 1; i < nv; i++) {
+            const double dx = R.P[i].x - x0, dy = R.P[i].y - y0;
+            const double q1 = (dx * bm.e2y - bm.e2x * dy) * bm.inv, q2 = (bm.e1x * dy - dx * bm.e1y) * bm.inv;
+            seg_add(S, p1, p2, q1, q2);
+            p1 = q1;
+            p2 = q2;
+        }
+        bary_of(bm, x0, y0, phi);
+        mom_shift(S, phi[1], phi[2]);
+    }
+    for (int i = 0; i < ncap; i++) {
+        bary_of(bm, R.cc[i].x, R.cc[i].y, phi);
+        point_add(S, phi[1], phi[2], R.cw[i] / c.area);
+    }
+    M = Mom<T>{(T)S.s0, (T)S.s1, (T)S.s2, (T)S.s11, (T)S.s22, (T)S.s12};
+    return true;
+}
+
+// inner points that the rule spends on a region (the counted qp-pairs)
+__device__ __forceinline__ int region_points(const NumArgs &A, int kind, int nv, int ncap)
+{
+    if (kind == nlg::KIND_WHOLE && ncap == 0) return A.inner.n;
+    return (nv >= 3 ? (nv - 2) * A.inner.n : 0) + ncap;
+}
+
+// an item's moments M at outer point q = o, added onto owner own's sums (rows 0-11), its s0 onto
+// the outer point's.  FP32 sums: rounded to the grids fxs and gs (integer adds, any order).
+template <typename T, typename Fx>
+__device__ __forceinline__ void item_add(const OuterPt &o, const Mom<T> &M, Fx (*acc)[32], Fx *s0q, int own, int q,
+                                         float fxs, T area, float gs)
+{
+    constexpr bool f32 = sizeof(T) == sizeof(float);
+    const T W = f32 ? (T)o.Wf * (T)fxs : (T)o.W;   // fxs: a power of two
+    const T w0 = W * (f32 ? (T)o.l0f : (T)o.l0), w1 = W * (f32 ? (T)o.l1f : (T)o.l1);
+    const T w2 = W * (f32 ? (T)o.l2f : (T)o.l2);
+    auto put = [&](Fx *p, T v) {
+        if constexpr (f32) atomicAdd(p, __float2int_rn(v));
+        else atomicAdd(p, v);
+    };
+    put(&acc[0][own], w0 * M.s0); put(&acc[1][own], w0 * M.s1); put(&acc[2][own], w0 * M.s2);
+    put(&acc[3][own], w1 * M.s0); put(&acc[4][own], w1 * M.s1); put(&acc[5][own], w1 * M.s2);
+    put(&acc[6][own], w2 * M.s0); put(&acc[7][own], w2 * M.s1); put(&acc[8][own], w2 * M.s2);
+    put(&acc[9][own], W * M.s11); put(&acc[10][own], W * M.s22); put(&acc[11][own], W * M.s12);
+    put(&s0q[q], f32 ? area * (T)gs * M.s0 : area * M.s0);
+}
+
+// Interior candidates of T_a: T_b whole for every outer point (certified when the lists are built,
+// a relation symmetric in a and b).  The outer rules integrate quadratics exactly too, so the
+// pair's blocks are closed forms of the two areas: M_ab = c |T_a| |T_b| / 9 in all nine entries
+// (formed by the scatter: nothing is stored), M_aa = c |T_a| |T_b| (1 + delta_ij) / 12, and the
+// M_bb that T_a receives as the inner triangle of its symmetric pairs is the same sum again.
+template <int STS>
+__device__ __forceinline__ void interior_const(const NumArgs &A, int a, int lane, LaneAcc &acc)
+{
+    const D2 ba = {A.bx[a], A.by[a]};
+    double sum = 0.0;
+    for (int64_t e = A.nbr_ptr[a] + lane; e < A.nbr_split[a]; e += 32) {
+        const int b = A.nbr_idx[e];
+#ifdef NL_CHECKS
+        if (b < 0 || b >= A.K) {   // debug build: bad candidate recorded (bit 16) and skipped
+            atomicOr(A.err, 16);
+            continue;
+        }
+#endif
+        sum += A.area[b];
+        A.flag[e] = 1;
+        int q0 = 0, q1 = A.outer.n;
+        if (A.switch47) rule_range(A, ba, D2{A.bx[b], A.by[b]}, q0, q1);
+        const int nq = q1 - q0;
+        acc.qp += (uint32_t)(nq * A.inner.n);
+        acc.cnt += A.outer_support ? 1u : (uint32_t)nq;
+        if (want_stats<STS>(A))
+            for (int q = 0; q < (A.outer_support ? 1 : nq); q++)
+                acc.hsum += nlg::record_hash(a, b, q, nlg::KIND_WHOLE, 3, 0);
+    }
+    const double w = sum * A.area[a] * A.kc * (1.0 / 12.0) * 2.0;
+    for (int i = 0; i < 6; i++) acc.maa[i] += i < 3 ? 2.0 * w : w;
+}
+
+// Queue the round's marked items for k_deferred, ordered by owner lane and outer point (as
+// defer_flush); items past the queue's capacity are integrated by their owner lane.
+template <int BALL, int STS, typename Sh>
+__device__ __forceinline__ void const_defer_flush(const NumArgs &A, int a, int64_t base, Sh &sh, int lane, float fxs,
+                                                  LaneAcc &acc)
+{
+    const unsigned m = sh.dmask[lane];
+    const int cnt = __popc(m);
+    int inc = cnt;
+    for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, off);
+        if (lane >= off) inc += y;
+    }
+    const int total = __shfl_sync(0xffffffffu, inc, 31);
+    if (total == 0) return;
+    sh.dmask[lane] = 0;
+    int slot0 = 0;
+    if (lane == 0 && A.defer) slot0 = atomicAdd(A.defer_n, total);
+    slot0 = __shfl_sync(0xffffffffu, slot0, 0);
+    int slot = slot0 + inc - cnt;
+    for (unsigned rest = m; rest; rest &= rest - 1, slot++) {
+        const int q = __ffs(rest) - 1;
+        if (A.defer && slot < A.defer_cap) {
+            A.defer[slot] = DeferItem{base + lane, a, (A.prob << 8) | q};
+            continue;
+        }
+        const CandData &cd = sh.cand[lane];
+        const OuterPt &o = sh.sq[q];
+        nlg::F2 dl[3];
+        for (int i = 0; i < 3; i++) { dl[i].x = cd.vlx[i] - o.lx; dl[i].y = cd.vly[i] - o.ly; }
+        Mom<float> M;
+        int nv, kind, ncap;
+        if (!exact_const_item<BALL, float>(A, cd.b, dl, o.x, o.y, M, nv, kind, ncap)) continue;
+        item_add<float>(o, M, sh.acc, sh.s0q, lane, q, fxs, cd.akcf, A.s0q_grid);
+        sh.hit[lane] = 1;
+        acc.cnt++;
+        acc.qp += (uint32_t)region_points(A, kind, nv, ncap);
+        if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, cd.b, q - cd.q0, kind, nv, ncap);
+    }
+}
+
+// The boundary candidates of outer triangle a, 32 at a time (one a lane): classification of every
+// (q, b) in FP32 in lockstep, whole ones summed on the spot (their moments are 1), cut ones queued
+// and drained by all lanes.
+template <int BALL, typename T, int STS>
+__device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstShared<BALL, T> &sh, int lane,
+                                               LaneAcc &acc)
+{
+    constexpr bool f32 = sizeof(T) == sizeof(float);
+    using Fx = typename ConstShared<BALL, T>::Fx;
+    const D2 ba = {A.bx[a], A.by[a]};
+    const float4 bah = bary_hilo(A, a);
+    const int64_t es = A.nbr_split[a], e1 = A.nbr_ptr[a + 1];
+    const int nq_all = A.outer.n;
+    // FP32 sums: one grid for all pairs of T_a (every moment is at most 1 on a part of T_b)
+    float fxs = 0.f, inv_s = 0.f;
+    if (f32) {
+        const float r = fx_outer_bound(sh.sq, nq_all);
+        const int e = ((__float_as_int(fmaxf(r, 1e-25f)) >> 23) & 0xff) - 126;   // r < 2^e
+        fxs = __int_as_float((127 + 29 - e) << 23);
+        inv_s = 1.f / fxs;
+    }
+    for (int q = lane; q < NL_MAXQ; q += 32) sh.s0q[q] = (Fx)0;
+    // sum of |T_b| over the whole items of outer point q = lane: exact integers (FP32 path: on the
+    // grid s0q_grid; FP64 path: 50-bit fixed point in two limbs, area_grid = 2^50 / a power of two
+    // above the largest area)
+    int ws_f = 0;
+    unsigned long long ws_hi = 0, ws_lo = 0;
+    __syncwarp();
+    for (int64_t base = es; base < e1; base += 32) {
+        const int64_t e = base + lane;
+        const bool valid = e < e1;
+        int q0 = 0, q1 = 0;
+        CandData c;
+        c.b = a;
+        c.akcf = 0.f;
+        unsigned a_hi = 0, a_lo = 0;
+        int a_fx = 0;
+        if (valid) {
+            int b = A.nbr_idx[e];
+#ifdef NL_CHECKS
+            if (b < 0 || b >= A.K) {   // debug build: bad candidate recorded (bit 16), replaced by a
+                atomicOr(A.err, 16);
+                b = a;
+            }
+#endif
+            load_cand(A, b, ba, bah, c, q1);
+            q0 = c.q0;
+            sh.cand[lane] = c;
+            if constexpr (f32) {
+                a_fx = __float2int_rn(c.akcf * A.s0q_grid);
+            } else {
+                const int64_t K = A.K;
+                Cand64 d;
+                d.x0 = A.tx[b];
+                d.y0 = A.ty[b];
+                d.e1x = A.tx[K + b] - d.x0;
+                d.e1y = A.ty[K + b] - d.y0;
+                d.e2x = A.tx[2 * K + b] - d.x0;
+                d.e2y = A.ty[2 * K + b] - d.y0;
+                d.area = A.area[b];
+                d.inv = 0.5 / d.area;
+                sh.c64[lane] = d;
+                const unsigned long long fx = __double2ull_rn(d.area * A.area_grid);
+                a_hi = (unsigned)(fx >> 25);
+                a_lo = (unsigned)fx & ((1u << 25) - 1u);
+            }
+        }
+        for (int i = 0; i < 12; i++) sh.acc[i][lane] = (Fx)0;
+        sh.dmask[lane] = 0;
+        sh.hit[lane] = 0;
+        int nqueue = 0, nwhole = 0;
+        T u0 = 0, u1 = 0, u2 = 0;   // sum of W_q phi_a,i over the outer points that see all of T_b
+        __syncwarp();
+        for (int q = 0; q < nq_all; q++) {
+            const bool active = valid && q >= q0 && q < q1;
+            const OuterPt &o = sh.sq[q];
+            int cls = nlg::CLS_EMPTY;
+            if (active) {
+                nlg::F2 dl[3];
+                cls = classify_item<kGeoBall<BALL>, T>(A, c, o, dl);
+            }
+            const bool whole = cls == nlg::CLS_WHOLE;
+            if (whole) {
+                const T W = f32 ? (T)o.Wf : (T)o.W;
+                u0 += W * (f32 ? (T)o.l0f : (T)o.l0);
+                u1 += W * (f32 ? (T)o.l1f : (T)o.l1);
+                u2 += W * (f32 ? (T)o.l2f : (T)o.l2);
+                nwhole++;
+                if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, c.b, q - q0, nlg::KIND_WHOLE, 3, 0);
+            }
+            if constexpr (f32) {
+                const int t = __reduce_add_sync(0xffffffffu, whole ? a_fx : 0);
+                if (lane == q) ws_f += t;
+            } else {
+                const unsigned th = __reduce_add_sync(0xffffffffu, whole ? a_hi : 0u);
+                const unsigned tl = __reduce_add_sync(0xffffffffu, whole ? a_lo : 0u);
+                if (lane == q) {
+                    ws_hi += th;
+                    ws_lo += tl;
+                }
+            }
+            const unsigned me = __ballot_sync(0xffffffffu, cls == nlg::CLS_EXACT);
+            if (cls == nlg::CLS_EXACT)
+                sh.queue[nqueue + __popc(me & ((1u << lane) - 1u))] = (unsigned short)((lane << 8) | q);
+            nqueue += __popc(me);
+        }
+        acc.cnt += (uint32_t)nwhole;
+        acc.qp += (uint32_t)(nwhole * A.inner.n);
+        __syncwarp();
+        // cut items, 32 at a time; the ones the FP64 geometry has to decide are marked for
+        // k_deferred (FP32 path) or compacted at the front of the queue (FP64 path)
+        int nslow = 0;
+        for (int r0 = 0; r0 < nqueue; r0 += 32) {
+            const bool live = r0 + lane < nqueue;
+            const unsigned it = sh.queue[live ? r0 + lane : r0];   // the other lanes follow along
+            const int own = it >> 8, q = it & 0xff;
+            const CandData &cd = sh.cand[own];
+            const OuterPt &o = sh.sq[q];
+            nlg::F2 d[3];
+            for (int k = 0; k < 3; k++) { d[k].x = cd.vlx[k] - o.lx; d[k].y = cd.vly[k] - o.ly; }
+            Mom<T> M;
+            int nv = 0, kind = nlg::KIND_PARTIAL, ncap = 0, r = -1;
+            T area = (T)cd.akcf;
+            if constexpr (BALL == NL_BALL_BARYCENTER || BALL == NL_BALL_OVERLAP) {
+                // FP64 predicate on the whole triangle
+            } else if constexpr (BALL == kBallNgonAny) {
+                if constexpr (f32) {
+                    int which = 0;
+                    bool cut = false;
+                    const int n = nlg::clip_ngon_f32_sh<true>(d, A.geo.err0, A.geo, sh.clip, lane, &which, &cut);
+                    r = n < 0 ? -1 : n < 3 ? 0 : 1;
+                    if (r == 1) {
+                        const Frame<float> f = {-d[0].x, -d[0].y, cd.e1x, cd.e1y, cd.e2x, cd.e2y, cd.binv};
+                        // about the polygon's first vertex
+                        const float x0 = sh.clip.x[which][0][lane], y0 = sh.clip.y[which][0][lane];
+                        const Frame<float> w = {-x0, -y0, cd.e1x, cd.e1y, cd.e2x, cd.e2y, cd.binv};
+                        mom_set(M, 0.f);
+                        float p1 = 0.f, p2 = 0.f;
+                        for (int k = 1; k < n; k++) {
+                            float q1, q2;
+                            frame_l(w, sh.clip.x[which][k][lane], sh.clip.y[which][k][lane], q1, q2);
+                            seg_add(M, p1, p2, q1, q2);
+                            p1 = q1;
+                            p2 = q2;
+                        }
+                        frame_l(f, x0, y0, p1, p2);
+                        mom_shift(M, p1, p2);
+                        nv = n;
+                        kind = cut ? nlg::KIND_PARTIAL : nlg::KIND_WHOLE;
+                    }
+                }
+            } else if constexpr (f32) {
+                const Frame<float> f = {-d[0].x, -d[0].y, cd.e1x, cd.e1y, cd.e2x, cd.e2y, cd.binv};
+                r = cut_item<BALL, float>(A, live, d, f, BALL == NL_BALL_EXACTCAPS ? 1.f / area : 0.f, sh.corner, M,
+                                          nv, kind, ncap);
+            } else {
+                const Cand64 &w = sh.c64[own];
+                const Frame<double> f = {o.x - w.x0, o.y - w.y0, w.e1x, w.e1y, w.e2x, w.e2y, w.inv};
+                area = w.area;
+                r = cut_item<BALL, double>(A, live, d, f, 2.0 * w.inv, sh.corner, M, nv, kind, ncap);
+            }
+            if (live && r > 0) {
+                item_add<T>(o, M, sh.acc, sh.s0q, own, q, fxs, area, A.s0q_grid);
+                sh.hit[own] = 1;
+                acc.cnt++;
+                acc.qp += (uint32_t)region_points(A, kind, nv, ncap);
+                if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, cd.b, q - cd.q0, kind, nv, ncap);
+            }
+            const bool slow = live && r < 0;
+            if (f32 && slow) atomicOr(&sh.dmask[own], 1u << q);
+            if constexpr (!f32) {
+                const unsigned ms = __ballot_sync(0xffffffffu, slow);   // also: every lane has read its item
+                if (slow) sh.queue[nslow + __popc(ms & ((1u << lane) - 1u))] = (unsigned short)it;
+                nslow += __popc(ms);
+                __syncwarp();
+            }
+        }
+        __syncwarp();
+        if constexpr (f32) {
+            const_defer_flush<BALL, STS>(A, a, base, sh, lane, fxs, acc);
+            __syncwarp();
+        } else {
+            for (int i = lane; i < nslow; i += 32) {
+                const unsigned it = sh.queue[i];
+                const int own = it >> 8, q = it & 0xff;
+                const CandData &cd = sh.cand[own];
+                const OuterPt &o = sh.sq[q];
+                nlg::F2 d[3];
+                for (int k = 0; k < 3; k++) { d[k].x = cd.vlx[k] - o.lx; d[k].y = cd.vly[k] - o.ly; }
+                Mom<T> M;
+                int nv, kind, ncap;
+                if (!exact_const_item<BALL, T>(A, cd.b, d, o.x, o.y, M, nv, kind, ncap)) continue;
+                item_add<T>(o, M, sh.acc, sh.s0q, own, q, fxs, sh.c64[own].area, A.s0q_grid);
+                sh.hit[own] = 1;
+                acc.cnt++;
+                acc.qp += (uint32_t)region_points(A, kind, nv, ncap);
+                if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, cd.b, q - cd.q0, kind, nv, ncap);
+            }
+            __syncwarp();
+        }
+        if (valid) {   // the owner's pair
+            const int b = c.b;
+            T P[9], Q[3], mab[9], mbb[6];
+            const T us[3] = {u0, u1, u2}, uw = u0 + u1 + u2;
+            bool big = false;
+            for (int k = 0; k < 12; k++) {
+                T v;
+                if constexpr (f32) {
+                    const int iv = sh.acc[k][lane];
+                    big = big || iv >= (1 << 30) || iv <= -(1 << 30);
+                    v = (float)iv * inv_s;
+                } else {
+                    v = sh.acc[k][lane];
+                }
+                if (k < 9) P[k] = v + us[k / 3];
+                else Q[k - 9] = v + uw;
+            }
+            if (big) atomicOr(A.err, 256);
+            T akc;
+            if constexpr (f32) akc = c.akcf * A.kcf;
+            else akc = sh.c64[lane].area * A.kc;
+            pair_block<T>(akc, P, Q, mab, mbb);
+            const bool any = nwhole > 0 || sh.hit[lane] != 0;
+            A.flag[e] = any ? 1 : 0;
+            T *blk = (T *)A.blk;
+            for (int i = 0; i < 9; i++) blk[(int64_t)i * A.E + e] = mab[i];
+            if (any)
+                for (int i = 0; i < 6; i++) atomicAdd(&A.mbb[(int64_t)i * A.K + b], (double)mbb[i]);
+        }
+        __syncwarp();
+    }
+    // M_aa = c sum_q W_q phi_a(x_q) phi_a(x_q)^T sum_b int_{R(x_q, T_b)} 1, in FP64, one outer point a lane
+    if (lane < nq_all) {
+        const OuterPt &o = sh.sq[lane];
+        double t;
+        if constexpr (f32) {
+            const long long s = (long long)sh.s0q[lane] + ws_f;
+            if (s >= (1ll << 30) || s <= -(1ll << 30)) atomicOr(A.err, 256);
+            t = (double)s / (double)A.s0q_grid;
+        } else {
+            t = sh.s0q[lane] + (double)((ws_hi << 25) + ws_lo) / A.area_grid;
+        }
+        const double ws = o.W * t * A.kc;
+        acc.maa[0] += ws * o.l0 * o.l0; acc.maa[1] += ws * o.l1 * o.l1; acc.maa[2] += ws * o.l2 * o.l2;
+        acc.maa[3] += ws * o.l0 * o.l1; acc.maa[4] += ws * o.l0 * o.l2; acc.maa[5] += ws * o.l1 * o.l2;
+    }
+}
+
+// all candidates of outer triangle a; the per-triangle outputs are stored (the only kernel that
+// writes them before k_deferred adds)
+template <int BALL, typename T, int STS>
+__device__ __forceinline__ void const_outer(const NumArgs &A, int a, ConstShared<BALL, T> &sh, int lane)
+{
+    LaneAcc acc;
+    acc_zero(acc);
+    interior_const<STS>(A, a, lane, acc);
+    if constexpr (kSupportBall<BALL>) {
+        support_boundary<BALL, T>(A, a, lane, sh.clip, acc);
+    } else {
+        if constexpr (BALL == NL_BALL_NGON)
+            for (int k = lane; k <= A.geo.ngon_n; k += 32) {
+                const int kk = k == A.geo.ngon_n ? 0 : k;
+                sh.corner[k] = make_float2((float)A.geo.ngon[2 * kk], (float)A.geo.ngon[2 * kk + 1]);
+            }
+        stage_outer(A, a, sh.sq, lane);
+        __syncwarp();
+        boundary_const<BALL, T, STS>(A, a, sh, lane, acc);
+    }
+    finish_outer<STS>(A, a, acc, lane, kStore);
+}
+
+// Measured (32-gon, delta = 0.1, 96 x 96 cells jittered, 16-point outer rule, 30 M cut items, one
+// GB300): FP32 sums 1.6 ms against 4.2 ms for the point-by-point kernel it replaced (certified
+// Sutherland-Hodgman clip into shared memory, 7-point rule on every fan triangle) plus 0.5 ms of its
+// interior kernel; it issues in 71 % of the cycles with 25 of 32 lanes active.  FP64 sums 13.4 ms
+// against 99.3 + 17.2 ms, with the FP64 pipe (1/64 of the FP32 rate) busy 86 % of the time.
+template <typename T>
+constexpr int kConstBlocksPerSm = sizeof(T) == sizeof(float) ? 5 : 4;
+
+template <int BALL, typename T, int STS>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, kConstBlocksPerSm<T>) k_const(const NumArgs A)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ConstShared<BALL, T> &sh = ((ConstShared<BALL, T> *)smem_raw)[threadIdx.x >> 5];
+    const int a = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+    if (a < A.K) const_outer<BALL, T, STS>(A, a, sh, threadIdx.x & 31);
+}
+
+// a deferred item of the constant kernel (FP32 path): region and moments by the FP64 geometry, its
+// M_ab into the queue's value slots, its M_bb, M_aa and statistics onto their sums
+template <int BALL>
+__device__ __forceinline__ void deferred_const(const NumArgs &A, const DeferItem &d, float *dv, int cap, int slot)
+{
+    const int K = A.K, a = d.a, q = d.qp & 0xff;
+    const int64_t e = d.e;
+#ifdef NL_CHECKS
+    if (a < 0 || a >= K || e < 0 || e >= A.E || q >= A.outer.n) {   // debug build: bad item (bit 64), skipped
+        atomicOr(A.err, 64);
+        return;
+    }
+#endif
+    const int b = A.nbr_idx[e];
+    D2 Va[3];
+    for (int i = 0; i < 3; i++) { Va[i].x = A.tx[i * K + a]; Va[i].y = A.ty[i * K + a]; }
+    const OuterPt o = outer_point(A, a, Va, A.area[a], q);
+    const D2 ba = {A.bx[a], A.by[a]};
+    CandData c;
+    int q1;
+    load_cand(A, b, ba, bary_hilo(A, a), c, q1);
+    nlg::F2 dl[3];
+    for (int i = 0; i < 3; i++) { dl[i].x = c.vlx[i] - o.lx; dl[i].y = c.vly[i] - o.ly; }
+    Mom<float> M;
+    int kind, nv, ncap;
+    if (!exact_const_item<BALL, float>(A, b, dl, o.x, o.y, M, nv, kind, ncap)) {
+        for (int k = 0; k < kDeferVals; k++) dv[(int64_t)k * cap + slot] = 0.f;
+        return;
+    }
+    const float la[3] = {o.l0f, o.l1f, o.l2f};
+    float P[9], mab[9], mbb[6];
+    for (int i = 0; i < 3; i++) {
+        const float w = o.Wf * la[i];
+        P[3 * i] = w * M.s0;
+        P[3 * i + 1] = w * M.s1;
+        P[3 * i + 2] = w * M.s2;
+    }
+    const float Q[3] = {o.Wf * M.s11, o.Wf * M.s22, o.Wf * M.s12};
+    pair_block<float>(c.akcf * A.kcf, P, Q, mab, mbb);
+    for (int k = 0; k < kDeferVals; k++) dv[(int64_t)k * cap + slot] = mab[k];
+    for (int k = 0; k < 6; k++) atomicAdd(&A.mbb[(int64_t)k * K + b], (double)mbb[k]);
+    const double ws = o.W * A.kc * A.area[b] * (double)M.s0;
+    const double m[6] = {ws * o.l0 * o.l0, ws * o.l1 * o.l1, ws * o.l2 * o.l2,
+                         ws * o.l0 * o.l1, ws * o.l0 * o.l2, ws * o.l1 * o.l2};
+    for (int k = 0; k < 6; k++) atomicAdd(&A.maa[(int64_t)k * K + a], m[k]);
+    A.flag[e] = 1;
+    atomicAdd((unsigned long long *)&A.qp_a[a], (unsigned long long)region_points(A, kind, nv, ncap));
+    atomicAdd((unsigned long long *)&A.cnt_a[a], 1ull);
+    if (A.stats)
+        atomicAdd((unsigned long long *)&A.hash_a[a],
+                  (unsigned long long)nlg::record_hash(a, b, q - c.q0, kind, nv, ncap));
+}
+
+}  // namespace nlq

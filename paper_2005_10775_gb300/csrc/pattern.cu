@@ -500,12 +500,13 @@ template <typename T>
 __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int32_t *tri, const int64_t *ptr,
                                               const int32_t *idx, const uint8_t *flag, const T *blk,
                                               const int64_t *row_ptr, const int32_t *col, double *W, int *err,
-                                              int cap, int hbits, int a, int lane, T *sacc_t, int32_t *skey,
-                                              uint32_t *spk, const double *area, const int *fxe, float ws)
+                                              int cap, int hbits, int a, int lane, T *sacc_t, T *scom_t,
+                                              int32_t *skey, uint32_t *spk, const int64_t *split, double kc,
+                                              const double *area, const int *fxe, float ws)
 {
     constexpr bool kFx = sizeof(T) == sizeof(float);
     using Acc = typename std::conditional<kFx, int, T>::type;
-    Acc *sacc = reinterpret_cast<Acc *>(sacc_t);
+    Acc *sacc = reinterpret_cast<Acc *>(sacc_t), *scom = reinterpret_cast<Acc *>(scom_t);
     const int ar[3] = {tri[3 * a], tri[3 * a + 1], tri[3 * a + 2]};
 #ifdef NL_CHECKS
     // debug build: indices checked, a bad one recorded (bit 64) and its access skipped
@@ -532,6 +533,7 @@ __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int
         for (int k = lane; k < H; k += 32) {
             skey[k] = -1;
             spk[k] = 0xffffffffu;
+            scom[k] = (Acc)0;
         }
         for (int k = lane; k < 3 * cap; k += 32) sacc[k] = (Acc)0;
         __syncwarp();
@@ -550,10 +552,41 @@ __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int
         __syncwarp();
     }
     const float sc = pow2f(shift);
+    const int64_t e_int = split ? split[a] : ptr[a];
+    if (split) {
+        // the constant kernel's interior pairs: M_ab = c |T_a| |T_b| / 9 in all nine entries, so each
+        // node of T_b receives one value for the three rows together, summed per column (scom, by
+        // hash slot) and added to the rows below
+        const double ka = kc * area[a] * (1.0 / 9.0);
+        int64_t e = ptr[a] + lane;
+        int b = e < e_int ? idx[e] : 0;
+        for (; e < e_int; e += 32) {
+            const int64_t en = e + 32;
+            const int bnx = en < e_int ? idx[en] : 0;
+            const double m = ka * area[b];
+            if (!cached) {
+                T v[9];
+                for (int p = 0; p < 9; p++) v[p] = (T)m;
+                scatter_pair<T, Acc>(1, b, v, K, J, tri, row_ptr, col, W, err, false, H, hbits, ar, len, cap, sc,
+                                     sacc, skey, spk);
+            } else {
+                const int bn[3] = {tri[3 * b], tri[3 * b + 1], tri[3 * b + 2]};
+                Acc v;
+                if constexpr (kFx) v = -__float2int_rn((float)m * sc);
+                else v = -m;
+                for (int k = 0; k < 3; k++) {
+                    const int sl = hash_find(skey, H, hbits, bn[k]);
+                    if (sl >= 0) atomicAdd(&scom[sl], v);
+                    else atomicOr(err, 2);
+                }
+            }
+            b = bnx;
+        }
+    }
     // the next pair's loads are issued before this pair's lookups and adds: the DRAM latency
     // of one iteration overlaps the shared-memory work of the previous one
     const int64_t e_end = ptr[a + 1];
-    int64_t e = ptr[a] + lane;
+    int64_t e = e_int + lane;
     uint8_t f = 0;
     int b = 0;
     T v[9];
@@ -581,6 +614,19 @@ __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int
         for (int p = 0; p < 9; p++) v[p] = vn[p];
     }
     __syncwarp();
+    if (cached && split) {   // a column's slot holds its place in each row: every entry has one owner
+        for (int k = lane; k < H; k += 32) {
+            const Acc x = scom[k];
+            if (x == (Acc)0) continue;
+            const unsigned pk = spk[k];
+            for (int i = 0; i < 3; i++) {
+                const unsigned pos = (pk >> (10 * i)) & kPosAbsent;
+                if (pos < (unsigned)len[i]) sacc[i * cap + pos] += x;
+                else atomicOr(err, 2);
+            }
+        }
+        __syncwarp();
+    }
     if (cached) {
         const double inv = (double)pow2f(-shift);
         for (int i = 0; i < 3; i++)
@@ -617,40 +663,41 @@ __global__ void k_local_blocks(int K, const double *maa, double *mbb, const int6
     if (t < K) local_block(K, t, maa, mbb, lslot, W, err);
 }
 
-// shared memory of one warp of the scatter: row accumulators [3][cap] (T), hash keys and
-// packed positions [H] (cap a multiple of 4 keeps the int arrays aligned after a float array)
+// shared memory of one warp of the scatter: row accumulators [3][cap] (T), sums per column slot
+// [H] (T), hash keys and packed positions [H] (cap a multiple of 4 keeps the int arrays aligned)
 template <typename T>
 __host__ __device__ constexpr size_t scatter_warp_bytes(int cap, int hbits)
 {
-    return cap > 0 ? 3 * (size_t)cap * sizeof(T) + ((size_t)8 << hbits) : 0;
+    return cap > 0 ? 3 * (size_t)cap * sizeof(T) + ((8 + sizeof(T)) << hbits) : 0;
 }
 
 template <typename T>
 __device__ __forceinline__ void scatter_warp_smem(unsigned char *raw, int wib, int cap, int hbits, T *&sacc,
-                                                  int32_t *&skey, uint32_t *&spk)
+                                                  T *&scom, int32_t *&skey, uint32_t *&spk)
 {
     unsigned char *base = raw + (size_t)wib * scatter_warp_bytes<T>(cap, hbits);
     sacc = (T *)base;
-    skey = (int32_t *)(base + 3 * (size_t)cap * sizeof(T));
+    scom = sacc + 3 * (size_t)cap;
+    skey = (int32_t *)(scom + ((size_t)1 << hbits));
     spk = (uint32_t *)(skey + (1 << hbits));
 }
 
 template <typename T>
 __global__ void k_scatter(int K, int J, int64_t E, const int32_t *tri, const int64_t *ptr, const int32_t *idx,
                           const uint8_t *flag, const T *blk, const int64_t *row_ptr, const int32_t *col,
-                          double *W, int *err, int cap, int hbits, const double *area, const int *fxe,
-                          float ws)
+                          double *W, int *err, int cap, int hbits, const int64_t *split, double kc,
+                          const double *area, const int *fxe, float ws)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int a = blockIdx.x * (blockDim.x >> 5) + wib;
-    T *sacc;
+    T *sacc, *scom;
     int32_t *skey;
     uint32_t *spk;
-    scatter_warp_smem<T>(smem_raw, wib, cap, hbits, sacc, skey, spk);
+    scatter_warp_smem<T>(smem_raw, wib, cap, hbits, sacc, scom, skey, spk);
     if (a >= K) return;
-    scatter_outer<T>(K, J, E, tri, ptr, idx, flag, blk, row_ptr, col, W, err, cap, hbits, a, lane, sacc, skey,
-                     spk, area, fxe, ws);
+    scatter_outer<T>(K, J, E, tri, ptr, idx, flag, blk, row_ptr, col, W, err, cap, hbits, a, lane, sacc, scom, skey,
+                     spk, split, kc, area, fxe, ws);
 }
 
 // ---- batched scatter: every problem of a batch in one launch per value type ----
@@ -674,14 +721,15 @@ __global__ void k_scatter_batch(const ScatterArgs *__restrict__ S, const int64_t
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
     if (g >= koff[n]) return;
-    T *sacc;
+    T *sacc, *scom;
     int32_t *skey;
     uint32_t *spk;
-    scatter_warp_smem<T>(smem_raw, wib, cap, hbits, sacc, skey, spk);
+    scatter_warp_smem<T>(smem_raw, wib, cap, hbits, sacc, scom, skey, spk);
     const int p = batch_problem(koff, n, g);
     const ScatterArgs &A = S[p];
     scatter_outer<T>(A.K, A.J, A.E, A.tri, A.ptr, A.idx, A.flag, (const T *)A.blk, A.row_ptr, A.col, A.W,
-                     A.err, cap, hbits, (int)(g - koff[p]), lane, sacc, skey, spk, A.area, A.fxe, A.ws);
+                     A.err, cap, hbits, (int)(g - koff[p]), lane, sacc, scom, skey, spk, A.split, A.kc, A.area,
+                     A.fxe, A.ws);
 }
 
 // M_aa + M_bb of every triangle of every problem (koff: prefix sums of K)
@@ -966,7 +1014,9 @@ static nl_status launch_scatter(nl_ctx *ctx, nl_plan *P, nl_csr *out)
     const unsigned grid = (unsigned)((K + warps - 1) / warps);
     k_scatter<T><<<grid, 32 * warps, smem, ctx->stream>>>(K, P->J, P->E, P->tri, P->nbr_ptr, P->nbr_idx, P->flag,
                                                            (const T *)P->blk, out->row_ptr, out->col_idx,
-                                                           P->W, P->err, cap, hbits, P->area, P->fxe,
+                                                           P->W, P->err, cap, hbits,
+                                                           P->cfg.kernel == NL_KERNEL_CONST ? P->nbr_split : nullptr,
+                                                           P->cfg.kernel_c, P->area, P->fxe,
                                                            nl_outer_abs_weight(P)); ++ctx->launches;
     NL_CK(cudaGetLastError());
     k_local_blocks<<<(K + 255) / 256, 256, 0, ctx->stream>>>(K, P->maa, P->mbb, P->lslot, P->W, P->err);

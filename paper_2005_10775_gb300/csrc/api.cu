@@ -231,6 +231,8 @@ int nl_const_ball(const nl_plan *P)
     return P->cfg.ball == NL_BALL_NGON && !ngon_regular(P) ? nlq::kBallNgonAny : P->cfg.ball;
 }
 
+bool nl_uses_queue(bool inv, int ball) { return inv || ball == NL_BALL_NGON || ball == nlq::kBallNgonAny; }
+
 nl_status nl_fill_args(nl_ctx *ctx, const nl_plan *P, nlq::NumArgs &A, bool stats)
 {
     memset(&A, 0, sizeof A);
@@ -404,13 +406,15 @@ nl_status run_numeric(nl_ctx *ctx, nl_plan *P, bool stats, bool one_stream = fal
     if (s != NL_OK) return s;
     const int ball = P->cfg.kernel == NL_KERNEL_CONST ? nl_const_ball(P) : P->cfg.ball;
     if (P->cfg.prec == NL_PREC_FP64) return nl_launch_numeric_f64(ctx, A, ball, one_stream);
-    if (!P->defer) {
-        const int cap = nl_defer_cap(P->E) > P->defer_min ? nl_defer_cap(P->E) : P->defer_min;
-        nlq::DeferItem *q = nullptr;
-        if ((s = nl_alloc(ctx, &q, nlq::defer_alloc_items(cap))) != NL_OK) return s;
-        P->defer = q;
+    if (!P->defer_n) {
+        if (nl_uses_queue(P->cfg.kernel == NL_KERNEL_INV_DIST, ball)) {
+            const int cap = nl_defer_cap(P->E) > P->defer_min ? nl_defer_cap(P->E) : P->defer_min;
+            nlq::DeferItem *q = nullptr;
+            if ((s = nl_alloc(ctx, &q, nlq::defer_alloc_items(cap))) != NL_OK) return s;
+            P->defer = q;
+            P->defer_cap = cap;
+        }
         if ((s = nl_alloc(ctx, &P->defer_n, 1)) != NL_OK) return s;
-        P->defer_cap = cap;
     }
     A.defer = (nlq::DeferItem *)P->defer;
     A.dval = nlq::defer_values(A.defer, P->defer_cap);

@@ -75,12 +75,6 @@ struct Launch {                    // one persistent numeric launch
     int defer_cap = 0;
 };
 
-// does a boundary launch of this value type and ball queue items for the deferred kernel?
-bool uses_queue(bool f64, int ball)
-{
-    return !f64 && ball >= 0 && ball != NL_BALL_BARY_NOCAPS && ball != NL_BALL_BARY_APPROXCAPS;
-}
-
 struct ScatterGroup {              // one scatter launch: problems of one value type
     bool f64 = false;
     std::vector<int> probs;
@@ -737,7 +731,7 @@ nl_status nl_batch_create(nl_ctx *ctx, int32_t n, const nl_mesh *meshes, const n
     if ((s = nl_alloc(ctx, &b->counters, 2 * nlaunch)) != NL_OK) return fail(s);
     // one deferred-item queue per float boundary launch, sized by its problems' candidate pairs
     for (Launch &l : b->launches) {
-        if (!uses_queue(b->pgroups[l.prec].f64, l.ball)) continue;
+        if (b->pgroups[l.prec].f64 || l.ball < 0 || !nl_uses_queue(l.inv, l.ball)) continue;
         int64_t E = 0;
         for (int i : l.probs) E += b->P[i]->E;
         l.defer_cap = nl_defer_cap(E);

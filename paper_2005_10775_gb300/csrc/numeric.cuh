@@ -2209,6 +2209,8 @@ __global__ void __launch_bounds__(256)
 // ---------------------------------------------------------------------------
 // ball mode of the constant-kernel launches: cfg.ball, or nlq::kBallNgonAny (api.cu)
 int nl_const_ball(const nl_plan *P);
+// does the FP32 path queue this kernel and ball's FP64-decided items for the deferred kernel? (api.cu)
+bool nl_uses_queue(bool inv, int ball);
 // kernel arguments of one assembled problem (api.cu)
 nl_status nl_fill_args(nl_ctx *ctx, const nl_plan *P, nlq::NumArgs &A, bool stats);
 

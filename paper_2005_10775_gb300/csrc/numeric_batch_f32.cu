@@ -81,21 +81,22 @@ nl_status nl_launch_deferred_batch_f32(nl_ctx *ctx, int ball, bool inv, const nl
     nl_status s = nl_deferred_blocks(ctx, &blocks);
     if (s != NL_OK) return s;
     const unsigned threads = nlq::kWarpsPerBlock * 32;
-#define NL_CASE(B)                                                                                             \
-    case B:                                                                                                    \
-        if (inv) nlq::k_deferred_batch<B, true><<<blocks, threads, 0, ctx->stream>>>(dA, items, count, cap);   \
-        else nlq::k_deferred_batch<B, false><<<blocks, threads, 0, ctx->stream>>>(dA, items, count, cap);      \
-        break
-    switch (ball == nlq::kBallNgonAny ? (int)NL_BALL_NGON : ball) {
-        NL_CASE(NL_BALL_BARYCENTER);
-        NL_CASE(NL_BALL_NOCAPS);
-        NL_CASE(NL_BALL_APPROXCAPS);
-        NL_CASE(NL_BALL_EXACTCAPS);
-        NL_CASE(NL_BALL_NGON);
-        NL_CASE(NL_BALL_OVERLAP);
-    default: return nl_fail(ctx, NL_EINVAL, "no deferred items for this ball mode");
-    }
+    if (!inv) {   // the constant kernel queues the N-gon's items only
+        nlq::k_deferred_batch<NL_BALL_NGON, false><<<blocks, threads, 0, ctx->stream>>>(dA, items, count, cap);
+    } else {
+#define NL_CASE(B) \
+    case B: nlq::k_deferred_batch<B, true><<<blocks, threads, 0, ctx->stream>>>(dA, items, count, cap); break
+        switch (ball) {
+            NL_CASE(NL_BALL_BARYCENTER);
+            NL_CASE(NL_BALL_NOCAPS);
+            NL_CASE(NL_BALL_APPROXCAPS);
+            NL_CASE(NL_BALL_EXACTCAPS);
+            NL_CASE(NL_BALL_NGON);
+            NL_CASE(NL_BALL_OVERLAP);
+        default: return nl_fail(ctx, NL_EINVAL, "no deferred items for this ball mode");
+        }
 #undef NL_CASE
+    }
     ++ctx->launches;
     nlq::k_defer_merge_batch<float><<<blocks, 256, 0, ctx->stream>>>(dA, items, count, cap); ++ctx->launches;
     NL_CK(cudaGetLastError());

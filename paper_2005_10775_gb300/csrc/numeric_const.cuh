@@ -566,8 +566,7 @@ struct ConstShared {
     typename std::conditional<kClip, nlg::ClipBuf, NoClip>::type clip;
 };
 
-// The item's region by the FP64 geometry, its moments in T (from FP64 barycentric coordinates):
-// false for an empty region
+// The N-gon's region by the FP64 geometry and its moments: false for an empty region
 template <int BALL, typename T>
 __device__ __noinline__ bool exact_const_item(const NumArgs &A, int b, const nlg::F2 *dl, double xx, double xy,
                                               Mom<T> &M, int &nv, int &kind, int &ncap)
@@ -575,13 +574,13 @@ __device__ __noinline__ bool exact_const_item(const NumArgs &A, int b, const nlg
     const CandFp64 c = cand_fp64(A, b);
     const D2 x = {xx, xy};
     nlg::Region R;
-    nlg::make_region<kGeoBall<BALL>>(c.V, dl, c.bb, x, A.geo, R);
+    nlg::make_region<NL_BALL_NGON>(c.V, dl, c.bb, x, A.geo, R);
     if (R.overflow) atomicOr(A.err, 1);
     if (R.kind == nlg::KIND_NONE) return false;
     kind = R.kind;
     nv = R.nv;
     ncap = R.ncap;
-    if (kind == nlg::KIND_WHOLE && ncap == 0) {
+    if (kind == nlg::KIND_WHOLE) {
         mom_set(M, (T)1);
         return true;
     }
@@ -590,26 +589,244 @@ __device__ __noinline__ bool exact_const_item(const NumArgs &A, int b, const nlg
     Mom<double> S;
     mom_set(S, 0.0);
     double phi[3];
-    if (nv >= 3) {
-        const double x0 = R.P[0].x, y0 = R.P[0].y;   // about the polygon's first vertex
-        double p1 = 0.0, p2 = 0.0;
-        for (int i = 1; i < nv; i++) {
-            const double dx = R.P[i].x - x0, dy = R.P[i].y - y0;
-            const double q1 = (dx * bm.e2y - bm.e2x * dy) * bm.inv, q2 = (bm.e1x * dy - dx * bm.e1y) * bm.inv;
-            seg_add(S, p1, p2, q1, q2);
-            p1 = q1;
-            p2 = q2;
-        }
-        bary_of(bm, x0, y0, phi);
-        mom_shift(S, phi[1], phi[2]);
+    const double x0 = R.P[0].x, y0 = R.P[0].y;   // about the polygon's first vertex
+    double p1 = 0.0, p2 = 0.0;
+    for (int i = 1; i < nv; i++) {
+        const double dx = R.P[i].x - x0, dy = R.P[i].y - y0;
+        const double q1 = (dx * bm.e2y - bm.e2x * dy) * bm.inv, q2 = (bm.e1x * dy - dx * bm.e1y) * bm.inv;
+        seg_add(S, p1, p2, q1, q2);
+        p1 = q1;
+        p2 = q2;
     }
-    for (int i = 0; i < ncap; i++) {
-        bary_of(bm, R.cc[i].x, R.cc[i].y, phi);
-        point_add(S, phi[1], phi[2], R.cw[i] / c.area);
-    }
+    bary_of(bm, x0, y0, phi);
+    mom_shift(S, phi[1], phi[2]);
     M = Mom<T>{(T)S.s0, (T)S.s1, (T)S.s2, (T)S.s11, (T)S.s22, (T)S.s12};
     return true;
 }
+
+// The same for the balls whose FP64 decisions are a vertex or edge predicate: barycenter, overlap and
+// the disc walks.  FP32 leaves a few predicates of an item open (a vertex or a closest point within
+// tau of the circle); only those are taken in FP64, by the canonical expressions, and the walk's points
+// (vertex if inside, then the edge's roots) are linked as they come, with nothing kept in arrays: on
+// the uniform grid of the paper's protocol, whose outer points lie at distance delta of other vertices
+// (1.35 M open items at h = 0.0125), it replaced a queue and a second kernel that built every such
+// region in local memory (exactcaps: 3.2 ms there, 1.1 ms here; the whole assembly 5.3 -> 3.2 ms).
+template <typename T>
+struct WalkPt {
+    T l1, l2, x, y;   // barycentric coordinates; position relative to x (arc ends)
+    int tag;          // 0 vertex, 1 entry, 2 exit
+};
+
+template <int BALL, typename T>
+__device__ __noinline__ bool exact_disc_item(const NumArgs &A, int b, const nlg::F2 *dl, double xx, double xy,
+                                             Mom<T> &M, int &nv, int &kind, int &ncap)
+{
+    const nlg::GeoParams &g = A.geo;
+    const D2 x = {xx, xy};
+    ncap = 0;
+    if constexpr (BALL == NL_BALL_BARYCENTER || BALL == NL_BALL_OVERLAP) {
+        const CandFp64 c = cand_fp64(A, b);
+        mom_set(M, (T)1);
+        nv = 3;
+        kind = nlg::KIND_WHOLE;
+        return BALL == NL_BALL_BARYCENTER ? nlg::in_ball(c.bb, x, g.d2) : nlg::overlaps(c.V, x, g.d2);
+    } else {
+        constexpr bool f32 = sizeof(T) == sizeof(float);
+        const int K = A.K;
+        D2 V[3];
+        for (int i = 0; i < 3; i++) { V[i].x = A.tx[i * K + b]; V[i].y = A.ty[i * K + b]; }
+        T px[3], py[3];   // vertices relative to x
+        unsigned in = 0, open = 0;
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            if constexpr (f32) {
+                px[i] = dl[i].x;
+                py[i] = dl[i].y;
+            } else {
+                px[i] = nlg::sub(V[i].x, x.x);
+                py[i] = nlg::sub(V[i].y, x.y);
+            }
+            const float r = dl[i].x * dl[i].x + dl[i].y * dl[i].y;
+            if (r <= g.rin_m2) in |= 1u << i;
+            else if (!(r > g.rout_p2)) open |= 1u << i;
+        }
+        // The loops over the open vertices and edges (one vertex and its two edges as a rule) run once
+        // for all lanes, whichever theirs are: the FP64 pipe takes a warp instruction of one lane as
+        // long as one of 32.
+        auto vert = [&](int i) { return i == 0 ? V[0] : i == 1 ? V[1] : V[2]; };
+        for (unsigned w = open; w; w &= w - 1) {
+            const int i = __ffs(w) - 1;
+            if (nlg::in_ball(vert(i), x, g.d2)) in |= 1u << i;
+        }
+        unsigned eopen = open | ((open >> 1) | (open << 2));   // edges that start or end at an open vertex
+        eopen &= 7u;
+        int nr[3] = {0, 0, 0};
+        unsigned ents = 0;   // bit 2 i + k: root k of edge i enters
+        T t[3][2];
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            const int j = (i + 1) % 3;
+            t[i][0] = t[i][1] = 0;
+            if ((eopen >> i) & 1u) continue;
+            const bool pi = ((in >> i) & 1u) != 0, qi = ((in >> j) & 1u) != 0;
+            if (pi != qi) {
+                nr[i] = 1;
+                if (!pi) ents |= 1u << (2 * i);
+            } else if (!pi) {
+                const float fx = dl[j].x - dl[i].x, fy = dl[j].y - dl[i].y;
+                const float a = fx * fx + fy * fy, bq = dl[i].x * fx + dl[i].y * fy, cr = dl[i].x * fy - dl[i].y * fx;
+                if (bq < 0.f && -bq < a) {
+                    if (cr * cr <= g.rin_m2 * a) {
+                        nr[i] = 2;
+                        ents |= 1u << (2 * i);
+                    } else if (!(cr * cr > g.rout_p2 * a)) {
+                        eopen |= 1u << i;
+                    }
+                }
+            }
+        }
+        const unsigned ecert = ~eopen & 7u;
+        for (unsigned w = eopen; w; w &= w - 1) {
+            // the canonical roots (nlg::edge_roots); l = num / a lies in (0, 1) exactly when 0 < num < a
+            const int i = __ffs(w) - 1;
+            const D2 p = vert(i), q = vert(i == 2 ? 0 : i + 1);
+            using namespace nlg;
+            const double dx = sub(q.x, p.x), dy = sub(q.y, p.y), fx = sub(p.x, x.x), fy = sub(p.y, x.y);
+            const double a = add(mul(dx, dx), mul(dy, dy)), bh = add(mul(fx, dx), mul(fy, dy));
+            const double c = sub(add(mul(fx, fx), mul(fy, fy)), g.d2);
+            const double disc = sub(mul(bh, bh), mul(a, c));
+            int m = 0;
+            T u0 = 0, u1 = 0;
+            unsigned en = 0;
+            if (!(disc < 0.0)) {
+                const double sq = __dsqrt_rn(disc), n1 = sub(-bh, sq), n2 = add(-bh, sq);
+                const bool k1 = n1 > 0.0 && n1 < a, k2 = n2 > 0.0 && n2 < a;
+                m = (int)k1 + (int)k2;
+                if constexpr (f32) {
+                    const float ia = 1.f / (float)a;
+                    u0 = (float)(k1 ? n1 : n2) * ia;
+                    u1 = (float)n2 * ia;
+                } else {
+                    const double ia = 1.0 / a;
+                    u0 = (k1 ? n1 : n2) * ia;
+                    u1 = n2 * ia;
+                }
+                en = k1 && k2 ? 1u : (in >> i) & 1u ? 0u : 1u;
+            }
+#pragma unroll
+            for (int k = 0; k < 3; k++)
+                if (k == i) {
+                    nr[k] = m;
+                    t[k][0] = u0;
+                    t[k][1] = u1;
+                    ents |= en << (2 * k);
+                }
+        }
+        const T r2 = f32 ? (T)(g.deltaf * g.deltaf) : (T)g.d2;
+        const T e1x = px[1] - px[0], e1y = py[1] - py[0], e2x = px[2] - px[0], e2y = py[2] - py[0];
+        const T inv = (T)1 / (e1x * e2y - e2x * e1y);
+        mom_set(M, (T)0);
+        WalkPt<T> first = {0, 0, 0, 0, 0}, prev = first;
+        int n = 0, narc = 0;
+        // the piece of boundary from a to b; moments about the walk's first point
+        auto link = [&](const WalkPt<T> &a, const WalkPt<T> &c) {
+            T u1 = a.l1 - first.l1, u2 = a.l2 - first.l2;
+            const T w1 = c.l1 - first.l1, w2 = c.l2 - first.l2;
+            if (BALL != NL_BALL_NOCAPS && a.tag == 2 && c.tag == 1) {
+                narc++;
+                if constexpr (BALL == NL_BALL_APPROXCAPS) {
+                    // dyadic arc points, each by bisection from the ends
+                    const T rad = f32 ? (T)g.deltaf : (T)g.delta;
+                    const int m = 1 << g.cap_level;
+                    for (int j = 1; j < m; j++) {
+                        T ax = a.x, ay = a.y, bx = c.x, by = c.y, mx = 0, my = 0;
+                        for (int lo = 0, hi = m; hi - lo > 1;) {
+                            mx = ax + bx;
+                            my = ay + by;
+                            const T sc = rad / sqrt(mx * mx + my * my);
+                            mx *= sc;
+                            my *= sc;
+                            const int md = (lo + hi) >> 1;
+                            if (md == j) break;
+                            if (j < md) { hi = md; bx = mx; by = my; }
+                            else { lo = md; ax = mx; ay = my; }
+                        }
+                        const T cx = mx - px[0], cy = my - py[0];
+                        const T v1 = (cx * e2y - e2x * cy) * inv - first.l1;
+                        const T v2 = (e1x * cy - cx * e1y) * inv - first.l2;
+                        seg_add(M, u1, u2, v1, v2);
+                        u1 = v1;
+                        u2 = v2;
+                    }
+                } else if (ncap < 3) {   // exactcaps: centroid and area
+                    T cx, cy, w;
+                    if constexpr (f32) {
+                        nlg::cap_rule_f32(nlg::F2{a.x, a.y}, nlg::F2{c.x, c.y}, g, &cx, &cy, &w);
+                    } else {
+                        D2 cc;
+                        nlg::cap_rule(D2{a.x, a.y}, D2{c.x, c.y}, D2{0.0, 0.0}, g.delta, g.cap_printed, &cc, &w);
+                        cx = cc.x;
+                        cy = cc.y;
+                    }
+                    cx -= px[0];
+                    cy -= py[0];
+                    // w / |T_b| = 2 w / det
+                    point_add(M, (cx * e2y - e2x * cy) * inv - first.l1, (e1x * cy - cx * e1y) * inv - first.l2,
+                              (T)2 * w * inv);
+                    ncap++;
+                }
+            }
+            seg_add(M, u1, u2, w1, w2);
+        };
+        auto emit = [&](T l1, T l2, T qx, T qy, int tag) {
+            const WalkPt<T> q = {l1, l2, qx, qy, tag};
+            if (n == 0) first = q;
+            else link(prev, q);
+            prev = q;
+            n++;
+        };
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            const int j = (i + 1) % 3;
+            const bool pi = ((in >> i) & 1u) != 0;
+            if (pi) emit((T)(i == 1), (T)(i == 2), px[i], py[i], 0);
+            const T ex = px[j] - px[i], ey = py[j] - py[i];
+            const bool calc = ((ecert >> i) & 1u) != 0;
+#pragma unroll
+            for (int k = 0; k < 2; k++)
+                if (k < nr[i]) {
+                    const bool en = ((ents >> (2 * i + k)) & 1u) != 0;
+                    const T tk = calc ? disc_cross<T>(px[i], py[i], ex, ey, r2, !en) : t[i][k];
+                    T l1, l2;
+                    edge_l(i, tk, l1, l2);
+                    emit(l1, l2, px[i] + tk * ex, py[i] + tk * ey, en ? 1 : 2);
+                }
+        }
+        if (n > 1) link(prev, first);
+        int m = n;
+        if (BALL == NL_BALL_APPROXCAPS) m += narc * ((1 << g.cap_level) - 1);
+        nv = n >= 2 && m >= 3 ? m : 0;
+        kind = in == 7u && n == 3 ? nlg::KIND_WHOLE : nlg::KIND_PARTIAL;
+        if (kind == nlg::KIND_WHOLE) mom_set(M, (T)1);
+        else mom_shift(M, first.l1, first.l2);
+        return nv >= 3 || ncap > 0;
+    }
+}
+
+// region and moments of one item by the FP64 geometry
+template <int BALL, typename T>
+__device__ __forceinline__ bool exact_item(const NumArgs &A, int b, const nlg::F2 *dl, double xx, double xy,
+                                           Mom<T> &M, int &nv, int &kind, int &ncap)
+{
+    if constexpr (kGeoBall<BALL> == NL_BALL_NGON) return exact_const_item<BALL, T>(A, b, dl, xx, xy, M, nv, kind, ncap);
+    else return exact_disc_item<BALL, T>(A, b, dl, xx, xy, M, nv, kind, ncap);
+}
+
+// are the items that FP32 leaves open queued for k_deferred?  The N-gon's on the FP32 path: its FP64
+// clip keeps its polygons in local memory, and a warp that ran it for one lane would wait (about 0.2
+// such items a round on a jittered mesh; a disc item costs some 150 FP64 instructions).
+template <int BALL, typename T>
+constexpr bool kConstQueue = sizeof(T) == sizeof(float) && kGeoBall<BALL> == NL_BALL_NGON;
 
 // inner points that the rule spends on a region (the counted qp-pairs)
 __device__ __forceinline__ int region_points(const NumArgs &A, int kind, int nv, int ncap)
@@ -704,7 +921,7 @@ __device__ __forceinline__ void const_defer_flush(const NumArgs &A, int a, int64
         for (int i = 0; i < 3; i++) { dl[i].x = cd.vlx[i] - o.lx; dl[i].y = cd.vly[i] - o.ly; }
         Mom<float> M;
         int nv, kind, ncap;
-        if (!exact_const_item<BALL, float>(A, cd.b, dl, o.x, o.y, M, nv, kind, ncap)) continue;
+        if (!exact_item<BALL, float>(A, cd.b, dl, o.x, o.y, M, nv, kind, ncap)) continue;
         item_add<float>(o, M, sh.acc, sh.s0q, lane, q, fxs, cd.akcf, A.s0q_grid);
         sh.hit[lane] = 1;
         acc.cnt++;
@@ -740,6 +957,7 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
     // above the largest area)
     int ws_f = 0;
     unsigned long long ws_hi = 0, ws_lo = 0;
+    int nopen = 0;   // items the FP64 geometry decided here
     __syncwarp();
     for (int64_t base = es; base < e1; base += 32) {
         const int64_t e = base + lane;
@@ -823,7 +1041,7 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
         acc.qp += (uint32_t)(nwhole * A.inner.n);
         __syncwarp();
         // cut items, 32 at a time; the ones the FP64 geometry has to decide are marked for
-        // k_deferred (FP32 path) or compacted at the front of the queue (FP64 path)
+        // k_deferred (kConstQueue) or compacted at the front of the queue and done after the others
         int nslow = 0;
         for (int r0 = 0; r0 < nqueue; r0 += 32) {
             const bool live = r0 + lane < nqueue;
@@ -882,8 +1100,9 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
                 if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, cd.b, q - cd.q0, kind, nv, ncap);
             }
             const bool slow = live && r < 0;
-            if (f32 && slow) atomicOr(&sh.dmask[own], 1u << q);
-            if constexpr (!f32) {
+            if constexpr (kConstQueue<BALL, T>) {
+                if (slow) atomicOr(&sh.dmask[own], 1u << q);
+            } else {
                 const unsigned ms = __ballot_sync(0xffffffffu, slow);   // also: every lane has read its item
                 if (slow) sh.queue[nslow + __popc(ms & ((1u << lane) - 1u))] = (unsigned short)it;
                 nslow += __popc(ms);
@@ -891,10 +1110,11 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
             }
         }
         __syncwarp();
-        if constexpr (f32) {
+        if constexpr (kConstQueue<BALL, T>) {
             const_defer_flush<BALL, STS>(A, a, base, sh, lane, fxs, acc);
             __syncwarp();
         } else {
+            nopen += nslow;
             for (int i = lane; i < nslow; i += 32) {
                 const unsigned it = sh.queue[i];
                 const int own = it >> 8, q = it & 0xff;
@@ -904,8 +1124,11 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
                 for (int k = 0; k < 3; k++) { d[k].x = cd.vlx[k] - o.lx; d[k].y = cd.vly[k] - o.ly; }
                 Mom<T> M;
                 int nv, kind, ncap;
-                if (!exact_const_item<BALL, T>(A, cd.b, d, o.x, o.y, M, nv, kind, ncap)) continue;
-                item_add<T>(o, M, sh.acc, sh.s0q, own, q, fxs, sh.c64[own].area, A.s0q_grid);
+                if (!exact_item<BALL, T>(A, cd.b, d, o.x, o.y, M, nv, kind, ncap)) continue;
+                T area;
+                if constexpr (f32) area = cd.akcf;
+                else area = sh.c64[own].area;
+                item_add<T>(o, M, sh.acc, sh.s0q, own, q, fxs, area, A.s0q_grid);
                 sh.hit[own] = 1;
                 acc.cnt++;
                 acc.qp += (uint32_t)region_points(A, kind, nv, ncap);
@@ -944,6 +1167,7 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
         }
         __syncwarp();
     }
+    if (!kConstQueue<BALL, T> && nopen > 0 && lane == 0 && A.defer_n) atomicAdd(A.defer_n, nopen);
     // M_aa = c sum_q W_q phi_a(x_q) phi_a(x_q)^T sum_b int_{R(x_q, T_b)} 1, in FP64, one outer point a lane
     if (lane < nq_all) {
         const OuterPt &o = sh.sq[lane];
@@ -1026,7 +1250,7 @@ __device__ __forceinline__ void deferred_const(const NumArgs &A, const DeferItem
     for (int i = 0; i < 3; i++) { dl[i].x = c.vlx[i] - o.lx; dl[i].y = c.vly[i] - o.ly; }
     Mom<float> M;
     int kind, nv, ncap;
-    if (!exact_const_item<BALL, float>(A, b, dl, o.x, o.y, M, nv, kind, ncap)) {
+    if (!exact_item<BALL, float>(A, b, dl, o.x, o.y, M, nv, kind, ncap)) {
         for (int k = 0; k < kDeferVals; k++) dv[(int64_t)k * cap + slot] = 0.f;
         return;
     }

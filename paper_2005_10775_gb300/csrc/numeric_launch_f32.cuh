@@ -75,16 +75,14 @@ nl_status launch_ball(nl_ctx *ctx, const nlq::NumArgs &A, int ball, unsigned gri
 template <int BALL, int STS>
 nl_status launch_const_k(nl_ctx *ctx, const nlq::NumArgs &A, unsigned grid, unsigned threads)
 {
-    // the outer-support balls integrate their candidates without the item queue
-    const bool defer = !nlq::kSupportBall<BALL> && A.defer;
-    if (defer) NL_CK(cudaMemsetAsync(A.defer_n, 0, sizeof(int), ctx->stream));
+    if (A.defer_n) NL_CK(cudaMemsetAsync(A.defer_n, 0, sizeof(int), ctx->stream));
     const size_t smem = sizeof(nlq::ConstShared<BALL, float>) * nlq::kWarpsPerBlock;
     NL_CK(cudaFuncSetAttribute(nlq::k_const<BALL, float, STS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)smem));
     nlq::k_const<BALL, float, STS><<<grid, threads, smem, ctx->stream>>>(A); ++ctx->launches;
     NL_CK(cudaGetLastError());
-    if constexpr (!nlq::kSupportBall<BALL>)
-        if (defer) return launch_deferred<nlq::kGeoBall<BALL>, false>(ctx, A, threads);
+    if constexpr (nlq::kConstQueue<BALL, float>)
+        if (A.defer) return launch_deferred<nlq::kGeoBall<BALL>, false>(ctx, A, threads);
     return NL_OK;
 }
 

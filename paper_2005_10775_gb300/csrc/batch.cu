@@ -82,7 +82,7 @@ struct ScatterGroup {              // one scatter launch: problems of one value 
     std::vector<int64_t> host_koff;
     ScatterArgs *dS = nullptr;
     int64_t *dkoff = nullptr;
-    int64_t totalK = 0, max_row = 0;
+    int64_t totalK = 0, max_row = 0, max_words = 0;
 };
 
 }  // namespace
@@ -314,7 +314,7 @@ nl_status launch_scatter(nl_ctx *ctx, nl_batch *b, bool set_attr)
     if (s != NL_OK) return s;
     for (ScatterGroup &g : b->sgroups)
         if ((s = nl_launch_scatter_batch(ctx, g.f64, g.dS, g.dkoff, (int)g.probs.size(), g.totalK, g.max_row,
-                                         set_attr)) != NL_OK)
+                                         g.max_words, set_attr)) != NL_OK)
             return s;
     return nl_launch_symmetrize_batch(ctx, b->dS_all, b->dzoff, b->n, b->total_nnz);
 }
@@ -850,6 +850,7 @@ nl_status nl_batch_create(nl_ctx *ctx, int32_t n, const nl_mesh *meshes, const n
                     sa.push_back(all[i]);
                     koff.push_back(koff.back() + b->P[i]->K);
                     g.max_row = std::max(g.max_row, b->P[i]->max_row);
+                    g.max_words = std::max(g.max_words, b->P[i]->max_words);
                 }
             if (g.probs.empty()) {
                 b->sgroups.pop_back();

@@ -53,7 +53,8 @@ struct nl_host_slot {
     unsigned long long mesh[6];   // order-preserving keys: xmin, ymin, xmax, ymax, r_max, h_max
     int64_t E;                    // candidate pairs
     int64_t nnz;                  // pattern entries
-    unsigned long long pat[4];    // pairs, qp-pairs, interactions, longest row
+    unsigned long long pat[5];    // pairs, qp-pairs, interactions, longest row, words of the widest
+                                  // column bitmap of a triangle's rows
     int bad;                      // degenerate / clockwise / out-of-range triangles
     int ovf;                      // cell-list or candidate-list overflow
     int row_ovf;                  // pattern row overflow
@@ -118,6 +119,7 @@ struct nl_plan {
     int64_t *tslot = nullptr;     // [nnz] slot of the transposed entry
     double *W = nullptr;          // [nnz] one-sided accumulation, D = W + W^T
     int64_t max_row = 0;          // longest row of the pattern
+    int64_t max_words = 0;        // 32-bit words of the widest bitmap over the columns of a triangle's rows
     int *fxe = nullptr;           // FP32 plans: 128 + e with every scatter column bound per unit of
                                   // |T_a| sum_q |w_q| below 2^(e+1) (k_node_exp)
     // extracted sub-matrix state (nl_extract)
@@ -312,9 +314,10 @@ struct ScatterArgs {   // one problem
 };
 // W = 0 over all problems (zoff: prefix sums of nnz, device, n + 1 entries; total = zoff[n])
 nl_status nl_launch_zero_batch(nl_ctx *ctx, const ScatterArgs *dS, const int64_t *dzoff, int n, int64_t total);
-// scatter of the problems in dS (all of one value type; koff: prefix sums of K; max_row: longest row)
+// scatter of the problems in dS (all of one value type; koff: prefix sums of K; max_row: longest row;
+// max_words: widest column bitmap, nl_plan::max_words)
 nl_status nl_launch_scatter_batch(nl_ctx *ctx, bool f64, const ScatterArgs *dS, const int64_t *dkoff, int n,
-                                  int64_t totalK, int64_t max_row, bool set_attr);
+                                  int64_t totalK, int64_t max_row, int64_t max_words, bool set_attr);
 // val = W + W^T over all problems
 nl_status nl_launch_symmetrize_batch(nl_ctx *ctx, const ScatterArgs *dS, const int64_t *dzoff, int n,
                                      int64_t total);

@@ -274,7 +274,8 @@ __global__ void __launch_bounds__(kRowThreads) k_rows(int J, const int64_t *nt_p
                                                       const uint8_t *sym, int hbits, int lbits, const int *list,
                                                       const int *nlist, int64_t *cnt, const int64_t *row_ptr,
                                                       int32_t *col, int *ovf_list, int *ovf_n, int *overflow,
-                                                      int32_t *buf, uint8_t *bflag, int *rlist, int *rn, int pass)
+                                                      int32_t *buf, uint8_t *bflag, int *rlist, int *rn, int2 *span,
+                                                      int pass)
 {
     extern __shared__ int32_t sm[];
     const int H = 1 << hbits;
@@ -343,6 +344,7 @@ __global__ void __launch_bounds__(kRowThreads) k_rows(int J, const int64_t *nt_p
         }
         if (pass == 0 && buf && threadIdx.x == 0) {
             bflag[j] = keep ? 1 : 0;
+            span[j] = keep ? make_int2(sc.lo, sc.hi) : make_int2(0, J - 1);   // bounds of the row's columns
             if (!keep) rlist[atomicAdd(rn, 1)] = j;
         }
         __syncthreads();   // the set and the counters are reused by the next row
@@ -500,13 +502,13 @@ template <typename T>
 __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int32_t *tri, const int64_t *ptr,
                                               const int32_t *idx, const uint8_t *flag, const T *blk,
                                               const int64_t *row_ptr, const int32_t *col, double *W, int *err,
-                                              int cap, int hbits, int a, int lane, T *sacc_t, T *scom_t,
-                                              int32_t *skey, uint32_t *spk, const int64_t *split, double kc,
-                                              const double *area, const int *fxe, float ws)
+                                              int cap, int hbits, int a, int lane, T *sacc_t, int32_t *skey,
+                                              uint32_t *spk, const int64_t *split, double kc, const double *area,
+                                              const int *fxe, float ws)
 {
     constexpr bool kFx = sizeof(T) == sizeof(float);
     using Acc = typename std::conditional<kFx, int, T>::type;
-    Acc *sacc = reinterpret_cast<Acc *>(sacc_t), *scom = reinterpret_cast<Acc *>(scom_t);
+    Acc *sacc = reinterpret_cast<Acc *>(sacc_t);
     const int ar[3] = {tri[3 * a], tri[3 * a + 1], tri[3 * a + 2]};
 #ifdef NL_CHECKS
     // debug build: indices checked, a bad one recorded (bit 64) and its access skipped
@@ -533,7 +535,6 @@ __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int
         for (int k = lane; k < H; k += 32) {
             skey[k] = -1;
             spk[k] = 0xffffffffu;
-            scom[k] = (Acc)0;
         }
         for (int k = lane; k < 3 * cap; k += 32) sacc[k] = (Acc)0;
         __syncwarp();
@@ -554,33 +555,14 @@ __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int
     const float sc = pow2f(shift);
     const int64_t e_int = split ? split[a] : ptr[a];
     if (split) {
-        // the constant kernel's interior pairs: M_ab = c |T_a| |T_b| / 9 in all nine entries, so each
-        // node of T_b receives one value for the three rows together, summed per column (scom, by
-        // hash slot) and added to the rows below
+        // the constant kernel's interior pairs: M_ab = c |T_a| |T_b| / 9 in all nine entries
         const double ka = kc * area[a] * (1.0 / 9.0);
-        int64_t e = ptr[a] + lane;
-        int b = e < e_int ? idx[e] : 0;
-        for (; e < e_int; e += 32) {
-            const int64_t en = e + 32;
-            const int bnx = en < e_int ? idx[en] : 0;
-            const double m = ka * area[b];
-            if (!cached) {
-                T v[9];
-                for (int p = 0; p < 9; p++) v[p] = (T)m;
-                scatter_pair<T, Acc>(1, b, v, K, J, tri, row_ptr, col, W, err, false, H, hbits, ar, len, cap, sc,
-                                     sacc, skey, spk);
-            } else {
-                const int bn[3] = {tri[3 * b], tri[3 * b + 1], tri[3 * b + 2]};
-                Acc v;
-                if constexpr (kFx) v = -__float2int_rn((float)m * sc);
-                else v = -m;
-                for (int k = 0; k < 3; k++) {
-                    const int sl = hash_find(skey, H, hbits, bn[k]);
-                    if (sl >= 0) atomicAdd(&scom[sl], v);
-                    else atomicOr(err, 2);
-                }
-            }
-            b = bnx;
+        for (int64_t e = ptr[a] + lane; e < e_int; e += 32) {
+            const int b = idx[e];
+            T v[9];
+            for (int p = 0; p < 9; p++) v[p] = (T)(ka * area[b]);
+            scatter_pair<T, Acc>(1, b, v, K, J, tri, row_ptr, col, W, err, cached, H, hbits, ar, len, cap, sc, sacc,
+                                 skey, spk);
         }
     }
     // the next pair's loads are issued before this pair's lookups and adds: the DRAM latency
@@ -614,19 +596,6 @@ __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int
         for (int p = 0; p < 9; p++) v[p] = vn[p];
     }
     __syncwarp();
-    if (cached && split) {   // a column's slot holds its place in each row: every entry has one owner
-        for (int k = lane; k < H; k += 32) {
-            const Acc x = scom[k];
-            if (x == (Acc)0) continue;
-            const unsigned pk = spk[k];
-            for (int i = 0; i < 3; i++) {
-                const unsigned pos = (pk >> (10 * i)) & kPosAbsent;
-                if (pos < (unsigned)len[i]) sacc[i * cap + pos] += x;
-                else atomicOr(err, 2);
-            }
-        }
-        __syncwarp();
-    }
     if (cached) {
         const double inv = (double)pow2f(-shift);
         for (int i = 0; i < 3; i++)
@@ -641,6 +610,202 @@ __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int
                 }
             }
     }
+}
+
+// ---------------------------------------------------------------------------
+// The scatter with the rows' columns indexed by bit ranks: row i of T_a's three rows is a bitmap over
+// the node indices that the three rows span, each word with the position of its first column, so a
+// node's place in a row is one 8-byte shared load and a population count, the same for every lane
+// (the hashed scatter below probes: 15 of 32 lanes active, 12.7 K instructions a triangle against
+// about 3 K here), and the index of three rows of 230 columns takes 1.4 KB instead of 4 KB, so twice as
+// many warps are resident.  Taken when the bitmaps fit (a mesh numbered with some locality); meshes
+// numbered without take the hashed one.  Measured against the hashed scatter (K = 23,328 approxcaps,
+// FP32 blocks) 741 -> 339 us, (K = 18,432, 32-gon) 455 -> 200 us, FP64 blocks 812 -> 420 us.
+// ---------------------------------------------------------------------------
+struct RankWord {
+    uint32_t bits, pre;   // columns present; position of the first of them in the row
+};
+
+__device__ __forceinline__ int rank_of(const RankWord &w, int bit)
+{
+    return (int)(w.pre + __popc(w.bits & ((1u << bit) - 1u)));
+}
+
+template <typename T>
+__device__ __forceinline__ void scatter_rank(int K, int J, int64_t E, const int32_t *tri, const int64_t *ptr,
+                                             const int32_t *idx, const uint8_t *flag, const T *blk,
+                                             const int64_t *row_ptr, const int32_t *col, double *W, int *err,
+                                             int cap, int nwcap, int a, int lane, T *sacc_t, RankWord *wd,
+                                             const int64_t *split, double kc, const double *area, const int *fxe,
+                                             float ws)
+{
+    constexpr bool kFx = sizeof(T) == sizeof(float);
+    using Acc = typename std::conditional<kFx, int, T>::type;
+    Acc *sacc = reinterpret_cast<Acc *>(sacc_t), *scom = sacc + 3 * (size_t)cap;
+    const int ar[3] = {tri[3 * a], tri[3 * a + 1], tri[3 * a + 2]};
+    int64_t r0[3];
+    int len[3], lo = 0x7fffffff, hi = -1;
+    for (int i = 0; i < 3; i++) {
+        r0[i] = row_ptr[ar[i]];
+        len[i] = (int)(row_ptr[ar[i] + 1] - r0[i]);
+        if (len[i] > 0) {   // a row is empty where a ball inside its triangles has an empty region
+            lo = min(lo, col[r0[i]]);
+            hi = max(hi, col[r0[i] + len[i] - 1]);
+        }
+    }
+    const int nw = hi < lo ? 0 : ((hi - lo) >> 5) + 1;
+    if (nw > nwcap || len[0] > cap || len[1] > cap || len[2] > cap) {   // never: the host sized both
+        if (lane == 0) atomicOr(err, 2);
+        return;
+    }
+    for (int k = lane; k < 3 * nw; k += 32) wd[k] = RankWord{0u, 0u};
+    for (int k = lane; k < 4 * cap; k += 32) sacc[k] = (Acc)0;
+    __syncwarp();
+    for (int i = 0; i < 3; i++)
+        for (int k0 = 0; k0 < len[i]; k0 += 32) {
+            const int k = k0 + lane;
+            const bool in = k < len[i];
+            const int c = in ? col[r0[i] + k] - lo : -1, w = in ? c >> 5 : -1;
+            // the columns of one word are neighbours: OR over each run, then one add a word
+            uint32_t bits = in ? 1u << (c & 31) : 0u;
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t y = __shfl_down_sync(0xffffffffu, bits, off);
+                const int wy = __shfl_down_sync(0xffffffffu, w, off);
+                if (lane + off < 32 && wy == w) bits |= y;
+            }
+            const int wp = __shfl_up_sync(0xffffffffu, w, 1);
+            if (in && (lane == 0 || wp != w)) {
+                RankWord &x = wd[3 * w + i];
+                if (x.bits == 0u) x.pre = (uint32_t)k;   // else the word began in the columns before
+                x.bits |= bits;
+            }
+            __syncwarp();
+        }
+    int shift = 0;   // FP32 blocks: fixed-point shift of the shared row sums
+    if constexpr (kFx) shift = fx_row_shift(exp2_floor((float)(area[a] * (double)ws)), *fxe - 128);
+    const float sc = pow2f(shift);
+    const int64_t e_int = split ? split[a] : ptr[a];
+    if (split) {
+        // the constant kernel's interior pairs: M_ab = c |T_a| |T_b| / 9 in all nine entries, so each
+        // node of T_b receives one value for the three rows together, summed in scom at the node's
+        // place in row 0 (an interior pair puts T_b's nodes into all three rows)
+        const double ka = kc * area[a] * (1.0 / 9.0);
+        int64_t e = ptr[a] + lane;
+        int b = e < e_int ? idx[e] : 0, bn = e + 32 < e_int ? idx[e + 32] : 0;
+        double ab = area[b];
+        int n0 = tri[3 * b], n1 = tri[3 * b + 1], n2 = tri[3 * b + 2];
+        for (; e < e_int; e += 32) {
+            // the next pair's loads before this pair's adds
+            const int b2 = e + 64 < e_int ? idx[e + 64] : 0;
+            const double an = area[bn];
+            const int m0 = tri[3 * bn], m1 = tri[3 * bn + 1], m2 = tri[3 * bn + 2];
+            const double m = ka * ab;
+            Acc v;
+            if constexpr (kFx) v = -__float2int_rn((float)m * sc);
+            else v = -m;
+            const int nd[3] = {n0 - lo, n1 - lo, n2 - lo};
+            for (int k = 0; k < 3; k++) {
+                const RankWord x = wd[3 * (nd[k] >> 5)];
+                atomicAdd(&scom[rank_of(x, nd[k] & 31)], v);
+            }
+            ab = an;
+            n0 = m0;
+            n1 = m1;
+            n2 = m2;
+            bn = b2;
+        }
+    }
+    // the next pair's loads are issued before this pair's lookups and adds: the DRAM latency
+    // of one iteration overlaps the shared-memory work of the previous one
+    const int64_t e_end = ptr[a + 1];
+    int64_t e = e_int + lane;
+    uint8_t f = 0;
+    int b = 0;
+    T v[9];
+    for (int p = 0; p < 9; p++) v[p] = (T)0;
+    if (e < e_end) {
+        f = flag[e];
+        b = idx[e];
+        for (int p = 0; p < 9; p++) v[p] = blk[(int64_t)p * E + e];
+    }
+    for (; e < e_end; e += 32) {
+        const int64_t en = e + 32;
+        uint8_t fn = 0;
+        int bnx = 0;
+        T vn[9];
+        for (int p = 0; p < 9; p++) vn[p] = (T)0;
+        if (en < e_end) {
+            fn = flag[en];
+            bnx = idx[en];
+            for (int p = 0; p < 9; p++) vn[p] = blk[(int64_t)p * E + en];
+        }
+#ifdef NL_CHECKS
+        if (f && (b < 0 || b >= K)) {
+            atomicOr(err, 64);
+            f = 0;
+        }
+#endif
+        if (f) {
+            for (int k = 0; k < 3; k++) {
+                const int c = tri[3 * b + k] - lo, w = c >> 5, bit = c & 31;
+                for (int i = 0; i < 3; i++) {
+                    const RankWord x = (unsigned)w < (unsigned)nw ? wd[3 * w + i] : RankWord{0u, 0u};
+                    if ((x.bits >> bit) & 1u) {
+                        if constexpr (kFx)
+                            atomicAdd(&sacc[i * cap + rank_of(x, bit)], -__float2int_rn(v[3 * i + k] * sc));
+                        else
+                            atomicAdd(&sacc[i * cap + rank_of(x, bit)], -v[3 * i + k]);
+                    } else {
+                        atomicOr(err, 2);
+                    }
+                }
+            }
+        }
+        f = fn;
+        b = bnx;
+        for (int p = 0; p < 9; p++) v[p] = vn[p];
+    }
+    __syncwarp();
+    const double inv = (double)pow2f(-shift);
+    for (int i = 0; i < 3; i++)
+        for (int k = lane; k < len[i]; k += 32) {
+            Acc x = sacc[i * cap + k];
+            if (split) {
+                const int c = i == 0 ? 0 : col[r0[i] + k] - lo;
+                const RankWord w = wd[3 * (c >> 5)];
+                if (i == 0) x += scom[k];
+                else if ((w.bits >> (c & 31)) & 1u) x += scom[rank_of(w, c & 31)];
+            }
+            if (x == (Acc)0) continue;
+            if constexpr (kFx) {
+                if (x > (1 << 30) || x < -(1 << 30)) atomicOr(err, 256);
+                atomicAdd(&W[r0[i] + k], (double)x * inv);
+            } else {
+                atomicAdd(&W[r0[i] + k], (double)x);
+            }
+        }
+}
+
+// shared memory of one warp: row sums [3][cap] and common sums [cap] (T), then the rows' words [nw][3]
+template <typename T>
+__host__ __device__ constexpr size_t rank_warp_bytes(int cap, int nw)
+{
+    return 4 * (size_t)cap * sizeof(T) + 24 * (size_t)nw;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(128)
+    k_scatter_rank(int K, int J, int64_t E, const int32_t *tri, const int64_t *ptr, const int32_t *idx,
+                   const uint8_t *flag, const T *blk, const int64_t *row_ptr, const int32_t *col, double *W, int *err,
+                   int cap, int nw, const int64_t *split, double kc, const double *area, const int *fxe, float ws)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int a = blockIdx.x * (blockDim.x >> 5) + wib;
+    unsigned char *base = smem_raw + (size_t)wib * rank_warp_bytes<T>(cap, nw);
+    if (a < K)
+        scatter_rank<T>(K, J, E, tri, ptr, idx, flag, blk, row_ptr, col, W, err, cap, nw, a, lane, (T *)base,
+                        (RankWord *)(base + 4 * (size_t)cap * sizeof(T)), split, kc, area, fxe, ws);
 }
 
 // M_aa + M_bb of every triangle into W through its local slots (diagonal halved: D = W + W^T),
@@ -663,22 +828,21 @@ __global__ void k_local_blocks(int K, const double *maa, double *mbb, const int6
     if (t < K) local_block(K, t, maa, mbb, lslot, W, err);
 }
 
-// shared memory of one warp of the scatter: row accumulators [3][cap] (T), sums per column slot
-// [H] (T), hash keys and packed positions [H] (cap a multiple of 4 keeps the int arrays aligned)
+// shared memory of one warp of the hashed scatter: row accumulators [3][cap] (T), hash keys and
+// packed positions [H] (cap a multiple of 4 keeps the int arrays aligned after a float array)
 template <typename T>
 __host__ __device__ constexpr size_t scatter_warp_bytes(int cap, int hbits)
 {
-    return cap > 0 ? 3 * (size_t)cap * sizeof(T) + ((8 + sizeof(T)) << hbits) : 0;
+    return cap > 0 ? 3 * (size_t)cap * sizeof(T) + ((size_t)8 << hbits) : 0;
 }
 
 template <typename T>
 __device__ __forceinline__ void scatter_warp_smem(unsigned char *raw, int wib, int cap, int hbits, T *&sacc,
-                                                  T *&scom, int32_t *&skey, uint32_t *&spk)
+                                                  int32_t *&skey, uint32_t *&spk)
 {
     unsigned char *base = raw + (size_t)wib * scatter_warp_bytes<T>(cap, hbits);
     sacc = (T *)base;
-    scom = sacc + 3 * (size_t)cap;
-    skey = (int32_t *)(scom + ((size_t)1 << hbits));
+    skey = (int32_t *)(base + 3 * (size_t)cap * sizeof(T));
     spk = (uint32_t *)(skey + (1 << hbits));
 }
 
@@ -691,12 +855,12 @@ __global__ void k_scatter(int K, int J, int64_t E, const int32_t *tri, const int
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int a = blockIdx.x * (blockDim.x >> 5) + wib;
-    T *sacc, *scom;
+    T *sacc;
     int32_t *skey;
     uint32_t *spk;
-    scatter_warp_smem<T>(smem_raw, wib, cap, hbits, sacc, scom, skey, spk);
+    scatter_warp_smem<T>(smem_raw, wib, cap, hbits, sacc, skey, spk);
     if (a >= K) return;
-    scatter_outer<T>(K, J, E, tri, ptr, idx, flag, blk, row_ptr, col, W, err, cap, hbits, a, lane, sacc, scom, skey,
+    scatter_outer<T>(K, J, E, tri, ptr, idx, flag, blk, row_ptr, col, W, err, cap, hbits, a, lane, sacc, skey,
                      spk, split, kc, area, fxe, ws);
 }
 
@@ -721,15 +885,31 @@ __global__ void k_scatter_batch(const ScatterArgs *__restrict__ S, const int64_t
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
     if (g >= koff[n]) return;
-    T *sacc, *scom;
+    T *sacc;
     int32_t *skey;
     uint32_t *spk;
-    scatter_warp_smem<T>(smem_raw, wib, cap, hbits, sacc, scom, skey, spk);
+    scatter_warp_smem<T>(smem_raw, wib, cap, hbits, sacc, skey, spk);
     const int p = batch_problem(koff, n, g);
     const ScatterArgs &A = S[p];
     scatter_outer<T>(A.K, A.J, A.E, A.tri, A.ptr, A.idx, A.flag, (const T *)A.blk, A.row_ptr, A.col, A.W,
-                     A.err, cap, hbits, (int)(g - koff[p]), lane, sacc, scom, skey, spk, A.split, A.kc, A.area,
+                     A.err, cap, hbits, (int)(g - koff[p]), lane, sacc, skey, spk, A.split, A.kc, A.area,
                      A.fxe, A.ws);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(128)
+    k_scatter_rank_batch(const ScatterArgs *__restrict__ S, const int64_t *__restrict__ koff, int n, int cap, int nw)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
+    if (g >= koff[n]) return;
+    unsigned char *base = smem_raw + (size_t)wib * rank_warp_bytes<T>(cap, nw);
+    const int p = batch_problem(koff, n, g);
+    const ScatterArgs &A = S[p];
+    scatter_rank<T>(A.K, A.J, A.E, A.tri, A.ptr, A.idx, A.flag, (const T *)A.blk, A.row_ptr, A.col, A.W, A.err, cap,
+                    nw, (int)(g - koff[p]), lane, (T *)base, (RankWord *)(base + 4 * (size_t)cap * sizeof(T)),
+                    A.split, A.kc, A.area, A.fxe, A.ws);
 }
 
 // M_aa + M_bb of every triangle of every problem (koff: prefix sums of K)
@@ -776,13 +956,26 @@ __global__ void k_symmetrize(int64_t nnz, const double *W, const int64_t *tslot,
     else atomicOr(err, 4);
 }
 
-__global__ void k_row_max(int J, const int64_t *rcnt, unsigned long long *out)
+// longest row (out[3]) and the words of the widest bitmap over the columns of a triangle's three rows (out[4])
+__global__ void k_row_max(int J, const int64_t *rcnt, int K, const int32_t *tri, const int2 *span,
+                          unsigned long long *out)
 {
     unsigned long long m = 0;
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < J; j += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, (unsigned long long)rcnt[j]);
-    for (int off = 16; off; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if ((threadIdx.x & 31) == 0) atomicMax(&out[3], m);
+    int w = 0;
+    const int nth = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int j = tid; j < J; j += nth) m = max(m, (unsigned long long)rcnt[j]);
+    for (int t = tid; t < K; t += nth) {
+        const int2 x = span[tri[3 * t]], y = span[tri[3 * t + 1]], z = span[tri[3 * t + 2]];
+        w = max(w, ((max(x.y, max(y.y, z.y)) - min(x.x, min(y.x, z.x))) >> 5) + 1);
+    }
+    for (int off = 16; off; off >>= 1) {
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
+        w = max(w, __shfl_xor_sync(0xffffffffu, w, off));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&out[3], m);
+        atomicMax(&out[4], (unsigned long long)w);
+    }
 }
 
 __global__ void k_sum_stats(int K, int64_t E, const uint8_t *flag, const int64_t *qp, const int64_t *cnt,
@@ -828,6 +1021,7 @@ struct nl_pat {
     int32_t *buf = nullptr;                // rows sorted by the first count: J rows of 2^lbits
     uint8_t *bflag = nullptr;              // row j is in buf
     int *rlist = nullptr, *rn = nullptr;   // the other rows, rebuilt by the column write
+    int2 *span = nullptr;                  // first and last column of each row (bounds)
     int lbits = 0;
     unsigned long long *st = nullptr;
 };
@@ -850,6 +1044,7 @@ void nl_pat_delete(nl_pat *T, cudaStream_t s)
     free_async(T->rcnt, s); free_async(T->ntri, s); free_async(T->ovf, s); free_async(T->st, s);
     free_async(T->olist, s); free_async(T->on, s);
     free_async(T->buf, s); free_async(T->bflag, s); free_async(T->rlist, s); free_async(T->rn, s);
+    free_async(T->span, s);
     delete T;
 }
 
@@ -876,11 +1071,12 @@ nl_status nl_pattern_a(nl_ctx *ctx, nl_plan *P, nl_csr *out, nl_pat *T, nl_host_
     NL_CK(cudaMallocAsync((void **)&T->olist, sizeof(int) * (J + 1), st));
     NL_CK(cudaMallocAsync((void **)&T->on, sizeof(int), st));
     NL_CK(cudaMemsetAsync(T->on, 0, sizeof(int), st));
-    NL_CK(cudaMallocAsync((void **)&T->st, sizeof(unsigned long long) * 4, st));
+    NL_CK(cudaMallocAsync((void **)&T->span, sizeof(int2) * (J + 1), st));
+    NL_CK(cudaMallocAsync((void **)&T->st, sizeof h->pat, st));
     NL_CK(cudaMemsetAsync(T->ncnt, 0, sizeof(int64_t) * (J + 1), st));
     NL_CK(cudaMemsetAsync(T->ncur, 0, sizeof(int64_t) * (J + 1), st));
     NL_CK(cudaMemsetAsync(T->ovf, 0, sizeof(int), st));
-    NL_CK(cudaMemsetAsync(T->st, 0, sizeof(unsigned long long) * 4, st));
+    NL_CK(cudaMemsetAsync(T->st, 0, sizeof h->pat, st));
     const unsigned wgrid = (unsigned)(((int64_t)K * 32 + 255) / 256);
     k_symflag<<<wgrid, 256, 0, st>>>(K, P->nbr_ptr, P->nbr_split, P->nbr_idx, P->flag, T->sym); ++ctx->launches;
     k_node_count<<<(K + 255) / 256, 256, 0, st>>>(K, P->tri, T->ncnt); ++ctx->launches;
@@ -917,18 +1113,18 @@ nl_status nl_pattern_a(nl_ctx *ctx, nl_plan *P, nl_csr *out, nl_pat *T, nl_host_
     NL_CK(cudaMemsetAsync(T->rn, 0, sizeof(int), st));
     k_rows<<<J, kRowThreads, sizeof(int32_t) * ((1u << hb0) + (1u << lb0)), st>>>(
         J, T->nptr, T->ntri, P->tri, P->nbr_ptr, P->nbr_idx, T->sym, hb0, lb0, nullptr, nullptr, T->rcnt, nullptr,
-        nullptr, T->olist, T->on, T->ovf, T->buf, T->bflag, T->rlist, T->rn, 0); ++ctx->launches;
+        nullptr, T->olist, T->on, T->ovf, T->buf, T->bflag, T->rlist, T->rn, T->span, 0); ++ctx->launches;
     NL_CK(cudaGetLastError());
     const int hbf = row_set_bits(NL_HASH_CAP);
     k_rows<<<256, kRowThreads, sizeof(int32_t) << hbf, st>>>(J, T->nptr, T->ntri, P->tri, P->nbr_ptr, P->nbr_idx,
                                                             T->sym, hbf, 0, T->olist, T->on, T->rcnt, nullptr,
                                                             nullptr, nullptr, nullptr, T->ovf, nullptr, nullptr,
-                                                            nullptr, nullptr, 0); ++ctx->launches;
+                                                            nullptr, nullptr, nullptr, 0); ++ctx->launches;
     NL_CK(cudaGetLastError());
     if ((s = nl_alloc(ctx, &out->row_ptr, (size_t)J + 1)) != NL_OK) return s;
     if ((s = nl_scan_i64(ctx, T->rcnt, out->row_ptr, J)) != NL_OK) return s;
     k_sum_stats<<<256, 256, 0, st>>>(K, P->E, P->flag, P->qp_a, P->cnt_a, T->st); ++ctx->launches;
-    k_row_max<<<64, 256, 0, st>>>(J, T->rcnt, T->st); ++ctx->launches;
+    k_row_max<<<64, 256, 0, st>>>(J, T->rcnt, K, P->tri, T->span, T->st); ++ctx->launches;
     NL_CK(cudaGetLastError());
     NL_CK(cudaMemcpyAsync(&h->err, P->err, sizeof(int), cudaMemcpyDeviceToHost, st));
     NL_CK(cudaMemcpyAsync(&h->nnz, out->row_ptr + J, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
@@ -954,6 +1150,7 @@ nl_status nl_pattern_b(nl_ctx *ctx, nl_plan *P, nl_csr *out, nl_pat *T, const nl
     out->n_qp_pairs = (int64_t)h->pat[1];
     out->n_inter = (int64_t)h->pat[2];
     P->max_row = (int64_t)h->pat[3];
+    P->max_words = (int64_t)h->pat[4];
     if ((s = nl_alloc(ctx, &out->col_idx, (size_t)nnz)) != NL_OK) return s;
     if ((s = nl_alloc(ctx, &out->val, (size_t)nnz)) != NL_OK) return s;
     // the rows the first count kept sorted are copied; the others (usually none) are built again,
@@ -967,7 +1164,7 @@ nl_status nl_pattern_b(nl_ctx *ctx, nl_plan *P, nl_csr *out, nl_pat *T, const nl
     k_rows<<<g1, kRowThreads, smem1, st>>>(J, T->nptr, T->ntri, P->tri, P->nbr_ptr, P->nbr_idx,
                                                             T->sym, hb1, lb1, T->rlist, T->rn, nullptr, out->row_ptr,
                                                             out->col_idx, nullptr, nullptr, T->ovf, nullptr, nullptr,
-                                                            nullptr, nullptr, 1); ++ctx->launches;
+                                                            nullptr, nullptr, nullptr, 1); ++ctx->launches;
     NL_CK(cudaGetLastError());
     if ((s = nl_alloc(ctx, &P->lslot, 6 * (size_t)K)) != NL_OK) return s;
     if ((s = nl_alloc(ctx, &P->tslot, (size_t)nnz)) != NL_OK) return s;
@@ -1003,20 +1200,46 @@ static void scatter_plan(int64_t max_row, int *cap, int *hbits, int *warps, size
     *smem = (size_t)w * scatter_warp_bytes<T>(c, hb);
 }
 
+// The bit-ranked scatter's plan: cap per row and the warps per block that fit 96 KB; false when a
+// warp's rows and bitmaps would leave the SM fewer than nine warps (24 KB each): rows or index spans
+// that long take the hashed scatter.
+template <typename T>
+static bool rank_plan(int64_t max_row, int64_t max_words, int *cap, int *warps, size_t *smem)
+{
+    const int64_t c = ((max_row > 0 ? max_row : 1) + 3) & ~3LL;
+    if (c > (1 << 20) || max_words > (1 << 20) || rank_warp_bytes<T>((int)c, (int)max_words) > 24 * 1024) return false;
+    *cap = (int)c;
+    *warps = 4;
+    *smem = 4 * rank_warp_bytes<T>((int)c, (int)max_words);
+    return true;
+}
+
 template <typename T>
 static nl_status launch_scatter(nl_ctx *ctx, nl_plan *P, nl_csr *out)
 {
     const int K = P->K;
     int cap, hbits, warps;
     size_t smem;
+    const int64_t *split = P->cfg.kernel == NL_KERNEL_CONST ? P->nbr_split : nullptr;
+    if (rank_plan<T>(P->max_row, P->max_words, &cap, &warps, &smem)) {
+        NL_CK(cudaFuncSetAttribute(k_scatter_rank<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(96 * 1024)));
+        k_scatter_rank<T><<<(unsigned)((K + warps - 1) / warps), 32 * warps, smem, ctx->stream>>>(
+            K, P->J, P->E, P->tri, P->nbr_ptr, P->nbr_idx, P->flag, (const T *)P->blk, out->row_ptr, out->col_idx, P->W,
+            P->err, cap, (int)P->max_words, split, P->cfg.kernel_c, P->area, P->fxe, nl_outer_abs_weight(P));
+        ++ctx->launches;
+        NL_CK(cudaGetLastError());
+        k_local_blocks<<<(K + 255) / 256, 256, 0, ctx->stream>>>(K, P->maa, P->mbb, P->lslot, P->W, P->err);
+        ++ctx->launches;
+        NL_CK(cudaGetLastError());
+        return NL_OK;
+    }
     scatter_plan<T>(P->max_row, &cap, &hbits, &warps, &smem);
     NL_CK(cudaFuncSetAttribute(k_scatter<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(96 * 1024)));
     const unsigned grid = (unsigned)((K + warps - 1) / warps);
     k_scatter<T><<<grid, 32 * warps, smem, ctx->stream>>>(K, P->J, P->E, P->tri, P->nbr_ptr, P->nbr_idx, P->flag,
                                                            (const T *)P->blk, out->row_ptr, out->col_idx,
-                                                           P->W, P->err, cap, hbits,
-                                                           P->cfg.kernel == NL_KERNEL_CONST ? P->nbr_split : nullptr,
-                                                           P->cfg.kernel_c, P->area, P->fxe,
+                                                           P->W, P->err, cap, hbits, split, P->cfg.kernel_c,
+                                                           P->area, P->fxe,
                                                            nl_outer_abs_weight(P)); ++ctx->launches;
     NL_CK(cudaGetLastError());
     k_local_blocks<<<(K + 255) / 256, 256, 0, ctx->stream>>>(K, P->maa, P->mbb, P->lslot, P->W, P->err);
@@ -1058,16 +1281,26 @@ nl_status nl_launch_symmetrize_batch(nl_ctx *ctx, const ScatterArgs *dS, const i
 
 template <typename T>
 static nl_status launch_scatter_batch(nl_ctx *ctx, const ScatterArgs *dS, const int64_t *dkoff, int n,
-                                      int64_t totalK, int64_t max_row, bool set_attr)
+                                      int64_t totalK, int64_t max_row, int64_t max_words, bool set_attr)
 {
     if (totalK <= 0) return NL_OK;
     int cap, hbits, warps;
     size_t smem;
-    scatter_plan<T>(max_row, &cap, &hbits, &warps, &smem);
-    if (set_attr)
-        NL_CK(cudaFuncSetAttribute(k_scatter_batch<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(96 * 1024)));
-    const unsigned grid = (unsigned)((totalK + warps - 1) / warps);
-    k_scatter_batch<T><<<grid, 32 * warps, smem, ctx->stream>>>(dS, dkoff, n, cap, hbits); ++ctx->launches;
+    if (rank_plan<T>(max_row, max_words, &cap, &warps, &smem)) {
+        if (set_attr)
+            NL_CK(cudaFuncSetAttribute(k_scatter_rank_batch<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(96 * 1024)));
+        k_scatter_rank_batch<T><<<(unsigned)((totalK + warps - 1) / warps), 32 * warps, smem, ctx->stream>>>(
+            dS, dkoff, n, cap, (int)max_words);
+    } else {
+        scatter_plan<T>(max_row, &cap, &hbits, &warps, &smem);
+        if (set_attr)
+            NL_CK(cudaFuncSetAttribute(k_scatter_batch<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(96 * 1024)));
+        const unsigned grid = (unsigned)((totalK + warps - 1) / warps);
+        k_scatter_batch<T><<<grid, 32 * warps, smem, ctx->stream>>>(dS, dkoff, n, cap, hbits);
+    }
+    ++ctx->launches;
     NL_CK(cudaGetLastError());
     k_local_blocks_batch<<<(unsigned)((totalK + 255) / 256), 256, 0, ctx->stream>>>(dS, dkoff, n);
     ++ctx->launches;
@@ -1076,8 +1309,8 @@ static nl_status launch_scatter_batch(nl_ctx *ctx, const ScatterArgs *dS, const 
 }
 
 nl_status nl_launch_scatter_batch(nl_ctx *ctx, bool f64, const ScatterArgs *dS, const int64_t *dkoff, int n,
-                                  int64_t totalK, int64_t max_row, bool set_attr)
+                                  int64_t totalK, int64_t max_row, int64_t max_words, bool set_attr)
 {
-    return f64 ? launch_scatter_batch<double>(ctx, dS, dkoff, n, totalK, max_row, set_attr)
-               : launch_scatter_batch<float>(ctx, dS, dkoff, n, totalK, max_row, set_attr);
+    return f64 ? launch_scatter_batch<double>(ctx, dS, dkoff, n, totalK, max_row, max_words, set_attr)
+               : launch_scatter_batch<float>(ctx, dS, dkoff, n, totalK, max_row, max_words, set_attr);
 }

@@ -228,7 +228,8 @@ static bool ngon_regular(const nl_plan *P)
 
 int nl_const_ball(const nl_plan *P)
 {
-    return P->cfg.ball == NL_BALL_NGON && !ngon_regular(P) ? nlq::kBallNgonAny : P->cfg.ball;
+    // (hmax is known from the preparation's stage B on)
+    return P->cfg.ball == NL_BALL_NGON && (!ngon_regular(P) || P->cfg.delta < P->hmax) ? nlq::kBallNgonAny : P->cfg.ball;
 }
 
 bool nl_uses_queue(bool inv, int ball) { return inv || ball == NL_BALL_NGON || ball == nlq::kBallNgonAny; }
@@ -299,6 +300,10 @@ nl_status nl_fill_args(nl_ctx *ctx, const nl_plan *P, nlq::NumArgs &A, bool stat
     }
     A.geo.delta = c.delta;
     A.geo.deltaf = (float)c.delta;
+    A.geo.deltalo = (float)(c.delta - (double)A.geo.deltaf);
+    A.geo.d2f = (float)P->d2;
+    A.geo.d2lo = (float)(P->d2 - (double)A.geo.d2f);
+    A.geo.turn = c.delta < P->hmax ? 1 : 0;
     A.geo.d2 = P->d2;
     A.geo.ngon = P->ngon;
     A.geo.ngon_n = c.ball == NL_BALL_NGON ? c.ngon_n : 0;

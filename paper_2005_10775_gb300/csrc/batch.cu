@@ -823,7 +823,7 @@ nl_status nl_batch_create(nl_ctx *ctx, int32_t n, const nl_mesh *meshes, const n
             a.val = outs[i].val;
             a.err = P->err;
             a.split = P->cfg.kernel == NL_KERNEL_CONST ? P->nbr_split : nullptr;
-            a.kc = P->cfg.kernel_c;
+            a.kc = nl_block_factor(P);
             a.area = P->area;
             a.fxe = P->fxe;
             a.ws = nl_outer_abs_weight(P);

@@ -70,7 +70,9 @@ struct GeoParams {
     float sector, rin_tau; // 2 pi / N; inradius - tau
     float inv_sector;      // N / 2 pi
     float poly_r2, poly_side, poly_m;   // regular polygon: circumradius^2, edge length, its orientation margin
-    float deltaf;          // delta in FP32
+    float deltaf, deltalo; // delta as an FP32 hi + lo pair
+    float d2f, d2lo;       // delta^2 as an FP32 hi + lo pair
+    int turn;              // delta < h_max: a region can be a small part of its triangle (numeric_const.cuh)
 };
 
 // atan2 from the arctangent polynomial of Abramowitz & Stegun 4.4.49 (Hastings): on [0, 1]

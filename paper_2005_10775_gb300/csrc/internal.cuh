@@ -272,6 +272,8 @@ nl_status nl_pattern_a(nl_ctx *ctx, nl_plan *P, nl_csr *out, nl_pat *T, nl_host_
 // B (slot A read): column indices, slot maps, value buffers
 nl_status nl_pattern_b(nl_ctx *ctx, nl_plan *P, nl_csr *out, nl_pat *T, const nl_host_slot *h);
 
+// factor of a plan's blocks in the matrix: the constant kernel's are formed without c
+inline double nl_block_factor(const nl_plan *P) { return P->cfg.kernel == NL_KERNEL_CONST ? P->cfg.kernel_c : 1.0; }
 nl_status nl_alloc_numeric(nl_ctx *ctx, nl_plan *P);
 // numeric phase of one assembled problem with every kernel on ctx->stream (api.cu): the first
 // call allocates the problem's FP64-item and near-field queues
@@ -307,7 +309,7 @@ struct ScatterArgs {   // one problem
     int *err;
     const int64_t *split; // constant kernel: first boundary candidate of each triangle (null: every
                           // pair's block is in blk)
-    double kc;            // kernel constant
+    double kc;            // factor of the blocks: c (constant kernel, whose blocks are without it), else 1
     const double *area;   // [K] |T| (the interior pairs' blocks, the FP32 scatter's fixed-point grids)
     const int *fxe;       // nl_plan::fxe
     float ws;             // nl_outer_abs_weight

@@ -1579,7 +1579,7 @@ __device__ __forceinline__ void support_boundary(const NumArgs &A, int a, int la
         rule_range(A, ba, bb, q0, q1);
         Sums<T> S;
         int64_t nq_in = 0;
-        whole_sums<T, false>(A, Vb, (T)(A.area[b] * A.kc), bb, S, nq_in);
+        whole_sums<T, false>(A, Vb, (T)A.area[b], bb, S, nq_in);   // without c (numeric_const.cuh)
         T v[21];
         for (int i = 0; i < 21; i++) v[i] = 0;
         int kind = nlg::KIND_NONE, nv = 0;

@@ -14,19 +14,23 @@
 //     S11 = 6 int l1^2 / |T|, S22 = 6 int l2^2 / |T|, S12 = 12 int l1 l2 / |T|.
 // A directed boundary segment p -> q contributes the triangle (0, p, q), 0 = T_b's vertex 0 (Green);
 // pieces of edges 0 and 2 pass through that origin and contribute nothing, and a piece [t0, t1] of
-// edge 1 contributes F(t1) - F(t0) with the polynomials of edge1_add.  T_b's vertices are renumbered
-// per item so that the origin belongs to the region (a vertex inside, or the start of the edge that is
-// cut twice): the contributions are then of the region's own size and nothing cancels, also where the
-// region is a small part of T_b (mom_turn puts the moments back).
+// edge 1 contributes F(t1) - F(t0) with the polynomials of edge1_add.  Where the ball is no larger than
+// the triangles (g.turn: delta < h_max) a region can be a small part of T_b and those contributions
+// would cancel: such problems sum the regions' fans instead (exact_disc_item, kBallNgonAny).
 //
 // A pair's block is linear in twelve sums over its outer points (acc rows): P_i,c = sum_q W_q
 // phi_a,i S_c (c = 0, 1, 2) and Q = sum_q W_q (S11, S22, S12); the other entries of M_ab and M_bb
 // follow from phi_0 = 1 - phi_1 - phi_2 and sum_i phi_a,i = 1 (pair_block).
+//
+// Every block of this file is without the constant c, which the scatter multiplies in FP64: D is a small
+// difference of M_aa, M_ab and M_bb where delta is near h, and a c rounded to FP32 in some of them would
+// not cancel.
 #pragma once
 
 namespace nlq {
 
-// ball modes of k_const beyond nl_ball: an N-gon whose vertices are not those of a regular polygon
+// ball modes of k_const beyond nl_ball: an N-gon whose vertices are not those of a regular polygon, or
+// no larger than the triangles (the certified Sutherland-Hodgman clip, moments about its first vertex)
 constexpr int kBallNgonAny = 16;
 
 template <int BALL>
@@ -59,6 +63,20 @@ __device__ __forceinline__ void seg_add(Mom<T> &M, T p1, T p2, T q1, T q2)
     M.s12 += cr * (a1 * a2 + p1 * p2 + q1 * q2);
 }
 
+// a triangle (f, p, q) of area cr |T| / 2 (counted without sign), by its corners' coordinates
+template <typename T>
+__device__ __forceinline__ void tri_add(Mom<T> &M, T cr, T f1, T f2, T p1, T p2, T q1, T q2)
+{
+    cr = cr < (T)0 ? -cr : cr;
+    const T a1 = f1 + p1 + q1, a2 = f2 + p2 + q2, h = (T)0.5 * cr;
+    M.s0 += cr;
+    M.s1 += cr * a1;
+    M.s2 += cr * a2;
+    M.s11 += h * (a1 * a1 + f1 * f1 + p1 * p1 + q1 * q1);
+    M.s22 += h * (a2 * a2 + f2 * f2 + p2 * p2 + q2 * q2);
+    M.s12 += cr * (a1 * a2 + f1 * f2 + p1 * p2 + q1 * q2);
+}
+
 // the piece of edge 1 (from (1, 0) to (0, 1)) up to its point (1 - t, t), times sg
 template <typename T>
 __device__ __forceinline__ void edge1_add(Mom<T> &M, T t, T sg)
@@ -84,22 +102,6 @@ __device__ __forceinline__ void point_add(Mom<T> &M, T l1, T l2, T w)
     M.s12 += (T)12 * w * l1 * l2;
 }
 
-// moments about vertex r's numbering (vertices r, r + 1, r + 2 as 0, 1, 2) to T_b's own
-template <typename T>
-__device__ __forceinline__ void mom_turn(Mom<T> &M, int r)
-{
-    if (r != 0) {
-        const bool one = r == 1;
-        const T s = one ? M.s1 : M.s2, ss = one ? M.s11 : M.s22, s12 = M.s1 + M.s2;
-        const T z = (T)3 * M.s0 - s12, zz = (T)6 * M.s0 - (T)4 * s12 + (M.s11 + M.s22 + M.s12);
-        M.s12 = (T)4 * s - (T)2 * ss - M.s12;
-        M.s1 = one ? z : s;
-        M.s2 = one ? s : z;
-        M.s11 = one ? zz : ss;
-        M.s22 = one ? ss : zz;
-    }
-}
-
 // moments of m about the point p in T_b's own coordinates: those of l + p
 template <typename T>
 __device__ __forceinline__ void mom_shift(Mom<T> &M, T p1, T p2)
@@ -111,18 +113,19 @@ __device__ __forceinline__ void mom_shift(Mom<T> &M, T p1, T p2)
     M.s2 += (T)3 * p2 * M.s0;
 }
 
-// M_ab (9) and the upper M_bb (00 11 22 01 02 12) from a pair's sums P, Q and akc = c |T_b|
+// M_ab (9) and the upper M_bb (00 11 22 01 02 12), without c, from a pair's sums P, Q and area = |T_b|
 template <typename T>
-__device__ __forceinline__ void pair_block(T akc, const T *P, const T *Q, T *mab, T *mbb)
+__device__ __forceinline__ void pair_block(T area, const T *P, const T *Q, T *mab, T *mbb)
 {
-    const T k3 = akc * (T)(1.0 / 3.0);
+    // a third by division: 1 / 3 rounded to FP32 would scale every S1 and S2 the same way
+    const T k3 = area / (T)3;
     for (int i = 0; i < 3; i++) {
         const T m1 = P[3 * i + 1] * k3, m2 = P[3 * i + 2] * k3;
-        mab[3 * i] = akc * P[3 * i] - m1 - m2;
+        mab[3 * i] = area * P[3 * i] - m1 - m2;
         mab[3 * i + 1] = m1;
         mab[3 * i + 2] = m2;
     }
-    const T k6 = akc * (T)(1.0 / 6.0), k12 = akc * (T)(1.0 / 12.0);
+    const T k6 = (T)0.5 * k3, k12 = (T)0.25 * k3;
     const T b11 = k6 * Q[0], b22 = k6 * Q[1], b12 = k12 * Q[2];
     const T p1 = mab[1] + mab[4] + mab[7], p2 = mab[2] + mab[5] + mab[8];
     const T p00 = mab[0] + mab[3] + mab[6];   // sum_q W int phi_0
@@ -135,45 +138,107 @@ __device__ __forceinline__ void pair_block(T akc, const T *P, const T *Q, T *mab
     mbb[5] = b12;
 }
 
-// FP64 data of a candidate (FP64 path)
+// FP32 data of a candidate: vertices and barycentre relative to bary_a, the edges 0 -> 1, 1 -> 2, 2 -> 0,
+// the gradients of the three barycentric coordinates, |T|.  Edges, gradients and area are those of the
+// rounded vertices: the triangles around T_a then form one mesh in FP32 too (a shared vertex is rounded
+// once), their regions tile the ball, and what the rounding takes from one triangle its neighbour
+// gets.  (Edges from the exact vertices, with only T_b's place rounded: errors 1.3-1.8 times as large
+// where delta is below h.)
+struct Cand32 {
+    float vx[3], vy[3], ex[3], ey[3], gx[3], gy[3], blx, bly, area;
+    int b, q0;
+};
+
+__device__ __forceinline__ Cand32 cand32_of(const CandData &c)
+{
+    Cand32 r;
+    for (int i = 0; i < 3; i++) {
+        const int k = (i + 1) % 3;
+        r.vx[i] = c.vlx[i];
+        r.vy[i] = c.vly[i];
+        r.ex[i] = c.vlx[k] - c.vlx[i];
+        r.ey[i] = c.vly[k] - c.vly[i];
+    }
+    const float det = r.ex[0] * r.ey[1] - r.ex[1] * r.ey[0], inv = 1.f / det;
+    for (int i = 0; i < 3; i++) {   // the opposite edge turned, over the determinant
+        const int k = (i + 1) % 3;
+        r.gx[i] = -r.ey[k] * inv;
+        r.gy[i] = r.ex[k] * inv;
+    }
+    r.blx = c.blx;
+    r.bly = c.bly;
+    r.area = 0.5f * det;
+    r.b = c.b;
+    r.q0 = c.q0;
+    return r;
+}
+
+// the same in FP64 (FP64 path): vertex 0, vertices relative to it, edges, gradients of l1 and l2, |T|
 struct Cand64 {
-    double x0, y0, e1x, e1y, e2x, e2y, inv, area;   // vertex 0, edges 0 -> 1 and 0 -> 2, 1 / det, |T|
+    double x0, y0, v[3][2], e[3][2], g[2][2], area, pad;
 };
 struct CandNone {};
 
 template <typename T>
 using CandT = typename std::conditional<sizeof(T) == sizeof(double), Cand64, CandNone>::type;
 
-// Frame of one item: T_b's vertex 0 and edges relative to x, and 1 / det
-template <typename T>
-struct Frame {
-    T rx, ry;   // x - vertex 0
-    T e1x, e1y, e2x, e2y, inv;
+// T_b as one item sees it: start of edge i relative to x and its direction (read from the candidate's
+// shared data by the edge's index, so that nothing is selected between registers), barycentric
+// coordinates of a point relative to x
+struct View32 {
+    const Cand32 &c;
+    float lx, ly;   // x relative to bary_a
+    __device__ __forceinline__ View32(const Cand32 &c_, const OuterPt &o) : c(c_), lx(o.lx), ly(o.ly) {}
+    __device__ __forceinline__ void edge(int i, float &px, float &py, float &ex, float &ey) const
+    {
+        px = c.vx[i] - lx;
+        py = c.vy[i] - ly;
+        ex = c.ex[i];
+        ey = c.ey[i];
+    }
+    __device__ __forceinline__ void coords(float px, float py, float &l1, float &l2) const
+    {
+        const float cx = px - (c.vx[0] - lx), cy = py - (c.vy[0] - ly);
+        l1 = cx * c.gx[1] + cy * c.gy[1];
+        l2 = cx * c.gx[2] + cy * c.gy[2];
+    }
 };
 
-template <typename T>
-__device__ __forceinline__ void frame_l(const Frame<T> &f, T px, T py, T &l1, T &l2)   // p relative to x
-{
-    const T cx = px + f.rx, cy = py + f.ry;
-    l1 = (cx * f.e2y - f.e2x * cy) * f.inv;
-    l2 = (f.e1x * cy - cx * f.e1y) * f.inv;
-}
-
-// start p (relative to x) and direction e of edge i
-template <typename T>
-__device__ __forceinline__ void frame_edge(const Frame<T> &f, int i, T &px, T &py, T &ex, T &ey)
-{
-    px = (i == 0 ? (T)0 : i == 1 ? f.e1x : f.e2x) - f.rx;
-    py = (i == 0 ? (T)0 : i == 1 ? f.e1y : f.e2y) - f.ry;
-    ex = i == 0 ? f.e1x : i == 1 ? f.e2x - f.e1x : -f.e2x;
-    ey = i == 0 ? f.e1y : i == 1 ? f.e2y - f.e1y : -f.e2y;
-}
+struct View64 {
+    const Cand64 &c;
+    double rx, ry;   // x - vertex 0
+    __device__ __forceinline__ View64(const Cand64 &c_, const OuterPt &o) : c(c_), rx(o.x - c_.x0), ry(o.y - c_.y0) {}
+    __device__ __forceinline__ void edge(int i, double &px, double &py, double &ex, double &ey) const
+    {
+        ex = c.e[i][0];
+        ey = c.e[i][1];
+        const double vx = c.v[i][0], vy = c.v[i][1];
+        px = vx - rx;
+        py = vy - ry;
+    }
+    __device__ __forceinline__ void coords(double px, double py, double &l1, double &l2) const
+    {
+        const double cx = px + rx, cy = py + ry;
+        l1 = cx * c.g[0][0] + cy * c.g[0][1];
+        l2 = cx * c.g[1][0] + cy * c.g[1][1];
+    }
+};
 
 template <typename T>
 __device__ __forceinline__ T quot(T a, T b)
 {
-    if constexpr (sizeof(T) == sizeof(float)) return __fdividef(a, b);
-    else return a / b;
+    if constexpr (sizeof(T) == sizeof(float)) {
+        return __fdividef(a, b);
+    } else {
+        // Newton's iteration on 1 / b from the hardware's approximate reciprocal (2^-20), then one
+        // residual step on the quotient: five FP64 instructions, within an ulp for the normal numbers
+        // of a mesh (the correctly rounded division takes about twice as many)
+        double y;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+        y = fma(y, fma(-b, y, 1.0), y);
+        const double t = a * y;
+        return fma(fma(-b, t, a), y, t);
+    }
 }
 
 // the barycentric point at parameter t of edge i
@@ -336,14 +401,36 @@ __device__ __forceinline__ bool ngon_status(const nlg::F2 d[3], const nlg::GeoPa
     return sure;
 }
 
-// the parameter t of edge (p, e) where it leaves (enters) the disc
+// square root of d >= 0
 template <typename T>
-__device__ __forceinline__ T disc_cross(T px, T py, T ex, T ey, T r2, bool exit_)
+__device__ __forceinline__ T root(T d)
 {
-    const T a = ex * ex + ey * ey, b = px * ex + py * ey, c = px * px + py * py - r2;
+    if constexpr (sizeof(T) == sizeof(float)) {
+        return sqrtf(d);
+    } else {
+        // Newton's iteration on 1 / sqrt(d) from the hardware's approximate one (2^-20 or better), then
+        // one residual step on the root: six FP64 instructions
+        double y;
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(fmax(d, 1e-280)));
+        const double h = 0.5 * y;
+        double s = d * y;
+        s = fma(h, fma(-s, s, d), s);
+        return fma(h, fma(-s, s, d), s);
+    }
+}
+
+// the parameter t of edge (p, e) where it leaves (enters) the disc.  FP32: delta^2 in two parts (one
+// rounded delta^2 would shift every region the same way: 4.4e-8 instead of 3e-8 in the matrix)
+template <typename T>
+__device__ __forceinline__ T disc_cross(const nlg::GeoParams &g, T px, T py, T ex, T ey, bool exit_)
+{
+    const T a = ex * ex + ey * ey, b = px * ex + py * ey;
+    T c;
+    if constexpr (sizeof(T) == sizeof(float)) c = (px * px + py * py - g.d2f) - g.d2lo;
+    else c = px * px + py * py - g.d2;
     T ds = b * b - a * c;
     ds = ds > (T)0 ? ds : (T)0;
-    const T s = sqrt(ds);
+    const T s = root(ds);
     // roots of a t^2 + 2 b t + c without cancellation: the far one from w, the other from c / w
     const T w = b > (T)0 ? -(b + s) : s - b;
     const bool num = exit_ == (b <= (T)0);
@@ -370,33 +457,16 @@ __device__ __forceinline__ void corner_of(const NumArgs &A, const float2 *corner
 // certain FP32 predicates, its coordinates in T.  1 done, 0 empty region, -1 the FP64 geometry decides.
 // The vertex count, kind and cap count are those of the FP64 region (the records' content).
 // Every lane of the warp calls it (with data of some item: `live` says whether the lane's counts).
-template <int BALL, typename T>
-__device__ __forceinline__ int cut_item(const NumArgs &A, bool live, const nlg::F2 v[3], const Frame<T> &f0, T inv_area,
-                                        const float2 *corner, Mom<T> &M, int &nv, int &kind, int &ncap)
+// d: T_b's vertices relative to x; v32, f: T_b in FP32 and in T.
+template <int BALL, typename T, typename View>
+__device__ __forceinline__ int cut_item(const NumArgs &A, bool live, const nlg::F2 d[3], const View32 &v32,
+                                        const View &f, T inv_area, const float2 *corner, Mom<T> &M, int &nv,
+                                        int &kind, int &ncap)
 {
     constexpr bool kPoly = BALL == NL_BALL_NGON;
     const nlg::GeoParams &g = A.geo;
     unsigned in, dbl;
-    const bool sure = kPoly ? ngon_status(v, g, corner, in, dbl) : disc_status(v, g, in, dbl);
-    // the new vertex 0: the vertex inside, the first of two inside, the start of the edge cut twice
-    const unsigned who = in ? in : dbl;
-    const int rot = (who & 1u) && !(who & 4u && in) ? 0 : who & 4u ? (who & 2u ? 1 : 2) : who & 2u ? 1 : 0;
-    in = ((in >> rot) | (in << (3 - rot))) & 7u;
-    dbl = ((dbl >> rot) | (dbl << (3 - rot))) & 7u;
-    const nlg::F2 d[3] = {rot == 0 ? v[0] : rot == 1 ? v[1] : v[2], rot == 0 ? v[1] : rot == 1 ? v[2] : v[0],
-                          rot == 0 ? v[2] : rot == 1 ? v[0] : v[1]};
-    Frame<T> f = f0;
-    if (rot != 0) {
-        const T ox = rot == 1 ? f0.e1x : f0.e2x, oy = rot == 1 ? f0.e1y : f0.e2y;   // the new vertex 0
-        const T wx = rot == 1 ? f0.e2x : f0.e1x, wy = rot == 1 ? f0.e2y : f0.e1y;   // the other of 1, 2
-        f.rx = f0.rx - ox;
-        f.ry = f0.ry - oy;
-        const T tx = wx - ox, ty = wy - oy;
-        f.e1x = rot == 1 ? tx : -ox;
-        f.e1y = rot == 1 ? ty : -oy;
-        f.e2x = rot == 1 ? -ox : tx;
-        f.e2y = rot == 1 ? -oy : ty;
-    }
+    const bool sure = kPoly ? ngon_status(d, g, corner, in, dbl) : disc_status(d, g, in, dbl);
     const unsigned nxt = ((in >> 1) | (in << 2)) & 7u;   // bit i: the end of edge i is inside
     unsigned X = (in & ~nxt) | dbl;                      // edges that leave the ball
     const unsigned N = (~in & nxt) | dbl;                // edges that enter it
@@ -417,7 +487,7 @@ __device__ __forceinline__ int cut_item(const NumArgs &A, bool live, const nlg::
     }
     // a polygon region with two crossings and no vertex of T_b inside has its corners still to count
     if (kPoly && X != 0u) empty = false;
-    mom_set(M, in == 7u ? (T)1 : (T)0);
+    mom_set(M, in & 4u ? (T)1 : (T)0);   // edge 1 up to vertex 2
     ncap = 0;
     bool go = live && known && !empty;
     __syncwarp();
@@ -428,23 +498,23 @@ __device__ __forceinline__ int cut_item(const NumArgs &A, bool live, const nlg::
             // the next edge that enters, along the boundary of T_b
             const int i1 = i == 2 ? 0 : i + 1, i2 = i1 == 2 ? 0 : i1 + 1;
             const int j = (N >> i1) & 1u ? i1 : ((N >> i2) & 1u ? i2 : i);
-            T px, py, ex, ey, sx, sy, gx, gy, tx, tn;
-            frame_edge(f, i, px, py, ex, ey);
-            frame_edge(f, j, sx, sy, gx, gy);
+            // start relative to x and direction of the edge left (p, e) and of the edge entered (s, h)
+            T px, py, ex, ey, sx, sy, hx, hy, tx, tn;
+            f.edge(i, px, py, ex, ey);
+            f.edge(j, sx, sy, hx, hy);
             int kx = 0, kn = 0;
             if constexpr (kPoly) {
                 float s0, s1, n0, n1;
-                bool hx, hn;
-                const nlg::F2 p = i == 0 ? d[0] : i == 1 ? d[1] : d[2], pe = i == 0 ? d[1] : i == 1 ? d[2] : d[0];
-                const nlg::F2 e = {pe.x - p.x, pe.y - p.y};
-                const float ae = e.x * e.x + e.y * e.y;
-                kx = ngon_edge(p, e, ae, p.x * e.x + p.y * e.y, p.x * e.y - p.y * e.x, true, g, corner, &hx, &s0, &s1);
-                const nlg::F2 q = j == 0 ? d[0] : j == 1 ? d[1] : d[2], qe = j == 0 ? d[1] : j == 1 ? d[2] : d[0];
-                const nlg::F2 h = {qe.x - q.x, qe.y - q.y};
-                const float ah = h.x * h.x + h.y * h.y;
-                kn = ngon_edge(q, h, ah, q.x * h.x + q.y * h.y, q.x * h.y - q.y * h.x, false, g, corner, &hn, &n0, &n1);
+                bool hitx, hitn;
+                nlg::F2 p, e, q, h;
+                v32.edge(i, p.x, p.y, e.x, e.y);
+                v32.edge(j, q.x, q.y, h.x, h.y);
+                const float ae = e.x * e.x + e.y * e.y, ah = h.x * h.x + h.y * h.y;
+                kx = ngon_edge(p, e, ae, p.x * e.x + p.y * e.y, p.x * e.y - p.y * e.x, true, g, corner, &hitx, &s0, &s1);
+                kn = ngon_edge(q, h, ah, q.x * h.x + q.y * h.y, q.x * h.y - q.y * h.x, false, g, corner, &hitn, &n0, &n1);
                 const float m = g.tau * sqrtf(ae), mh = g.tau * sqrtf(ah);
-                known = hx && hn && s0 < -m && s1 > m && n0 > mh && n1 < -mh;
+                known = hitx && hitn && s0 < -m && s1 > m && n0 > mh && n1 < -mh;
+                // t from the line of the polygon edge
                 T ox, oy, ux, uy;
                 corner_of<T>(A, corner, kx, ox, oy);
                 corner_of<T>(A, corner, kx + 1, ux, uy);
@@ -455,18 +525,27 @@ __device__ __forceinline__ int cut_item(const NumArgs &A, bool live, const nlg::
                 corner_of<T>(A, corner, kn + 1, ux, uy);
                 ux -= ox;
                 uy -= oy;
-                tn = quot(uy * (sx - ox) - ux * (sy - oy), ux * gy - uy * gx);
+                tn = quot(uy * (sx - ox) - ux * (sy - oy), ux * hy - uy * hx);
                 if (kn == kx) {
                     // both on one polygon edge: the boundary runs along it from the exit to the entry, or
                     // (the polygon all but inside T_b) around it
-                    const T run = ((sx + tn * gx) - (px + tx * ex)) * ux + ((sy + tn * gy) - (py + tx * ey)) * uy;
-                    known = known && run > (T)(g.tau * g.poly_side);
+                    const float2 a0 = corner[kx], a1 = corner[kx + 1];
+                    const float wx = a1.x - a0.x, wy = a1.y - a0.y;
+                    float t, r;
+                    if constexpr (sizeof(T) == sizeof(float)) {
+                        t = tx;
+                        r = tn;
+                    } else {   // FP32 decides
+                        t = __fdividef(wy * (p.x - a0.x) - wx * (p.y - a0.y), wx * e.y - wy * e.x);
+                        r = __fdividef(wy * (q.x - a0.x) - wx * (q.y - a0.y), wx * h.y - wy * h.x);
+                    }
+                    const float run = ((q.x + r * h.x) - (p.x + t * e.x)) * wx + ((q.y + r * h.y) - (p.y + t * e.y)) * wy;
+                    known = known && run > g.poly_m;
                 }
                 go = known;
             } else {
-                const T r2 = sizeof(T) == sizeof(float) ? (T)(g.deltaf * g.deltaf) : (T)g.d2;
-                tx = disc_cross<T>(px, py, ex, ey, r2, true);
-                tn = disc_cross<T>(sx, sy, gx, gy, r2, false);
+                tx = disc_cross<T>(g, px, py, ex, ey, true);
+                tn = disc_cross<T>(g, sx, sy, hx, hy, false);
             }
             if (i == 1) edge1_add(M, tx, (T)1);
             if (j == 1) edge1_add(M, tn, (T)-1);
@@ -481,7 +560,7 @@ __device__ __forceinline__ int cut_item(const NumArgs &A, bool live, const nlg::
                     if (k >= g.ngon_n) k -= g.ngon_n;
                     T ox, oy, m1, m2;
                     corner_of<T>(A, corner, k, ox, oy);
-                    frame_l(f, ox, oy, m1, m2);
+                    f.coords(ox, oy, m1, m2);
                     seg_add(M, l1, l2, m1, m2);
                     l1 = m1;
                     l2 = m2;
@@ -489,31 +568,40 @@ __device__ __forceinline__ int cut_item(const NumArgs &A, bool live, const nlg::
             }
             if constexpr (BALL == NL_BALL_APPROXCAPS) {   // along the dyadic arc points
                 if (g.cap_level > 0) {
-                    const T ax = px + tx * ex, ay = py + tx * ey, bx = sx + tn * gx, by = sy + tn * gy;
+                    const T ax = px + tx * ex, ay = py + tx * ey, bx = sx + tn * hx, by = sy + tn * hy;
                     const T dl = sizeof(T) == sizeof(float) ? (T)g.deltaf : (T)g.delta;
                     auto mid = [&](T ux, T uy, T &ox, T &oy) {
                         T s;
-                        if constexpr (sizeof(T) == sizeof(float)) s = dl * rsqrtf(ux * ux + uy * uy);
-                        else s = dl / sqrt(ux * ux + uy * uy);
+                        if constexpr (sizeof(T) == sizeof(float)) {
+                            const float rs = rsqrtf(ux * ux + uy * uy);
+                            s = fmaf(dl, rs, g.deltalo * rs);
+                        } else {
+                            s = quot(dl, root(ux * ux + uy * uy));
+                        }
                         ox = ux * s;
                         oy = uy * s;
                     };
                     auto to = [&](T x, T y) {
                         T m1, m2;
-                        frame_l(f, x, y, m1, m2);
+                        f.coords(x, y, m1, m2);
                         seg_add(M, l1, l2, m1, m2);
                         l1 = m1;
                         l2 = m2;
                     };
+                    // the bisection's direction (a - x) + (b - x) points away from an arc beyond a half circle
+                    // (the ball all but inside T_b): such a polygon turns back, and its fan's areas count
+                    // without sign, as exact_disc_item takes them
+                    known = ax * bx + ay * by > (T)0 || ax * by - ay * bx > (T)1e-3 * dl * dl;
+                    go = known;
                     T mx, my;
                     mid(ax + bx, ay + by, mx, my);
                     if (g.cap_level == 2) {
-                        T hx, hy;
-                        mid(ax + mx, ay + my, hx, hy);
-                        to(hx, hy);
+                        T qx, qy;
+                        mid(ax + mx, ay + my, qx, qy);
+                        to(qx, qy);
                         to(mx, my);
-                        mid(mx + bx, my + by, hx, hy);
-                        to(hx, hy);
+                        mid(mx + bx, my + by, qx, qy);
+                        to(qx, qy);
                     } else {
                         to(mx, my);
                     }
@@ -521,7 +609,7 @@ __device__ __forceinline__ int cut_item(const NumArgs &A, bool live, const nlg::
             }
             seg_add(M, l1, l2, q1, q2);
             if constexpr (BALL == NL_BALL_EXACTCAPS) {
-                const T ax = px + tx * ex, ay = py + tx * ey, bx = sx + tn * gx, by = sy + tn * gy;
+                const T ax = px + tx * ex, ay = py + tx * ey, bx = sx + tn * hx, by = sy + tn * hy;
                 T cx, cy, w;
                 if constexpr (sizeof(T) == sizeof(float)) {
                     nlg::cap_rule_f32(nlg::F2{ax, ay}, nlg::F2{bx, by}, g, &cx, &cy, &w);
@@ -532,14 +620,13 @@ __device__ __forceinline__ int cut_item(const NumArgs &A, bool live, const nlg::
                     cy = cc.y;
                 }
                 T c1, c2;
-                frame_l(f, cx, cy, c1, c2);
+                f.coords(cx, cy, c1, c2);
                 point_add(M, c1, c2, w * inv_area);
                 ncap++;
             }
         }
         __syncwarp();
     }
-    mom_turn(M, rot);
     kind = in == 7u ? nlg::KIND_WHOLE : nlg::KIND_PARTIAL;
     nv = BALL == NL_BALL_EXACTCAPS && n < 3 ? 0 : n;
     return !known ? -1 : empty ? 0 : 1;
@@ -555,11 +642,15 @@ struct ConstShared {
     static constexpr bool kClip = sizeof(T) == sizeof(float) ? (BALL == kBallNgonAny || kSupportBall<BALL>) : kSupportBall<BALL>;
     using Fx = typename std::conditional<sizeof(T) == sizeof(float), int, T>::type;   // FP32 sums: fixed point
     CandT<T> c64[sizeof(T) == sizeof(double) ? 32 : 1];
+    T w[NL_MAXQ][4];           // per outer point: W phi_a,i (i = 0, 1, 2) and W
     OuterPt sq[NL_MAXQ];
-    CandData cand[32];
+    Cand32 cand[32];
     Fx acc[12][32];            // P (rows 0-8) and Q (9-11) of each lane's pair, value-major
     Fx s0q[NL_MAXQ];           // per outer point: sum of |T_b| S0 over the cut regions
-    unsigned dmask[32];        // outer points of each lane's candidate whose item the deferred kernel takes
+    unsigned dmask[32];        // FP32: outer points of each lane's candidate whose item the deferred kernel
+                               // takes; FP64: the lanes that hold moments for this lane's pair
+    typename std::conditional<sizeof(T) == sizeof(double), T, CandNone>::type mom[6][sizeof(T) == sizeof(double) ? 32 : 1];
+    unsigned char momq[sizeof(T) == sizeof(double) ? 32 : 1];   // FP64: moments on their way, their outer points
     float2 corner[65];         // the regular polygon's corners, corner[N] = corner[0]
     unsigned short queue[32 * NL_MAXQ];   // cut items (owner lane << 8 | q)
     unsigned char hit[32];     // the lane's pair has a non-empty cut region
@@ -619,11 +710,12 @@ struct WalkPt {
 
 template <int BALL, typename T>
 __device__ __noinline__ bool exact_disc_item(const NumArgs &A, int b, const nlg::F2 *dl, double xx, double xy,
-                                             Mom<T> &M, int &nv, int &kind, int &ncap)
+                                             Mom<T> &M, int &nv, int &kind, int &ncap, bool *used64)
 {
     const nlg::GeoParams &g = A.geo;
     const D2 x = {xx, xy};
     ncap = 0;
+    *used64 = true;
     if constexpr (BALL == NL_BALL_BARYCENTER || BALL == NL_BALL_OVERLAP) {
         const CandFp64 c = cand_fp64(A, b);
         mom_set(M, (T)1);
@@ -722,16 +814,23 @@ __device__ __noinline__ bool exact_disc_item(const NumArgs &A, int b, const nlg:
                     ents |= en << (2 * k);
                 }
         }
-        const T r2 = f32 ? (T)(g.deltaf * g.deltaf) : (T)g.d2;
         const T e1x = px[1] - px[0], e1y = py[1] - py[0], e2x = px[2] - px[0], e2y = py[2] - py[0];
         const T inv = (T)1 / (e1x * e2y - e2x * e1y);
         mom_set(M, (T)0);
         WalkPt<T> first = {0, 0, 0, 0, 0}, prev = first;
         int n = 0, narc = 0;
-        // the piece of boundary from a to b; moments about the walk's first point
+        // the piece of boundary from a to c: triangles of the region's fan from its first point, their
+        // areas from positions, their moments from the corners' coordinates (nothing cancels)
         auto link = [&](const WalkPt<T> &a, const WalkPt<T> &c) {
-            T u1 = a.l1 - first.l1, u2 = a.l2 - first.l2;
-            const T w1 = c.l1 - first.l1, w2 = c.l2 - first.l2;
+            T u1 = a.l1, u2 = a.l2, ux = a.x, uy = a.y;
+            auto to = [&](T v1, T v2, T vx, T vy) {
+                const T cr = (ux - first.x) * (vy - first.y) - (vx - first.x) * (uy - first.y);
+                tri_add(M, cr * inv, first.l1, first.l2, u1, u2, v1, v2);
+                u1 = v1;
+                u2 = v2;
+                ux = vx;
+                uy = vy;
+            };
             if (BALL != NL_BALL_NOCAPS && a.tag == 2 && c.tag == 1) {
                 narc++;
                 if constexpr (BALL == NL_BALL_APPROXCAPS) {
@@ -752,11 +851,7 @@ __device__ __noinline__ bool exact_disc_item(const NumArgs &A, int b, const nlg:
                             else { lo = md; ax = mx; ay = my; }
                         }
                         const T cx = mx - px[0], cy = my - py[0];
-                        const T v1 = (cx * e2y - e2x * cy) * inv - first.l1;
-                        const T v2 = (e1x * cy - cx * e1y) * inv - first.l2;
-                        seg_add(M, u1, u2, v1, v2);
-                        u1 = v1;
-                        u2 = v2;
+                        to((cx * e2y - e2x * cy) * inv, (e1x * cy - cx * e1y) * inv, mx, my);
                     }
                 } else if (ncap < 3) {   // exactcaps: centroid and area
                     T cx, cy, w;
@@ -771,12 +866,11 @@ __device__ __noinline__ bool exact_disc_item(const NumArgs &A, int b, const nlg:
                     cx -= px[0];
                     cy -= py[0];
                     // w / |T_b| = 2 w / det
-                    point_add(M, (cx * e2y - e2x * cy) * inv - first.l1, (e1x * cy - cx * e1y) * inv - first.l2,
-                              (T)2 * w * inv);
+                    point_add(M, (cx * e2y - e2x * cy) * inv, (e1x * cy - cx * e1y) * inv, (T)2 * w * inv);
                     ncap++;
                 }
             }
-            seg_add(M, u1, u2, w1, w2);
+            to(c.l1, c.l2, c.x, c.y);
         };
         auto emit = [&](T l1, T l2, T qx, T qy, int tag) {
             const WalkPt<T> q = {l1, l2, qx, qy, tag};
@@ -796,7 +890,7 @@ __device__ __noinline__ bool exact_disc_item(const NumArgs &A, int b, const nlg:
             for (int k = 0; k < 2; k++)
                 if (k < nr[i]) {
                     const bool en = ((ents >> (2 * i + k)) & 1u) != 0;
-                    const T tk = calc ? disc_cross<T>(px[i], py[i], ex, ey, r2, !en) : t[i][k];
+                    const T tk = calc ? disc_cross<T>(g, px[i], py[i], ex, ey, !en) : t[i][k];
                     T l1, l2;
                     edge_l(i, tk, l1, l2);
                     emit(l1, l2, px[i] + tk * ex, py[i] + tk * ey, en ? 1 : 2);
@@ -808,18 +902,18 @@ __device__ __noinline__ bool exact_disc_item(const NumArgs &A, int b, const nlg:
         nv = n >= 2 && m >= 3 ? m : 0;
         kind = in == 7u && n == 3 ? nlg::KIND_WHOLE : nlg::KIND_PARTIAL;
         if (kind == nlg::KIND_WHOLE) mom_set(M, (T)1);
-        else mom_shift(M, first.l1, first.l2);
+        *used64 = (open | eopen) != 0u;
         return nv >= 3 || ncap > 0;
     }
 }
 
-// region and moments of one item by the FP64 geometry
+// region and moments of one item by the FP64 geometry (*used64 = false: FP32 was certain after all)
 template <int BALL, typename T>
 __device__ __forceinline__ bool exact_item(const NumArgs &A, int b, const nlg::F2 *dl, double xx, double xy,
-                                           Mom<T> &M, int &nv, int &kind, int &ncap)
+                                           Mom<T> &M, int &nv, int &kind, int &ncap, bool *used64)
 {
     if constexpr (kGeoBall<BALL> == NL_BALL_NGON) return exact_const_item<BALL, T>(A, b, dl, xx, xy, M, nv, kind, ncap);
-    else return exact_disc_item<BALL, T>(A, b, dl, xx, xy, M, nv, kind, ncap);
+    else return exact_disc_item<BALL, T>(A, b, dl, xx, xy, M, nv, kind, ncap, used64);
 }
 
 // are the items that FP32 leaves open queued for k_deferred?  The N-gon's on the FP32 path: its FP64
@@ -835,31 +929,55 @@ __device__ __forceinline__ int region_points(const NumArgs &A, int kind, int nv,
     return (nv >= 3 ? (nv - 2) * A.inner.n : 0) + ncap;
 }
 
-// an item's moments M at outer point q = o, added onto owner own's sums (rows 0-11), its s0 onto
-// the outer point's.  FP32 sums: rounded to the grids fxs and gs (integer adds, any order).
-template <typename T, typename Fx>
-__device__ __forceinline__ void item_add(const OuterPt &o, const Mom<T> &M, Fx (*acc)[32], Fx *s0q, int own, int q,
-                                         float fxs, T area, float gs)
+// An item's moments M at an outer point of weights w, added onto owner own's sums (rows 0-11), its s0 onto
+// the outer point's.  FP32 sums: rounded to the grids fxs and gs (native integer adds, any order).
+__device__ __forceinline__ void item_add(const float *w, const Mom<float> &M, int (*acc)[32], int *s0q, int own,
+                                         float fxs, float area, float gs)
 {
-    constexpr bool f32 = sizeof(T) == sizeof(float);
-    const T W = f32 ? (T)o.Wf * (T)fxs : (T)o.W;   // fxs: a power of two
-    const T w0 = W * (f32 ? (T)o.l0f : (T)o.l0), w1 = W * (f32 ? (T)o.l1f : (T)o.l1);
-    const T w2 = W * (f32 ? (T)o.l2f : (T)o.l2);
-    auto put = [&](Fx *p, T v) {
-        if constexpr (f32) atomicAdd(p, __float2int_rn(v));
-        else atomicAdd(p, v);
-    };
-    put(&acc[0][own], w0 * M.s0); put(&acc[1][own], w0 * M.s1); put(&acc[2][own], w0 * M.s2);
-    put(&acc[3][own], w1 * M.s0); put(&acc[4][own], w1 * M.s1); put(&acc[5][own], w1 * M.s2);
-    put(&acc[6][own], w2 * M.s0); put(&acc[7][own], w2 * M.s1); put(&acc[8][own], w2 * M.s2);
-    put(&acc[9][own], W * M.s11); put(&acc[10][own], W * M.s22); put(&acc[11][own], W * M.s12);
-    put(&s0q[q], f32 ? area * (T)gs * M.s0 : area * M.s0);
+    const float w0 = w[0] * fxs, w1 = w[1] * fxs, w2 = w[2] * fxs, W = w[3] * fxs;   // fxs: a power of two
+    auto put = [&](int k, float v) { atomicAdd(&acc[k][own], __float2int_rn(v)); };
+    put(0, w0 * M.s0); put(1, w0 * M.s1); put(2, w0 * M.s2);
+    put(3, w1 * M.s0); put(4, w1 * M.s1); put(5, w1 * M.s2);
+    put(6, w2 * M.s0); put(7, w2 * M.s1); put(8, w2 * M.s2);
+    put(9, W * M.s11); put(10, W * M.s22); put(11, W * M.s12);
+    atomicAdd(s0q, __float2int_rn(area * gs * M.s0));
+}
+
+// FP64 sums: an FP64 shared atomic is a loop of compare-and-swaps with an FP64 add in each, and the FP64
+// pipe is what bounds the kernel.  So the lanes leave their moments in shared memory, and each owner
+// takes the ones of its pair into its own column: one fused multiply-add a value.  Every lane calls it.
+template <typename Sh>
+__device__ __forceinline__ void items_gather(Sh &sh, bool has, int own, int q, const Mom<double> &M, int lane)
+{
+    if (has) {
+        sh.mom[0][lane] = M.s0; sh.mom[1][lane] = M.s1; sh.mom[2][lane] = M.s2;
+        sh.mom[3][lane] = M.s11; sh.mom[4][lane] = M.s22; sh.mom[5][lane] = M.s12;
+        sh.momq[lane] = (unsigned char)q;
+        atomicOr(&sh.dmask[own], 1u << lane);
+        atomicAdd(&sh.s0q[q], sh.c64[own].area * M.s0);
+    }
+    __syncwarp();
+    unsigned from = sh.dmask[lane];
+    sh.dmask[lane] = 0;
+    while (from) {
+        const int i = __ffs(from) - 1;
+        from &= from - 1;
+        const double *w = sh.w[sh.momq[i]];
+        const double s0 = sh.mom[0][i], s1 = sh.mom[1][i], s2 = sh.mom[2][i];
+        for (int k = 0; k < 3; k++) {
+            sh.acc[3 * k][lane] += w[k] * s0;
+            sh.acc[3 * k + 1][lane] += w[k] * s1;
+            sh.acc[3 * k + 2][lane] += w[k] * s2;
+        }
+        for (int k = 0; k < 3; k++) sh.acc[9 + k][lane] += w[3] * sh.mom[3 + k][i];
+    }
+    __syncwarp();
 }
 
 // Interior candidates of T_a: T_b whole for every outer point (certified when the lists are built,
 // a relation symmetric in a and b).  The outer rules integrate quadratics exactly too, so the
-// pair's blocks are closed forms of the two areas: M_ab = c |T_a| |T_b| / 9 in all nine entries
-// (formed by the scatter: nothing is stored), M_aa = c |T_a| |T_b| (1 + delta_ij) / 12, and the
+// pair's blocks are closed forms of the two areas: M_ab = |T_a| |T_b| / 9 in all nine entries
+// (formed by the scatter: nothing is stored), M_aa = |T_a| |T_b| (1 + delta_ij) / 12, and the
 // M_bb that T_a receives as the inner triangle of its symmetric pairs is the same sum again.
 template <int STS>
 __device__ __forceinline__ void interior_const(const NumArgs &A, int a, int lane, LaneAcc &acc)
@@ -885,7 +1003,7 @@ __device__ __forceinline__ void interior_const(const NumArgs &A, int a, int lane
             for (int q = 0; q < (A.outer_support ? 1 : nq); q++)
                 acc.hsum += nlg::record_hash(a, b, q, nlg::KIND_WHOLE, 3, 0);
     }
-    const double w = sum * A.area[a] * A.kc * (1.0 / 12.0) * 2.0;
+    const double w = sum * A.area[a] * (1.0 / 12.0) * 2.0;
     for (int i = 0; i < 6; i++) acc.maa[i] += i < 3 ? 2.0 * w : w;
 }
 
@@ -915,14 +1033,15 @@ __device__ __forceinline__ void const_defer_flush(const NumArgs &A, int a, int64
             A.defer[slot] = DeferItem{base + lane, a, (A.prob << 8) | q};
             continue;
         }
-        const CandData &cd = sh.cand[lane];
+        const Cand32 &cd = sh.cand[lane];
         const OuterPt &o = sh.sq[q];
         nlg::F2 dl[3];
-        for (int i = 0; i < 3; i++) { dl[i].x = cd.vlx[i] - o.lx; dl[i].y = cd.vly[i] - o.ly; }
+        for (int i = 0; i < 3; i++) { dl[i].x = cd.vx[i] - o.lx; dl[i].y = cd.vy[i] - o.ly; }
         Mom<float> M;
         int nv, kind, ncap;
-        if (!exact_item<BALL, float>(A, cd.b, dl, o.x, o.y, M, nv, kind, ncap)) continue;
-        item_add<float>(o, M, sh.acc, sh.s0q, lane, q, fxs, cd.akcf, A.s0q_grid);
+        bool used64;
+        if (!exact_item<BALL, float>(A, cd.b, dl, o.x, o.y, M, nv, kind, ncap, &used64)) continue;
+        item_add(sh.w[q], M, sh.acc, &sh.s0q[q], lane, fxs, cd.area, A.s0q_grid);
         sh.hit[lane] = 1;
         acc.cnt++;
         acc.qp += (uint32_t)region_points(A, kind, nv, ncap);
@@ -952,6 +1071,14 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
         inv_s = 1.f / fxs;
     }
     for (int q = lane; q < NL_MAXQ; q += 32) sh.s0q[q] = (Fx)0;
+    for (int q = lane; q < nq_all; q += 32) {
+        const OuterPt &o = sh.sq[q];
+        const T W = f32 ? (T)o.Wf : (T)o.W;
+        sh.w[q][0] = W * (f32 ? (T)o.l0f : (T)o.l0);
+        sh.w[q][1] = W * (f32 ? (T)o.l1f : (T)o.l1);
+        sh.w[q][2] = W * (f32 ? (T)o.l2f : (T)o.l2);
+        sh.w[q][3] = W;
+    }
     // sum of |T_b| over the whole items of outer point q = lane: exact integers (FP32 path: on the
     // grid s0q_grid; FP64 path: 50-bit fixed point in two limbs, area_grid = 2^50 / a power of two
     // above the largest area)
@@ -978,7 +1105,7 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
 #endif
             load_cand(A, b, ba, bah, c, q1);
             q0 = c.q0;
-            sh.cand[lane] = c;
+            sh.cand[lane] = cand32_of(c);
             if constexpr (f32) {
                 a_fx = __float2int_rn(c.akcf * A.s0q_grid);
             } else {
@@ -986,12 +1113,22 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
                 Cand64 d;
                 d.x0 = A.tx[b];
                 d.y0 = A.ty[b];
-                d.e1x = A.tx[K + b] - d.x0;
-                d.e1y = A.ty[K + b] - d.y0;
-                d.e2x = A.tx[2 * K + b] - d.x0;
-                d.e2y = A.ty[2 * K + b] - d.y0;
+                const double x1 = A.tx[K + b], y1 = A.ty[K + b], x2 = A.tx[2 * K + b], y2 = A.ty[2 * K + b];
                 d.area = A.area[b];
-                d.inv = 0.5 / d.area;
+                const double inv = quot(0.5, d.area);
+                d.v[0][0] = d.v[0][1] = 0.0;
+                d.v[1][0] = d.e[0][0] = x1 - d.x0;
+                d.v[1][1] = d.e[0][1] = y1 - d.y0;
+                d.v[2][0] = x2 - d.x0;
+                d.v[2][1] = y2 - d.y0;
+                d.e[1][0] = x2 - x1;
+                d.e[1][1] = y2 - y1;
+                d.e[2][0] = -d.v[2][0];
+                d.e[2][1] = -d.v[2][1];
+                d.g[0][0] = inv * d.v[2][1];
+                d.g[0][1] = -inv * d.v[2][0];
+                d.g[1][0] = -inv * d.v[1][1];
+                d.g[1][1] = inv * d.v[1][0];
                 sh.c64[lane] = d;
                 const unsigned long long fx = __double2ull_rn(d.area * A.area_grid);
                 a_hi = (unsigned)(fx >> 25);
@@ -1002,6 +1139,7 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
         sh.dmask[lane] = 0;
         sh.hit[lane] = 0;
         int nqueue = 0, nwhole = 0;
+        unsigned cutq = 0;   // outer points whose region of this lane's candidate is cut
         T u0 = 0, u1 = 0, u2 = 0;   // sum of W_q phi_a,i over the outer points that see all of T_b
         __syncwarp();
         for (int q = 0; q < nq_all; q++) {
@@ -1014,10 +1152,9 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
             }
             const bool whole = cls == nlg::CLS_WHOLE;
             if (whole) {
-                const T W = f32 ? (T)o.Wf : (T)o.W;
-                u0 += W * (f32 ? (T)o.l0f : (T)o.l0);
-                u1 += W * (f32 ? (T)o.l1f : (T)o.l1);
-                u2 += W * (f32 ? (T)o.l2f : (T)o.l2);
+                u0 += sh.w[q][0];
+                u1 += sh.w[q][1];
+                u2 += sh.w[q][2];
                 nwhole++;
                 if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, c.b, q - q0, nlg::KIND_WHOLE, 3, 0);
             }
@@ -1032,10 +1169,16 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
                     ws_lo += tl;
                 }
             }
-            const unsigned me = __ballot_sync(0xffffffffu, cls == nlg::CLS_EXACT);
-            if (cls == nlg::CLS_EXACT)
-                sh.queue[nqueue + __popc(me & ((1u << lane) - 1u))] = (unsigned short)((lane << 8) | q);
-            nqueue += __popc(me);
+            if (cls == nlg::CLS_EXACT) cutq |= 1u << q;
+        }
+        // the cut items, every lane's first, then every lane's second, ...: neighbours in the queue have
+        // different owners and outer points, so their adds rarely meet on one address
+        for (unsigned m = __ballot_sync(0xffffffffu, cutq != 0u); m; m = __ballot_sync(0xffffffffu, cutq != 0u)) {
+            if (cutq) {
+                sh.queue[nqueue + __popc(m & ((1u << lane) - 1u))] = (unsigned short)((lane << 8) | (__ffs(cutq) - 1));
+                cutq &= cutq - 1;
+            }
+            nqueue += __popc(m);
         }
         acc.cnt += (uint32_t)nwhole;
         acc.qp += (uint32_t)(nwhole * A.inner.n);
@@ -1047,13 +1190,13 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
             const bool live = r0 + lane < nqueue;
             const unsigned it = sh.queue[live ? r0 + lane : r0];   // the other lanes follow along
             const int own = it >> 8, q = it & 0xff;
-            const CandData &cd = sh.cand[own];
+            const Cand32 &cd = sh.cand[own];
             const OuterPt &o = sh.sq[q];
             nlg::F2 d[3];
-            for (int k = 0; k < 3; k++) { d[k].x = cd.vlx[k] - o.lx; d[k].y = cd.vly[k] - o.ly; }
+            for (int k = 0; k < 3; k++) { d[k].x = cd.vx[k] - o.lx; d[k].y = cd.vy[k] - o.ly; }
             Mom<T> M;
             int nv = 0, kind = nlg::KIND_PARTIAL, ncap = 0, r = -1;
-            T area = (T)cd.akcf;
+            T area = (T)cd.area;
             if constexpr (BALL == NL_BALL_BARYCENTER || BALL == NL_BALL_OVERLAP) {
                 // FP64 predicate on the whole triangle
             } else if constexpr (BALL == kBallNgonAny) {
@@ -1063,37 +1206,42 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
                     const int n = nlg::clip_ngon_f32_sh<true>(d, A.geo.err0, A.geo, sh.clip, lane, &which, &cut);
                     r = n < 0 ? -1 : n < 3 ? 0 : 1;
                     if (r == 1) {
-                        const Frame<float> f = {-d[0].x, -d[0].y, cd.e1x, cd.e1y, cd.e2x, cd.e2y, cd.binv};
                         // about the polygon's first vertex
                         const float x0 = sh.clip.x[which][0][lane], y0 = sh.clip.y[which][0][lane];
-                        const Frame<float> w = {-x0, -y0, cd.e1x, cd.e1y, cd.e2x, cd.e2y, cd.binv};
                         mom_set(M, 0.f);
                         float p1 = 0.f, p2 = 0.f;
                         for (int k = 1; k < n; k++) {
-                            float q1, q2;
-                            frame_l(w, sh.clip.x[which][k][lane], sh.clip.y[which][k][lane], q1, q2);
+                            const float dx = sh.clip.x[which][k][lane] - x0, dy = sh.clip.y[which][k][lane] - y0;
+                            const float q1 = dx * cd.gx[1] + dy * cd.gy[1], q2 = dx * cd.gx[2] + dy * cd.gy[2];
                             seg_add(M, p1, p2, q1, q2);
                             p1 = q1;
                             p2 = q2;
                         }
-                        frame_l(f, x0, y0, p1, p2);
+                        View32(cd, o).coords(x0, y0, p1, p2);
                         mom_shift(M, p1, p2);
                         nv = n;
                         kind = cut ? nlg::KIND_PARTIAL : nlg::KIND_WHOLE;
                     }
                 }
             } else if constexpr (f32) {
-                const Frame<float> f = {-d[0].x, -d[0].y, cd.e1x, cd.e1y, cd.e2x, cd.e2y, cd.binv};
-                r = cut_item<BALL, float>(A, live, d, f, BALL == NL_BALL_EXACTCAPS ? 1.f / area : 0.f, sh.corner, M,
-                                          nv, kind, ncap);
+                const View32 v(cd, o);
+                if (!A.geo.turn)
+                    r = cut_item<BALL, float>(A, live, d, v, v, BALL == NL_BALL_EXACTCAPS ? 1.f / area : 0.f, sh.corner,
+                                              M, nv, kind, ncap);
             } else {
                 const Cand64 &w = sh.c64[own];
-                const Frame<double> f = {o.x - w.x0, o.y - w.y0, w.e1x, w.e1y, w.e2x, w.e2y, w.inv};
                 area = w.area;
-                r = cut_item<BALL, double>(A, live, d, f, 2.0 * w.inv, sh.corner, M, nv, kind, ncap);
+                if (!A.geo.turn)
+                    r = cut_item<BALL, double>(A, live, d, View32(cd, o), View64(w, o),
+                                               BALL == NL_BALL_EXACTCAPS ? 1.0 / area : 0.0, sh.corner, M, nv, kind,
+                                               ncap);
+            }
+            if constexpr (f32) {
+                if (live && r > 0) item_add(sh.w[q], M, sh.acc, &sh.s0q[q], own, fxs, area, A.s0q_grid);
+            } else {
+                items_gather(sh, live && r > 0, own, q, M, lane);
             }
             if (live && r > 0) {
-                item_add<T>(o, M, sh.acc, sh.s0q, own, q, fxs, area, A.s0q_grid);
                 sh.hit[own] = 1;
                 acc.cnt++;
                 acc.qp += (uint32_t)region_points(A, kind, nv, ncap);
@@ -1114,32 +1262,38 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
             const_defer_flush<BALL, STS>(A, a, base, sh, lane, fxs, acc);
             __syncwarp();
         } else {
-            nopen += nslow;
-            for (int i = lane; i < nslow; i += 32) {
-                const unsigned it = sh.queue[i];
+            for (int i0 = 0; i0 < nslow; i0 += 32) {
+                const bool live = i0 + lane < nslow;
+                const unsigned it = sh.queue[live ? i0 + lane : i0];
                 const int own = it >> 8, q = it & 0xff;
-                const CandData &cd = sh.cand[own];
+                const Cand32 &cd = sh.cand[own];
                 const OuterPt &o = sh.sq[q];
-                nlg::F2 d[3];
-                for (int k = 0; k < 3; k++) { d[k].x = cd.vlx[k] - o.lx; d[k].y = cd.vly[k] - o.ly; }
                 Mom<T> M;
-                int nv, kind, ncap;
-                if (!exact_item<BALL, T>(A, cd.b, d, o.x, o.y, M, nv, kind, ncap)) continue;
-                T area;
-                if constexpr (f32) area = cd.akcf;
-                else area = sh.c64[own].area;
-                item_add<T>(o, M, sh.acc, sh.s0q, own, q, fxs, area, A.s0q_grid);
-                sh.hit[own] = 1;
-                acc.cnt++;
-                acc.qp += (uint32_t)region_points(A, kind, nv, ncap);
-                if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, cd.b, q - cd.q0, kind, nv, ncap);
+                int nv = 0, kind = 0, ncap = 0;
+                bool has = false, used64 = kGeoBall<BALL> == NL_BALL_NGON;
+                if (live) {
+                    nlg::F2 d[3];
+                    for (int k = 0; k < 3; k++) { d[k].x = cd.vx[k] - o.lx; d[k].y = cd.vy[k] - o.ly; }
+                    has = exact_item<BALL, T>(A, cd.b, d, o.x, o.y, M, nv, kind, ncap, &used64);
+                    nopen += used64;
+                }
+                if constexpr (f32) {
+                    if (has) item_add(sh.w[q], M, sh.acc, &sh.s0q[q], own, fxs, cd.area, A.s0q_grid);
+                } else {
+                    items_gather(sh, has, own, q, M, lane);
+                }
+                if (has) {
+                    sh.hit[own] = 1;
+                    acc.cnt++;
+                    acc.qp += (uint32_t)region_points(A, kind, nv, ncap);
+                    if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, cd.b, q - cd.q0, kind, nv, ncap);
+                }
             }
             __syncwarp();
         }
         if (valid) {   // the owner's pair
             const int b = c.b;
             T P[9], Q[3], mab[9], mbb[6];
-            const T us[3] = {u0, u1, u2}, uw = u0 + u1 + u2;
             bool big = false;
             for (int k = 0; k < 12; k++) {
                 T v;
@@ -1150,14 +1304,21 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
                 } else {
                     v = sh.acc[k][lane];
                 }
-                if (k < 9) P[k] = v + us[k / 3];
-                else Q[k - 9] = v + uw;
+                if (k < 9) P[k] = v;
+                else Q[k - 9] = v;
             }
             if (big) atomicOr(A.err, 256);
-            T akc;
-            if constexpr (f32) akc = c.akcf * A.kcf;
-            else akc = sh.c64[lane].area * A.kc;
-            pair_block<T>(akc, P, Q, mab, mbb);
+            T area;
+            if constexpr (f32) area = c.akcf;
+            else area = sh.c64[lane].area;
+            pair_block<T>(f32 ? (T)sh.cand[lane].area : area, P, Q, mab, mbb);
+            // the outer points that see all of T_b: their moments are 1, the blocks |T_b| u_i / 3 and
+            // |T_b| sum_i u_i (1 + delta_ij) / 12 (kept apart from the cut ones, whose block is formed by
+            // differences: in FP32 those would round the larger, whole part)
+            const T k3 = area / (T)3, us[3] = {u0 * k3, u1 * k3, u2 * k3};
+            for (int i = 0; i < 9; i++) mab[i] += us[i / 3];
+            const T kw = (us[0] + us[1] + us[2]) * (T)0.25;
+            for (int i = 0; i < 6; i++) mbb[i] += i < 3 ? (T)2 * kw : kw;
             const bool any = nwhole > 0 || sh.hit[lane] != 0;
             A.flag[e] = any ? 1 : 0;
             T *blk = (T *)A.blk;
@@ -1167,10 +1328,9 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
         }
         __syncwarp();
     }
-    if (!kConstQueue<BALL, T> && nopen > 0 && lane == 0 && A.defer_n) atomicAdd(A.defer_n, nopen);
-    // M_aa = c sum_q W_q phi_a(x_q) phi_a(x_q)^T sum_b int_{R(x_q, T_b)} 1, in FP64, one outer point a lane
+    if (!kConstQueue<BALL, T> && nopen > 0 && A.defer_n) atomicAdd(A.defer_n, nopen);
+    // M_aa / c = sum_q W_q phi_a(x_q) phi_a(x_q)^T sum_b int_{R(x_q, T_b)} 1, in FP64, one outer point a lane
     if (lane < nq_all) {
-        const OuterPt &o = sh.sq[lane];
         double t;
         if constexpr (f32) {
             const long long s = (long long)sh.s0q[lane] + ws_f;
@@ -1179,9 +1339,13 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
         } else {
             t = sh.s0q[lane] + (double)((ws_hi << 25) + ws_lo) / A.area_grid;
         }
-        const double ws = o.W * t * A.kc;
-        acc.maa[0] += ws * o.l0 * o.l0; acc.maa[1] += ws * o.l1 * o.l1; acc.maa[2] += ws * o.l2 * o.l2;
-        acc.maa[3] += ws * o.l0 * o.l1; acc.maa[4] += ws * o.l0 * o.l2; acc.maa[5] += ws * o.l1 * o.l2;
+        // W phi_a,i and W as the pairs' sums have them (FP32 path: rounded to FP32): M_aa, M_ab and M_bb are
+        // then the blocks of one square (sum_i phi_a,i u_i - u(y))^2, and what rounding the weights costs
+        // is not enlarged by the difference that D takes of them
+        const double w0 = (double)sh.w[lane][0], w1 = (double)sh.w[lane][1], w2 = (double)sh.w[lane][2];
+        const double s = t / (double)sh.w[lane][3];
+        acc.maa[0] += s * w0 * w0; acc.maa[1] += s * w1 * w1; acc.maa[2] += s * w2 * w2;
+        acc.maa[3] += s * w0 * w1; acc.maa[4] += s * w0 * w2; acc.maa[5] += s * w1 * w2;
     }
 }
 
@@ -1209,10 +1373,11 @@ __device__ __forceinline__ void const_outer(const NumArgs &A, int a, ConstShared
 }
 
 // Measured (32-gon, delta = 0.1, 96 x 96 cells jittered, 16-point outer rule, 30 M cut items, one
-// GB300): FP32 sums 1.6 ms against 4.2 ms for the point-by-point kernel it replaced (certified
+// GB300): FP32 sums 1.50 ms against 4.2 ms for the point-by-point kernel it replaced (certified
 // Sutherland-Hodgman clip into shared memory, 7-point rule on every fan triangle) plus 0.5 ms of its
-// interior kernel; it issues in 71 % of the cycles with 25 of 32 lanes active.  FP64 sums 13.4 ms
-// against 99.3 + 17.2 ms, with the FP64 pipe (1/64 of the FP32 rate) busy 86 % of the time.
+// interior kernel; it issues in 71 % of the cycles with 24 of 32 lanes active.  FP64 sums 10.2 ms
+// against 99.3 + 17.2 ms, with the FP64 pipe (1/64 of the FP32 rate) busy 87 % of the time: every FP64
+// instruction saved counts there, whatever it costs elsewhere.
 template <typename T>
 constexpr int kConstBlocksPerSm = sizeof(T) == sizeof(float) ? 5 : 4;
 
@@ -1250,7 +1415,8 @@ __device__ __forceinline__ void deferred_const(const NumArgs &A, const DeferItem
     for (int i = 0; i < 3; i++) { dl[i].x = c.vlx[i] - o.lx; dl[i].y = c.vly[i] - o.ly; }
     Mom<float> M;
     int kind, nv, ncap;
-    if (!exact_item<BALL, float>(A, b, dl, o.x, o.y, M, nv, kind, ncap)) {
+    bool used64;
+    if (!exact_item<BALL, float>(A, b, dl, o.x, o.y, M, nv, kind, ncap, &used64)) {
         for (int k = 0; k < kDeferVals; k++) dv[(int64_t)k * cap + slot] = 0.f;
         return;
     }
@@ -1263,10 +1429,10 @@ __device__ __forceinline__ void deferred_const(const NumArgs &A, const DeferItem
         P[3 * i + 2] = w * M.s2;
     }
     const float Q[3] = {o.Wf * M.s11, o.Wf * M.s22, o.Wf * M.s12};
-    pair_block<float>(c.akcf * A.kcf, P, Q, mab, mbb);
+    pair_block<float>(c.akcf, P, Q, mab, mbb);
     for (int k = 0; k < kDeferVals; k++) dv[(int64_t)k * cap + slot] = mab[k];
     for (int k = 0; k < 6; k++) atomicAdd(&A.mbb[(int64_t)k * K + b], (double)mbb[k]);
-    const double ws = o.W * A.kc * A.area[b] * (double)M.s0;
+    const double ws = o.W * A.area[b] * (double)M.s0;
     const double m[6] = {ws * o.l0 * o.l0, ws * o.l1 * o.l1, ws * o.l2 * o.l2,
                          ws * o.l0 * o.l1, ws * o.l0 * o.l2, ws * o.l1 * o.l2};
     for (int k = 0; k < 6; k++) atomicAdd(&A.maa[(int64_t)k * K + a], m[k]);

@@ -12,6 +12,7 @@
 // and of the summed M_bb of its pairs (diagonals halved).  The transposed blocks come
 // from the final W + W^T pass through the transposed-slot map.
 #include <cuda_runtime.h>
+#include <math.h>
 
 #include <stdlib.h>
 
@@ -127,14 +128,15 @@ __global__ void k_node_fill(int K, const int32_t *tri, const int64_t *start, int
 
 // FP32 scatter: exponent of a bound on what node j's column of a row of T_a receives per unit
 // of sum_q |W_q| (that is, per |T_a| sum_q |w_q|).  Each triangle T_b at j adds at most
-// s0max(T_b), a bound on int_{S cap T_b} gamma(x, y) dy over all points x and sets S: kc |T_b|
-// for a constant kernel, c 2 sqrt(pi |T_b|) for c / |x - y| (1/r integrated over the disc of
+// s0max(T_b), a bound on int_{S cap T_b} gamma(x, y) dy over all points x and sets S: |T_b| for
+// the constant kernel (its blocks are without c), c 2 sqrt(pi |T_b|) for c / |x - y| (1/r integrated over the disc of
 // area |T_b| centred at x, the largest such integral), each with the per-point margin of the
 // numeric phase (1.25, 2.5 for the singular quadrature).  The bound taken, (triangles at j) x
 // max s0max, is order-free and so the same in every run.  fxe (zeroed) receives 128 + the
 // largest floor(log2) of it in FP32 over the nodes (an integer maximum: the same in every run).
+// cap: a bound on it from the ball (the regions around j lie in one disc), or infinity.
 __global__ void k_node_exp(int J, const int64_t *nptr, const int32_t *ntri, const double *area, int inv, double c,
-                           int *fxe)
+                           double cap, int *fxe)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= J) return;
@@ -143,7 +145,7 @@ __global__ void k_node_exp(int J, const int64_t *nptr, const int32_t *ntri, cons
         const double A = area[ntri[s]];
         m = fmax(m, inv ? 2.5 * c * 2.0 * sqrt(3.14159265358979323846 * A) : 1.25 * c * A);
     }
-    const double nb = (double)(nptr[j + 1] - nptr[j]) * m;
+    const double nb = fmin((double)(nptr[j + 1] - nptr[j]) * m, cap);
     int e = nb < 1e38 ? ((__float_as_int((float)nb) >> 23) & 255) - 127 : 126;
     e = e < -126 ? -126 : (e > 126 ? 126 : e);
     atomicMax(fxe, e + 128);
@@ -451,7 +453,8 @@ template <typename T, typename Acc>
 __device__ __forceinline__ void scatter_pair(uint8_t f, int b, const T *v, int K, int J, const int32_t *tri,
                                              const int64_t *row_ptr, const int32_t *col, double *W, int *err,
                                              bool cached, int H, int hbits, const int *ar, const int *len, int cap,
-                                             float sc, Acc *sacc, const int32_t *skey, const uint32_t *spk)
+                                             float sc, double kc, Acc *sacc, const int32_t *skey,
+                                             const uint32_t *spk)
 {
     if (!f) return;
 #ifdef NL_CHECKS
@@ -492,7 +495,7 @@ __device__ __forceinline__ void scatter_pair(uint8_t f, int b, const T *v, int K
                     continue;
                 }
 #endif
-                if (sl >= 0) atomicAdd(&W[sl], -(double)v[3 * i + k]); else atomicOr(err, 2);
+                if (sl >= 0) atomicAdd(&W[sl], -(double)v[3 * i + k] * kc); else atomicOr(err, 2);
             }
         }
     }
@@ -555,13 +558,13 @@ __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int
     const float sc = pow2f(shift);
     const int64_t e_int = split ? split[a] : ptr[a];
     if (split) {
-        // the constant kernel's interior pairs: M_ab = c |T_a| |T_b| / 9 in all nine entries
-        const double ka = kc * area[a] * (1.0 / 9.0);
+        // the constant kernel's interior pairs: M_ab / c = |T_a| |T_b| / 9 in all nine entries
+        const double ka = area[a] * (1.0 / 9.0);
         for (int64_t e = ptr[a] + lane; e < e_int; e += 32) {
             const int b = idx[e];
             T v[9];
             for (int p = 0; p < 9; p++) v[p] = (T)(ka * area[b]);
-            scatter_pair<T, Acc>(1, b, v, K, J, tri, row_ptr, col, W, err, cached, H, hbits, ar, len, cap, sc, sacc,
+            scatter_pair<T, Acc>(1, b, v, K, J, tri, row_ptr, col, W, err, cached, H, hbits, ar, len, cap, sc, kc, sacc,
                                  skey, spk);
         }
     }
@@ -589,7 +592,7 @@ __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int
         } else {
             for (int p = 0; p < 9; p++) vn[p] = (T)0;
         }
-        scatter_pair<T, Acc>(f, b, v, K, J, tri, row_ptr, col, W, err, cached, H, hbits, ar, len, cap, sc, sacc,
+        scatter_pair<T, Acc>(f, b, v, K, J, tri, row_ptr, col, W, err, cached, H, hbits, ar, len, cap, sc, kc, sacc,
                              skey, spk);
         f = fn;
         b = bnx;
@@ -597,7 +600,7 @@ __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int
     }
     __syncwarp();
     if (cached) {
-        const double inv = (double)pow2f(-shift);
+        const double inv = (double)pow2f(-shift) * kc;
         for (int i = 0; i < 3; i++)
             for (int k = lane; k < len[i]; k += 32) {
                 const Acc x = sacc[i * cap + k];
@@ -606,7 +609,7 @@ __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int
                     if (x > (1 << 30) || x < -(1 << 30)) atomicOr(err, 256);
                     atomicAdd(&W[r0[i] + k], (double)x * inv);
                 } else {
-                    atomicAdd(&W[r0[i] + k], (double)x);
+                    atomicAdd(&W[r0[i] + k], (double)x * kc);
                 }
             }
     }
@@ -686,10 +689,10 @@ __device__ __forceinline__ void scatter_rank(int K, int J, int64_t E, const int3
     const float sc = pow2f(shift);
     const int64_t e_int = split ? split[a] : ptr[a];
     if (split) {
-        // the constant kernel's interior pairs: M_ab = c |T_a| |T_b| / 9 in all nine entries, so each
+        // the constant kernel's interior pairs: M_ab / c = |T_a| |T_b| / 9 in all nine entries, so each
         // node of T_b receives one value for the three rows together, summed in scom at the node's
         // place in row 0 (an interior pair puts T_b's nodes into all three rows)
-        const double ka = kc * area[a] * (1.0 / 9.0);
+        const double ka = area[a] * (1.0 / 9.0);
         int64_t e = ptr[a] + lane;
         int b = e < e_int ? idx[e] : 0, bn = e + 32 < e_int ? idx[e + 32] : 0;
         double ab = area[b];
@@ -766,7 +769,7 @@ __device__ __forceinline__ void scatter_rank(int K, int J, int64_t E, const int3
         for (int p = 0; p < 9; p++) v[p] = vn[p];
     }
     __syncwarp();
-    const double inv = (double)pow2f(-shift);
+    const double inv = (double)pow2f(-shift) * kc;
     for (int i = 0; i < 3; i++)
         for (int k = lane; k < len[i]; k += 32) {
             Acc x = sacc[i * cap + k];
@@ -781,7 +784,7 @@ __device__ __forceinline__ void scatter_rank(int K, int J, int64_t E, const int3
                 if (x > (1 << 30) || x < -(1 << 30)) atomicOr(err, 256);
                 atomicAdd(&W[r0[i] + k], (double)x * inv);
             } else {
-                atomicAdd(&W[r0[i] + k], (double)x);
+                atomicAdd(&W[r0[i] + k], (double)x * kc);
             }
         }
 }
@@ -811,10 +814,10 @@ __global__ void __launch_bounds__(128)
 // M_aa + M_bb of every triangle into W through its local slots (diagonal halved: D = W + W^T),
 // leaving mbb zeroed (the numeric phase also zeroes it before it sums)
 __device__ __forceinline__ void local_block(int K, int t, const double *maa, double *mbb, const int64_t *lslot,
-                                            double *W, int *err)
+                                            double *W, int *err, double kc)
 {
     for (int p = 0; p < 6; p++) {
-        double v = maa[(int64_t)p * K + t] + mbb[(int64_t)p * K + t];
+        double v = (maa[(int64_t)p * K + t] + mbb[(int64_t)p * K + t]) * kc;
         mbb[(int64_t)p * K + t] = 0.0;
         if (p < 3) v *= 0.5;
         const int64_t sl = lslot[(int64_t)p * K + t];
@@ -822,10 +825,11 @@ __device__ __forceinline__ void local_block(int K, int t, const double *maa, dou
     }
 }
 
-__global__ void k_local_blocks(int K, const double *maa, double *mbb, const int64_t *lslot, double *W, int *err)
+__global__ void k_local_blocks(int K, const double *maa, double *mbb, const int64_t *lslot, double *W, int *err,
+                               double kc)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < K) local_block(K, t, maa, mbb, lslot, W, err);
+    if (t < K) local_block(K, t, maa, mbb, lslot, W, err, kc);
 }
 
 // shared memory of one warp of the hashed scatter: row accumulators [3][cap] (T), hash keys and
@@ -919,7 +923,7 @@ __global__ void k_local_blocks_batch(const ScatterArgs *__restrict__ S, const in
     if (g >= koff[n]) return;
     const int p = batch_problem(koff, n, g);
     const ScatterArgs &A = S[p];
-    local_block(A.K, (int)(g - koff[p]), A.maa, A.mbb, A.lslot, A.W, A.err);
+    local_block(A.K, (int)(g - koff[p]), A.maa, A.mbb, A.lslot, A.W, A.err, A.kc);
 }
 
 __global__ void k_zero_batch(const ScatterArgs *__restrict__ S, const int64_t *__restrict__ zoff, int n)
@@ -1087,9 +1091,21 @@ nl_status nl_pattern_a(nl_ctx *ctx, nl_plan *P, nl_csr *out, nl_pat *T, nl_host_
         nl_free(P->fxe, st);
         if ((s = nl_alloc(ctx, &P->fxe, 1)) != NL_OK) return s;
         NL_CK(cudaMemsetAsync(P->fxe, 0, sizeof(int), st));
+        // the constant kernel's cut regions lie in the disc of the ball: where delta is near the triangles'
+        // size that bounds a column more closely than the triangles around its node do
+        const int ball = P->cfg.ball;
+        const bool disc = P->cfg.kernel == NL_KERNEL_CONST &&
+                          (ball == NL_BALL_NOCAPS || ball == NL_BALL_APPROXCAPS || ball == NL_BALL_EXACTCAPS ||
+                           ball == NL_BALL_NGON);
+        double rad = P->cfg.delta;
+        for (size_t k = 0; k + 1 < P->ngon_host.size(); k += 2)
+            rad = fmax(rad, hypot(P->ngon_host[k], P->ngon_host[k + 1]));
+        // (approxcaps: a fan that turns back counts its areas without sign, at most twice the disc)
+        const double cap = disc ? (ball == NL_BALL_APPROXCAPS ? 2.5 : 1.25) * 3.14159265358979323846 * rad * rad : HUGE_VAL;
         k_node_exp<<<(J + 255) / 256, 256, 0, st>>>(J, T->nptr, T->ntri, P->area,
                                                     P->cfg.kernel == NL_KERNEL_INV_DIST ? 1 : 0,
-                                                    fabs(P->cfg.kernel_c), P->fxe); ++ctx->launches;
+                                                    P->cfg.kernel == NL_KERNEL_INV_DIST ? fabs(P->cfg.kernel_c) : 1.0,
+                                                    cap, P->fxe); ++ctx->launches;
     }
     NL_CK(cudaFuncSetAttribute(k_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)(sizeof(int32_t) * (NL_HASH_CAP + kListCap))));
@@ -1225,10 +1241,11 @@ static nl_status launch_scatter(nl_ctx *ctx, nl_plan *P, nl_csr *out)
         NL_CK(cudaFuncSetAttribute(k_scatter_rank<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(96 * 1024)));
         k_scatter_rank<T><<<(unsigned)((K + warps - 1) / warps), 32 * warps, smem, ctx->stream>>>(
             K, P->J, P->E, P->tri, P->nbr_ptr, P->nbr_idx, P->flag, (const T *)P->blk, out->row_ptr, out->col_idx, P->W,
-            P->err, cap, (int)P->max_words, split, P->cfg.kernel_c, P->area, P->fxe, nl_outer_abs_weight(P));
+            P->err, cap, (int)P->max_words, split, nl_block_factor(P), P->area, P->fxe, nl_outer_abs_weight(P));
         ++ctx->launches;
         NL_CK(cudaGetLastError());
-        k_local_blocks<<<(K + 255) / 256, 256, 0, ctx->stream>>>(K, P->maa, P->mbb, P->lslot, P->W, P->err);
+        k_local_blocks<<<(K + 255) / 256, 256, 0, ctx->stream>>>(K, P->maa, P->mbb, P->lslot, P->W, P->err,
+                                                               nl_block_factor(P));
         ++ctx->launches;
         NL_CK(cudaGetLastError());
         return NL_OK;
@@ -1238,11 +1255,12 @@ static nl_status launch_scatter(nl_ctx *ctx, nl_plan *P, nl_csr *out)
     const unsigned grid = (unsigned)((K + warps - 1) / warps);
     k_scatter<T><<<grid, 32 * warps, smem, ctx->stream>>>(K, P->J, P->E, P->tri, P->nbr_ptr, P->nbr_idx, P->flag,
                                                            (const T *)P->blk, out->row_ptr, out->col_idx,
-                                                           P->W, P->err, cap, hbits, split, P->cfg.kernel_c,
+                                                           P->W, P->err, cap, hbits, split, nl_block_factor(P),
                                                            P->area, P->fxe,
                                                            nl_outer_abs_weight(P)); ++ctx->launches;
     NL_CK(cudaGetLastError());
-    k_local_blocks<<<(K + 255) / 256, 256, 0, ctx->stream>>>(K, P->maa, P->mbb, P->lslot, P->W, P->err);
+    k_local_blocks<<<(K + 255) / 256, 256, 0, ctx->stream>>>(K, P->maa, P->mbb, P->lslot, P->W, P->err,
+                                                               nl_block_factor(P));
     ++ctx->launches;
     NL_CK(cudaGetLastError());
     return NL_OK;

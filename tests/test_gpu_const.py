@@ -47,6 +47,8 @@ CASES = [
     ("ngon", 14, 0.2, 0.2, "switch47", {"off": ("turned", 5)}),
     ("nocaps", 10, 0.05, 0.2, "dunavant7", {}),
     ("approxcaps", 14, 0.2, 0.2, "dunavant7", {"cap_m": 1}),
+    ("approxcaps", 10, 0.05, 0.2, "dunavant7", {}),                   # arcs beyond a half circle
+    ("approxcaps", 10, 0.05, 0.2, "dunavant7", {"cap_m": 4}),
     ("approxcaps", 14, 0.2, 0.2, "switch47", {"cap_m": 4}),
     ("approxcaps", 14, 0.2, 0.2, "dunavant7", {"cap_m": 8}),         # past the FP32 walk: FP64 regions
     ("exactcaps", 14, 0.2, 0.0, "switch47", {}),

@@ -530,28 +530,27 @@ __device__ __forceinline__ int clip_ngon_f32_sh(const F2 dl[3], float err0, cons
     }
     *cut = false;
     uint64_t mask = ngon_pass_mask(dl, g);
-    while (mask && n > 0) {
+    // One exit: an uncertain sign ends the loops through `sure`, so that the warp's lanes meet again after
+    // every pass and vertex (returns inside the loops let them drift apart to the end of the item).
+    bool sure = true;
+    while (mask && n > 0 && sure) {
         const int k = __ffsll((long long)mask) - 1;
         mask &= mask - 1;
         const float ox = g.of[k][0], oy = g.of[k][1], ex = g.ef[k][0], ey = g.ef[k][1];
         const float el = g.mk[k] * g.inv_tau;   // |e_k|
         const float elu = el * kU9, elc = el * kU3o;
-        // a pass over a convex polygon keeps at most n + 1 vertices (certified signs keep the exact
-        // combinatorics), so a list of fewer than kClipCap vertices cannot outgrow the buffer
-        if (n >= kClipCap) return -1;
         const int nxt = cur ^ 1;
         int m = 0;
         bool all_in = true;
         float sx = cb.x[cur][n - 1][lane], sy = cb.y[cur][n - 1][lane], se = cb.e[cur][n - 1][lane];
         float so = ex * (sy - oy) - ey * (sx - ox);
         float su = fmaf(el, se, fmaf(elu, fabsf(sx - ox) + fabsf(sy - oy), elc));
-        // one vertex step: false when its sign is not certain
-        auto step = [&](int i) -> bool {
+        auto step = [&](int i) {
             const float px = cb.x[cur][i][lane], py = cb.y[cur][i][lane], pe = cb.e[cur][i][lane];
             const float po = ex * (py - oy) - ey * (px - ox);
             // |e_k| (err + 3 u |o_k|_1 + 9 u |r|_1), the bound above
             const float pu = fmaf(el, pe, fmaf(elu, fabsf(px - ox) + fabsf(py - oy), elc));
-            if (!(fabsf(po) > pu)) return false;
+            sure = sure && fabsf(po) > pu;
             const bool p_in = po > 0.f, s_in = so > 0.f;
             all_in = all_in && p_in;
             if (p_in != s_in) {
@@ -575,25 +574,25 @@ __device__ __forceinline__ int clip_ngon_f32_sh(const F2 dl[3], float err0, cons
                 m++;
             }
             sx = px; sy = py; se = pe; so = po; su = pu;
-            return true;
         };
+        // a pass over a convex polygon keeps at most n + 1 vertices (certified signs keep the exact
+        // combinatorics), so a list of fewer than kClipCap vertices cannot outgrow the buffer
+        sure = n < kClipCap;
         if constexpr (UNROLL) {
 #pragma unroll
-            for (int i = 0; i < kClipCap - 1; i++) {   // n < kClipCap
-                if (i >= n) break;
-                if (!step(i)) return -1;
-            }
+            for (int i = 0; i < kClipCap - 1; i++)   // n < kClipCap
+                if (sure && i < n) step(i);
         } else {
-            for (int i = 0; i < n; i++)
-                if (!step(i)) return -1;
+            for (int i = 0; sure && i < n; i++) step(i);
         }
-        if (all_in) continue;   // identity pass: keep the current list
-        *cut = true;
-        cur = nxt;
-        n = m;
+        if (!all_in) {   // else an identity pass: keep the current list
+            *cut = true;
+            cur = nxt;
+            n = m;
+        }
     }
     *which = cur;
-    return n;
+    return sure ? n : -1;
 }
 
 // Near field of the singular kernel for a whole T_b: near iff dist(x, T_b) < diam(T_b).

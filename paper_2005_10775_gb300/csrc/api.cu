@@ -388,17 +388,23 @@ nl_status nl_alloc_numeric(nl_ctx *ctx, nl_plan *P)
 {
     nl_status s;
     const size_t tsz = P->cfg.prec == NL_PREC_FP64 ? sizeof(double) : sizeof(float);
-    if ((s = nl_alloc(ctx, &P->flag, (size_t)P->E)) != NL_OK) return s;
-    unsigned char *blk = nullptr;
-    if ((s = nl_alloc(ctx, &blk, tsz * 9 * (size_t)(P->E ? P->E : 1))) != NL_OK) return s;
-    P->blk = blk;
-    if ((s = nl_alloc(ctx, &P->mbb, 6 * (size_t)P->K)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->maa, 6 * (size_t)P->K)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->qp_a, (size_t)P->K)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->cnt_a, (size_t)P->K)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->hash_a, (size_t)P->K)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->err, 1)) != NL_OK) return s;
-    NL_CK(cudaMemsetAsync(P->err, 0, sizeof(int), ctx->stream));
+    const size_t k = (size_t)P->K, e = (size_t)P->E;
+    nl_carver c;
+    const size_t err = c.add<int>(1), fxe = c.add<int>(1), zero = c.n;
+    const size_t mbb = c.add<double>(6 * k), maa = c.add<double>(6 * k), qp = c.add<int64_t>(k), cnt = c.add<int64_t>(k);
+    const size_t hash = c.add<uint64_t>(k), flag = c.add<uint8_t>(e), blk = c.add<char>(9 * tsz * (e ? e : 1));
+    if ((s = nl_alloc(ctx, &P->slab[1], c.n)) != NL_OK) return s;
+    char *p = P->slab[1];
+    P->err = (int *)(p + err);
+    P->fxe = (int *)(p + fxe);
+    P->mbb = (double *)(p + mbb);
+    P->maa = (double *)(p + maa);
+    P->qp_a = (int64_t *)(p + qp);
+    P->cnt_a = (int64_t *)(p + cnt);
+    P->hash_a = (uint64_t *)(p + hash);
+    P->flag = (uint8_t *)(p + flag);
+    P->blk = p + blk;
+    NL_CK(cudaMemsetAsync(p, 0, zero, ctx->stream));   // err, fxe
     return NL_OK;
 }
 
@@ -464,10 +470,6 @@ nl_status nl_assemble_step_c(nl_ctx *ctx, nl_plan *P, nl_prep *T, nl_pat *Q, nl_
     if (ev_num) NL_CK(cudaEventRecord(ev_num, ctx->stream));
     if ((s = run_numeric(ctx, P, false, one_stream)) != NL_OK) return s;
     if (ev_sym) NL_CK(cudaEventRecord(ev_sym, ctx->stream));
-    h->deferred = 0;
-    h->near = 0;
-    if (P->defer_n) NL_CK(cudaMemcpyAsync(&h->deferred, P->defer_n, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    if (P->near_n) NL_CK(cudaMemcpyAsync(&h->near, P->near_n, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
     return nl_pattern_a(ctx, P, out, Q, h);
 }
 
@@ -481,16 +483,17 @@ nl_status nl_assemble_step_d(nl_ctx *ctx, nl_plan *P, nl_pat *Q, const nl_host_s
     // A full queue of FP64-decided or near-field items leaves the excess to the boundary
     // kernel's lanes, and which items those are depends on the scheduling.  Queues that hold
     // them all (kept for every re-assembly of this plan) make the values independent of it.
-    const bool dfull = P->defer && h->deferred > P->defer_cap && !nl_defer_cap_fixed();
-    const bool nfull = P->near_n && P->near_cap > 0 && h->near > P->near_cap && !nl_near_cap_fixed();
+    const int64_t deferred = (int64_t)h->pat[kPatDeferred], near = (int64_t)h->pat[kPatNear];
+    const bool dfull = P->defer && deferred > P->defer_cap && !nl_defer_cap_fixed();
+    const bool nfull = P->near_n && P->near_cap > 0 && near > P->near_cap && !nl_near_cap_fixed();
     if (dfull) {
-        const int64_t want = (int64_t)h->deferred + h->deferred / 4;
+        const int64_t want = deferred + deferred / 4;
         P->defer_min = (int)(want > (int64_t(1) << 24) ? (int64_t(1) << 24) : want);
         nl_free(P->defer, ctx->stream);
         nl_free(P->defer_n, ctx->stream);
     }
     if (nfull) {
-        const int64_t want = (int64_t)h->near + h->near / 4;
+        const int64_t want = near + near / 4;
         P->near_min = (int)(want > (int64_t(1) << 30) ? (int64_t(1) << 30) : want);
         nl_free(P->nearq, ctx->stream);
         nl_free(P->otab, ctx->stream);
@@ -505,12 +508,10 @@ nl_status nl_assemble_step_d(nl_ctx *ctx, nl_plan *P, nl_pat *Q, const nl_host_s
 void nl_plan_free(nl_plan *P, cudaStream_t s)
 {
     if (!P) return;
-    nl_free(P->tri, s); nl_free(P->tx, s); nl_free(P->ty, s); nl_free(P->bx, s); nl_free(P->by, s);
-    nl_free(P->rad, s); nl_free(P->area, s); nl_free(P->akc, s); nl_free(P->hl, s); nl_free(P->ngon, s); nl_free(P->nbr_ptr, s); nl_free(P->nbr_idx, s);
-    nl_free(P->nbr_split, s); nl_free(P->flag, s); nl_free(P->blk, s); nl_free(P->maa, s); nl_free(P->qp_a, s);
-    nl_free(P->cnt_a, s); nl_free(P->hash_a, s); nl_free(P->lslot, s); nl_free(P->mbb, s); nl_free(P->tslot, s); nl_free(P->W, s);
-    nl_free(P->val32, s); nl_free(P->x32, s); nl_free(P->err, s); nl_free(P->defer, s); nl_free(P->defer_n, s);
-    nl_free(P->nearq, s); nl_free(P->near_n, s); nl_free(P->otab, s); nl_free(P->fxe, s);
+    for (char *&p : P->slab) nl_free(p, s);
+    nl_free(P->nbr_ptr, s); nl_free(P->nbr_idx, s); nl_free(P->nbr_split, s);
+    nl_free(P->val32, s); nl_free(P->x32, s); nl_free(P->defer, s); nl_free(P->defer_n, s);
+    nl_free(P->nearq, s); nl_free(P->near_n, s); nl_free(P->otab, s);
 }
 
 nl_status nl_host_slots(nl_ctx *ctx, int n, nl_host_slot **out)
@@ -572,15 +573,17 @@ nl_status nl_create(nl_ctx **out, int device, void *stream)
     for (int k = 0; e == cudaSuccess && k <= nl_ctx::kSideStreams; k++)
         e = cudaEventCreateWithFlags(&ctx->side_ev[k], cudaEventDisableTiming);
     if (e == cudaSuccess) {
-        // keep freed pool memory cached by this process (up to 8 GiB) instead of handing it
+        // keep freed pool memory cached by this process (up to 16 GiB, of 277) instead of handing it
         // back to the driver at every synchronisation: later assemblies allocate without
-        // driver calls.  This is a property of the process's pool, not of the device.
+        // driver calls.  Two matrices of the largest workloads (K = 96,800: about 5 GB each with
+        // their pair blocks) fit; with 8 GiB every assembly there mapped memory again (24.6 against
+        // 17.5 ms).  This is a property of the process's pool, not of the device.
         cudaMemPool_t pool;
         if (cudaDeviceGetDefaultMemPool(&pool, device) == cudaSuccess) {
             uint64_t thr = 0;
             if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr) == cudaSuccess &&
-                thr < (uint64_t(8) << 30)) {
-                thr = uint64_t(8) << 30;
+                thr < (uint64_t(16) << 30)) {
+                thr = uint64_t(16) << 30;
                 cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
             }
         }
@@ -647,7 +650,7 @@ nl_status nl_assemble(nl_ctx *ctx, const nl_mesh *mesh, const nl_config *cfg, nl
     if ((e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess) goto cuda_fail;
     if ((s = nl_assemble_step_c(ctx, P, T, Q, h, out, false, ctx->ev[1], ctx->ev[2])) != NL_OK) goto fail;
     if ((e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess) goto cuda_fail;
-    ctx->last_fp64_items = h->deferred;
+    ctx->last_fp64_items = (int64_t)h->pat[kPatDeferred];
     if ((s = nl_assemble_step_d(ctx, P, Q, h, out, false, ctx->ev[3])) != NL_OK) goto fail;
     if ((e = cudaEventRecord(ctx->ev[4], ctx->stream)) != cudaSuccess) goto cuda_fail;
     nl_prep_delete(T, ctx->stream);

@@ -607,7 +607,7 @@ nl_status assemble_pipelined(nl_ctx *ctx, int n, const nl_mesh *meshes, const nl
                 fail_at = i;
                 return finish(nl_cuda_fail(ctx, q, "a batch problem's stream"));
             }
-            if (step[i] == 3) fp64_items += h[i].deferred;
+            if (step[i] == 3) fp64_items += (int64_t)h[i].pat[kPatDeferred];
             if ((s = issue(i)) != NL_OK) {
                 fail_at = i;
                 return finish(s);

@@ -49,18 +49,24 @@ __device__ __forceinline__ int nl_block_scan(int v, int *wsum, int *total)
 // words).  The phases copy them, stream-ordered, into pinned slots owned by the
 // context; the host reads a slot only after synchronising the stream, so a batch of
 // problems needs one synchronisation per phase instead of one per problem.
+constexpr int kPatWords = 10;
 struct nl_host_slot {
-    unsigned long long mesh[6];   // order-preserving keys: xmin, ymin, xmax, ymax, r_max, h_max
+    unsigned long long mesh[6];   // order-preserving keys: xmin, ymin (complemented), xmax, ymax, r_max, h_max
+    unsigned long long bad;       // degenerate / clockwise / out-of-range triangles (copied with mesh)
     int64_t E;                    // candidate pairs
-    int64_t nnz;                  // pattern entries
-    unsigned long long pat[5];    // pairs, qp-pairs, interactions, longest row, words of the widest
-                                  // column bitmap of a triangle's rows
-    int bad;                      // degenerate / clockwise / out-of-range triangles
+    unsigned long long pat[kPatWords];   // what the symbolic stage A leaves (one copy)
     int ovf;                      // cell-list or candidate-list overflow
-    int row_ovf;                  // pattern row overflow
-    int err;                      // numeric-phase error word
-    int deferred;                 // FP32 path: items the FP64 geometry decided
-    int near;                     // FP32 path, singular kernel: near-field items queued for k_near
+};
+
+// words of nl_host_slot::pat
+enum {
+    kPatPairs, kPatQp, kPatInter, kPatMaxRow,
+    kPatMaxWords,   // words of the widest column bitmap of a triangle's rows
+    kPatNnz,        // pattern entries
+    kPatErr,        // numeric-phase error word
+    kPatRowOvf,     // pattern row overflow
+    kPatDeferred,   // FP32 path: items the FP64 geometry decided
+    kPatNear        // FP32 path, singular kernel: near-field items queued for k_near
 };
 
 struct nl_ctx {
@@ -88,8 +94,23 @@ nl_status nl_side_streams(nl_ctx *ctx);
 // pinned host slots for n problems (grown on demand; invalidates earlier slot pointers)
 nl_status nl_host_slots(nl_ctx *ctx, int n, nl_host_slot **out);
 
+// Several device arrays of one lifetime in one allocation: add() them, allocate total() bytes once, and
+// turn the offsets into pointers.  (An assembly's fifty small arrays, each with its own stream-ordered
+// allocation and release and many with a memset, kept the host busier than the GPU on small problems.)
+struct nl_carver {
+    size_t n = 0;
+    template <class T>
+    size_t add(size_t count)
+    {
+        const size_t at = n;
+        n += ((count ? count : 1) * sizeof(T) + 255) & ~(size_t)255;
+        return at;
+    }
+};
+
 // Device-resident state of one assembled problem (held by nl_csr.priv).
 struct nl_plan {
+    char *slab[3] = {nullptr, nullptr, nullptr};   // the allocations that hold the mesh, numeric and slot arrays
     cudaStream_t stream = nullptr;   // stream the buffers were allocated on (freed stream-ordered)
     int K = 0, J = 0;
     nl_config cfg{};

@@ -15,6 +15,7 @@
 // index) and per-triangle candidate lists sorted by triangle index.
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stddef.h>
 #include <string.h>
 
 #include <new>
@@ -137,13 +138,14 @@ __global__ void __launch_bounds__(1024) k_scan_one(const int64_t *in, int64_t *o
 // ---------------------------------------------------------------------------
 __global__ void k_prepare(int K, int J, const int32_t *__restrict__ tri, const double *__restrict__ vx,
                           const double *__restrict__ vy, double *tx, double *ty, double *bx, double *by,
-                          double *rad, double *area, double *diam, float4 *cf, double kc, float *akc, int *bad)
+                          double *rad, double *area, double *diam, float4 *cf, double kc, float *akc,
+                          unsigned long long *bad)
 {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= K) return;
     int i0 = tri[3 * t], i1 = tri[3 * t + 1], i2 = tri[3 * t + 2];
     if (i0 < 0 || i1 < 0 || i2 < 0 || i0 >= J || i1 >= J || i2 >= J) {
-        atomicAdd(bad, 1);
+        atomicAdd(bad, 1ull);
         return;
     }
     double x0 = vx[i0], y0 = vy[i0], x1 = vx[i1], y1 = vy[i1], x2 = vx[i2], y2 = vy[i2];
@@ -170,7 +172,7 @@ __global__ void k_prepare(int K, int J, const int32_t *__restrict__ tri, const d
     double cr = (x1 - x0) * (y2 - y0) - (x2 - x0) * (y1 - y0);
     area[t] = 0.5 * fabs(cr);
     akc[t] = (float)(0.5 * fabs(cr) * kc);
-    if (!(cr > 0.0)) atomicAdd(bad, 1);
+    if (!(cr > 0.0)) atomicAdd(bad, 1ull);
 }
 
 // Every FP64 coordinate v as an FP32 pair hi = fl32(v), lo = fl32(v - hi) (v - hi is exact in
@@ -218,7 +220,8 @@ inline double stat_value(unsigned long long k)
 }
 
 // bounding box of the barycenters, largest barycenter radius and largest diameter; block sums
-// in shared memory, one atomic per block and statistic (keys preset: minima ~0, maxima 0)
+// in shared memory, one atomic per block and statistic.  Minima are kept as maxima of the complemented
+// keys, so that one memset to zero presets them all.
 __global__ void k_mesh_stats(int K, const double *bx, const double *by, const double *rad, const double *diam,
                              unsigned long long *key)
 {
@@ -243,7 +246,7 @@ __global__ void k_mesh_stats(int K, const double *bx, const double *by, const do
         const int i = threadIdx.x;
         double r = s[i][0];
         for (int k = 1; k < nw; k++) r = i < kStatXmax ? fmin(r, s[i][k]) : fmax(r, s[i][k]);
-        if (i < kStatXmax) atomicMin(&key[i], stat_key(r));
+        if (i < kStatXmax) atomicMax(&key[i], ~stat_key(r));
         else atomicMax(&key[i], stat_key(r));
     }
 }
@@ -510,9 +513,9 @@ double nl_polygon_inradius(const double *o, int N)
 struct nl_prep {
     void *dvx = nullptr, *dvy = nullptr, *dtri = nullptr;
     bool own_vx = false, own_vy = false, own_tri = false;
+    char *slab[2] = {nullptr, nullptr};   // the allocations that hold the arrays of stages A and B
     double *diam = nullptr;
-    int *bad = nullptr;
-    unsigned long long *st = nullptr;   // k_mesh_stats keys
+    unsigned long long *st = nullptr;   // k_mesh_stats keys, then the count of bad triangles
     float4 *cf = nullptr;
     Grid g{};
     int ncell = 0;
@@ -538,9 +541,7 @@ void prep_release(nl_prep *T, cudaStream_t s)
     free_async(vx, s); free_async(vy, s); free_async(tr, s);
     T->dvx = T->dvy = T->dtri = nullptr;
     T->own_vx = T->own_vy = T->own_tri = false;
-    free_async(T->diam, s); free_async(T->bad, s); free_async(T->st, s); free_async(T->cf, s);
-    free_async(T->cell, s); free_async(T->bucket, s); free_async(T->ccnt, s); free_async(T->cstart, s);
-    free_async(T->cursor, s); free_async(T->cnt, s); free_async(T->ovf, s);
+    free_async(T->slab[0], s); free_async(T->slab[1], s);
 }
 }  // namespace
 
@@ -564,20 +565,30 @@ nl_status nl_prepare_a(nl_ctx *ctx, const nl_mesh *mesh, const nl_config *cfg, n
     if ((s = nl_stage(ctx, mesh->vx, sizeof(double) * J, &T->dvx, &T->own_vx)) != NL_OK) return s;
     if ((s = nl_stage(ctx, mesh->vy, sizeof(double) * J, &T->dvy, &T->own_vy)) != NL_OK) return s;
     if ((s = nl_stage(ctx, mesh->tri, sizeof(int32_t) * 3 * K, &T->dtri, &T->own_tri)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->tri, 3 * (size_t)K)) != NL_OK) return s;
+    {
+        const size_t k = (size_t)K;
+        nl_carver c;
+        const size_t tri = c.add<int32_t>(3 * k), tx = c.add<double>(3 * k), ty = c.add<double>(3 * k);
+        const size_t bx = c.add<double>(k), by = c.add<double>(k), rad = c.add<double>(k), area = c.add<double>(k);
+        const size_t akc = c.add<float>(k), hl = c.add<float>(16 * k);
+        const size_t ngon = c.add<double>(cfg->ball == NL_BALL_NGON ? 2 * (size_t)cfg->ngon_n : 0);
+        if ((s = nl_alloc(ctx, &P->slab[0], c.n)) != NL_OK) return s;
+        char *p = P->slab[0];
+        P->tri = (int32_t *)(p + tri);
+        P->tx = (double *)(p + tx);
+        P->ty = (double *)(p + ty);
+        P->bx = (double *)(p + bx);
+        P->by = (double *)(p + by);
+        P->rad = (double *)(p + rad);
+        P->area = (double *)(p + area);
+        P->akc = (float *)(p + akc);
+        P->hl = (float *)(p + hl);
+        P->ngon = cfg->ball == NL_BALL_NGON ? (double *)(p + ngon) : nullptr;
+    }
     NL_CK(cudaMemcpyAsync(P->tri, T->dtri, sizeof(int32_t) * 3 * K, cudaMemcpyDeviceToDevice, ctx->stream));
-    if ((s = nl_alloc(ctx, &P->tx, 3 * (size_t)K)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->ty, 3 * (size_t)K)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->bx, K)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->by, K)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->rad, K)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->area, K)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->akc, K)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->hl, 16 * (size_t)K)) != NL_OK) return s;
     if (cfg->ball == NL_BALL_NGON) {
         const size_t nb = sizeof(double) * 2 * cfg->ngon_n;
         P->ngon_host.resize(2 * (size_t)cfg->ngon_n);
-        if ((s = nl_alloc(ctx, &P->ngon, 2 * (size_t)cfg->ngon_n)) != NL_OK) return s;
         if (nl_is_device_ptr(cfg->ngon_offsets)) {
             NL_CK(cudaMemcpyAsync(P->ngon, cfg->ngon_offsets, nb, cudaMemcpyDeviceToDevice, ctx->stream));
             NL_CK(cudaMemcpyAsync(P->ngon_host.data(), cfg->ngon_offsets, nb, cudaMemcpyDeviceToHost, ctx->stream));
@@ -588,18 +599,20 @@ nl_status nl_prepare_a(nl_ctx *ctx, const nl_mesh *mesh, const nl_config *cfg, n
         }
         P->rin = nl_polygon_inradius(P->ngon_host.data(), cfg->ngon_n);
     }
-    NL_CK(cudaMallocAsync((void **)&T->diam, sizeof(double) * K, ctx->stream));
-    NL_CK(cudaMallocAsync((void **)&T->bad, sizeof(int), ctx->stream));
-    NL_CK(cudaMallocAsync((void **)&T->st, sizeof(unsigned long long) * kStats, ctx->stream));
-    NL_CK(cudaMemsetAsync(T->st, 0xff, sizeof(unsigned long long) * kStatXmax, ctx->stream));
-    NL_CK(cudaMemsetAsync(T->st + kStatXmax, 0, sizeof(unsigned long long) * (kStats - kStatXmax), ctx->stream));
-    NL_CK(cudaMemsetAsync(T->bad, 0, sizeof(int), ctx->stream));
-    NL_CK(cudaMallocAsync((void **)&T->cf, sizeof(float4) * K, ctx->stream));
+    {
+        nl_carver c;
+        const size_t stt = c.add<unsigned long long>(kStats + 1), diam = c.add<double>(K), cf = c.add<float4>(K);
+        if ((s = nl_alloc(ctx, &T->slab[0], c.n)) != NL_OK) return s;
+        T->st = (unsigned long long *)(T->slab[0] + stt);
+        T->diam = (double *)(T->slab[0] + diam);
+        T->cf = (float4 *)(T->slab[0] + cf);
+    }
+    NL_CK(cudaMemsetAsync(T->st, 0, sizeof(unsigned long long) * (kStats + 1), ctx->stream));
     k_prepare<<<(K + 255) / 256, 256, 0, ctx->stream>>>(K, J, (const int32_t *)T->dtri, (const double *)T->dvx,
                                                         (const double *)T->dvy, P->tx, P->ty, P->bx, P->by,
                                                         P->rad, P->area, T->diam, T->cf,
                                                         cfg->kernel == NL_KERNEL_CONST ? 1.0 : cfg->kernel_c, P->akc,
-                                                        T->bad); ++ctx->launches;
+                                                        T->st + kStats); ++ctx->launches;
     k_hilo<<<(K + 255) / 256, 256, 0, ctx->stream>>>(K, P->tx, P->ty, P->bx, P->by, P->hl); ++ctx->launches;
     NL_CK(cudaGetLastError());
     {
@@ -608,9 +621,10 @@ nl_status nl_prepare_a(nl_ctx *ctx, const nl_mesh *mesh, const nl_config *cfg, n
         ++ctx->launches;
     }
     NL_CK(cudaGetLastError());
-    static_assert(sizeof(unsigned long long) * kStats == sizeof(h->mesh), "mesh statistics slot");
-    NL_CK(cudaMemcpyAsync(h->mesh, T->st, sizeof h->mesh, cudaMemcpyDeviceToHost, ctx->stream));
-    NL_CK(cudaMemcpyAsync(&h->bad, T->bad, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    static_assert(sizeof(unsigned long long) * kStats == sizeof(h->mesh) &&
+                      offsetof(nl_host_slot, bad) == offsetof(nl_host_slot, mesh) + sizeof(h->mesh),
+                  "mesh statistics slot");
+    NL_CK(cudaMemcpyAsync(h->mesh, T->st, sizeof h->mesh + sizeof h->bad, cudaMemcpyDeviceToHost, ctx->stream));
     return NL_OK;
 }
 
@@ -619,19 +633,18 @@ nl_status nl_prepare_b(nl_ctx *ctx, nl_plan *P, nl_prep *T, nl_host_slot *h)
     const int K = P->K;
     const nl_config *cfg = &P->cfg;
     cudaStream_t st = ctx->stream;
-    // the staged inputs and the statistics buffers are no longer needed
+    // the staged inputs are no longer needed
     {
         void *vx = T->own_vx ? T->dvx : nullptr, *vy = T->own_vy ? T->dvy : nullptr;
         void *tr = T->own_tri ? T->dtri : nullptr;
         free_async(vx, st); free_async(vy, st); free_async(tr, st);
         T->dvx = T->dvy = T->dtri = nullptr;
         T->own_vx = T->own_vy = T->own_tri = false;
-        free_async(T->diam, st); free_async(T->bad, st); free_async(T->st, st);
     }
     MeshStats hst;
-    hst.xmin = stat_value(h->mesh[kStatXmin]);
+    hst.xmin = stat_value(~h->mesh[kStatXmin]);
     hst.xmax = stat_value(h->mesh[kStatXmax]);
-    hst.ymin = stat_value(h->mesh[kStatYmin]);
+    hst.ymin = stat_value(~h->mesh[kStatYmin]);
     hst.ymax = stat_value(h->mesh[kStatYmax]);
     hst.rmax = stat_value(h->mesh[kStatRmax]);
     hst.hmax = stat_value(h->mesh[kStatHmax]);
@@ -653,18 +666,26 @@ nl_status nl_prepare_b(nl_ctx *ctx, nl_plan *P, nl_prep *T, nl_host_slot *h)
     g.ny = (int)floor(Ly / cs) + 1;
     const int ncell = g.nx * g.ny;
     T->ncell = ncell;
-    NL_CK(cudaMallocAsync((void **)&T->cell, sizeof(int32_t) * K, st));
-    NL_CK(cudaMallocAsync((void **)&T->bucket, sizeof(int32_t) * K, st));
-    NL_CK(cudaMallocAsync((void **)&T->ccnt, sizeof(int64_t) * (ncell + 1), st));
-    NL_CK(cudaMallocAsync((void **)&T->cstart, sizeof(int64_t) * (ncell + 1), st));
-    NL_CK(cudaMallocAsync((void **)&T->cursor, sizeof(int64_t) * (ncell + 1), st));
-    NL_CK(cudaMallocAsync((void **)&T->ovf, sizeof(int), st));
-    NL_CK(cudaMemsetAsync(T->ccnt, 0, sizeof(int64_t) * (ncell + 1), st));
-    NL_CK(cudaMemsetAsync(T->cursor, 0, sizeof(int64_t) * (ncell + 1), st));
-    NL_CK(cudaMemsetAsync(T->ovf, 0, sizeof(int), st));
+    nl_status s;
+    {
+        const size_t k = (size_t)K, nc = (size_t)ncell + 1;
+        nl_carver c;
+        const size_t ccnt = c.add<int64_t>(nc), cursor = c.add<int64_t>(nc), ovf = c.add<int>(1), zero = c.n;
+        const size_t cell = c.add<int32_t>(k), bucket = c.add<int32_t>(k), cstart = c.add<int64_t>(nc);
+        const size_t cnt = c.add<int64_t>(k);
+        if ((s = nl_alloc(ctx, &T->slab[1], c.n)) != NL_OK) return s;
+        char *p = T->slab[1];
+        T->ccnt = (int64_t *)(p + ccnt);
+        T->cursor = (int64_t *)(p + cursor);
+        T->ovf = (int *)(p + ovf);
+        T->cell = (int32_t *)(p + cell);
+        T->bucket = (int32_t *)(p + bucket);
+        T->cstart = (int64_t *)(p + cstart);
+        T->cnt = (int64_t *)(p + cnt);
+        NL_CK(cudaMemsetAsync(p, 0, zero, st));   // ccnt, cursor, ovf
+    }
     k_cell_count<<<(K + 255) / 256, 256, 0, st>>>(K, g, P->bx, P->by, T->cell, T->ccnt); ++ctx->launches;
     NL_CK(cudaGetLastError());
-    nl_status s;
     if ((s = nl_scan_i64(ctx, T->ccnt, T->cstart, ncell)) != NL_OK) return s;
     k_cell_fill<<<(K + 255) / 256, 256, 0, st>>>(K, T->cell, T->cstart, T->cursor, T->bucket); ++ctx->launches;
     NL_CK(cudaGetLastError());
@@ -672,7 +693,6 @@ nl_status nl_prepare_b(nl_ctx *ctx, nl_plan *P, nl_prep *T, nl_host_slot *h)
     NL_CK(cudaGetLastError());
     // candidate counts and their prefix sum
     if ((s = nl_alloc(ctx, &P->nbr_ptr, (size_t)K + 1)) != NL_OK) return s;
-    NL_CK(cudaMallocAsync((void **)&T->cnt, sizeof(int64_t) * K, st));
     const unsigned wblocks = (unsigned)(((int64_t)K * 32 + 255) / 256);
     k_candidates<<<wblocks, 256, 0, st>>>(K, g, (float)cfg->delta, T->cf, T->cstart, T->bucket, T->cnt, nullptr,
                                           nullptr, 0); ++ctx->launches;

@@ -961,9 +961,17 @@ __global__ void k_symmetrize(int64_t nnz, const double *W, const int64_t *tslot,
 }
 
 // longest row (out[3]) and the words of the widest bitmap over the columns of a triangle's three rows (out[4])
+// and the other numbers the host reads here: entries, error word, queue counts (null: 0)
 __global__ void k_row_max(int J, const int64_t *rcnt, int K, const int32_t *tri, const int2 *span,
+                          const int64_t *row_ptr, const int *err, const int *defer_n, const int *near_n,
                           unsigned long long *out)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        out[kPatNnz] = (unsigned long long)row_ptr[J];
+        out[kPatErr] = (unsigned long long)(unsigned)*err;
+        out[kPatDeferred] = defer_n ? (unsigned long long)*defer_n : 0ull;
+        out[kPatNear] = near_n ? (unsigned long long)*near_n : 0ull;
+    }
     unsigned long long m = 0;
     int w = 0;
     const int nth = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -977,8 +985,8 @@ __global__ void k_row_max(int J, const int64_t *rcnt, int K, const int32_t *tri,
         w = max(w, __shfl_xor_sync(0xffffffffu, w, off));
     }
     if ((threadIdx.x & 31) == 0) {
-        atomicMax(&out[3], m);
-        atomicMax(&out[4], (unsigned long long)w);
+        atomicMax(&out[kPatMaxRow], m);
+        atomicMax(&out[kPatMaxWords], (unsigned long long)w);
     }
 }
 
@@ -1017,6 +1025,7 @@ __global__ void k_sum_stats(int K, int64_t E, const uint8_t *flag, const int64_t
 }  // namespace
 
 struct nl_pat {
+    char *slab[2] = {nullptr, nullptr};   // the allocations that hold the arrays below
     uint8_t *sym = nullptr;
     int64_t *ncnt = nullptr, *nptr = nullptr, *ncur = nullptr, *rcnt = nullptr;
     int32_t *ntri = nullptr;
@@ -1044,11 +1053,7 @@ void free_async(T *&p, cudaStream_t s)
 void nl_pat_delete(nl_pat *T, cudaStream_t s)
 {
     if (!T) return;
-    free_async(T->sym, s); free_async(T->ncnt, s); free_async(T->nptr, s); free_async(T->ncur, s);
-    free_async(T->rcnt, s); free_async(T->ntri, s); free_async(T->ovf, s); free_async(T->st, s);
-    free_async(T->olist, s); free_async(T->on, s);
-    free_async(T->buf, s); free_async(T->bflag, s); free_async(T->rlist, s); free_async(T->rn, s);
-    free_async(T->span, s);
+    free_async(T->slab[0], s); free_async(T->slab[1], s);
     delete T;
 }
 
@@ -1065,22 +1070,32 @@ nl_status nl_pattern_a(nl_ctx *ctx, nl_plan *P, nl_csr *out, nl_pat *T, nl_host_
     const int K = P->K, J = P->J;
     cudaStream_t st = ctx->stream;
     nl_status s;
-    NL_CK(cudaMallocAsync((void **)&T->sym, P->E ? P->E : 1, st));
-    NL_CK(cudaMallocAsync((void **)&T->ncnt, sizeof(int64_t) * (J + 1), st));
-    NL_CK(cudaMallocAsync((void **)&T->nptr, sizeof(int64_t) * (J + 1), st));
-    NL_CK(cudaMallocAsync((void **)&T->ncur, sizeof(int64_t) * (J + 1), st));
-    NL_CK(cudaMallocAsync((void **)&T->rcnt, sizeof(int64_t) * (J + 1), st));
-    NL_CK(cudaMallocAsync((void **)&T->ntri, sizeof(int32_t) * 3 * (size_t)K, st));
-    NL_CK(cudaMallocAsync((void **)&T->ovf, sizeof(int), st));
-    NL_CK(cudaMallocAsync((void **)&T->olist, sizeof(int) * (J + 1), st));
-    NL_CK(cudaMallocAsync((void **)&T->on, sizeof(int), st));
-    NL_CK(cudaMemsetAsync(T->on, 0, sizeof(int), st));
-    NL_CK(cudaMallocAsync((void **)&T->span, sizeof(int2) * (J + 1), st));
-    NL_CK(cudaMallocAsync((void **)&T->st, sizeof h->pat, st));
-    NL_CK(cudaMemsetAsync(T->ncnt, 0, sizeof(int64_t) * (J + 1), st));
-    NL_CK(cudaMemsetAsync(T->ncur, 0, sizeof(int64_t) * (J + 1), st));
-    NL_CK(cudaMemsetAsync(T->ovf, 0, sizeof(int), st));
-    NL_CK(cudaMemsetAsync(T->st, 0, sizeof h->pat, st));
+    {
+        const size_t j = (size_t)J + 1;
+        nl_carver c;
+        const size_t ncnt = c.add<int64_t>(j), ncur = c.add<int64_t>(j), on = c.add<int>(1), rn = c.add<int>(1);
+        const size_t stt = c.add<unsigned long long>(kPatWords), zero = c.n;
+        const size_t nptr = c.add<int64_t>(j), rcnt = c.add<int64_t>(j), ntri = c.add<int32_t>(3 * (size_t)K);
+        const size_t olist = c.add<int>(j), rlist = c.add<int>(j), bflag = c.add<uint8_t>(j), span = c.add<int2>(j);
+        const size_t sym = c.add<uint8_t>((size_t)P->E);
+        if ((s = nl_alloc(ctx, &T->slab[0], c.n)) != NL_OK) return s;
+        char *p = T->slab[0];
+        T->ncnt = (int64_t *)(p + ncnt);
+        T->ncur = (int64_t *)(p + ncur);
+        T->on = (int *)(p + on);
+        T->rn = (int *)(p + rn);
+        T->st = (unsigned long long *)(p + stt);
+        T->ovf = (int *)(T->st + kPatRowOvf);   // little-endian: the low half of the word
+        T->nptr = (int64_t *)(p + nptr);
+        T->rcnt = (int64_t *)(p + rcnt);
+        T->ntri = (int32_t *)(p + ntri);
+        T->olist = (int *)(p + olist);
+        T->rlist = (int *)(p + rlist);
+        T->bflag = (uint8_t *)(p + bflag);
+        T->span = (int2 *)(p + span);
+        T->sym = (uint8_t *)(p + sym);
+        NL_CK(cudaMemsetAsync(p, 0, zero, st));   // the counters and the statistics
+    }
     const unsigned wgrid = (unsigned)(((int64_t)K * 32 + 255) / 256);
     k_symflag<<<wgrid, 256, 0, st>>>(K, P->nbr_ptr, P->nbr_split, P->nbr_idx, P->flag, T->sym); ++ctx->launches;
     k_node_count<<<(K + 255) / 256, 256, 0, st>>>(K, P->tri, T->ncnt); ++ctx->launches;
@@ -1088,9 +1103,6 @@ nl_status nl_pattern_a(nl_ctx *ctx, nl_plan *P, nl_csr *out, nl_pat *T, nl_host_
     if ((s = nl_scan_i64(ctx, T->ncnt, T->nptr, J)) != NL_OK) return s;
     k_node_fill<<<(K + 255) / 256, 256, 0, st>>>(K, P->tri, T->nptr, T->ncur, T->ntri); ++ctx->launches;
     if (P->cfg.prec != NL_PREC_FP64 && J > 0) {
-        nl_free(P->fxe, st);
-        if ((s = nl_alloc(ctx, &P->fxe, 1)) != NL_OK) return s;
-        NL_CK(cudaMemsetAsync(P->fxe, 0, sizeof(int), st));
         // the constant kernel's cut regions lie in the disc of the ball: where delta is near the triangles'
         // size that bounds a column more closely than the triangles around its node do
         const int ball = P->cfg.ball;
@@ -1122,11 +1134,8 @@ nl_status nl_pattern_a(nl_ctx *ctx, nl_plan *P, nl_csr *out, nl_pat *T, nl_host_
     }
     const int lb0 = hb0 - 1;
     T->lbits = lb0;
-    NL_CK(cudaMallocAsync((void **)&T->buf, sizeof(int32_t) * ((size_t)J << lb0), st));
-    NL_CK(cudaMallocAsync((void **)&T->bflag, (size_t)J + 1, st));
-    NL_CK(cudaMallocAsync((void **)&T->rlist, sizeof(int) * (J + 1), st));
-    NL_CK(cudaMallocAsync((void **)&T->rn, sizeof(int), st));
-    NL_CK(cudaMemsetAsync(T->rn, 0, sizeof(int), st));
+    if ((s = nl_alloc(ctx, &T->slab[1], sizeof(int32_t) * ((size_t)J << lb0))) != NL_OK) return s;
+    T->buf = (int32_t *)T->slab[1];
     k_rows<<<J, kRowThreads, sizeof(int32_t) * ((1u << hb0) + (1u << lb0)), st>>>(
         J, T->nptr, T->ntri, P->tri, P->nbr_ptr, P->nbr_idx, T->sym, hb0, lb0, nullptr, nullptr, T->rcnt, nullptr,
         nullptr, T->olist, T->on, T->ovf, T->buf, T->bflag, T->rlist, T->rn, T->span, 0); ++ctx->launches;
@@ -1140,11 +1149,9 @@ nl_status nl_pattern_a(nl_ctx *ctx, nl_plan *P, nl_csr *out, nl_pat *T, nl_host_
     if ((s = nl_alloc(ctx, &out->row_ptr, (size_t)J + 1)) != NL_OK) return s;
     if ((s = nl_scan_i64(ctx, T->rcnt, out->row_ptr, J)) != NL_OK) return s;
     k_sum_stats<<<256, 256, 0, st>>>(K, P->E, P->flag, P->qp_a, P->cnt_a, T->st); ++ctx->launches;
-    k_row_max<<<64, 256, 0, st>>>(J, T->rcnt, K, P->tri, T->span, T->st); ++ctx->launches;
+    k_row_max<<<64, 256, 0, st>>>(J, T->rcnt, K, P->tri, T->span, out->row_ptr, P->err, P->defer_n, P->near_n, T->st);
+    ++ctx->launches;
     NL_CK(cudaGetLastError());
-    NL_CK(cudaMemcpyAsync(&h->err, P->err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    NL_CK(cudaMemcpyAsync(&h->nnz, out->row_ptr + J, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    NL_CK(cudaMemcpyAsync(&h->row_ovf, T->ovf, sizeof(int), cudaMemcpyDeviceToHost, st));
     NL_CK(cudaMemcpyAsync(h->pat, T->st, sizeof h->pat, cudaMemcpyDeviceToHost, st));
     return NL_OK;
 }
@@ -1154,19 +1161,20 @@ nl_status nl_pattern_b(nl_ctx *ctx, nl_plan *P, nl_csr *out, nl_pat *T, const nl
     const int K = P->K, J = P->J;
     cudaStream_t st = ctx->stream;
     nl_status s;
-    if (h->row_ovf) return nl_fail(ctx, NL_EUNSUPPORTED, "a matrix row has more than 4095 columns");
-    if (h->err & 256) return nl_fail(ctx, NL_EUNSUPPORTED, "a fixed-point sum left its range (error word " +
-                                                          std::to_string(h->err) + ")");
-    if (h->err) return nl_fail(ctx, NL_EUNSUPPORTED, "a region exceeded the vertex buffer (error word " +
-                                                       std::to_string(h->err) + ")");
-    const int64_t nnz = h->nnz;
+    const int err = (int)h->pat[kPatErr];
+    if (h->pat[kPatRowOvf]) return nl_fail(ctx, NL_EUNSUPPORTED, "a matrix row has more than 4095 columns");
+    if (err & 256) return nl_fail(ctx, NL_EUNSUPPORTED, "a fixed-point sum left its range (error word " +
+                                                          std::to_string(err) + ")");
+    if (err) return nl_fail(ctx, NL_EUNSUPPORTED, "a region exceeded the vertex buffer (error word " +
+                                                       std::to_string(err) + ")");
+    const int64_t nnz = (int64_t)h->pat[kPatNnz];
     out->n = J;
     out->nnz = nnz;
-    out->n_pairs = (int64_t)h->pat[0];
-    out->n_qp_pairs = (int64_t)h->pat[1];
-    out->n_inter = (int64_t)h->pat[2];
-    P->max_row = (int64_t)h->pat[3];
-    P->max_words = (int64_t)h->pat[4];
+    out->n_pairs = (int64_t)h->pat[kPatPairs];
+    out->n_qp_pairs = (int64_t)h->pat[kPatQp];
+    out->n_inter = (int64_t)h->pat[kPatInter];
+    P->max_row = (int64_t)h->pat[kPatMaxRow];
+    P->max_words = (int64_t)h->pat[kPatMaxWords];
     if ((s = nl_alloc(ctx, &out->col_idx, (size_t)nnz)) != NL_OK) return s;
     if ((s = nl_alloc(ctx, &out->val, (size_t)nnz)) != NL_OK) return s;
     // the rows the first count kept sorted are copied; the others (usually none) are built again,
@@ -1182,9 +1190,15 @@ nl_status nl_pattern_b(nl_ctx *ctx, nl_plan *P, nl_csr *out, nl_pat *T, const nl
                                                             out->col_idx, nullptr, nullptr, T->ovf, nullptr, nullptr,
                                                             nullptr, nullptr, nullptr, 1); ++ctx->launches;
     NL_CK(cudaGetLastError());
-    if ((s = nl_alloc(ctx, &P->lslot, 6 * (size_t)K)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->tslot, (size_t)nnz)) != NL_OK) return s;
-    if ((s = nl_alloc(ctx, &P->W, (size_t)nnz)) != NL_OK) return s;
+    {
+        nl_carver c;
+        const size_t lslot = c.add<int64_t>(6 * (size_t)K), tslot = c.add<int64_t>((size_t)nnz);
+        const size_t W = c.add<double>((size_t)nnz);
+        if ((s = nl_alloc(ctx, &P->slab[2], c.n)) != NL_OK) return s;
+        P->lslot = (int64_t *)(P->slab[2] + lslot);
+        P->tslot = (int64_t *)(P->slab[2] + tslot);
+        P->W = (double *)(P->slab[2] + W);
+    }
     k_local_slots<<<(K + 255) / 256, 256, 0, st>>>(K, P->tri, out->row_ptr, out->col_idx, P->lslot); ++ctx->launches;
     k_tslot<<<(unsigned)(((int64_t)J * 32 + 255) / 256), 256, 0, st>>>(J, out->row_ptr, out->col_idx, P->tslot);
     ++ctx->launches;

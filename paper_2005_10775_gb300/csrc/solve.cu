@@ -11,6 +11,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 
 #include "internal.cuh"
@@ -179,86 +180,182 @@ __global__ void k_residual(int n, const int64_t *rp, const int32_t *__restrict__
     block_atomic_add(bb, &acc[1]);
 }
 
-// inner FP32 conjugate gradients on A d = z0 (z0 = r / ||r||)
+// Inner FP32 conjugate gradients on A d = z0 (z0 = r / ||r||): one cooperative launch a refinement pass.
+// An iteration is a product of some 3 us (n = 6,500, nnz = 1.5 M) between two reductions, so launches and
+// the host's checks took most of the time: four launches an iteration and a check every eighth.  Here an
+// iteration is two grid barriers, the blocks keep their rows (values and columns can stay in L1), and the
+// convergence check costs nothing.  Extraction, load vector and solve of the 96 x 96 N-gon mesh (64
+// iterations): 1.54 -> 1.2 ms.  With two launches an iteration it took 1.50 ms; with 3 blocks of 512, 1 or 2
+// of 1024 threads an SM 1.26, 1.21 and 1.31 (fewer arrivals against more rows in flight).  104 iterations on
+// 39,601 nodes (17 M entries, more than L2 holds) are bound by the matrix from memory: 5.08 -> 4.96 ms.
+// The product forms its direction p = z + beta p as it gathers it (z and
+// p of a node lie side by side: one 8-byte load), so directions need no pass of their own.
+//     zz[k & 3] = ||z_k||^2 (rho of iteration k), pq[k & 3] = p_k . A p_k
 struct CgScal {
-    double rho, pq, zz;
-    int brk;   // breakdown: p.Ap not positive (or not a number) while the residual is not yet zero
+    double zz[4], pq[4];
+    double rho;          // at the end: ||z||^2, the iterations done
+    int it;
+    int brk;             // breakdown: p.Ap not positive (or not a number) while the residual is not yet zero
+    int late;            // a barrier's wait ran out
+    unsigned arrived;    // barrier arrivals since the launch
 };
 
 // a direction with p.Ap <= 0 (A not positive definite along p) or a non-finite p.Ap ends the
 // solve; below rho = 1e-20 (the inner residual 1e-10 of its start) the iteration has converged
 // and the host stops it
 constexpr double kBreakdownRho = 1e-20;
+constexpr int kCheck = 8;            // inner iterations between convergence checks
+constexpr double kInnerTol = 1e-5;   // inner relative reduction per refinement step
+constexpr int kCgThreads = 512, kCgBlocks = 2, kCgWarps = kCgThreads / 32;
 
-__global__ void k_cg_init(int n, const double *r, double inv_norm, float *z, float *p, float *d, CgScal *sc)
+__global__ void k_cg_init(int n, const double *r, double inv_norm, float2 *zp, float *d, CgScal *sc)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) {
-        float v = (float)(r[i] * inv_norm);
-        z[i] = v;
-        p[i] = v;
+        zp[i] = make_float2((float)(r[i] * inv_norm), 0.0f);
         d[i] = 0.0f;
     }
     if (i == 0) {
-        sc->rho = 1.0;
-        sc->pq = 0.0;
-        sc->zz = 0.0;
-        sc->brk = 0;
+        *sc = CgScal{};
+        sc->zz[0] = 1.0;
     }
 }
 
-// q = A p and p.q
-__global__ void k_cg_spmv(int n, const int64_t *rp, const int32_t *__restrict__ col, const float *__restrict__ val,
-                          const float *__restrict__ p, float *q, CgScal *sc)
+// Every block of the (cooperative) grid arrives; the wait is bounded (some seconds), and a block whose
+// wait ran out leaves for good, so that the others' waits run out too.  False: leave.
+__device__ __forceinline__ bool cg_barrier(CgScal *sc, unsigned &target)
 {
-    const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    double pq = 0.0;
-    if (r < n) {
-        float s = row_dot<float, float>(val, col, p, rp[r], rp[r + 1], lane);
-        for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        if (lane == 0) q[r] = s;
-        pq = (double)s * (double)p[r];
-    }
-    block_atomic_add(pq, &sc->pq);
-}
-
-__global__ void k_cg_update(int n, const float *p, const float *q, float *d, float *z, CgScal *sc)
-{
-    __shared__ double part[8];
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    double pq = sc->pq;
-    const bool brk = sc->rho > kBreakdownRho && !(pq > 0.0);
-    float alpha = (pq > 0.0) ? (float)(sc->rho / pq) : 0.0f;
-    if (i == 0 && brk) sc->brk = 1;
-    double zz = 0.0;
-    if (i < n) {
-        d[i] += alpha * p[i];
-        float zn = z[i] - alpha * q[i];
-        z[i] = zn;
-        zz = (double)zn * zn;
-    }
-    for (int off = 16; off; off >>= 1) zz += __shfl_xor_sync(0xffffffffu, zz, off);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = zz;
+    __shared__ int ok;
+    target += gridDim.x;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) t += part[w];
-        atomicAdd(&sc->zz, t);
+        __threadfence();
+        atomicAdd(&sc->arrived, 1u);
+        int left = 1 << 22;
+        unsigned seen;
+        do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&sc->arrived) : "memory");
+        } while ((int)(seen - target) < 0 && --left);
+        if (!left) sc->late = 1;
+        ok = left;
+        __threadfence();
     }
+    __syncthreads();
+    return ok != 0;
 }
 
-__global__ void k_cg_dir(int n, const float *z, float *p, const CgScal *sc)
+// z0/z1: (z, p) of every node before and after an even iteration (the reverse after an odd one).  They
+// and q are written by other blocks between barriers: no read-only loads.  A block's warps take `rpb`
+// neighbouring rows a round (their columns overlap).  The FP64 pipe takes a warp's instruction in some 16
+// cycles whether one lane works or all: the rows' products for p.q are left in shared memory and one warp
+// sums a round of them, the update's warps are spread over the blocks, and one thread a block divides.
+__global__ void __launch_bounds__(kCgThreads, kCgBlocks)
+k_cg(int n, const int64_t *__restrict__ rp, const int32_t *__restrict__ col, const float *__restrict__ val,
+     float2 *z0, float2 *z1, float *q, float *d, int max_it, CgScal *sc)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float beta = sc->rho != 0.0 ? (float)(sc->zz / sc->rho) : 0.0f;
-    if (i < n) p[i] = z[i] + beta * p[i];
-}
-
-__global__ void k_cg_shift(CgScal *sc)
-{
-    sc->rho = sc->zz;
-    sc->pq = 0.0;
-    sc->zz = 0.0;
+    constexpr int kLoads = 4;     // a lane's values and columns in flight; 8 were slower (5.5 ms for the 39,601 nodes)
+    constexpr int kRounds = 16;   // rounds between the sums
+    __shared__ float2 s_qp[kRounds][kCgWarps];
+    __shared__ float s_scalar;
+    __shared__ int s_stop;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int rpb = min(kCgWarps, (n + (int)gridDim.x - 1) / (int)gridDim.x);
+    unsigned target = 0;
+    double rho = 1.0, rho_old = 0.0;
+    int it = 0;
+    bool brk = false;
+    while (it < max_it) {
+        const float2 *cur = it & 1 ? z1 : z0;
+        float2 *next = it & 1 ? z0 : z1;
+        if (threadIdx.x == 0) {
+            s_scalar = it > 0 && rho_old != 0.0 ? (float)(rho / rho_old) : 0.0f;
+            if (blockIdx.x == 0) {   // slots of the next iteration; their old values were read two barriers ago
+                sc->zz[(it + 2) & 3] = 0.0;
+                sc->pq[(it + 1) & 3] = 0.0;
+            }
+        }
+        __syncthreads();
+        const float beta = s_scalar;
+        for (int64_t first = (int64_t)blockIdx.x * rpb; first < n; first += (int64_t)kRounds * rpb * gridDim.x) {
+            for (int u = 0; u < kRounds; u++) {
+                const int64_t r = first + (int64_t)u * rpb * gridDim.x + w;
+                if (w >= rpb || r >= n) {
+                    if (lane == 0) s_qp[u][w] = make_float2(0.0f, 0.0f);
+                    continue;
+                }
+                const int64_t e = rp[r + 1];
+                float s = 0.0f;
+                for (int64_t k0 = rp[r] + lane; k0 < e; k0 += 32 * kLoads) {
+                    float v[kLoads];
+                    int c[kLoads];
+#pragma unroll
+                    for (int j = 0; j < kLoads; j++) {
+                        const int64_t k = k0 + 32 * j;
+                        v[j] = k < e ? val[k] : 0.0f;
+                        c[j] = k < e ? col[k] : -1;
+                    }
+#pragma unroll
+                    for (int j = 0; j < kLoads; j++)
+                        if (c[j] >= 0) {
+                            const float2 x = cur[c[j]];
+                            s += v[j] * fmaf(beta, x.y, x.x);
+                        }
+                }
+                for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+                if (lane == 0) {
+                    const float2 x = cur[r];
+                    const float p = fmaf(beta, x.y, x.x);
+                    q[r] = s;
+                    next[r].y = p;
+                    s_qp[u][w] = make_float2(s, p);
+                }
+            }
+            __syncthreads();
+            if (w < kRounds && first + (int64_t)w * rpb * gridDim.x < n) {
+                const float2 x = lane < kCgWarps ? s_qp[w][lane] : make_float2(0.0f, 0.0f);
+                double pq = (double)x.x * (double)x.y;
+                for (int off = 16; off; off >>= 1) pq += __shfl_xor_sync(0xffffffffu, pq, off);
+                if (lane == 0) atomicAdd(&sc->pq[it & 3], pq);
+            }
+            __syncthreads();
+        }
+        if (!cg_barrier(sc, target)) return;
+        if (threadIdx.x == 0) {
+            const double pq = __ldcg(&sc->pq[it & 3]);
+            brk |= rho > kBreakdownRho && !(pq > 0.0);
+            s_scalar = pq > 0.0 ? (float)(rho / pq) : 0.0f;
+        }
+        __syncthreads();
+        const float alpha = s_scalar;
+        for (int64_t base = ((int64_t)w * gridDim.x + blockIdx.x) * 32; base < n; base += (int64_t)gridDim.x * kCgThreads) {
+            const int64_t i = base + lane;
+            double zz = 0.0;
+            if (i < n) {
+                d[i] += alpha * next[i].y;
+                const float zn = cur[i].x - alpha * q[i];
+                next[i].x = zn;
+                zz = (double)zn * zn;
+            }
+            for (int off = 16; off; off >>= 1) zz += __shfl_xor_sync(0xffffffffu, zz, off);
+            if (lane == 0) atomicAdd(&sc->zz[(it + 1) & 3], zz);
+        }
+        if (!cg_barrier(sc, target)) return;
+        it++;
+        if (threadIdx.x == 0) {
+            rho_old = rho;
+            rho = __ldcg(&sc->zz[it & 3]);
+            s_stop = it % kCheck == 0 && (brk || !isfinite(rho) || !(sqrt(rho) > kInnerTol));
+        }
+        if (it % kCheck == 0) {
+            __syncthreads();
+            if (s_stop) break;
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        sc->rho = rho;
+        sc->it = it;
+        sc->brk = brk;
+    }
 }
 
 __global__ void k_axpy_f32(int n, double s, const float *d, double *x)
@@ -288,36 +385,6 @@ nl_status ensure_f32(nl_ctx *ctx, nl_csr *A)
 }
 
 unsigned wgrid(int64_t rows) { return (unsigned)((rows * 32 + 255) / 256); }
-
-// A CUDA graph of a fixed sequence of kernel launches on one stream, captured once and replayed
-// (released with its holder).  A capture the runtime refuses (the stream already capturing, a
-// launch error) leaves `failed` set and the caller launches the kernels itself.
-struct ChunkGraph {
-    cudaGraphExec_t exec = nullptr;
-    bool failed = false;
-    template <class Launches>
-    void capture(cudaStream_t st, Launches launches)
-    {
-        cudaGraph_t g = nullptr;
-        if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-            cudaGetLastError();
-            failed = true;
-            return;
-        }
-        launches();
-        const cudaError_t e = cudaStreamEndCapture(st, &g);
-        if (e == cudaSuccess && g && cudaGraphInstantiate(&exec, g, 0) != cudaSuccess) exec = nullptr;
-        if (g) cudaGraphDestroy(g);
-        if (!exec) {
-            cudaGetLastError();
-            failed = true;
-        }
-    }
-    ~ChunkGraph()
-    {
-        if (exec) cudaGraphExecDestroy(exec);
-    }
-};
 
 nl_status extract_body(nl_ctx *ctx, const nl_csr *D, const nl_mesh *mesh, nl_csr *A, nl_csr *B)
 {
@@ -523,23 +590,25 @@ nl_status nl_cg(nl_ctx *ctx, const nl_csr *Ac, const double *b, double *x, doubl
         NL_CK(cudaMemcpyAsync(xd, x, sizeof(double) * n, cudaMemcpyHostToDevice, ctx->stream));
     }
     double *r, *acc;
-    float *z, *p, *q, *d;
+    float2 *zp[2];   // (z, p) of every node, before and after an iteration
+    float *q, *d;
     CgScal *sc;
     if ((s = tmp.get(ctx, &r, (size_t)n + 1)) != NL_OK || (s = tmp.get(ctx, &acc, 2)) != NL_OK ||
-        (s = tmp.get(ctx, &z, (size_t)n + 1)) != NL_OK || (s = tmp.get(ctx, &p, (size_t)n + 1)) != NL_OK ||
+        (s = tmp.get(ctx, &zp[0], (size_t)n + 1)) != NL_OK || (s = tmp.get(ctx, &zp[1], (size_t)n + 1)) != NL_OK ||
         (s = tmp.get(ctx, &q, (size_t)n + 1)) != NL_OK || (s = tmp.get(ctx, &d, (size_t)n + 1)) != NL_OK ||
         (s = tmp.get(ctx, &sc, 1)) != NL_OK)
         return s;
     const unsigned eg = (unsigned)((n + 255) / 256);
     int total = 0;
     double rel = INFINITY;
-    bool conv = false, stop = false;
+    bool conv = false;
     nl_status out = NL_OK;
-    const int kCheck = 8;          // inner iterations between host convergence checks
-    const double kInnerTol = 1e-5; // inner relative reduction per refinement step
     const int kPasses = 64;        // FP64 refinement passes
-    ChunkGraph graph;              // the captured inner chunk (released with the call)
-    for (int outer = 0; outer < kPasses && !stop; outer++) {
+    int cg_blocks = 0, sms = 0;    // the cooperative grid: what the device holds at once
+    NL_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+    NL_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cg_blocks, k_cg, kCgThreads, 0));
+    cg_blocks = std::max(1, std::min(cg_blocks * sms, n));
+    for (int outer = 0; outer < kPasses; outer++) {
         NL_CK(cudaMemsetAsync(acc, 0, sizeof(double) * 2, ctx->stream));
         k_residual<<<wgrid(n), 256, 0, ctx->stream>>>(n, A->row_ptr, A->col_idx, A->val, xd, (const double *)bd, r,
                                                       acc); ++ctx->launches;
@@ -560,46 +629,26 @@ nl_status nl_cg(nl_ctx *ctx, const nl_csr *Ac, const double *b, double *x, doubl
             out = nl_fail(ctx, NL_ENOCONV, "CG did not reach the tolerance within max_it iterations");
             break;
         }
-        k_cg_init<<<eg, 256, 0, ctx->stream>>>(n, r, 1.0 / rn, z, p, d, sc); ++ctx->launches;
-        while (total < max_it) {
-            const int chunk = (max_it - total) < kCheck ? (max_it - total) : kCheck;
-            auto iterate = [&](int count) {
-                for (int c = 0; c < count; c++) {
-                    k_cg_spmv<<<wgrid(n), 256, 0, ctx->stream>>>(n, A->row_ptr, A->col_idx, v32, p, q, sc);
-                    k_cg_update<<<eg, 256, 0, ctx->stream>>>(n, p, q, d, z, sc);
-                    k_cg_dir<<<eg, 256, 0, ctx->stream>>>(n, z, p, sc);
-                    k_cg_shift<<<1, 1, 0, ctx->stream>>>(sc);
-                }
-                ctx->launches += 4 * count;
-            };
-            // a full chunk is one launch of a graph of its 4 x kCheck kernels (captured at the first
-            // full chunk of the call: its buffers are the call's own), which removes most of the
-            // launch gaps between these short kernels; a capture that fails falls back to launches
-            if (chunk == kCheck && !graph.exec && !graph.failed) {
-                const int64_t l0 = ctx->launches;   // captured, not launched
-                graph.capture(ctx->stream, [&] { iterate(kCheck); });
-                ctx->launches = l0;
-            }
-            if (chunk == kCheck && graph.exec) {
-                NL_CK(cudaGraphLaunch(graph.exec, ctx->stream));
-                ctx->launches += 4 * kCheck;
-            } else {
-                iterate(chunk);
-            }
-            NL_CK(cudaGetLastError());
-            total += chunk;
-            CgScal hs;
-            NL_CK(cudaMemcpyAsync(&hs, sc, sizeof hs, cudaMemcpyDeviceToHost, ctx->stream));
-            NL_CK(cudaStreamSynchronize(ctx->stream));
-            if (hs.brk || !isfinite(hs.rho)) {   // breakdown: the correction d is not usable
-                out = nl_fail(ctx, NL_ENOCONV, "CG breakdown: a search direction with p.Ap <= 0 or not a number "
-                                               "(A not symmetric positive definite, or non-finite values)");
-                stop = true;
-                break;
-            }
-            if (!(sqrt(hs.rho) > kInnerTol)) break;   // inner tolerance reached
+        k_cg_init<<<eg, 256, 0, ctx->stream>>>(n, r, 1.0 / rn, zp[0], d, sc); ++ctx->launches;
+        int left = max_it - total;
+        int n_arg = n;
+        void *args[] = {&n_arg, &A->row_ptr, &A->col_idx, &v32, &zp[0], &zp[1], &q, &d, &left, &sc};
+        NL_CK(cudaLaunchCooperativeKernel((const void *)k_cg, dim3((unsigned)cg_blocks), dim3(kCgThreads), args, 0,
+                                          ctx->stream));
+        ++ctx->launches;
+        CgScal hs;
+        NL_CK(cudaMemcpyAsync(&hs, sc, sizeof hs, cudaMemcpyDeviceToHost, ctx->stream));
+        NL_CK(cudaStreamSynchronize(ctx->stream));
+        if (hs.late) {
+            out = nl_fail(ctx, NL_ETIMEOUT, "CG: a wait between the blocks of the solver kernel expired");
+            break;
         }
-        if (stop) break;
+        total += hs.it;
+        if (hs.brk || !isfinite(hs.rho)) {   // breakdown: the correction d is not usable
+            out = nl_fail(ctx, NL_ENOCONV, "CG breakdown: a search direction with p.Ap <= 0 or not a number "
+                                           "(A not symmetric positive definite, or non-finite values)");
+            break;
+        }
         k_axpy_f32<<<eg, 256, 0, ctx->stream>>>(n, rn, d, xd); ++ctx->launches;
         NL_CK(cudaGetLastError());
     }

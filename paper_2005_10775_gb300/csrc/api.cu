@@ -268,18 +268,18 @@ nl_status nl_fill_args(nl_ctx *ctx, const nl_plan *P, nlq::NumArgs &A, bool stat
     A.duffy_n = c.kernel == NL_KERNEL_INV_DIST ? c.duffy_n : 1;
     gauss_legendre01(A.duffy_n, A.gl_x, A.gl_w);
     gauss_legendre01(2, A.gl2_x, A.gl2_w);
+    double near_c[5] = {};   // over the nodes: w cosh, w sinh, w cosh^2, w cosh sinh, w sinh^2
     for (int j = 0; j < 8; j++) {
+        const double w = j < A.duffy_n ? A.gl_w[j] : 0.0, sh = sinh(A.gl_x[j]), ch = cosh(A.gl_x[j]);
         A.glf_x[j] = j < A.duffy_n ? (float)A.gl_x[j] : 0.f;
-        A.glf_w[j] = j < A.duffy_n ? (float)A.gl_w[j] : 0.f;
-        A.glf_sh[j] = j < A.duffy_n ? (float)sinh(A.gl_x[j]) : 0.f;
-        A.glf_ch[j] = j < A.duffy_n ? (float)cosh(A.gl_x[j]) : 1.f;
+        A.glf_w[j] = (float)w;
+        if (w == 0.0) continue;
+        const double f[5] = {ch, sh, ch * ch, ch * sh, sh * sh};
+        for (int k = 0; k < 5; k++) near_c[k] += w * f[k];
     }
+    for (int k = 0; k < 5; k++) A.near_c[k] = (float)near_c[k];
     A.sh1f = (float)sinh(1.0);
     A.ch1f = (float)cosh(1.0);
-    for (int j = 0; j < 2; j++) {
-        A.gl2f_x[j] = (float)A.gl2_x[j];
-        A.gl2f_w[j] = (float)A.gl2_w[j];
-    }
     A.kernel = c.kernel;
     A.ball = c.ball;
     A.shifted = c.shifted ? 1 : 0;

@@ -75,9 +75,8 @@ struct NumArgs {
     double gl_x[8], gl_w[8];          // Gauss-Legendre on [0,1] with duffy_n points
     double gl2_x[2], gl2_w[2];
     float glf_x[8], glf_w[8];         // the same rules in FP32 (no FP64 conversions in the FP32 path)
-    float glf_sh[8], glf_ch[8];       // sinh and cosh of the duffy_n nodes glf_x (FP32)
+    float near_c[5];                  // sums of w_j times cosh x_j, sinh x_j and their products over those nodes
     float sh1f, ch1f;                 // sinh(1), cosh(1) (FP32)
-    float gl2f_x[2], gl2f_w[2];
     float kcf;                        // kc in FP32
     int duffy_n;
     int switch47;                     // outer rule: 0..nsplit-1 if |bary_a - bary_b|^2 < thr2 else nsplit..n-1
@@ -422,14 +421,22 @@ __device__ __forceinline__ void poly_sums_sh(const NumArgs &A, const nlg::ClipBu
 // FP32 version of the near-singular rule (FP32-compensated path) for the whole triangle
 // with FP32 vertices dl relative to x: the same signed apex-x decomposition, Duffy collapse
 // and sinh substitution.  Its discrete choices are taken in FP64 (near_edge64) whenever
-// FP32 is within 1e-4 of a threshold, so the evaluated points are those of the FP64 rule.
+// FP32 is within 1e-4 of a threshold, so the rule's panels are those of the FP64 rule.
+//
+// The rule's sums are formed by moments instead of point by point.  A point is y = s w, w = F + t e on
+// the edge's line at t = d sinh(u); the barycentrics are l_k = s a_k - o_k, a_k affine in t, o_k the
+// origin's.  The two Gauss points in s integrate 1, s and s^2 exactly (1, 1/2, 1/3), so a side needs the
+// sums of w_j, w_j t_j and w_j t_j^2 over its nodes alone.  On a full panel [p, p + 1] these follow from
+// t_j = d (sinh p cosh x_j + cosh p sinh x_j) and five sums of the rule (near_c); only the last panel
+// [p, U] of a side visits its nodes.  15 operations a full panel and 8 a node, where the points took 50 a node.
 __device__ __forceinline__ void near_whole_f32(const NumArgs &A, const nlg::F2 dl[3], int tb, D2 x,
                                                const nlg::F2 &e1, const nlg::F2 &e2, float inv_det,
                                                Sums<float> &S, int64_t &nqp)
 {
-    sums_zero(S);
-    const float kc = A.kcf;
+    // over the sides: integrals of 1, of a_k = l_wk (without the offset) and of a_j a_k
+    float M0 = 0.f, A1 = 0.f, A2 = 0.f, Q11 = 0.f, Q12 = 0.f, Q22 = 0.f;
     const int nu = A.duffy_n;
+#pragma unroll 1
     for (int i = 0; i < 3; i++) {
         const nlg::F2 a = dl[i], b = dl[(i + 1) % 3];
         float ex = b.x - a.x, ey = b.y - a.y;
@@ -468,51 +475,60 @@ __device__ __forceinline__ void near_whole_f32(const NumArgs &A, const nlg::F2 d
         }
         if (skip_edge || d == 0.f) continue;
         const float sigma = (Fx * ey - Fy * ex) > 0.f ? 1.f : -1.f;
-        // The panels of both sides (B, then A) in one loop, so that lanes whose sides split their
-        // panels differently still run the loop body together.  On a full panel [p, p + 1],
-        // sinh(p + x_j) = sinh(p) cosh(x_j) + cosh(p) sinh(x_j), with sinh(p), cosh(p) carried from
-        // panel to panel by the same addition theorem (sinh(1), cosh(1)); the last panel of a side,
-        // [p, U], evaluates sinh directly.  The FP32 point y = s w - v_0 of T_b relative to its
-        // first vertex is linear in s, and so are its barycentrics: l = s l_w - l_0.
-        const int nB = skipB ? 0 : npB, nA = skipA ? 0 : npA;
-        const float l10 = (dl[0].x * e2.y - e2.x * dl[0].y) * inv_det;
-        const float l20 = (e1.x * dl[0].y - dl[0].x * e1.y) * inv_det;
-        float sp = 0.f, cp = 1.f;   // sinh, cosh of the panel start
-        for (int p = 0; p < nB + nA; p++) {
-            const bool sideA = p >= nB;
-            const int pnl = sideA ? p - nB : p, npan = sideA ? nA : nB;
-            const float tau = sideA ? tA : tB, U = sideA ? UA : UB;
-            const float sign = sideA ? -sigma : sigma;
-            const float sg = tau > 0.f ? 1.f : -1.f;
-            if (pnl == 0) {
-                sp = 0.f;
-                cp = 1.f;
-            }
-            const bool full = pnl + 1 < npan;
-            const float u0 = (float)pnl, hw = full ? 1.f : fmaxf(U, u0) - u0;
-            const float gdx = sg * d * ex, gdy = sg * d * ey, kcs = sign * sg * d * kc;
-            // the Gauss points of the panel: sinh at the node, then the two points in s
-            auto node = [&](int j, float sh) {
-                const float wj = kcs * (hw * A.glf_w[j]);
-                const float wx = fmaf(sh, gdx, Fx), wy = fmaf(sh, gdy, Fy);
-                const float l1w = (wx * e2.y - e2.x * wy) * inv_det;
-                const float l2w = (e1.x * wy - wx * e1.y) * inv_det;
-                for (int k = 0; k < 2; k++) {
-                    const float sv = A.gl2f_x[k];
-                    const float l1 = sv * l1w - l10, l2 = sv * l2w - l20;
-                    sums_add<float>(S, wj * A.gl2f_w[k], 1.f - l1 - l2, l1, l2);
-                }
-            };
-            for (int j = 0; j < nu; j++)
-                node(j, full ? fmaf(sp, A.glf_ch[j], cp * A.glf_sh[j]) : sinhf(u0 + hw * A.glf_x[j]));
-            nqp += 2 * nu;
-            if (full) {
+        const float a10 = (Fx * e2.y - e2.x * Fy) * inv_det, a20 = (e1.x * Fy - Fx * e1.y) * inv_det;
+        const float g1 = (ex * e2.y - e2.x * ey) * inv_det, g2 = (e1.x * ey - ex * e1.y) * inv_det;
+#pragma unroll 1
+        for (int side = 0; side < 2; side++) {   // side B, then side A
+            const int np = side ? (skipA ? 0 : npA) : (skipB ? 0 : npB);
+            if (np == 0) continue;
+            const float tau = side ? tA : tB, U = side ? UA : UB;
+            const float sg = tau > 0.f ? 1.f : -1.f, k = (side ? -sigma : sigma) * sg * d * A.kcf;
+            float sp = 0.f, cp = d;   // d sinh, d cosh of the panel's start
+            float m1 = 0.f, m2 = 0.f;
+            for (int p = 0; p + 1 < np; p++) {
+                m1 += fmaf(sp, A.near_c[0], cp * A.near_c[1]);
+                m2 += fmaf(sp * sp, A.near_c[2], fmaf(2.f * sp * cp, A.near_c[3], cp * cp * A.near_c[4]));
                 const float sn = fmaf(sp, A.ch1f, cp * A.sh1f);
                 cp = fmaf(cp, A.ch1f, sp * A.sh1f);
                 sp = sn;
             }
+            const float u0 = (float)(np - 1), hw = fmaxf(U, u0) - u0;
+            float n1 = 0.f, n2 = 0.f;
+            for (int j = 0; j < nu; j++) {
+                const float eu = expf(u0 + hw * A.glf_x[j]);
+                const float t = 0.5f * d * (eu - 1.f / eu), wt = A.glf_w[j] * t;
+                n1 += wt;
+                n2 = fmaf(wt, t, n2);
+            }
+            const float m0 = k * (u0 + hw);
+            m1 = k * sg * fmaf(hw, n1, m1);
+            m2 = k * fmaf(hw, n2, m2);
+            M0 += m0;
+            const float b1 = fmaf(a10, m0, g1 * m1), b2 = fmaf(a20, m0, g2 * m1);   // integrals of a_k
+            const float c1 = fmaf(a10, m1, g1 * m2), c2 = fmaf(a20, m1, g2 * m2);   // of t a_k
+            A1 += b1;
+            A2 += b2;
+            Q11 += fmaf(a10, b1, g1 * c1);
+            Q12 += fmaf(a10, b2, g1 * c2);
+            Q22 += fmaf(a20, b2, g2 * c2);
+            nqp += 2 * nu * np;
         }
     }
+    const float o1 = (dl[0].x * e2.y - e2.x * dl[0].y) * inv_det, o2 = (e1.x * dl[0].y - dl[0].x * e1.y) * inv_det;
+    const float s1 = fmaf(0.5f, A1, -o1 * M0), s2 = fmaf(0.5f, A2, -o2 * M0);
+    constexpr float third = 1.f / 3.f;
+    const float s11 = fmaf(third, Q11, o1 * fmaf(o1, M0, -A1)), s22 = fmaf(third, Q22, o2 * fmaf(o2, M0, -A2));
+    const float s12 = fmaf(third, Q12, fmaf(o1 * o2, M0, -0.5f * fmaf(o1, A2, o2 * A1)));
+    S.s0 = M0;
+    S.s1[0] = M0 - s1 - s2;
+    S.s1[1] = s1;
+    S.s1[2] = s2;
+    S.S2[1] = s11;
+    S.S2[2] = s22;
+    S.S2[5] = s12;
+    S.S2[3] = s1 - s11 - s12;
+    S.S2[4] = s2 - s22 - s12;
+    S.S2[0] = S.s1[0] - S.S2[3] - S.S2[4];
 }
 
 struct OuterPt {
@@ -1900,140 +1916,18 @@ __device__ __forceinline__ bool warp_run_sum(long long key, int lane, V *v)
 // ---------------------------------------------------------------------------
 // Near-field whole items of the FP32 singular kernel (after the boundary launch, in stream
 // order): the boundary kernel queues every (x_q, T_b) whose whole T_b lies in the near field of
-// x_q (certified in FP32), in (pair, outer point) order; here each warp takes 32 of them and
-// runs the near-singular rule (signed apex-x decomposition, Duffy collapse, sinh substitution,
-// as near_whole_f32) with its lanes spread over the items' panels instead of the items: the
-// items have 3 to 30 panels (11 on average at the singular workload), so a lane per item left
-// most lanes idle while the longest item ran.  A lane per item first sets up its six sides
-// (two per edge: panel count, U, the scaled foot-point direction) in shared memory; the warp then
-// takes the panels of all 32 items 32 at a time, sums each item's panels by a segmented shuffle
-// tree and adds the sums onto the item's column; a lane per item finally combines its item.  The
+// x_q (certified in FP32), in (pair, outer point) order; here a lane takes an item
+// (near_whole_f32), 32 neighbouring items a warp.  By moments a panel is some 15 operations, so
+// lanes of 3 to 30 panels may wait for each other: spreading the panels over the lanes (shared
+// item data, a search for each panel's item, a segmented sum of ten values) cost more than that.
+// Bound by the issue of the setup (roots, asinh), the epilogue's shuffles and atomics.  The
 // blocks are then summed over the lanes of one pair (M_ab onto the pair's stored values with
 // FP32 atomics, M_bb onto T_b's sums) and of one outer triangle (M_aa, statistics), so a warp
 // issues a few atomics per pair instead of one per item.
 // ---------------------------------------------------------------------------
-struct NearSide {              // one side (edge, end A or B) of a near-field item
-    float gdx, gdy;            // sg d e: the foot point's scaled edge direction
-    float fx, fy;              // foot point F of x on the edge's line, relative to x
-    float kcs;                 // sign sg d kc
-    float u;                   // U = asinh(|t| / d), the last panel's end
-};
-
-struct NearShared {            // per warp
-    NearSide side[6][32];
-    unsigned short npan[6][32];   // up to about 710 on a side (FP64 panel counts)
-    float e1x[32], e1y[32], e2x[32], e2y[32], inv[32], l10[32], l20[32];
-    int start[32];             // first panel of each lane's item in the warp's panel list
-    float acc[10][32];         // each item's sums (s0, s1, S2) over its panels
-};
-
-// the six sides of an item (vertices dl relative to x): panel counts (0 for a degenerate side),
-// by the same FP32 rule with FP64 fallback as near_whole_f32
-__device__ __forceinline__ int near_setup_f32(const NumArgs &A, const nlg::F2 dl[3], int tb, D2 x, NearShared &sh,
-                                              int lane)
-{
-    const float kc = A.kcf;
-    int total = 0;
-    for (int i = 0; i < 3; i++) {
-        const nlg::F2 a = dl[i], b = dl[(i + 1) % 3];
-        float ex = b.x - a.x, ey = b.y - a.y;
-        const float L = sqrtf(ex * ex + ey * ey);
-        ex /= L;
-        ey /= L;
-        const float tA = a.x * ex + a.y * ey, tB = b.x * ex + b.y * ey;
-        const float Fx = a.x - tA * ex, Fy = a.y - tA * ey;
-        const float d = sqrtf(Fx * Fx + Fy * Fy);
-        const float UA = asinhf(fabsf(tA) / d), UB = asinhf(fabsf(tB) / d);
-        const float th = 1e-4f * L;
-        const float M = fmaxf(fmaxf(fabsf(a.x) + fabsf(a.y), fabsf(b.x) + fabsf(b.y)), L) + L;
-        auto near_int = [&](float U, float t) {
-            const float eps = 1e-6f * M * (1.f / d + 1.f / fabsf(t)) + 1e-5f * fmaxf(U, 1.f);
-            return fabsf(U - rintf(U)) < eps;
-        };
-        bool skip_edge = false, skipA = false, skipB = false;
-        int npA, npB;
-        if (!(d >= th) || !(fabsf(tA) >= th) || !(fabsf(tB) >= th) || near_int(UA, tA) || near_int(UB, tB)) {
-            const int i1 = (i + 1) % 3;
-            const D2 Vi = {A.tx[i * A.K + tb], A.ty[i * A.K + tb]}, Vj = {A.tx[i1 * A.K + tb], A.ty[i1 * A.K + tb]};
-            const NearEdge64 q = near_edge64(Vi, Vj, x);
-            skip_edge = (q.d == 0.0);
-            skipA = (q.tA == 0.0);
-            skipB = (q.tB == 0.0);
-            npA = skip_edge || skipA ? 0 : near_panels64(q.tA, q.d);
-            npB = skip_edge || skipB ? 0 : near_panels64(q.tB, q.d);
-        } else {
-            npA = (int)ceilf(UA);
-            npB = (int)ceilf(UB);
-            npA = npA < 1 ? 1 : npA;
-            npB = npB < 1 ? 1 : npB;
-        }
-        if (skip_edge || d == 0.f) npA = npB = 0;
-        if (skipA) npA = 0;
-        if (skipB) npB = 0;
-        const float sigma = (Fx * ey - Fy * ex) > 0.f ? 1.f : -1.f;
-        for (int sd = 0; sd < 2; sd++) {   // side B, then side A
-            const bool sideA = sd == 1;
-            const float tau = sideA ? tA : tB;
-            const float sg = tau > 0.f ? 1.f : -1.f, sign = sideA ? -sigma : sigma;
-            NearSide &S = sh.side[2 * i + sd][lane];
-            S.gdx = sg * d * ex;
-            S.gdy = sg * d * ey;
-            S.fx = Fx;
-            S.fy = Fy;
-            S.kcs = sign * sg * d * kc;
-            S.u = sideA ? UA : UB;
-            const int np = sideA ? npA : npB;
-            sh.npan[2 * i + sd][lane] = (unsigned short)np;
-            total += np;
-        }
-    }
-    return total;
-}
-
-// the item data of a near-field item that its panels use (barycentric frame of T_b)
-struct NearItem {
-    float e1x, e1y, e2x, e2y, inv, l10, l20;
-};
-
-// panel pnl of a side with npan panels (side data sd, item frame it) added onto S
-__device__ __forceinline__ void near_panel_f32(const NumArgs &A, const NearSide &sd, int npan, const NearItem &it,
-                                               int pnl, float S[10])
-{
-    const bool full = pnl + 1 < npan;
-    const float u0 = (float)pnl, hw = full ? 1.f : fmaxf(sd.u, u0) - u0;
-    // on a full panel [p, p + 1], sinh(p + x_j) = sinh(p) cosh(x_j) + cosh(p) sinh(x_j); the last
-    // panel [p, U] evaluates sinh directly
-    float sp = 0.f, cp = 1.f;
-    if (full && pnl > 0) {
-        const float ep = expf(u0), em = 1.f / ep;
-        sp = 0.5f * (ep - em);
-        cp = 0.5f * (ep + em);
-    }
-    const int nu = A.duffy_n;
-    for (int j = 0; j < nu; j++) {
-        const float sh_ = full ? fmaf(sp, A.glf_ch[j], cp * A.glf_sh[j]) : sinhf(u0 + hw * A.glf_x[j]);
-        const float wj = sd.kcs * (hw * A.glf_w[j]);
-        const float wx = fmaf(sh_, sd.gdx, sd.fx), wy = fmaf(sh_, sd.gdy, sd.fy);
-        const float l1w = (wx * it.e2y - it.e2x * wy) * it.inv;
-        const float l2w = (it.e1x * wy - wx * it.e1y) * it.inv;
-        for (int k = 0; k < 2; k++) {
-            const float sv = A.gl2f_x[k];
-            const float l1 = sv * l1w - it.l10, l2 = sv * l2w - it.l20, l0 = 1.f - l1 - l2;
-            const float w = wj * A.gl2f_w[k];
-            const float w0 = w * l0, w1 = w * l1, w2 = w * l2;
-            S[0] += w;
-            S[1] += w0; S[2] += w1; S[3] += w2;
-            S[4] += w0 * l0; S[5] += w1 * l1; S[6] += w2 * l2;
-            S[7] += w0 * l1; S[8] += w0 * l2; S[9] += w1 * l2;
-        }
-    }
-}
-
 template <int BALL>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_near(const NumArgs A)
 {
-    __shared__ NearShared near_sh[kWarpsPerBlock];
-    NearShared &sh = near_sh[threadIdx.x >> 5];
     const int n = min(*A.near_n, A.near_cap);
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -2042,7 +1936,9 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_near(const NumArgs A)
     for (int64_t base = warp0 * 32; base < n; base += nwarps * 32) {
         const int64_t i = base + lane;
         long long ke = -1, ka = -1;
-        int b = 0, q = 0, q0 = 0, np = 0;
+        int b = 0, q = 0, q0 = 0;
+        int64_t nq = 0;
+        Sums<float> S;
         DeferItem d = {0, 0, 0};
         OuterPt o;
         if (i < n) {
@@ -2065,65 +1961,16 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_near(const NumArgs A)
                 q0 = c.q0;
                 nlg::F2 dl[3];
                 for (int k = 0; k < 3; k++) { dl[k].x = c.vlx[k] - o.lx; dl[k].y = c.vly[k] - o.ly; }
-                sh.e1x[lane] = c.e1x;
-                sh.e1y[lane] = c.e1y;
-                sh.e2x[lane] = c.e2x;
-                sh.e2y[lane] = c.e2y;
-                sh.inv[lane] = c.binv;
-                sh.l10[lane] = (dl[0].x * c.e2y - c.e2x * dl[0].y) * c.binv;
-                sh.l20[lane] = (c.e1x * dl[0].y - dl[0].x * c.e1y) * c.binv;
-                np = near_setup_f32(A, dl, b, D2{o.x, o.y}, sh, lane);
+                near_whole_f32(A, dl, b, D2{o.x, o.y}, nlg::F2{c.e1x, c.e1y}, nlg::F2{c.e2x, c.e2y}, c.binv, S, nq);
                 ke = d.e;
                 ka = a;
             }
         }
-        // the warp's panel list: item j's panels start at start[j]
-        int incl = np;
-        for (int off = 1; off < 32; off <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += y;
-        }
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
-        sh.start[lane] = incl - np;
-        for (int k = 0; k < 10; k++) sh.acc[k][lane] = 0.f;
         __syncwarp();
-        for (int t0 = 0; t0 < total; t0 += 32) {
-            const int t = t0 + lane;
-            float S[10];
-            for (int k = 0; k < 10; k++) S[k] = 0.f;
-            long long key = -1;
-            int it = 0;
-            if (t < total) {
-                // the last item whose panels start at or before t (an item without panels shares
-                // its start with the next one)
-                int lo = 0, hi = 31;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (sh.start[mid] <= t) lo = mid; else hi = mid - 1;
-                }
-                it = lo;
-                int r = t - sh.start[it], side = 0;
-                while (side < 5 && r >= (int)sh.npan[side][it]) r -= (int)sh.npan[side++][it];
-                const NearItem itd = {sh.e1x[it], sh.e1y[it], sh.e2x[it], sh.e2y[it], sh.inv[it], sh.l10[it],
-                                      sh.l20[it]};
-                near_panel_f32(A, sh.side[side][it], (int)sh.npan[side][it], itd, r, S);
-                key = it;
-            }
-            // the panels of one item are adjacent: one shared add per item and pass
-            if (warp_run_sum<10>(key, lane, S))
-                for (int k = 0; k < 10; k++) sh.acc[k][it] += S[k];
-            __syncwarp();
-        }
         float w[21];
         for (int k = 0; k < 21; k++) w[k] = 0.f;
-        int64_t nq = 0;
         if (ka >= 0) {
-            Sums<float> S;
-            S.s0 = sh.acc[0][lane];
-            for (int k = 0; k < 3; k++) S.s1[k] = sh.acc[1 + k][lane];
-            for (int k = 0; k < 6; k++) S.S2[k] = sh.acc[4 + k][lane];
             combine<float>(o, S, w);
-            nq = 2 * (int64_t)A.duffy_n * np;
             A.flag[d.e] = 1;
         }
         __syncwarp();

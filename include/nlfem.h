@@ -140,9 +140,9 @@ const char *nl_last_error(nl_ctx *ctx);
    pairs with a non-empty region) and the numeric scatter.  *out receives a new
    library-owned n x n CSR (n = mesh->nv).  Synchronises the stream three times (to
    size the candidate-search grid, the candidate lists and the pattern); device memory
-   comes from the device's stream-ordered pool on the context's stream.  The interior
-   candidates' quadrature runs on a second stream of the context, concurrently with the
-   boundary candidates' (ordered after the context's stream's earlier work, which waits
+   comes from the device's stream-ordered pool on the context's stream.  The singular kernel's
+   interior candidates' quadrature runs on a second stream of the context, concurrently with the
+   boundary candidates'; the constant kernel takes both in one launch (ordered after the context's stream's earlier work, which waits
    for it before anything that follows).  The pattern's
    first row count uses a hash set of 2^b slots, b from the mean candidate list;
    NL_ROW_SET_BITS=b (6..13) in the environment sets it instead (the pattern does not
@@ -163,8 +163,8 @@ nl_status nl_assemble_numeric(nl_ctx *ctx, nl_csr *inout);
        so the whole batch waits on the host three times, not three times per problem,
        with the problems spread over eight streams of the context (joined by events);
      - runs the numeric phase (pair geometry + quadrature) of all problems either in one
-       pair of persistent launches (interior candidates, then boundary candidates) per value
-       type x ball x kernel type present, whose warps take work items (a run of outer
+       persistent launch per value type x ball x kernel type present (the singular kernel's
+       interior candidates in one launch per value type before it), whose warps take work items (a run of outer
        triangles of one problem) from a global counter, or as each problem's own kernels
        over several streams (the autotuner's choice, below);
      - scatters all problems in one launch per value type;
@@ -194,8 +194,8 @@ typedef struct {
                              candidates x outer points x inner points per triangle) */
     int32_t blocks;       /* persistent grid of the first boundary-candidate launch (blocks of 128 threads)
                              under the chosen schedule */
-    int32_t launches;     /* numeric launches per run: one interior launch per value type, one boundary
-                             launch per value type x ball x kernel type */
+    int32_t launches;     /* numeric launches per run: one launch per value type x ball x kernel type, and
+                             one for the singular kernel's interior candidates per value type */
     int32_t source;       /* NL_SCHED_*: how the schedule was chosen */
     int32_t n_tried;      /* schedules timed by the autotuner in this nl_batch_create */
     double tuned_ms;      /* numeric phase of the batch with the chosen schedule (NL_SCHED_TUNED; median of 3) */

@@ -361,12 +361,26 @@ nl_status nl_fill_args(nl_ctx *ctx, const nl_plan *P, nlq::NumArgs &A, bool stat
     A.geo.b_in2 = (float)((c.delta - tau) * (c.delta - tau));
     A.geo.b_out2 = (float)((c.delta + tau) * (c.delta + tau));
     for (int r = 0; r < A.inner.n; r++) {
-        A.fin[r] = make_float4((float)A.inner.l[r][0], (float)A.inner.l[r][1], (float)A.inner.l[r][2],
-                               (float)A.inner.w[r]);
+        const double *l = A.inner.l[r], w = A.inner.w[r];
+        A.fin[r] = make_float4((float)l[0], (float)l[1], (float)l[2], (float)w);
+        A.fq[r][0] = make_float4((float)(w * l[0] * l[0]), (float)(w * l[1] * l[1]), (float)(w * l[2] * l[2]),
+                                 (float)(w * l[0] * l[1]));
+        A.fq[r][1] = make_float4((float)(w * l[0] * l[2]), (float)(w * l[1] * l[2]), (float)l[1], (float)l[2]);
+    }
+    for (int k = 0; k < 6; k++) {
+        const int i = k < 3 ? k : (k == 5 ? 1 : 0), j = k < 3 ? k : (k == 3 ? 1 : 2);
+        double lost = 0.0, kept = 0.0;
+        for (int r = 0; r < A.inner.n; r++) {
+            const float4 f = A.fq[r][k >> 2];
+            const float c = (k & 3) == 0 ? f.x : (k & 3) == 1 ? f.y : (k & 3) == 2 ? f.z : f.w;
+            lost += A.inner.w[r] * A.inner.l[r][i] * A.inner.l[r][j] - (double)c;
+            kept += c;
+        }
+        A.fq_lo[k] = kept != 0.0 ? (float)(lost / kept) : 0.f;
+    }
     for (int q = 0; q < A.outer.n; q++)
         A.fout[q] = make_float4((float)A.outer.l[q][0], (float)A.outer.l[q][1], (float)A.outer.l[q][2],
                                 (float)A.outer.w[q]);
-    }
     A.flag = P->flag;
     A.blk = P->blk;
     A.mbb = P->mbb;

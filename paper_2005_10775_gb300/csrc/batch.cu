@@ -7,9 +7,9 @@
 //     so a batch synchronises three times in all, with the problems spread over the
 //     context's eight side streams (problem i on stream i mod 8, joined by events);
 //   * the numeric phase of every problem runs in a few persistent launches: the
-//     interior candidates of all problems of a value type (nlq::k_interior_batch), then
-//     the boundary candidates of all problems of a ball mode x kernel type
-//     (nlq::k_boundary_batch); warps take work items (a run of `chunk` outer triangles
+//     candidates of all constant-kernel problems of a ball mode (nlq::k_const_batch); for the
+//     singular kernel the interior candidates of all problems of a value type
+//     (nlq::k_interior_batch), then the boundary candidates by ball mode (nlq::k_boundary_batch); warps take work items (a run of `chunk` outer triangles
 //     of one problem) from the launch's global counter;
 //   * the scatter of every problem runs in one launch per value type;
 //   * numeric phase + scatter are captured once in a CUDA graph (nl_batch_run).

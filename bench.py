@@ -31,17 +31,24 @@ if ROOT not in sys.path:
 
 METRIC = "assembly qp-pairs/s & ms/matrix, FP32-comp vs FP64 GPU at rel err <=1e-6"
 UNIT = "qp-pairs/s"
-# algorithmic work per unit, counted from the quadrature of Secs. 5-6 and the local
-# blocks of Sec. 7.2: the inner-point
-# evaluation (map, phi_b, omega, s0, s1, S2) and the per-(T_a, q, T_b) outer combination
+# algorithmic work per unit.  Singular kernel (Secs. 5-6 and the local blocks of Sec. 7.2): the inner-point
+# evaluation (map, phi_b, omega, s0, s1, S2) and the per-(T_a, q, T_b) outer combination.  The constant
+# kernel's regions are integrated by moments, which is what the inner rules compute (they are exact
+# for quadratics): no inner points, 20 flop an edge of a region with three edges at least.  n_qp_pairs still counts
+# the points of those rules, the metric's unit.
 FLOP_PER_QP = 37.0
 FLOP_PER_INTER = 48.0
+FLOP_PER_REGION = 60.0
+
+
+def algorithmic_flop(kernel, n_qp, n_inter):
+    if kernel == "const":
+        return (FLOP_PER_REGION + FLOP_PER_INTER) * n_inter
+    return FLOP_PER_QP * n_qp + FLOP_PER_INTER * n_inter
+
+
 SMS, FP32_LANES = 152, 128
 FP64_NOMINAL_TFLOPS = 1.25   # GB300 FP64 rate (nominal); the measured one comes from nl_fma_peak
-# DRAM bytes (read + write) of the numeric phase (k_interior + k_boundary + k_deferred) of
-# one assembly, from one ncu capture of the current kernels (profiles/k_boundary_<workload>.md)
-NCU_TRAFFIC = {"ngon32_96": (380.4e6, "ncu dram__bytes_read.sum + dram__bytes_write.sum of k_interior + k_boundary "
-                                      "+ k_deferred + k_defer_merge, profiles/numeric_traffic_ngon32_96.md")}
 
 
 def parse():
@@ -333,7 +340,7 @@ def batch_bench(args, nl, ctx, stream, dev, world, dist, rank, cpu_seconds=None)
     peaks, src = measured_peaks()
     sm_mhz = float(peaks.get("sm_max_mhz", 2070.0))
     peak = SMS * FP32_LANES * 2 * sm_mhz * 1e6 / 1e12
-    achieved = (FLOP_PER_QP * n_qp + FLOP_PER_INTER * n_inter) / (phases[1] / 1e3) / 1e12
+    achieved = algorithmic_flop("const", n_qp, n_inter) / (phases[1] / 1e3) / 1e12
     Ks = [p.mesh.nt for p in probs]
     line = {
         "metric": METRIC, "value": n_qp * world / (ms_batch / 1e3), "unit": UNIT, "n_gpus": world,
@@ -361,7 +368,7 @@ def batch_bench(args, nl, ctx, stream, dev, world, dist, rank, cpu_seconds=None)
         "fp64": fp64,
         "speedup_fp32c_vs_fp64": (fp64["ms_per_step"] / ms_batch) if fp64 else None,
         "roofline": {"bound": "alu",
-                     "kernel": "k_interior_batch + k_boundary_batch + k_deferred_batch (pair geometry + quadrature, "
+                     "kernel": "k_const_batch + k_deferred_batch (pair geometry + quadrature, "
                                "all problems)",
                      "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                      "peak_source": f"FP32 FMA: {SMS} SMs x {FP32_LANES} lanes x 2 x {sm_mhz:.0f} MHz "
@@ -555,7 +562,7 @@ def config_entry(args, nl, ctx, name, stream, dev, dist, flush, world, rank, pea
     t64, ph64, st64, _, _ = time_assembly(nl, ctx, mesh, cfg_for("fp64"), fp64_steps, 1, stream, flush, dev, dist)
     n_pairs, n_qp, n_inter, nnz, n_fp64 = st32
     ms32, ms64 = t32 / steps, t64 / fp64_steps
-    flop = FLOP_PER_QP * n_qp + FLOP_PER_INTER * n_inter
+    flop = algorithmic_flop(p.kernel, n_qp, n_inter)
     a32 = flop / (ph32[1] / 1e3) / 1e12
     a64 = flop / (ph64[1] / 1e3) / 1e12
     e = {"workload": name, "K": p.mesh.nt, "ball": f"{p.ball}{p.ngon_n or ''}", "delta": p.delta,
@@ -708,7 +715,7 @@ def main():
     peaks = alu_peaks(nl, ctx)
     peak = peaks["fp32_derived_tflops"]
     numeric_ms = phase[1]
-    achieved = (FLOP_PER_QP * n_qp + FLOP_PER_INTER * n_inter) / (numeric_ms / 1e3) / 1e12
+    achieved = algorithmic_flop(p.kernel, n_qp, n_inter) / (numeric_ms / 1e3) / 1e12
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
@@ -724,14 +731,14 @@ def main():
         "fp64": fp64,
         "speedup_fp32c_vs_fp64": (fp64["ms_per_step"] / ms_step) if fp64 else None,
         "fp32c_vs_fp64_max_rel_err": err32,
-        "roofline": {"bound": "alu", "kernel": "k_interior + k_boundary + k_deferred + k_defer_merge (+ k_near for the "
-                               "singular kernel): pair geometry + quadrature",
+        "roofline": {"bound": "alu", "kernel": ("k_const (+ k_deferred + k_defer_merge)" if p.kernel == "const" else
+                                "k_interior + k_boundary + k_near + k_deferred + k_defer_merge")
+                     + ": pair geometry + quadrature",
                      "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                      "peak_source": f"FP32 FMA: {SMS} SMs x {FP32_LANES} lanes x 2 x {peaks['sm_max_mhz']:.0f} MHz "
                                     f"(clock from MEASURED_PEAKS.json, {peaks['clock_source']})",
                      "frac_of_measured_fp32": achieved / peaks["fp32_measured_tflops"],
-                     "traffic": NCU_TRAFFIC[args.workload][0] if args.workload in NCU_TRAFFIC else None,
-                     "traffic_source": NCU_TRAFFIC[args.workload][1] if args.workload in NCU_TRAFFIC else None},
+                     "traffic": None, "traffic_source": None},
         "fma_peaks": peaks,
         "clocks": ck,
         "solve": solve,
@@ -739,7 +746,7 @@ def main():
         "e2e": e2e,
     }
     if fp64:
-        a64 = (FLOP_PER_QP * n_qp + FLOP_PER_INTER * n_inter) / (fp64["numeric_ms"] / 1e3) / 1e12
+        a64 = algorithmic_flop(p.kernel, n_qp, n_inter) / (fp64["numeric_ms"] / 1e3) / 1e12
         line["roofline"]["fp64_path"] = {"achieved": a64, "peak_fp64_measured": peaks["fp64_measured_tflops"],
                                          "frac": a64 / peaks["fp64_measured_tflops"]}
     if rank == 0 and not args.no_cpu_baseline:

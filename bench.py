@@ -34,16 +34,17 @@ UNIT = "qp-pairs/s"
 # algorithmic work per unit.  Singular kernel (Secs. 5-6 and the local blocks of Sec. 7.2): the inner-point
 # evaluation (map, phi_b, omega, s0, s1, S2) and the per-(T_a, q, T_b) outer combination.  The constant
 # kernel's regions are integrated by moments, which is what the inner rules compute (they are exact
-# for quadratics): no inner points, 20 flop an edge of a region with three edges at least.  n_qp_pairs still counts
-# the points of those rules, the metric's unit.
+# for quadratics): no inner points, and a triangle inside every outer point's ball is one product of the two rules'
+# sums.  Its count is a lower estimate, 30 flop an interaction (T_a, q, T_b): its classification and,
+# averaged over whole and cut regions, the moments.  n_qp_pairs counts the rules' points, the metric's unit.
 FLOP_PER_QP = 37.0
 FLOP_PER_INTER = 48.0
-FLOP_PER_REGION = 60.0
+FLOP_PER_INTER_CONST = 30.0
 
 
 def algorithmic_flop(kernel, n_qp, n_inter):
     if kernel == "const":
-        return (FLOP_PER_REGION + FLOP_PER_INTER) * n_inter
+        return FLOP_PER_INTER_CONST * n_inter
     return FLOP_PER_QP * n_qp + FLOP_PER_INTER * n_inter
 
 

@@ -113,6 +113,11 @@ struct nl_plan {
     char *slab[3] = {nullptr, nullptr, nullptr};   // the allocations that hold the mesh, numeric and slot arrays
     cudaStream_t stream = nullptr;   // stream the buffers were allocated on (freed stream-ordered)
     int K = 0, J = 0;
+    // The plan holds its geometry in lengths of its own, the mesh's times 2^k with delta in [1, 2): exact, and
+    // FP32 then holds areas, their products (the constant kernel's blocks) and the fourth powers of lengths in
+    // the predicates whatever unit the mesh is in (in nanometres given in metres they would underflow).  cfg
+    // has delta and c in these units (c times 2^-4k, or 2^-3k for c / |x - y|), so the matrix comes out in the
+    // mesh's.
     nl_config cfg{};
     double d2 = 0.0, hmax = 0.0, rmax = 0.0, rin = 0.0;
     // mesh (device)

@@ -136,8 +136,9 @@ __global__ void __launch_bounds__(1024) k_scan_one(const int64_t *in, int64_t *o
 // ---------------------------------------------------------------------------
 // preprocessing
 // ---------------------------------------------------------------------------
+// scale: the plan's lengths per mesh length (a power of two, nl_plan::cfg)
 __global__ void k_prepare(int K, int J, const int32_t *__restrict__ tri, const double *__restrict__ vx,
-                          const double *__restrict__ vy, double *tx, double *ty, double *bx, double *by,
+                          const double *__restrict__ vy, double scale, double *tx, double *ty, double *bx, double *by,
                           double *rad, double *area, double *diam, float4 *cf, double kc, float *akc,
                           unsigned long long *bad)
 {
@@ -148,7 +149,8 @@ __global__ void k_prepare(int K, int J, const int32_t *__restrict__ tri, const d
         atomicAdd(bad, 1ull);
         return;
     }
-    double x0 = vx[i0], y0 = vy[i0], x1 = vx[i1], y1 = vy[i1], x2 = vx[i2], y2 = vy[i2];
+    double x0 = vx[i0] * scale, y0 = vy[i0] * scale, x1 = vx[i1] * scale, y1 = vy[i1] * scale;
+    double x2 = vx[i2] * scale, y2 = vy[i2] * scale;
     tx[t] = x0; tx[K + t] = x1; tx[2 * K + t] = x2;
     ty[t] = y0; ty[K + t] = y1; ty[2 * K + t] = y2;
     // barycentre ((v0 + v1) + v2) / 3, round-to-nearest, no contraction
@@ -560,7 +562,13 @@ nl_status nl_prepare_a(nl_ctx *ctx, const nl_mesh *mesh, const nl_config *cfg, n
     P->K = K;
     P->J = J;
     P->cfg = *cfg;
-    P->d2 = cfg->delta * cfg->delta;
+    int unit = 0;   // 2^unit: the plan's lengths per mesh length
+    frexp(cfg->delta, &unit);
+    unit = 1 - unit;
+    unit = unit < -1000 ? -1000 : (unit > 1000 ? 1000 : unit);
+    P->cfg.delta = ldexp(cfg->delta, unit);
+    P->cfg.kernel_c = ldexp(cfg->kernel_c, (cfg->kernel == NL_KERNEL_CONST ? -4 : -3) * unit);
+    P->d2 = P->cfg.delta * P->cfg.delta;
     nl_status s;
     if ((s = nl_stage(ctx, mesh->vx, sizeof(double) * J, &T->dvx, &T->own_vx)) != NL_OK) return s;
     if ((s = nl_stage(ctx, mesh->vy, sizeof(double) * J, &T->dvy, &T->own_vy)) != NL_OK) return s;
@@ -590,13 +598,13 @@ nl_status nl_prepare_a(nl_ctx *ctx, const nl_mesh *mesh, const nl_config *cfg, n
         const size_t nb = sizeof(double) * 2 * cfg->ngon_n;
         P->ngon_host.resize(2 * (size_t)cfg->ngon_n);
         if (nl_is_device_ptr(cfg->ngon_offsets)) {
-            NL_CK(cudaMemcpyAsync(P->ngon, cfg->ngon_offsets, nb, cudaMemcpyDeviceToDevice, ctx->stream));
             NL_CK(cudaMemcpyAsync(P->ngon_host.data(), cfg->ngon_offsets, nb, cudaMemcpyDeviceToHost, ctx->stream));
             NL_CK(cudaStreamSynchronize(ctx->stream));
         } else {
             memcpy(P->ngon_host.data(), cfg->ngon_offsets, nb);
-            NL_CK(cudaMemcpyAsync(P->ngon, P->ngon_host.data(), nb, cudaMemcpyHostToDevice, ctx->stream));
         }
+        for (double &o : P->ngon_host) o = ldexp(o, unit);
+        NL_CK(cudaMemcpyAsync(P->ngon, P->ngon_host.data(), nb, cudaMemcpyHostToDevice, ctx->stream));
         P->rin = nl_polygon_inradius(P->ngon_host.data(), cfg->ngon_n);
     }
     {
@@ -609,9 +617,9 @@ nl_status nl_prepare_a(nl_ctx *ctx, const nl_mesh *mesh, const nl_config *cfg, n
     }
     NL_CK(cudaMemsetAsync(T->st, 0, sizeof(unsigned long long) * (kStats + 1), ctx->stream));
     k_prepare<<<(K + 255) / 256, 256, 0, ctx->stream>>>(K, J, (const int32_t *)T->dtri, (const double *)T->dvx,
-                                                        (const double *)T->dvy, P->tx, P->ty, P->bx, P->by,
-                                                        P->rad, P->area, T->diam, T->cf,
-                                                        cfg->kernel == NL_KERNEL_CONST ? 1.0 : cfg->kernel_c, P->akc,
+                                                        (const double *)T->dvy, ldexp(1.0, unit), P->tx, P->ty,
+                                                        P->bx, P->by, P->rad, P->area, T->diam, T->cf,
+                                                        cfg->kernel == NL_KERNEL_CONST ? 1.0 : P->cfg.kernel_c, P->akc,
                                                         T->st + kStats); ++ctx->launches;
     k_hilo<<<(K + 255) / 256, 256, 0, ctx->stream>>>(K, P->tx, P->ty, P->bx, P->by, P->hl); ++ctx->launches;
     NL_CK(cudaGetLastError());

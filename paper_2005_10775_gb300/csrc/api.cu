@@ -293,10 +293,6 @@ nl_status nl_fill_args(nl_ctx *ctx, const nl_plan *P, nlq::NumArgs &A, bool stat
         int e = 0;
         frexp(bound > 1e-30 ? bound : 1e-30, &e);   // bound < 2^e
         A.s0q_grid = (float)ldexp(1.0, 30 - e);
-        // FP64 sums of areas: 2^50 on a power of two above the largest area a triangle of
-        // barycentre radius r_max can have (27/8 of the equilateral one's r^2 is above 3 sqrt(3)/4)
-        frexp(4.0 * P->rmax * P->rmax, &e);
-        A.area_grid = ldexp(1.0, 50 - e);
     }
     A.geo.delta = c.delta;
     A.geo.deltaf = (float)c.delta;

@@ -109,7 +109,6 @@ struct NumArgs {
     OuterPt *otab;                    // [K][outer.n] outer points as the boundary kernel staged them (read by
                                       // k_near; with the near-field queue only)
     int prob;                         // index of this problem in a batched launch's argument array
-    double area_grid;                 // constant kernel, FP64: scale of the fixed-point sums of areas
     float s0q_grid;                   // FP32 boundary kernel: scale of the fixed-point sums of s0 per
                                       // outer point (a power of two; the bound on a sum maps below 2^30)
 };

@@ -1079,11 +1079,7 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
         sh.w[q][2] = W * (f32 ? (T)o.l2f : (T)o.l2);
         sh.w[q][3] = W;
     }
-    // sum of |T_b| over the whole items of outer point q = lane: exact integers (FP32 path: on the
-    // grid s0q_grid; FP64 path: 50-bit fixed point in two limbs, area_grid = 2^50 / a power of two
-    // above the largest area)
-    int ws_f = 0;
-    unsigned long long ws_hi = 0, ws_lo = 0;
+    double ws = 0.0;   // sum of |T_b| over the whole items of outer point q = lane
     int nopen = 0;   // items the FP64 geometry decided here
     __syncwarp();
     for (int64_t base = es; base < e1; base += 32) {
@@ -1093,8 +1089,7 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
         CandData c;
         c.b = a;
         c.akcf = 0.f;
-        unsigned a_hi = 0, a_lo = 0;
-        int a_fx = 0;
+        T area_b = 0;
         if (valid) {
             int b = A.nbr_idx[e];
 #ifdef NL_CHECKS
@@ -1107,7 +1102,7 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
             q0 = c.q0;
             sh.cand[lane] = cand32_of(c);
             if constexpr (f32) {
-                a_fx = __float2int_rn(c.akcf * A.s0q_grid);
+                area_b = c.akcf;
             } else {
                 const int64_t K = A.K;
                 Cand64 d;
@@ -1130,10 +1125,26 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
                 d.g[1][0] = -inv * d.v[1][1];
                 d.g[1][1] = inv * d.v[1][0];
                 sh.c64[lane] = d;
-                const unsigned long long fx = __double2ull_rn(d.area * A.area_grid);
-                a_hi = (unsigned)(fx >> 25);
-                a_lo = (unsigned)fx & ((1u << 25) - 1u);
+                area_b = d.area;
             }
+        }
+        // The round's areas as integers, so that 32 of them are summed in one or two instructions and in no
+        // order: 27 bits (FP32; an area has 24) or 54 in two limbs (FP64; an area has 53) under the power of
+        // two above the round's largest area.  A grid of the mesh's largest area took the small triangles
+        // of a graded mesh down to 1e-9 of themselves.
+        constexpr int kExpBias = f32 ? 127 : 1023, kBits = f32 ? 27 : 54;
+        unsigned ef;   // exponent field of the largest area
+        if constexpr (f32) ef = (unsigned)__float_as_int(area_b) >> 23;
+        else ef = (unsigned)__double2hiint(area_b) >> 20;
+        ef = max(__reduce_max_sync(0xffffffffu, ef), (unsigned)kBits + 1u);
+        unsigned a_hi = 0, a_lo, r_hi = 0, r_lo = 0;
+        if constexpr (f32) {
+            a_lo = __float2uint_rn(area_b * __int_as_float((2 * kExpBias + kBits - 1 - (int)ef) << 23));
+        } else {
+            const unsigned long long fx =
+                __double2ull_rn(area_b * __hiloint2double((2 * kExpBias + kBits - 1 - (int)ef) << 20, 0));
+            a_hi = (unsigned)(fx >> 27);
+            a_lo = (unsigned)fx & ((1u << 27) - 1u);
         }
         for (int i = 0; i < 12; i++) sh.acc[i][lane] = (Fx)0;
         sh.dmask[lane] = 0;
@@ -1158,19 +1169,16 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
                 nwhole++;
                 if (want_stats<STS>(A)) acc.hsum += nlg::record_hash(a, c.b, q - q0, nlg::KIND_WHOLE, 3, 0);
             }
-            if constexpr (f32) {
-                const int t = __reduce_add_sync(0xffffffffu, whole ? a_fx : 0);
-                if (lane == q) ws_f += t;
-            } else {
+            const unsigned tl = __reduce_add_sync(0xffffffffu, whole ? a_lo : 0u);
+            if (lane == q) r_lo = tl;
+            if constexpr (!f32) {
                 const unsigned th = __reduce_add_sync(0xffffffffu, whole ? a_hi : 0u);
-                const unsigned tl = __reduce_add_sync(0xffffffffu, whole ? a_lo : 0u);
-                if (lane == q) {
-                    ws_hi += th;
-                    ws_lo += tl;
-                }
+                if (lane == q) r_hi = th;
             }
             if (cls == nlg::CLS_EXACT) cutq |= 1u << q;
         }
+        if constexpr (f32) ws += (double)r_lo * (double)__int_as_float(((int)ef + 1 - kBits) << 23);
+        else ws += (double)(((unsigned long long)r_hi << 27) + r_lo) * __hiloint2double(((int)ef + 1 - kBits) << 20, 0);
         // the cut items, every lane's first, then every lane's second, ...: neighbours in the queue have
         // different owners and outer points, so their adds rarely meet on one address
         for (unsigned m = __ballot_sync(0xffffffffu, cutq != 0u); m; m = __ballot_sync(0xffffffffu, cutq != 0u)) {
@@ -1333,11 +1341,11 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
     if (lane < nq_all) {
         double t;
         if constexpr (f32) {
-            const long long s = (long long)sh.s0q[lane] + ws_f;
-            if (s >= (1ll << 30) || s <= -(1ll << 30)) atomicOr(A.err, 256);
-            t = (double)s / (double)A.s0q_grid;
+            const int s = sh.s0q[lane];
+            if (s >= (1 << 30) || s <= -(1 << 30)) atomicOr(A.err, 256);
+            t = (double)s / (double)A.s0q_grid + ws;
         } else {
-            t = sh.s0q[lane] + (double)((ws_hi << 25) + ws_lo) / A.area_grid;
+            t = sh.s0q[lane] + ws;
         }
         // W phi_a,i and W as the pairs' sums have them (FP32 path: rounded to FP32): M_aa, M_ab and M_bb are
         // then the blocks of one square (sum_i phi_a,i u_i - u(y))^2, and what rounding the weights costs

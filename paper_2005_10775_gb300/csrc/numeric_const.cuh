@@ -50,6 +50,17 @@ __device__ __forceinline__ void mom_set(Mom<T> &M, T v)
     M.s0 = M.s1 = M.s2 = M.s11 = M.s22 = M.s12 = v;
 }
 
+// a thin triangle's moments (its Cand32 area is negative): every one lies in [0, 1]
+__device__ __forceinline__ void mom_hold(Mom<float> &M)
+{
+    M.s0 = fminf(fmaxf(M.s0, 0.f), 1.f);
+    M.s1 = fminf(fmaxf(M.s1, 0.f), 1.f);
+    M.s2 = fminf(fmaxf(M.s2, 0.f), 1.f);
+    M.s11 = fminf(fmaxf(M.s11, 0.f), 1.f);
+    M.s22 = fminf(fmaxf(M.s22, 0.f), 1.f);
+    M.s12 = fminf(fmaxf(M.s12, 0.f), 1.f);
+}
+
 // boundary segment p -> q, (l1, l2) coordinates
 template <typename T>
 __device__ __forceinline__ void seg_add(Mom<T> &M, T p1, T p2, T q1, T q2)
@@ -143,7 +154,9 @@ __device__ __forceinline__ void pair_block(T area, const T *P, const T *Q, T *ma
 // rounded vertices: the triangles around T_a then form one mesh in FP32 too (a shared vertex is rounded
 // once), their regions tile the ball, and what the rounding takes from one triangle its neighbour
 // gets.  (Edges from the exact vertices, with only T_b's place rounded: errors 1.3-1.8 times as large
-// where delta is below h.)
+// where delta is below h.)  Thin triangles, whose height the vertices' rounding reaches, keep the exact edges
+// and area (as -area), and their moments are held to [0, 1] (mom_hold): a rounded one can have no area
+// or a negative one.  (The 23 words keep lanes that read their own candidate in distinct banks.)
 struct Cand32 {
     float vx[3], vy[3], ex[3], ey[3], gx[3], gy[3], blx, bly, area;
     int b, q0;
@@ -159,7 +172,17 @@ __device__ __forceinline__ Cand32 cand32_of(const CandData &c)
         r.ex[i] = c.vlx[k] - c.vlx[i];
         r.ey[i] = c.vly[k] - c.vly[i];
     }
-    const float det = r.ex[0] * r.ey[1] - r.ex[1] * r.ey[0], inv = 1.f / det;
+    float det = r.ex[0] * r.ey[1] - r.ex[1] * r.ey[0];
+    // the vertices' rounding moves det by up to 8u (2 + L) L (delta < 2, L the longer of two edges): by
+    // more than 6 % here
+    const float L = fmaxf(fabsf(c.e1x) + fabsf(c.e1y), fabsf(c.e2x) + fabsf(c.e2y));
+    const bool thin = c.akcf < 4e-6f * (2.f + L) * L;
+    if (thin) {
+        r.ex[0] = c.e1x; r.ex[1] = c.e2x - c.e1x; r.ex[2] = -c.e2x;
+        r.ey[0] = c.e1y; r.ey[1] = c.e2y - c.e1y; r.ey[2] = -c.e2y;
+        det = 2.f * c.akcf;
+    }
+    const float inv = 1.f / det;
     for (int i = 0; i < 3; i++) {   // the opposite edge turned, over the determinant
         const int k = (i + 1) % 3;
         r.gx[i] = -r.ey[k] * inv;
@@ -167,7 +190,7 @@ __device__ __forceinline__ Cand32 cand32_of(const CandData &c)
     }
     r.blx = c.blx;
     r.bly = c.bly;
-    r.area = 0.5f * det;
+    r.area = thin ? -c.akcf : 0.5f * det;
     r.b = c.b;
     r.q0 = c.q0;
     return r;
@@ -709,8 +732,8 @@ struct WalkPt {
 };
 
 template <int BALL, typename T>
-__device__ __noinline__ bool exact_disc_item(const NumArgs &A, int b, const nlg::F2 *dl, double xx, double xy,
-                                             Mom<T> &M, int &nv, int &kind, int &ncap, bool *used64)
+__device__ __noinline__ bool exact_disc_item(const NumArgs &A, int b, float area32, const nlg::F2 *dl, double xx,
+                                             double xy, Mom<T> &M, int &nv, int &kind, int &ncap, bool *used64)
 {
     const nlg::GeoParams &g = A.geo;
     const D2 x = {xx, xy};
@@ -815,7 +838,8 @@ __device__ __noinline__ bool exact_disc_item(const NumArgs &A, int b, const nlg:
                 }
         }
         const T e1x = px[1] - px[0], e1y = py[1] - py[0], e2x = px[2] - px[0], e2y = py[2] - py[0];
-        const T inv = (T)1 / (e1x * e2y - e2x * e1y);
+        const bool thin = f32 && area32 < 0.f;   // Cand32
+        const T inv = (T)1 / (thin ? (T)(-2.f * area32) : e1x * e2y - e2x * e1y);
         mom_set(M, (T)0);
         WalkPt<T> first = {0, 0, 0, 0, 0}, prev = first;
         int n = 0, narc = 0;
@@ -902,18 +926,21 @@ __device__ __noinline__ bool exact_disc_item(const NumArgs &A, int b, const nlg:
         nv = n >= 2 && m >= 3 ? m : 0;
         kind = in == 7u && n == 3 ? nlg::KIND_WHOLE : nlg::KIND_PARTIAL;
         if (kind == nlg::KIND_WHOLE) mom_set(M, (T)1);
+        if constexpr (f32)
+            if (thin) mom_hold(M);
         *used64 = (open | eopen) != 0u;
         return nv >= 3 || ncap > 0;
     }
 }
 
-// region and moments of one item by the FP64 geometry (*used64 = false: FP32 was certain after all)
+// region and moments of one item by the FP64 geometry (*used64 = false: FP32 was certain after all);
+// area32: the candidate's Cand32 area
 template <int BALL, typename T>
-__device__ __forceinline__ bool exact_item(const NumArgs &A, int b, const nlg::F2 *dl, double xx, double xy,
+__device__ __forceinline__ bool exact_item(const NumArgs &A, int b, float area32, const nlg::F2 *dl, double xx, double xy,
                                            Mom<T> &M, int &nv, int &kind, int &ncap, bool *used64)
 {
     if constexpr (kGeoBall<BALL> == NL_BALL_NGON) return exact_const_item<BALL, T>(A, b, dl, xx, xy, M, nv, kind, ncap);
-    else return exact_disc_item<BALL, T>(A, b, dl, xx, xy, M, nv, kind, ncap, used64);
+    else return exact_disc_item<BALL, T>(A, b, area32, dl, xx, xy, M, nv, kind, ncap, used64);
 }
 
 // are the items that FP32 leaves open queued for k_deferred?  The N-gon's on the FP32 path: its FP64
@@ -1040,8 +1067,8 @@ __device__ __forceinline__ void const_defer_flush(const NumArgs &A, int a, int64
         Mom<float> M;
         int nv, kind, ncap;
         bool used64;
-        if (!exact_item<BALL, float>(A, cd.b, dl, o.x, o.y, M, nv, kind, ncap, &used64)) continue;
-        item_add(sh.w[q], M, sh.acc, &sh.s0q[q], lane, fxs, cd.area, A.s0q_grid);
+        if (!exact_item<BALL, float>(A, cd.b, cd.area, dl, o.x, o.y, M, nv, kind, ncap, &used64)) continue;
+        item_add(sh.w[q], M, sh.acc, &sh.s0q[q], lane, fxs, fabsf(cd.area), A.s0q_grid);
         sh.hit[lane] = 1;
         acc.cnt++;
         acc.qp += (uint32_t)region_points(A, kind, nv, ncap);
@@ -1204,7 +1231,7 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
             for (int k = 0; k < 3; k++) { d[k].x = cd.vx[k] - o.lx; d[k].y = cd.vy[k] - o.ly; }
             Mom<T> M;
             int nv = 0, kind = nlg::KIND_PARTIAL, ncap = 0, r = -1;
-            T area = (T)cd.area;
+            T area = (T)fabsf(cd.area);
             if constexpr (BALL == NL_BALL_BARYCENTER || BALL == NL_BALL_OVERLAP) {
                 // FP64 predicate on the whole triangle
             } else if constexpr (BALL == kBallNgonAny) {
@@ -1245,7 +1272,10 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
                                                ncap);
             }
             if constexpr (f32) {
-                if (live && r > 0) item_add(sh.w[q], M, sh.acc, &sh.s0q[q], own, fxs, area, A.s0q_grid);
+                if (live && r > 0) {
+                    if (cd.area < 0.f) mom_hold(M);
+                    item_add(sh.w[q], M, sh.acc, &sh.s0q[q], own, fxs, area, A.s0q_grid);
+                }
             } else {
                 items_gather(sh, live && r > 0, own, q, M, lane);
             }
@@ -1282,11 +1312,11 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
                 if (live) {
                     nlg::F2 d[3];
                     for (int k = 0; k < 3; k++) { d[k].x = cd.vx[k] - o.lx; d[k].y = cd.vy[k] - o.ly; }
-                    has = exact_item<BALL, T>(A, cd.b, d, o.x, o.y, M, nv, kind, ncap, &used64);
+                    has = exact_item<BALL, T>(A, cd.b, cd.area, d, o.x, o.y, M, nv, kind, ncap, &used64);
                     nopen += used64;
                 }
                 if constexpr (f32) {
-                    if (has) item_add(sh.w[q], M, sh.acc, &sh.s0q[q], own, fxs, cd.area, A.s0q_grid);
+                    if (has) item_add(sh.w[q], M, sh.acc, &sh.s0q[q], own, fxs, fabsf(cd.area), A.s0q_grid);
                 } else {
                     items_gather(sh, has, own, q, M, lane);
                 }
@@ -1319,7 +1349,7 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
             T area;
             if constexpr (f32) area = c.akcf;
             else area = sh.c64[lane].area;
-            pair_block<T>(f32 ? (T)sh.cand[lane].area : area, P, Q, mab, mbb);
+            pair_block<T>(f32 ? (T)fabsf(sh.cand[lane].area) : area, P, Q, mab, mbb);
             // the outer points that see all of T_b: their moments are 1, the blocks |T_b| u_i / 3 and
             // |T_b| sum_i u_i (1 + delta_ij) / 12 (kept apart from the cut ones, whose block is formed by
             // differences: in FP32 those would round the larger, whole part)
@@ -1424,7 +1454,7 @@ __device__ __forceinline__ void deferred_const(const NumArgs &A, const DeferItem
     Mom<float> M;
     int kind, nv, ncap;
     bool used64;
-    if (!exact_item<BALL, float>(A, b, dl, o.x, o.y, M, nv, kind, ncap, &used64)) {
+    if (!exact_item<BALL, float>(A, b, 0.f, dl, o.x, o.y, M, nv, kind, ncap, &used64)) {
         for (int k = 0; k < kDeferVals; k++) dv[(int64_t)k * cap + slot] = 0.f;
         return;
     }

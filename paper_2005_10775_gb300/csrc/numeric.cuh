@@ -349,14 +349,17 @@ __device__ __forceinline__ void whole_sums(const NumArgs &A, const D2 V[3], T ar
     nqp += n;
 }
 
-// inner sums over the region R of the singular kernel c / |x - y|
+// Inner sums over the region R.  Only the singular kernel c / |x - y| comes here, yet the kernel's type is read at
+// run time: with the other one's branches gone the lanes of the FP64 boundary kernel met again less often (6.2 of
+// 32 active instead of 7.4, 23 % more FP64 instructions: 33 -> 40 ms for nocaps on 40 x 40 cells).
 template <typename T>
 __device__ __forceinline__ void inner_sums(const NumArgs &A, const nlg::Region &R, const D2 V[3], double area_b,
                                            D2 x, Sums<T> &S, int64_t &nqp)
 {
     sums_zero(S);
+    const bool inv = (A.kernel == NL_KERNEL_INV_DIST);
     const RuleTab &ri = A.inner;
-    if (R.nv >= 3 && nlg::is_near(R, V, x)) {
+    if (inv && R.nv >= 3 && nlg::is_near(R, V, x)) {
         BaryMap bm = bary_map(V);
         Sums<double> Sd;
         sums_zero(Sd);
@@ -368,13 +371,18 @@ __device__ __forceinline__ void inner_sums(const NumArgs &A, const nlg::Region &
         // the region is T_b itself: phi_b at the rule points are the rule's barycentrics
         const T ar = (T)area_b;
         T lx[3], ly[3];
-        for (int i = 0; i < 3; i++) { lx[i] = (T)(V[i].x - x.x); ly[i] = (T)(V[i].y - x.y); }
+        if (inv)
+            for (int i = 0; i < 3; i++) { lx[i] = (T)(V[i].x - x.x); ly[i] = (T)(V[i].y - x.y); }
         for (int r = 0; r < ri.n; r++) {
             T p0 = (T)ri.l[r][0], p1 = (T)ri.l[r][1], p2 = (T)ri.l[r][2];
             T w = (T)ri.w[r] * ar;
-            T dx = p0 * lx[0] + p1 * lx[1] + p2 * lx[2];
-            T dy = p0 * ly[0] + p1 * ly[1] + p2 * ly[2];
-            w = w * (T)A.kc / sqrt(dx * dx + dy * dy);
+            if (inv) {
+                T dx = p0 * lx[0] + p1 * lx[1] + p2 * lx[2];
+                T dy = p0 * ly[0] + p1 * ly[1] + p2 * ly[2];
+                w = w * (T)A.kc / sqrt(dx * dx + dy * dy);
+            } else {
+                w = w * (T)A.kc;
+            }
             sums_add<T>(S, w, p0, p1, p2);
         }
         nqp += ri.n;
@@ -404,9 +412,13 @@ __device__ __forceinline__ void inner_sums(const NumArgs &A, const nlg::Region &
                     T p1 = m0 * f0[1] + m1 * fk[1] + m2 * fn[1];
                     T p2 = m0 * f0[2] + m1 * fk[2] + m2 * fn[2];
                     w *= art;
-                    T dx = m0 * l0x + m1 * lkx + m2 * lnx;
-                    T dy = m0 * l0y + m1 * lky + m2 * lny;
-                    w = w * (T)A.kc / sqrt(dx * dx + dy * dy);
+                    if (inv) {
+                        T dx = m0 * l0x + m1 * lkx + m2 * lnx;
+                        T dy = m0 * l0y + m1 * lky + m2 * lny;
+                        w = w * (T)A.kc / sqrt(dx * dx + dy * dy);
+                    } else {
+                        w = w * (T)A.kc;
+                    }
                     sums_add<T>(S, w, p0, p1, p2);
                 }
                 nqp += ri.n;
@@ -418,8 +430,12 @@ __device__ __forceinline__ void inner_sums(const NumArgs &A, const nlg::Region &
             double ph[3];
             bary_of(bm, R.cc[c].x, R.cc[c].y, ph);
             T w = (T)R.cw[c];
-            double dx = R.cc[c].x - x.x, dy = R.cc[c].y - x.y;
-            w = w * (T)(A.kc / sqrt(dx * dx + dy * dy));
+            if (inv) {
+                double dx = R.cc[c].x - x.x, dy = R.cc[c].y - x.y;
+                w = w * (T)(A.kc / sqrt(dx * dx + dy * dy));
+            } else {
+                w = w * (T)A.kc;
+            }
             sums_add<T>(S, w, (T)ph[0], (T)ph[1], (T)ph[2]);
             nqp++;
         }
@@ -962,7 +978,7 @@ struct BoundaryShared {
 
 constexpr int kQueueCap = 32 * NL_MAXQ;
 
-template <int BALL, typename T>
+template <int BALL, typename T, bool EDGES>
 __device__ __forceinline__ int classify_item(const NumArgs &A, const CandData &c, const OuterPt &o, nlg::F2 dl[3])
 {
     for (int i = 0; i < 3; i++) { dl[i].x = c.vlx[i] - o.lx; dl[i].y = c.vly[i] - o.ly; }
@@ -977,7 +993,7 @@ __device__ __forceinline__ int classify_item(const NumArgs &A, const CandData &c
         if (nlg::dist2_origin_triangle(dl) > A.geo.rout_p2) return nlg::CLS_EMPTY;
         return nlg::CLS_EXACT;
     }
-    return nlg::classify_vertices(dl, A.geo.rin_m2, A.geo.rout_p2);
+    return nlg::classify_vertices<EDGES>(dl, A.geo.rin_m2, A.geo.rout_p2);
 }
 
 // one undecided (q, b): build the region exactly as the FP64 geometry would and integrate it
@@ -1013,6 +1029,14 @@ __device__ __forceinline__ void fan_tri_sums(const NumArgs &A, nlg::Col px, nlg:
     sums_close(S);
 }
 
+// A triangle outside the disc that the tangent's test (nlg::classify_vertices) missed, by its edges' distances: asked
+// where the horizon is below the triangles' size and the tangent misses many, which the near field's test
+// would send to the FP64 geometry (64 x 64 cells, N-gon, 147 -> 142 ms).  Elsewhere the test costs more.
+__device__ __forceinline__ bool missed_empty(const NumArgs &A, const nlg::F2 dl[3])
+{
+    return A.geo.turn && nlg::classify_vertices<true>(dl, -1.f, A.geo.rout_p2) == nlg::CLS_EMPTY;
+}
+
 // FP32 region of one undecided (q, b) of the balls whose region is a polygon (N-gon, nocaps,
 // approxcaps), left in the lane's clip-buffer column (buffer *which): 1 with its vertex count n
 // and kind, 0 empty, -1 the FP64 geometry decides (as exact_item_f32)
@@ -1022,6 +1046,7 @@ __device__ __forceinline__ int exact_region_f32(const NumArgs &A, const CandData
 {
     nlg::F2 dl[3];
     for (int i = 0; i < 3; i++) { dl[i].x = c.vlx[i] - o.lx; dl[i].y = c.vly[i] - o.ly; }
+    if (missed_empty(A, dl)) return 0;
     if (nlg::near_f32(dl, cand_diam(c), A.geo.tau) != 0) return -1;
     which = 0;
     if (BALL == NL_BALL_NGON) {
@@ -1049,6 +1074,7 @@ __device__ __forceinline__ int exact_item_f32(const NumArgs &A, const CandData &
     if (sizeof(T) == sizeof(float) && (BALL == NL_BALL_NOCAPS || BALL == NL_BALL_APPROXCAPS)) {
         nlg::F2 dl[3];
         for (int i = 0; i < 3; i++) { dl[i].x = c.vlx[i] - o.lx; dl[i].y = c.vly[i] - o.ly; }
+        if (missed_empty(A, dl)) return 0;
         if (nlg::near_f32(dl, cand_diam(c), A.geo.tau) != 0)
             return -1;
         int k = nlg::KIND_PARTIAL;
@@ -1073,6 +1099,7 @@ __device__ __forceinline__ int exact_item_f32(const NumArgs &A, const CandData &
     if (sizeof(T) == sizeof(float) && BALL == NL_BALL_EXACTCAPS) {
         nlg::F2 dl[3];
         for (int i = 0; i < 3; i++) { dl[i].x = c.vlx[i] - o.lx; dl[i].y = c.vly[i] - o.ly; }
+        if (missed_empty(A, dl)) return 0;
         if (nlg::near_f32(dl, cand_diam(c), A.geo.tau) != 0)
             return -1;
         int nc = 0, k = nlg::KIND_PARTIAL;
@@ -1438,7 +1465,7 @@ __device__ __forceinline__ void boundary_outer(const NumArgs &A, int a, Boundary
             int cls = nlg::CLS_EMPTY;
             if (active) {
                 nlg::F2 dl[3];
-                cls = classify_item<BALL, T>(A, c, sh.sq[q], dl);
+                cls = classify_item<BALL, T, sizeof(T) == sizeof(double)>(A, c, sh.sq[q], dl);
                 // singular kernel: whole items in the near field take the near rule (certified
                 // in FP32; undecided ones the FP64 path)
                 if (cls == nlg::CLS_WHOLE) {

@@ -1186,7 +1186,7 @@ __device__ __forceinline__ void boundary_const(const NumArgs &A, int a, ConstSha
             int cls = nlg::CLS_EMPTY;
             if (active) {
                 nlg::F2 dl[3];
-                cls = classify_item<kGeoBall<BALL>, T>(A, c, o, dl);
+                cls = classify_item<kGeoBall<BALL>, T, false>(A, c, o, dl);
             }
             const bool whole = cls == nlg::CLS_WHOLE;
             if (whole) {

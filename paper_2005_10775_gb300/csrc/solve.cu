@@ -186,8 +186,9 @@ __global__ void k_residual(int n, const int64_t *rp, const int32_t *__restrict__
 // iteration is two grid barriers, the blocks keep their rows (values and columns can stay in L1), and the
 // convergence check costs nothing.  Extraction, load vector and solve of the 96 x 96 N-gon mesh (64
 // iterations): 1.54 -> 1.2 ms.  With two launches an iteration it took 1.50 ms; with 3 blocks of 512, 1 or 2
-// of 1024 threads an SM 1.26, 1.21 and 1.31 (fewer arrivals against more rows in flight).  104 iterations on
-// 39,601 nodes (17 M entries, more than L2 holds) are bound by the matrix from memory: 5.08 -> 4.96 ms.
+// of 1024 threads an SM 1.26, 1.21 and 1.31 (fewer arrivals against more rows in flight).  A matrix that L2 does
+// not hold is bound by its entries from memory: 18 M entries 2.69 -> 2.08 ms, 27 M 16.4 -> 15.3 ms (with every
+// iteration in the same order 2.8 and 17.7 ms, slower than with four launches).
 // The product forms its direction p = z + beta p as it gathers it (z and
 // p of a node lie side by side: one 8-byte load), so directions need no pass of their own.
 //     zz[k & 3] = ||z_k||^2 (rho of iteration k), pq[k & 3] = p_k . A p_k
@@ -260,6 +261,7 @@ k_cg(int n, const int64_t *__restrict__ rp, const int32_t *__restrict__ col, con
     __shared__ int s_stop;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int rpb = min(kCgWarps, (n + (int)gridDim.x - 1) / (int)gridDim.x);
+    const int stride = rpb * (int)gridDim.x, rounds = (n - 1) / stride + 1, row0 = (int)blockIdx.x * rpb + w;
     unsigned target = 0;
     double rho = 1.0, rho_old = 0.0;
     int it = 0;
@@ -276,9 +278,14 @@ k_cg(int n, const int64_t *__restrict__ rp, const int32_t *__restrict__ col, con
         }
         __syncthreads();
         const float beta = s_scalar;
-        for (int64_t first = (int64_t)blockIdx.x * rpb; first < n; first += (int64_t)kRounds * rpb * gridDim.x) {
-            for (int u = 0; u < kRounds; u++) {
-                const int64_t r = first + (int64_t)u * rpb * gridDim.x + w;
+        // rounds in alternating order: an iteration begins with the rows that the last one left in the caches.
+        // Two rounds unrolled: one was 15 % slower on 18 M entries, four 7 %
+        for (int t0 = 0; t0 < rounds; t0 += kRounds) {
+            const int nu = min(kRounds, rounds - t0);
+#pragma unroll 2
+            for (int u = 0; u < nu; u++) {
+                const int t = it & 1 ? rounds - 1 - t0 - u : t0 + u;
+                const int64_t r = (int64_t)t * stride + row0;
                 if (w >= rpb || r >= n) {
                     if (lane == 0) s_qp[u][w] = make_float2(0.0f, 0.0f);
                     continue;
@@ -311,7 +318,7 @@ k_cg(int n, const int64_t *__restrict__ rp, const int32_t *__restrict__ col, con
                 }
             }
             __syncthreads();
-            if (w < kRounds && first + (int64_t)w * rpb * gridDim.x < n) {
+            if (w < nu) {
                 const float2 x = lane < kCgWarps ? s_qp[w][lane] : make_float2(0.0f, 0.0f);
                 double pq = (double)x.x * (double)x.y;
                 for (int off = 16; off; off >>= 1) pq += __shfl_xor_sync(0xffffffffu, pq, off);

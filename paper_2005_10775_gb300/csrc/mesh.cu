@@ -84,8 +84,10 @@ __global__ void k_copy1(int64_t *dst, const int64_t *src) { *dst = *src; }
 // next tile's loads issued before the current tile's sums.  An assembly scans four arrays of K or J
 // counts; as three to five launches each they were a sixth of a small assembly's kernel time (K = 2048:
 // 46 of 287 us, 15 us here; the assembly from host to host 515 -> 474 us).
+// Two tiles at most: one block takes 5.1 us for 2,048 counts, 10.2 for 8,192, 16.4 for 16,641, 28.7 for
+// 32,768 and 78.8 for 96,800, the four launches of many blocks 14.4 to 16.6 us for all of them.
 constexpr int kScanOneItems = 8;
-constexpr int kScanOneMax = 1 << 17;   // larger arrays are scanned by many blocks
+constexpr int kScanOneMax = 1 << 14;
 
 __global__ void __launch_bounds__(1024) k_scan_one(const int64_t *in, int64_t *out, int n)
 {

@@ -691,8 +691,10 @@ __device__ __forceinline__ void scatter_rank(int K, int J, int64_t E, const int3
     if (split) {
         // the constant kernel's interior pairs: M_ab / c = |T_a| |T_b| / 9 in all nine entries, so each
         // node of T_b receives one value for the three rows together, summed in scom at the node's
-        // place in row 0 (an interior pair puts T_b's nodes into all three rows)
-        const double ka = area[a] * (1.0 / 9.0);
+        // place in row 0 (an interior pair puts T_b's nodes into all three rows).  FP32 blocks: on a grid
+        // eight times finer than the rows' (a ninth of an area product a pair, where the rows' bound has at
+        // least 1.25): on a uniform mesh every pair rounds the same way
+        const double ka = area[a] * (1.0 / 9.0) * (kFx ? 8.0 * (double)sc : 1.0);
         int64_t e = ptr[a] + lane;
         int b = e < e_int ? idx[e] : 0, bn = e + 32 < e_int ? idx[e + 32] : 0;
         double ab = area[b];
@@ -704,7 +706,7 @@ __device__ __forceinline__ void scatter_rank(int K, int J, int64_t E, const int3
             const int m0 = tri[3 * bn], m1 = tri[3 * bn + 1], m2 = tri[3 * bn + 2];
             const double m = ka * ab;
             Acc v;
-            if constexpr (kFx) v = -__float2int_rn((float)m * sc);
+            if constexpr (kFx) v = -__double2int_rn(m);
             else v = -m;
             const int nd[3] = {n0 - lo, n1 - lo, n2 - lo};
             for (int k = 0; k < 3; k++) {
@@ -769,22 +771,23 @@ __device__ __forceinline__ void scatter_rank(int K, int J, int64_t E, const int3
         for (int p = 0; p < 9; p++) v[p] = vn[p];
     }
     __syncwarp();
-    const double inv = (double)pow2f(-shift) * kc;
+    const double inv = 0.125 * (double)pow2f(-shift) * kc;
     for (int i = 0; i < 3; i++)
         for (int k = lane; k < len[i]; k += 32) {
-            Acc x = sacc[i * cap + k];
+            const Acc x = sacc[i * cap + k];
+            Acc y = (Acc)0;   // the interior pairs'
             if (split) {
                 const int c = i == 0 ? 0 : col[r0[i] + k] - lo;
                 const RankWord w = wd[3 * (c >> 5)];
-                if (i == 0) x += scom[k];
-                else if ((w.bits >> (c & 31)) & 1u) x += scom[rank_of(w, c & 31)];
+                if (i == 0) y = scom[k];
+                else if ((w.bits >> (c & 31)) & 1u) y = scom[rank_of(w, c & 31)];
             }
-            if (x == (Acc)0) continue;
             if constexpr (kFx) {
-                if (x > (1 << 30) || x < -(1 << 30)) atomicOr(err, 256);
-                atomicAdd(&W[r0[i] + k], (double)x * inv);
+                if (x > (1 << 30) || x < -(1 << 30) || y < -(1 << 30)) atomicOr(err, 256);
+                const long long t = 8ll * x + y;   // one conversion to FP64
+                if (t != 0) atomicAdd(&W[r0[i] + k], (double)t * inv);
             } else {
-                atomicAdd(&W[r0[i] + k], (double)x * kc);
+                if (x + y != (Acc)0) atomicAdd(&W[r0[i] + k], (double)(x + y) * kc);
             }
         }
 }

@@ -859,14 +859,19 @@ __device__ __noinline__ bool exact_disc_item(const NumArgs &A, int b, float area
                 narc++;
                 if constexpr (BALL == NL_BALL_APPROXCAPS) {
                     // dyadic arc points, each by bisection from the ends
-                    const T rad = f32 ? (T)g.deltaf : (T)g.delta;
                     const int m = 1 << g.cap_level;
                     for (int j = 1; j < m; j++) {
                         T ax = a.x, ay = a.y, bx = c.x, by = c.y, mx = 0, my = 0;
                         for (int lo = 0, hi = m; hi - lo > 1;) {
                             mx = ax + bx;
                             my = ay + by;
-                            const T sc = rad / sqrt(mx * mx + my * my);
+                            T sc;
+                            if constexpr (f32) {   // both parts of delta in one rounding (disc_cross)
+                                const float rs = 1.f / sqrtf(mx * mx + my * my);
+                                sc = fmaf(g.deltaf, rs, g.deltalo * rs);
+                            } else {
+                                sc = g.delta / sqrt(mx * mx + my * my);
+                            }
                             mx *= sc;
                             my *= sc;
                             const int md = (lo + hi) >> 1;

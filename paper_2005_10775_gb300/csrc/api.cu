@@ -3,6 +3,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <mutex>
 #include <new>
 #include <string>
 
@@ -524,6 +525,81 @@ void nl_plan_free(nl_plan *P, cudaStream_t s)
     nl_free(P->nearq, s); nl_free(P->near_n, s); nl_free(P->otab, s);
 }
 
+// What the process's default pool keeps of the memory that is freed to it, instead of handing it back to the driver
+// at every synchronisation (later assemblies then allocate without driver calls): 8 GiB, and while a context
+// assembles larger problems as much as they use.  A program that assembles again while the last matrix lives
+// needs both (K = 96,800: about 5 GB each with their pair blocks; with 8 GiB kept every assembly mapped memory
+// again, 24.6 against 16.4 ms).  What is in use when an assembly ends says how much, so the amount falls again
+// with smaller problems, and to 8 GiB with the last context.  (The pool's high-water mark would say it too, but
+// setting it back at every call made such an assembly 0.25 ms longer.)  A threshold that the program itself sets is left as it is.
+namespace {
+constexpr uint64_t kPoolKeep = uint64_t(8) << 30;
+
+struct PoolState {
+    std::mutex lock;
+    int users = 0;           // contexts on the device
+    uint64_t base = 0, set = 0;
+};
+PoolState pool_state[64];
+
+PoolState *pool_of(int device, cudaMemPool_t *pool)
+{
+    if (device < 0 || device >= 64 || cudaDeviceGetDefaultMemPool(pool, device) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return &pool_state[device];
+}
+
+// threshold to `want`, if it is still the one set last
+void pool_set(PoolState *p, cudaMemPool_t pool, uint64_t want)
+{
+    uint64_t thr = 0;
+    if (want != p->set && cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr) == cudaSuccess &&
+        thr == p->set && cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &want) == cudaSuccess)
+        p->set = want;
+}
+
+void pool_open(int device)
+{
+    cudaMemPool_t pool;
+    PoolState *p = pool_of(device, &pool);
+    if (!p) return;
+    std::lock_guard<std::mutex> hold(p->lock);
+    uint64_t thr = 0;
+    if (p->users++ == 0 && cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr) == cudaSuccess) {
+        p->set = thr;
+        p->base = thr > kPoolKeep ? thr : kPoolKeep;
+        pool_set(p, pool, p->base);
+    }
+}
+
+void pool_close(int device)
+{
+    cudaMemPool_t pool;
+    PoolState *p = pool_of(device, &pool);
+    if (!p) return;
+    std::lock_guard<std::mutex> hold(p->lock);
+    if (--p->users == 0) pool_set(p, pool, p->base);
+}
+}  // namespace
+
+void nl_pool_follow(nl_ctx *ctx)
+{
+    cudaMemPool_t pool;
+    PoolState *p = pool_of(ctx->device, &pool);
+    if (!p) return;
+    std::lock_guard<std::mutex> hold(p->lock);
+    uint64_t used = 0;
+    if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess) {
+        // half as much again for the temporaries of the next assembly and the pieces between; down only when
+        // a quarter would do (a program frees its last matrix now before, now after the next call)
+        const uint64_t want = used + used / 2;
+        if (want > p->set || want < p->set / 4) pool_set(p, pool, want > p->base ? want : p->base);
+    }
+    cudaGetLastError();
+}
+
 nl_status nl_host_slots(nl_ctx *ctx, int n, nl_host_slot **out)
 {
     if (n < 1) n = 1;
@@ -583,20 +659,8 @@ nl_status nl_create(nl_ctx **out, int device, void *stream)
     for (int k = 0; e == cudaSuccess && k <= nl_ctx::kSideStreams; k++)
         e = cudaEventCreateWithFlags(&ctx->side_ev[k], cudaEventDisableTiming);
     if (e == cudaSuccess) {
-        // keep freed pool memory cached by this process (up to 16 GiB, of 277) instead of handing it
-        // back to the driver at every synchronisation: later assemblies allocate without
-        // driver calls.  Two matrices of the largest workloads (K = 96,800: about 5 GB each with
-        // their pair blocks) fit; with 8 GiB every assembly there mapped memory again (24.6 against
-        // 17.5 ms).  This is a property of the process's pool, not of the device.
-        cudaMemPool_t pool;
-        if (cudaDeviceGetDefaultMemPool(&pool, device) == cudaSuccess) {
-            uint64_t thr = 0;
-            if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr) == cudaSuccess &&
-                thr < (uint64_t(16) << 30)) {
-                thr = uint64_t(16) << 30;
-                cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
-            }
-        }
+        pool_open(device);
+        ctx->pooled = true;
         cudaGetLastError();
     }
     if (e != cudaSuccess) {
@@ -623,6 +687,7 @@ void nl_destroy(nl_ctx *ctx)
         if (ctx->side_ev[k]) cudaEventDestroy(ctx->side_ev[k]);
     if (ctx->slots) cudaFreeHost(ctx->slots);
     nl_tune_cache_free(ctx->tune);
+    if (ctx->pooled) pool_close(ctx->device);
     if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
 }
@@ -665,6 +730,7 @@ nl_status nl_assemble(nl_ctx *ctx, const nl_mesh *mesh, const nl_config *cfg, nl
     if ((e = cudaEventRecord(ctx->ev[4], ctx->stream)) != cudaSuccess) goto cuda_fail;
     nl_prep_delete(T, ctx->stream);
     nl_pat_delete(Q, ctx->stream);
+    nl_pool_follow(ctx);
     return NL_OK;
 cuda_fail:
     s = nl_cuda_fail(ctx, e, "stream operation");

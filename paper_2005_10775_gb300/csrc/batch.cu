@@ -620,6 +620,7 @@ nl_status assemble_pipelined(nl_ctx *ctx, int n, const nl_mesh *meshes, const nl
     s = finish(NL_OK);
     if (cudaEventRecord(ctx->ev[4], st) != cudaSuccess) return nl_fail(ctx, NL_ECUDA, "cudaEventRecord");
     ctx->last_fp64_items = fp64_items;
+    nl_pool_follow(ctx);
     return s;
 }
 
@@ -903,6 +904,7 @@ nl_status nl_batch_create(nl_ctx *ctx, int32_t n, const nl_mesh *meshes, const n
     T.assign(n, nullptr);
     Q.assign(n, nullptr);
     if ((s = phase_check(ctx, b, "release of the temporaries")) != NL_OK) return fail(s);
+    nl_pool_follow(ctx);
     *batch = b;
     return NL_OK;
 }

@@ -73,6 +73,7 @@ struct nl_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
+    bool pooled = false;   // counted among the device pool's users (api.cu)
     std::string err;
     cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     double last_ms[4] = {0, 0, 0, 0};
@@ -91,6 +92,8 @@ struct nl_ctx {
 // the context's side streams and their events (created on first use)
 nl_status nl_side_streams(nl_ctx *ctx);
 
+// at the end of an assembly: the pool keeps as much as the assembly used (api.cu)
+void nl_pool_follow(nl_ctx *ctx);
 // pinned host slots for n problems (grown on demand; invalidates earlier slot pointers)
 nl_status nl_host_slots(nl_ctx *ctx, int n, nl_host_slot **out);
 

@@ -667,13 +667,15 @@ nl_status nl_prepare_b(nl_ctx *ctx, nl_plan *P, nl_prep *T, nl_host_slot *h)
     double R = (cfg->delta + 2.0 * hst.rmax) * (1.0 + 2e-5);
     double Lx = hst.xmax - hst.xmin, Ly = hst.ymax - hst.ymin, L = fmax(fmax(Lx, Ly), 1e-300);
     double cs = fmin(R, L / sqrt(fmax(K / 32.0, 1.0)));
+    cs = fmax(cs, L / 8192.0);   // parts of a mesh far from each other: nx ny stays an int
     Grid &g = T->g;
     g.cs = cs;
-    g.m = (int)ceil(R / cs);
     g.x0 = hst.xmin;
     g.y0 = hst.ymin;
     g.nx = (int)floor(Lx / cs) + 1;
     g.ny = (int)floor(Ly / cs) + 1;
+    // cells of reach; a mesh far smaller than the horizon has the whole grid in it (R / cs is no int there)
+    g.m = (int)fmin(ceil(R / cs), (double)(g.nx > g.ny ? g.nx : g.ny));
     const int ncell = g.nx * g.ny;
     T->ncell = ncell;
     nl_status s;

@@ -440,12 +440,15 @@ __device__ __forceinline__ int exp2_floor(float x)
 
 // Fixed-point shift of the rows of T_a: the sum a column of node j receives is below
 // 2^(ea + 1) 2^(ej + 1) (ea: exponent of |T_a| sum_q |w_q|, ej the largest node exponent of
-// k_node_exp), so every sum scaled by 2^s stays below 2^30.
+// k_node_exp), so every sum scaled by 2^s stays below 2^30.  Above 126 (every triangle of the mesh below
+// 4e-8 horizons, and so every pair interior, or the candidate lists would overflow) the scale 2^s is
+// beyond FP32: the interior pairs are scaled in FP64, anything else is an error (bit 256).
 __device__ __forceinline__ int fx_row_shift(int ea, int ej)
 {
     const int s = 28 - ea - ej;
-    return s < -126 ? -126 : (s > 126 ? 126 : s);
+    return s < -126 ? -126 : s;
 }
+__device__ __forceinline__ double pow2d(int s) { return __hiloint2double((s + 1023) << 20, 0); }
 
 // One pair (a, b) of the scatter: flag f, its M_ab block v, added to the three rows of T_a's
 // nodes (shared sums, fixed point for FP32 blocks, when cached; else FP64 atomics on W).
@@ -551,11 +554,12 @@ __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int
                 }
                 atomicAnd(&spk[sl], ~((kPosAbsent ^ (unsigned)k) << (10 * i)));
             }
-        cached = !__any_sync(0xffffffffu, full);   // a full table: this triangle searches in global memory
         if constexpr (kFx) shift = fx_row_shift(exp2_floor((float)(area[a] * (double)ws)), *fxe - 128);
+        // a full table: this triangle searches in global memory
+        cached = !__any_sync(0xffffffffu, full) && shift <= 126;
         __syncwarp();
     }
-    const float sc = pow2f(shift);
+    const float sc = pow2f(min(shift, 126));
     const int64_t e_int = split ? split[a] : ptr[a];
     if (split) {
         // the constant kernel's interior pairs: M_ab / c = |T_a| |T_b| / 9 in all nine entries
@@ -600,7 +604,7 @@ __device__ __forceinline__ void scatter_outer(int K, int J, int64_t E, const int
     }
     __syncwarp();
     if (cached) {
-        const double inv = (double)pow2f(-shift) * kc;
+        const double inv = pow2d(-shift) * kc;
         for (int i = 0; i < 3; i++)
             for (int k = lane; k < len[i]; k += 32) {
                 const Acc x = sacc[i * cap + k];
@@ -686,7 +690,7 @@ __device__ __forceinline__ void scatter_rank(int K, int J, int64_t E, const int3
         }
     int shift = 0;   // FP32 blocks: fixed-point shift of the shared row sums
     if constexpr (kFx) shift = fx_row_shift(exp2_floor((float)(area[a] * (double)ws)), *fxe - 128);
-    const float sc = pow2f(shift);
+    const float sc = pow2f(min(shift, 126));
     const int64_t e_int = split ? split[a] : ptr[a];
     if (split) {
         // the constant kernel's interior pairs: M_ab / c = |T_a| |T_b| / 9 in all nine entries, so each
@@ -694,7 +698,7 @@ __device__ __forceinline__ void scatter_rank(int K, int J, int64_t E, const int3
         // place in row 0 (an interior pair puts T_b's nodes into all three rows).  FP32 blocks: on a grid
         // eight times finer than the rows' (a ninth of an area product a pair, where the rows' bound has at
         // least 1.25): on a uniform mesh every pair rounds the same way
-        const double ka = area[a] * (1.0 / 9.0) * (kFx ? 8.0 * (double)sc : 1.0);
+        const double ka = area[a] * (1.0 / 9.0) * (kFx ? pow2d(shift + 3) : 1.0);
         int64_t e = ptr[a] + lane;
         int b = e < e_int ? idx[e] : 0, bn = e + 32 < e_int ? idx[e + 32] : 0;
         double ab = area[b];
@@ -723,6 +727,7 @@ __device__ __forceinline__ void scatter_rank(int K, int J, int64_t E, const int3
     // the next pair's loads are issued before this pair's lookups and adds: the DRAM latency
     // of one iteration overlaps the shared-memory work of the previous one
     const int64_t e_end = ptr[a + 1];
+    if (shift > 126 && e_int < e_end && lane == 0) atomicOr(err, 256);
     int64_t e = e_int + lane;
     uint8_t f = 0;
     int b = 0;
@@ -771,7 +776,7 @@ __device__ __forceinline__ void scatter_rank(int K, int J, int64_t E, const int3
         for (int p = 0; p < 9; p++) v[p] = vn[p];
     }
     __syncwarp();
-    const double inv = 0.125 * (double)pow2f(-shift) * kc;
+    const double inv = pow2d(-shift - 3) * kc;
     for (int i = 0; i < 3; i++)
         for (int k = lane; k < len[i]; k += 32) {
             const Acc x = sacc[i * cap + k];

@@ -352,14 +352,16 @@ __device__ __forceinline__ void whole_sums(const NumArgs &A, const D2 V[3], T ar
 // Inner sums over the region R.  Only the singular kernel c / |x - y| comes here, yet the kernel's type is read at
 // run time: with the other one's branches gone the lanes of the FP64 boundary kernel met again less often (6.2 of
 // 32 active instead of 7.4, 23 % more FP64 instructions: 33 -> 40 ms for nocaps on 40 x 40 cells).
+// True for a near region, whose caps (exactcaps) are the caller's to add.
 template <typename T>
-__device__ __forceinline__ void inner_sums(const NumArgs &A, const nlg::Region &R, const D2 V[3], double area_b,
+__device__ __forceinline__ bool inner_sums(const NumArgs &A, const nlg::Region &R, const D2 V[3], double area_b,
                                            D2 x, Sums<T> &S, int64_t &nqp)
 {
     sums_zero(S);
     const bool inv = (A.kernel == NL_KERNEL_INV_DIST);
     const RuleTab &ri = A.inner;
-    if (inv && R.nv >= 3 && nlg::is_near(R, V, x)) {
+    const bool near = inv && R.nv >= 3 && nlg::is_near(R, V, x);
+    if (near) {
         BaryMap bm = bary_map(V);
         Sums<double> Sd;
         sums_zero(Sd);
@@ -440,6 +442,7 @@ __device__ __forceinline__ void inner_sums(const NumArgs &A, const nlg::Region &
             nqp++;
         }
     }
+    return near;
 }
 
 // inner sums over a fanned polygon in FP32 coordinates relative to x, held in the lane's columns
@@ -1171,7 +1174,20 @@ __device__ __noinline__ bool exact_item_fp64(const NumArgs &A, const CandData &c
         const nlg::F2 e1 = {c.e1x, c.e1y}, e2 = {c.e2x, c.e2y};
         near_whole_f32(A, dl, c.b, x, e1, e2, c.binv, *(Sums<float> *)&S, nq);
     } else {
-        inner_sums<T>(A, R, Vb, c64.area, x, S, nq);
+        const bool near = inner_sums<T>(A, R, Vb, c64.area, x, S, nq);
+        // a near region's caps: one point each, as a far one's
+        if constexpr (BALL == NL_BALL_EXACTCAPS) {
+            if (near && R.ncap > 0) {
+                const BaryMap bm = bary_map(Vb);
+                for (int k = 0; k < R.ncap; k++) {
+                    double ph[3];
+                    bary_of(bm, R.cc[k].x, R.cc[k].y, ph);
+                    const double dx = R.cc[k].x - x.x, dy = R.cc[k].y - x.y;
+                    sums_add<T>(S, (T)(R.cw[k] * (A.kc / sqrt(dx * dx + dy * dy))), (T)ph[0], (T)ph[1], (T)ph[2]);
+                    nq++;
+                }
+            }
+        }
     }
     return true;
 }

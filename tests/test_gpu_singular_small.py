@@ -1,6 +1,6 @@
 """The singular kernel with a horizon below the triangles' size, where many triangles outside the disc pass the
-tangent's empty test and an edge-distance test takes them out: records and pattern bit-exact with the FP64
-oracle, values within the paths' stated accuracies."""
+tangent's empty test and an edge-distance test takes them out, and regions in the near field have caps: records
+and pattern bit-exact with the FP64 oracle, values within the paths' stated accuracies."""
 import numpy as np
 import pytest
 
@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 TOL = {"fp64": 1e-12, "fp32c": 1e-6}
 
 
-@pytest.mark.parametrize("ball", ["ngon", "nocaps", "approxcaps"])
+@pytest.mark.parametrize("ball", ["ngon", "nocaps", "approxcaps", "exactcaps"])
 @pytest.mark.parametrize("prec", ["fp64", "fp32c"])
 def test_singular_small_horizon(ball, prec):
     from paper_2005_10775_gb300 import nlfem as nl

@@ -76,8 +76,10 @@ typedef enum {
 } nl_kernel;
 
 typedef enum {
-    NL_PREC_FP64 = 0,         /* geometry and quadrature in FP64 */
-    NL_PREC_FP32_COMP = 1     /* geometry in FP64; quadrature in FP32 with FP64 (compensated) long sums */
+    /* Which vertices lie in the ball and which edges cross it is decided in FP32 where FP32 is certain and in FP64
+       elsewhere, so that it is the FP64 geometry's decision in both. */
+    NL_PREC_FP64 = 0,         /* regions' coordinates and quadrature in FP64 */
+    NL_PREC_FP32_COMP = 1     /* regions' coordinates and quadrature in FP32 with FP64 (compensated) long sums */
 } nl_prec;
 
 typedef struct nl_ctx nl_ctx;
@@ -140,10 +142,12 @@ const char *nl_last_error(nl_ctx *ctx);
    pairs with a non-empty region) and the numeric scatter.  *out receives a new
    library-owned n x n CSR (n = mesh->nv).  Synchronises the stream three times (to
    size the candidate-search grid, the candidate lists and the pattern); device memory
-   comes from the device's stream-ordered pool on the context's stream.  The singular kernel's
+   comes from the device's stream-ordered pool on the context's stream, which keeps 8 GiB of freed
+   memory for the process, or as much as the latest assemblies left in use.  The singular kernel's
    interior candidates' quadrature runs on a second stream of the context, concurrently with the
-   boundary candidates'; the constant kernel takes both in one launch (ordered after the context's stream's earlier work, which waits
-   for it before anything that follows).  The pattern's
+   boundary candidates' (ordered after the context's stream's earlier work, which waits
+   for it before anything that follows); the constant kernel takes both in one launch.  The mesh may be
+   in any unit of length.  The pattern's
    first row count uses a hash set of 2^b slots, b from the mean candidate list;
    NL_ROW_SET_BITS=b (6..13) in the environment sets it instead (the pattern does not
    depend on it: rows that fill the set are counted again in a full one). */

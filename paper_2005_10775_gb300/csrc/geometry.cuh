@@ -543,8 +543,8 @@ struct ClipBuf {
     float x[2][kClipCap][32], y[2][kClipCap][32], e[2][kClipCap][32];
 };
 
-// UNROLL: the vertex loop unrolled over the capacity (constant kernel, when it integrated its fans point by
-// point: numeric phase 4.82 -> 4.69 ms; the singular kernel's larger boundary kernel lost more to instruction fetch)
+// UNROLL: the vertex loop unrolled over the capacity (the constant kernel's irregular or large polygons,
+// kBallNgonAny; the singular kernel's larger boundary kernel lost more to instruction fetch)
 template <bool UNROLL = false>
 __device__ __forceinline__ int clip_ngon_f32_sh(const F2 dl[3], float err0, const GeoParams &g, ClipBuf &cb,
                                                 int lane, int *which, bool *cut)

@@ -667,7 +667,8 @@ nl_status nl_prepare_b(nl_ctx *ctx, nl_plan *P, nl_prep *T, nl_host_slot *h)
     double R = (cfg->delta + 2.0 * hst.rmax) * (1.0 + 2e-5);
     double Lx = hst.xmax - hst.xmin, Ly = hst.ymax - hst.ymin, L = fmax(fmax(Lx, Ly), 1e-300);
     double cs = fmin(R, L / sqrt(fmax(K / 32.0, 1.0)));
-    cs = fmax(cs, L / 8192.0);   // parts of a mesh far from each other: nx ny stays an int
+    // parts of a mesh far from each other: nx ny stays an int
+    while ((floor(Lx / cs) + 1.0) * (floor(Ly / cs) + 1.0) > 1073741824.0) cs *= 2.0;
     Grid &g = T->g;
     g.cs = cs;
     g.x0 = hst.xmin;
